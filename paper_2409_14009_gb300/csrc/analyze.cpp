@@ -426,6 +426,11 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
   // takes 256 to cut the number of dependent launches.
   const bool tc_modes = h->opt.precision == CHOL_PREC_TF32 || h->opt.precision == CHOL_PREC_BF16;
   const bool mixed = h->opt.precision != CHOL_PREC_FP64;
+  // binary64 updates on the tensor cores: their operand blocks are 64 columns wide
+  const bool split64 = !mixed && nb == 64;
+  h->split.assign(split64 ? ns : 0, SplitDev{});
+  h->sgt_tasks.clear(); h->sgs_tasks.clear(); h->split_tasks.clear();
+  h->split_slab_rows = h->split_exps = h->split_trows = h->split_texps = 0;
   const int tg = tc_modes ? kTileTC : kTile;
   std::vector<std::vector<int32_t>> by_level(h->nlevels);
   for (int32_t J = 0; J < ns; ++J) by_level[h->level[J]].push_back(J);
@@ -612,6 +617,21 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
         }
         if (pass == 0) st.gemm_next = (int32_t)h->gemm_tasks.size() - st.gemm_b;
       }
+      // the same tiles for the tensor cores, 128 rows high
+      st.sgt_b = (int32_t)h->sgt_tasks.size();
+      for (int pass = 0; split64 && pass < 2; ++pass) {
+        for (int32_t J : large) {
+          const SnodeDev& d = h->snodes[J];
+          if (d.s <= k0) continue;
+          const int32_t kb = std::min(nb, d.s - k0);
+          for (int32_t c0 = k0 + kb; c0 < d.s; c0 += kTile) {
+            if ((pass == 0) != (c0 == k0 + kb)) continue;
+            for (int32_t r0 = c0; r0 < d.len; r0 += 2 * kTile) h->sgt_tasks.push_back({J, k0, r0, c0});
+          }
+        }
+        if (pass == 0) st.sgt_next = (int32_t)h->sgt_tasks.size() - st.sgt_b;
+      }
+      st.sgt_n = (int32_t)h->sgt_tasks.size() - st.sgt_b;
       st.potrf_n = (int32_t)h->potrf_list.size() - st.potrf_b;
       st.trsm_n = (int32_t)h->trsm_tasks.size() - st.trsm_b;
       st.gemm_n = (int32_t)h->gemm_tasks.size() - st.gemm_b;
@@ -632,6 +652,41 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
         for (int32_t r0 = c0; r0 < b; r0 += tg) h->syrk_tasks.push_back({J, 0, r0, c0});
     }
     P.syrk_n = (int32_t)h->syrk_tasks.size() - P.syrk_b;
+    P.sgs_b = (int32_t)h->sgs_tasks.size();
+    P.sgr_b = (int32_t)h->split_tasks.size();
+    if (split64) {
+      int64_t so = 0, se = 0, to = 0, te = 0;
+      for (int32_t J : large) {
+        const SnodeDev& d = h->snodes[J];
+        const int32_t b = d.len - d.s;
+        SplitDev& z = h->split[J];
+        // a 128-row tile starts at a multiple of 64 below the last row
+        z.srows = (b + 63) / 64 * 64 + 64;
+        z.trows = (d.len + 63) / 64 * 64 + 64;
+        z.sblk = (d.s + 31) / 32;
+        if (b > 0) {
+          z.soff = so;
+          z.srow0 = se;
+          so += (int64_t)z.sblk * kSplitSlices * z.srows;
+          se += z.srows;
+          for (int32_t r0 = 0; r0 < b; r0 += 64) h->split_tasks.push_back({J, 0, r0, 0});
+          for (int32_t c0 = 0; c0 < b; c0 += kTile)
+            for (int32_t r0 = c0; r0 < b; r0 += 2 * kTile) h->sgs_tasks.push_back({J, 0, r0, c0});
+        }
+        if (d.s > nb) {
+          z.toff = to;
+          z.trow0 = te;
+          to += 2 * (int64_t)kSplitSlices * z.trows;
+          te += z.trows;
+        }
+      }
+      h->split_slab_rows = std::max(h->split_slab_rows, so);
+      h->split_exps = std::max(h->split_exps, se);
+      h->split_trows = std::max(h->split_trows, to);
+      h->split_texps = std::max(h->split_texps, te);
+    }
+    P.sgs_n = (int32_t)h->sgs_tasks.size() - P.sgs_b;
+    P.sgr_n = (int32_t)h->split_tasks.size() - P.sgr_b;
     // triangular solves over every supernode of the level: the diagonal
     // triangles as 64-row blocks in dependency order (one cooperative launch per
     // level and direction), then one panel product per level for the

@@ -26,6 +26,16 @@ struct DeviceState {
   AsmTask* asm_tasks = nullptr;
   AsmSeg* asm_segs = nullptr;
   TriItemHost* tri = nullptr;   // solve: diagonal-triangle items
+  int sg_ready = 0;             // binary64 updates on the tensor cores: 1 = in use, -1 = not
+  unsigned char* sg_slab = nullptr;              // slices of a level's off-diagonal rows
+  int32_t* sg_exps = nullptr;                    // ... and their row exponents
+  unsigned char* sgt_slab[2] = {nullptr, nullptr};   // slices of a 64-column block, by step parity
+  int32_t* sgt_exps[2] = {nullptr, nullptr};
+  SplitDev* sg_dev = nullptr;
+  TileTask* sg_split = nullptr;
+  TileTask* sg_syrk = nullptr;
+  TileTask* sg_trail = nullptr;
+  int32_t* sg_err = nullptr;    // a tile gave up waiting
   int4* rlb_pairs = nullptr;    // RLB: (K, c0, c1, -) of every (J, K) pair, J-major
   int32_t* rlb_pbeg = nullptr;  // RLB: first pair of every supernode
   double* zrr_ws = nullptr;     // adjoint: Z_RR workspace when there is no update workspace (RLB)
@@ -191,3 +201,11 @@ inline int chol_factored_here(const chol_handle* h) {
   return cur == h->dev->device ? CHOL_OK : CHOL_ESTATE;
 }
 int chol_dalloc(chol_handle* h, void** p, size_t bytes);
+
+// binary64 updates on the tensor cores (split_gemm.cu)
+int chol_sg_ensure(chol_handle* h);
+void chol_sg_release(chol_handle* h);
+void chol_sg_split_block(chol_handle* h, const StepRange& s, int buf, cudaStream_t st);
+void chol_sg_trailing(chol_handle* h, const TileTask* tasks, int n, int grid, int buf, cudaStream_t st);
+void chol_sg_syrk(chol_handle* h, const LevelPlan& P, cudaStream_t st);
+int chol_sg_status(chol_handle* h);

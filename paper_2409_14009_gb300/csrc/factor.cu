@@ -658,6 +658,16 @@ int chol_dalloc(chol_handle* h, void** p, size_t bytes) {
   if (bytes == 0) return CHOL_OK;
   if (h->opt.device_mem_cap > 0 && D->bytes + (int64_t)bytes > h->opt.device_mem_cap) return CHOL_ENOMEM;
   cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && D->sg_ready == 1) {
+    // the tensor-core updates' workspaces are the part that can be done without
+    cudaGetLastError();
+    if (D->graph_exec) {   // captured with them
+      cudaGraphExecDestroy(D->graph_exec);
+      D->graph_exec = nullptr;
+    }
+    chol_sg_release(h);
+    e = cudaMalloc(p, bytes);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
@@ -681,7 +691,8 @@ void chol_device_free(chol_handle* h) {
                   D->ssmall, D->Zp, D->Tw, D->Ww, D->Uh, D->a_col, D->a_row, D->adj_xb, D->perm, D->status, D->part, D->scalar_dev, D->Y, D->W,
                   D->mx_diagpos, D->mx_aij, D->mx_d, D->mx_fallbacks, D->csr_ptr, D->csr_col, D->csr_src,
                   D->csr_val, D->Lbf, D->tmaps, D->tc_err, D->R, D->Z, D->Pv, D->Q, D->red, D->Y32, D->W32,
-                  D->rhs_scale, D->host_vals, D->host_rhs, D->panel, D->pflags, D->dinv, D->split_part, D->split_cnt, D->hand32};
+                  D->rhs_scale, D->host_vals, D->host_rhs, D->panel, D->pflags, D->dinv, D->split_part, D->split_cnt, D->hand32, D->sg_slab, D->sg_exps, D->sgt_slab[0], D->sgt_slab[1],
+                  D->sgt_exps[0], D->sgt_exps[1], D->sg_dev, D->sg_split, D->sg_syrk, D->sg_trail, D->sg_err};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (D->status_host) cudaFreeHost(D->status_host);
@@ -842,6 +853,7 @@ int enqueue_factor_fp64(chol_handle* h, const double* values, cudaStream_t st) {
     CHOL_CUDA_TRY(cudaStreamWaitEvent(D->hstream, D->lev[2], 0));
     st = D->hstream;
   }
+  const bool sg = D->sg_ready == 1;   // updates on the tensor cores
   bool inv_pending = false;
   for (const LevelPlan& P : h->levels) {
     NvtxRange nvtx_level("level", (long long)(&P - h->levels.data()));
@@ -874,7 +886,13 @@ int enqueue_factor_fp64(chol_handle* h, const double* values, cudaStream_t st) {
         KScope ks(h, CHOL_K_TRSM, st, s.trsm_flops, 16.0 * kTrsmRows * nb * s.trsm_n);
         k_trsm<<<s.trsm_n, kTrsmThreads, 0, st>>>(D->sn, D->trsm + s.trsm_b, nb, D->L);
       }
-      const int nrest = s.gemm_n - s.gemm_next;
+      const int gemm_n = sg ? s.sgt_n : s.gemm_n, gemm_next = sg ? s.sgt_next : s.gemm_next;
+      const int nrest = gemm_n - gemm_next;
+      const int buf = (int)(k & 1);   // step k + 2 reuses step k's slices: its rest has joined by then
+      if (sg && gemm_n > 0) {
+        KScope ks(h, CHOL_K_GEMM, st, 0.0, 22.0 * 128.0 * nb * gemm_next);
+        chol_sg_split_block(h, s, buf, st);
+      }
       if (nrest > 0) {
         CHOL_CUDA_TRY(cudaEventRecord(D->lev[0], st));   // step k's panel is final
         CHOL_CUDA_TRY(cudaStreamWaitEvent(D->lstream, D->lev[0], 0));
@@ -883,16 +901,19 @@ int enqueue_factor_fp64(chol_handle* h, const double* values, cudaStream_t st) {
         CHOL_CUDA_TRY(cudaStreamWaitEvent(st, D->lev[1], 0));   // step k-1's rest
         rest_pending = false;
       }
-      if (s.gemm_n > 0) {
-        const double frac = (double)s.gemm_next / s.gemm_n;
-        if (s.gemm_next > 0) {
-          KScope ks(h, CHOL_K_GEMM, st, s.gemm_flops * frac, 16.0 * kTile * kTile * s.gemm_next);
-          k_gemm_trailing<<<s.gemm_next, kGemmThreads, 0, st>>>(D->sn, D->gemm + s.gemm_b, nb, D->L);
+      if (gemm_n > 0) {
+        const double frac = (double)gemm_next / gemm_n;
+        const double tile_bytes = 16.0 * kTile * kTile * (sg ? 2 : 1);
+        if (gemm_next > 0) {
+          KScope ks(h, CHOL_K_GEMM, st, s.gemm_flops * frac, tile_bytes * gemm_next);
+          if (sg) chol_sg_trailing(h, D->sg_trail + s.sgt_b, gemm_next, D->sms, buf, st);
+          else k_gemm_trailing<<<gemm_next, kGemmThreads, 0, st>>>(D->sn, D->gemm + s.gemm_b, nb, D->L);
         }
         if (nrest > 0) {
-          KScope ks(h, CHOL_K_GEMM, D->lstream, s.gemm_flops * (1.0 - frac), 16.0 * kTile * kTile * nrest);
-          k_gemm_trailing<<<nrest, kGemmThreads, 0, D->lstream>>>(D->sn, D->gemm + s.gemm_b + s.gemm_next, nb,
-                                                                  D->L);
+          KScope ks(h, CHOL_K_GEMM, D->lstream, s.gemm_flops * (1.0 - frac), tile_bytes * nrest);
+          if (sg) chol_sg_trailing(h, D->sg_trail + s.sgt_b + gemm_next, nrest, INT_MAX, buf, D->lstream);
+          else
+            k_gemm_trailing<<<nrest, kGemmThreads, 0, D->lstream>>>(D->sn, D->gemm + s.gemm_b + gemm_next, nb, D->L);
           CHOL_CUDA_TRY(cudaEventRecord(D->lev[1], D->lstream));
           rest_pending = true;
         }
@@ -909,7 +930,10 @@ int enqueue_factor_fp64(chol_handle* h, const double* values, cudaStream_t st) {
     }
     if (P.syrk_n > 0) {
       KScope ks(h, CHOL_K_SYRK, st, P.syrk_flops, 8.0 * kTile * kTile * P.syrk_n);
-      if (rlb)
+      if (sg) {
+        ks.launches(2);
+        chol_sg_syrk(h, P, st);
+      } else if (rlb)
         k_syrk_rlb<<<P.syrk_n, kGemmThreads, 0, st>>>(D->sn, D->syrk + P.syrk_b, D->rlb_pairs, D->rlb_pbeg, D->rows,
                                                        D->L);
       else
@@ -1009,6 +1033,7 @@ extern "C" int chol_factor(chol_handle* h, const double* values, void* stream) {
   h->factored = false;
   h->selinv_valid = false;
   if (h->opt.precision != CHOL_PREC_FP64 && (rc = chol_mixed_ensure(h))) return rc;
+  if (h->opt.precision == CHOL_PREC_FP64 && (rc = chol_sg_ensure(h))) return rc;
   h->bounds_code = 0;
 #ifdef CHOL_BOUNDS_CHECK
   if (bc_begin(h) || chol_bc_begin_mixed(h)) return CHOL_ECUDA;
@@ -1079,6 +1104,8 @@ int chol_finish_factor(chol_handle* h, cudaStream_t st) {
   CHOL_CUDA_TRY(cudaMemcpyAsync(D->status_host, D->status, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   if (h->opt.precision != CHOL_PREC_FP64)
     CHOL_CUDA_TRY(cudaMemcpyAsync(&D->status_host[1], D->mx_fallbacks, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+  else if (D->sg_ready == 1)
+    CHOL_CUDA_TRY(cudaMemcpyAsync(&D->status_host[3], D->sg_err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   CHOL_CUDA_TRY(cudaStreamSynchronize(st));
   if (h->opt.precision != CHOL_PREC_FP64) {
     h->fp64_fallbacks = D->status_host[1];
@@ -1099,6 +1126,8 @@ int chol_finish_factor(chol_handle* h, cudaStream_t st) {
   if (h->opt.precision != CHOL_PREC_FP64) {
     const int rc = chol_tc_status(h);
     if (rc) return rc;
+  } else if (const int rc = chol_sg_status(h)) {
+    return rc;
   }
   {
     const int rc = chol_solve_status(h);

@@ -36,6 +36,17 @@ struct SnodeDev {
   int32_t ld;    // leading dimension of the panel
 };
 
+// Binary64 updates on the tensor cores (split_gemm.cuh): where the slices of a
+// supernode's rows lie, in units of 64-byte slice rows, and its row exponents.
+// s*: the off-diagonal rows over all columns (SYRK operands, per level);
+// t*: the panel's rows over the current 64-column block (trailing update).
+struct SplitDev {
+  int64_t soff, toff;    // first slice row
+  int64_t srow0, trow0;  // first exponent
+  int32_t srows, trows;  // rows per slice (a multiple of 64, at least 64 past the last row's tile)
+  int32_t sblk, pad;     // 32-column blocks of the SYRK operand
+};
+
 // Blocked large-supernode task: supernode J, column step k0, tile origin (r0, c0).
 struct TileTask {
   int32_t J, k0, r0, c0;
@@ -74,6 +85,7 @@ struct AsmSeg {
 struct StepRange {
   int32_t potrf_b, potrf_n, trsm_b, trsm_n, gemm_b, gemm_n, ogemm_b, ogemm_n, ok0, okb;
   int32_t gemm_next, ogemm_next;
+  int32_t sgt_b, sgt_n, sgt_next;   // binary64 on the tensor cores: 128 x 64 trailing tiles (in sgt_tasks), next column first
   int32_t panel_b, panel_n, panel_ticket, join_rest;
   double potrf_flops, trsm_flops, gemm_flops, ogemm_flops, panel_flops;
 };
@@ -102,6 +114,8 @@ struct LevelPlan {
   int32_t small_max_panel;    // largest len*s among them (shared memory sizing)
   std::vector<StepRange> steps;
   int32_t syrk_b, syrk_n;     // U tiles (in syrk_tasks)
+  int32_t sgs_b, sgs_n;       // binary64 on the tensor cores: U tiles of 128 x 64 (in sgs_tasks)
+  int32_t sgr_b, sgr_n;       // ... and the 64-row tasks that split their operands (in split_tasks)
   int32_t asm_b, asm_n;       // assembly tasks, one CTA each
   int32_t asmw_n;             // then (from asm_b + asm_n) small tasks, one warp each
   int32_t tri_b, tri_n;       // diagonal-triangle solve items (in tri_items), dependency order
@@ -166,6 +180,11 @@ struct chol_handle {
   // schedule
   std::vector<LevelPlan> levels;
   std::vector<int32_t> level_snodes, small_list, potrf_list;
+  // binary64 updates on the tensor cores (block_cols = 64 only): slice layout per
+  // supernode, tile and split tasks, workspace sizes (64-byte slice rows, exponents)
+  std::vector<SplitDev> split;
+  std::vector<TileTask> sgt_tasks, sgs_tasks, split_tasks;
+  int64_t split_slab_rows = 0, split_exps = 0, split_trows = 0, split_texps = 0;
   std::vector<TileTask> trsm_tasks, gemm_tasks, syrk_tasks, bpanel_tasks;
   std::vector<TriItemHost> tri_items;          // solve: diagonal-triangle blocks per level
   int32_t tri_nflags = 0;                      // solve: one flag per 64-row diagonal block
@@ -194,6 +213,7 @@ struct chol_handle {
 
 // Tile sizes shared by the schedule builder and the kernels.
 constexpr int kTile = 64;        // SIMT GEMM/SYRK tile edge
+constexpr int kSplitSlices = 7;  // bf16 slices of a binary64 operand (split_gemm.cuh)
 constexpr int kTileTC = 128;     // tensor-core (tcgen05) GEMM/SYRK tile edge
 constexpr int kTcOuter = 256;    // outer column block of the tensor-core trailing update
 constexpr int kAsmCols = 32;     // assembly task width (target columns)

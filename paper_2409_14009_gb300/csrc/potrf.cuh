@@ -37,12 +37,15 @@ __device__ __forceinline__ void pk_coord(int e, int kb, int& r, int& c) {
 // Square root of a pivot and its reciprocal. binary32 (the low-precision
 // factor of the mixed modes, refined in binary64 afterwards): the hardware
 // reciprocal square root rsqrtf (a few ulps) and sqrt(d) = d rsqrt(d), which
-// keeps the pivot chain short. binary64: on this GPU every FP64 instruction of the serial pivot chain holds
-// the narrow FP64 pipe for many cycles, and sqrt plus a division expand to
-// long dependent sequences; instead the reciprocal square root starts from the
-// binary32 estimate and takes two Newton-Raphson steps y <- y (3 - d y^2) / 2
-// (each roughly doubles the correct bits: ~23 -> ~46 -> full precision, within
-// a few ulps), then sqrt(d) = d y. Pivots outside the binary32 normal range
+// keeps the pivot chain short. binary64: every FP64 instruction holds the
+// narrow FP64 pipe for about 64 cycles a warp, conversions included, and sqrt
+// plus a division expand to long dependent sequences. Instead d = m 4^k with
+// 1 <= m < 4 (exponent bits), the binary32 estimate y of 1/sqrt(m) crosses the
+// formats as integers, and one third-order step (the binomial series of
+// (1 - e)^(-1/2), e = 1 - m y^2 ~ 2^-21, cut after e^2: the next term is
+// 5/16 e^3 ~ 2^-65) gives full precision within an ulp in four dependent
+// operations (two Newton-Raphson steps and two conversions took eight). The
+// result for d 4^k is that for d scaled by 2^k, bit for bit. Subnormal pivots
 // take sqrt and a division.
 __device__ __forceinline__ void pivot_root(float d, bool bad, float& root, float& rroot) {
   rroot = bad ? __int_as_float(0x7fc00000) : rsqrtf(d);
@@ -52,12 +55,20 @@ __device__ __forceinline__ void pivot_root(double d, bool bad, double& root, dou
   if (bad) {
     root = __longlong_as_double(0x7ff8000000000000LL);
     rroot = root;
-  } else if (d > 1e-30 && d < 1e30) {
-    double y = (double)rsqrtf((float)d);
-    y = y * fma(-0.5 * d, y * y, 1.5);
-    y = y * fma(-0.5 * d, y * y, 1.5);
-    root = d * y;
-    rroot = y;
+  } else if (d >= 2.2250738585072014e-308 && d < INFINITY) {
+    const int hi = __double2hiint(d), lo = __double2loint(d);
+    const int k2 = ((hi >> 20) - 1023) & ~1;               // d = m 2^k2, k2 even
+    const int mh = hi - k2 * (1 << 20);
+    const double m = __hiloint2double(mh, lo);
+    // binary32 of m, truncated: exponent rebiased, 23 bits of mantissa
+    const float mf = __int_as_float(((mh - ((1023 - 127) << 20)) << 3) | (int)((unsigned)lo >> 29));
+    const int yb = __float_as_int(rsqrtf(mf));             // 1/2 < y <= 1
+    const double y = __hiloint2double((yb >> 3) + ((1023 - 127) << 20), (int)((unsigned)yb << 29));
+    const double e = fma(-m, y * y, 1.0);
+    const double r = fma(y * e, fma(0.375, e, 0.5), y);
+    const double q = m * r;
+    rroot = __hiloint2double(__double2hiint(r) - (k2 / 2) * (1 << 20), __double2loint(r));
+    root = __hiloint2double(__double2hiint(q) + (k2 / 2) * (1 << 20), __double2loint(q));
   } else {
     root = sqrt(d);
     rroot = 1.0 / root;

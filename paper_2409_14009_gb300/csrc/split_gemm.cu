@@ -1,0 +1,362 @@
+// split_gemm.cu -- the binary64 factor's updates on the tensor cores
+// (split_gemm.cuh): operand splitting, the panel's trailing update, the update
+// matrices U_J = L_RJ L_RJ^T and the RLB form of the latter.
+//
+// Kernels
+//   k_sg_split_block  rows below a 64-column block of a panel, one exponent per
+//                     row of the block (the trailing update's operands)
+//   k_sg_split_rows   the off-diagonal rows L_RJ, one exponent per row over all
+//                     of J's columns (the SYRK's operands)
+//   k_sg_trailing     C -= A B^T on the panel, K = one 64-column block
+//   k_sg_syrk         U_J tiles, any K; RLB: subtracted from the ancestors
+#include "device.h"
+#include "split_gemm.cuh"
+
+namespace {
+
+constexpr int kSplitThreads = 256;
+
+__device__ __forceinline__ uint32_t abs_high(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
+
+// 128 rows [r0, r0 + 128) of the column block [k0, k0 + 64): thread (r, half)
+// owns 32 columns of a row in registers (loads coalesced along the rows).
+// HBM-bound: 8 bytes read and 14 written per entry.
+__global__ void __launch_bounds__(kSplitThreads)
+k_sg_split_block(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, const TileTask* __restrict__ tasks,
+                 const double* __restrict__ L, unsigned char* __restrict__ slab, int32_t* __restrict__ exps) {
+  __shared__ uint32_t hmax[2][sg::kM];
+  const TileTask t = tasks[blockIdx.x];
+  const SnodeDev d = sn[t.J];
+  const SplitDev z = sd[t.J];
+  const int r = threadIdx.x & (sg::kM - 1), half = threadIdx.x / sg::kM;
+  const int row = t.r0 + r, c0 = t.k0 + 32 * half;
+  const double* G = L + d.loff + row;
+  double x[32];
+  uint32_t m = 0;
+#pragma unroll
+  for (int c = 0; c < 32; ++c) {
+    x[c] = (row < d.len && c0 + c < d.s) ? G[(int64_t)(c0 + c) * d.ld] : 0.0;
+    m = max(m, abs_high(x[c]));
+  }
+  hmax[half][r] = m;
+  __syncthreads();
+  const int32_t e = sg::row_exponent(max(hmax[0][r], hmax[1][r]));
+  if (row >= z.trows) return;
+  if (half == 0) exps[z.trow0 + row] = e;
+  unsigned char* out = slab + (z.toff + (int64_t)half * sg::kSlices * z.trows) * 64;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    double y[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) y[i] = e == sg::kExpNaN ? 0.0 : x[8 * c + i];
+    uint4 w[sg::kSlices];
+    sg::digits8(y, e, w);
+#pragma unroll
+    for (int q = 0; q < sg::kSlices; ++q)
+      *reinterpret_cast<uint4*>(out + (int64_t)q * z.trows * 64 + sg::chunk_offset(row, c)) = w[q];
+  }
+}
+
+// 64 off-diagonal rows of J and all its columns: a first pass over the entries
+// for the rows' exponents, a second (from L2) for the digits; the four thread
+// groups take every fourth K block.
+__global__ void __launch_bounds__(kSplitThreads)
+k_sg_split_rows(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, const TileTask* __restrict__ tasks,
+                const double* __restrict__ L, unsigned char* __restrict__ slab, int32_t* __restrict__ exps) {
+  __shared__ uint32_t hmax[4][64];
+  const TileTask t = tasks[blockIdx.x];
+  const SnodeDev d = sn[t.J];
+  const SplitDev z = sd[t.J];
+  const int b = d.len - d.s;
+  const int r = threadIdx.x & 63, g = threadIdx.x >> 6;
+  const int row = t.r0 + r;
+  const bool in = row < b;
+  const double* G = L + d.loff + d.s + row;
+  uint32_t m = 0;
+  if (in) {
+#pragma unroll 8
+    for (int c = g; c < d.s; c += 4) m = max(m, abs_high(G[(int64_t)c * d.ld]));
+  }
+  hmax[g][r] = m;
+  __syncthreads();
+  const int32_t e = sg::row_exponent(max(max(hmax[0][r], hmax[1][r]), max(hmax[2][r], hmax[3][r])));
+  if (g == 0) exps[z.srow0 + row] = e;
+  for (int k = g; k * sg::kBlockK < d.s; k += 4) {
+    unsigned char* out = slab + (z.soff + (int64_t)k * sg::kSlices * z.srows) * 64;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      double y[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int col = k * sg::kBlockK + 8 * c + i;
+        y[i] = (in && col < d.s && e != sg::kExpNaN) ? G[(int64_t)col * d.ld] : 0.0;
+      }
+      uint4 w[sg::kSlices];
+      sg::digits8(y, e, w);
+#pragma unroll
+      for (int q = 0; q < sg::kSlices; ++q)
+        *reinterpret_cast<uint4*>(out + (int64_t)q * z.srows * 64 + sg::chunk_offset(row, c)) = w[q];
+    }
+  }
+}
+
+__device__ __forceinline__ uint32_t smem_base(const unsigned char* p) { return (tc::smem_u32(p) + 1023u) & ~1023u; }
+
+// Trailing update of the panel, step k0: 128 x 64 tiles, K = 64. One chunk per
+// tile, so the epilogue reads all seven accumulators of eight columns at a
+// time; the entries of C are loaded one batch ahead.
+__global__ void __launch_bounds__(sg::kThreads, 1)
+k_sg_trailing(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, const TileTask* __restrict__ tasks,
+              int ntasks, const unsigned char* __restrict__ slab, const int32_t* __restrict__ exps,
+              double* __restrict__ L, int* err) {
+  extern __shared__ unsigned char sg_smem[];
+  __shared__ __align__(8) sg::Shared S;
+  const uint32_t base = smem_base(sg_smem);
+  const uint32_t tmem = sg::setup(S);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  auto next = [&](int i, sg::Tile& t) {
+    const int64_t q = blockIdx.x + (int64_t)i * gridDim.x;
+    if (q >= ntasks) return false;
+    const TileTask k = tasks[q];
+    const SplitDev z = sd[k.J];
+    t.a = {slab + z.toff * 64, exps + z.trow0, z.trows, k.r0};
+    t.b = {slab + z.toff * 64, exps + z.trow0, z.trows, k.c0};
+    t.nblk = 2;
+    return true;
+  };
+  if (warp == sg::kEpiWarps) {
+    if (lane == 0) sg::copy_loop(S, base, next, err);
+  } else if (warp == sg::kEpiWarps + 1) {
+    if (lane == 0) sg::mma_loop(S, base, tmem, next, err);
+  } else {
+    sg::Tile t;
+    for (int i = 0; next(i, t); ++i) {
+      const TileTask k = tasks[blockIdx.x + (int64_t)i * gridDim.x];
+      const SnodeDev d = sn[k.J];
+      const int r = k.r0 + (warp & 3) * 32 + lane, c0 = k.c0 + (warp >> 2) * 32;
+      const bool in = r < d.len;
+      const int32_t ea = in ? t.a.exps[r] : 0;
+      double* C = L + d.loff + r;
+      double cv[2][8];
+      auto load = [&](int cb, double (&v)[8]) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const int col = c0 + 8 * cb + c;
+          v[c] = (in && col < d.s && r >= col) ? C[(int64_t)col * d.ld] : 0.0;
+        }
+      };
+      load(0, cv[0]);
+      if (!sg::epi_wait(S, sg::kSlices - 1, i, err)) break;
+      tc::fence_after();
+#pragma unroll
+      for (int cb = 0; cb < 4; ++cb) {
+        if (cb < 3) load(cb + 1, cv[(cb + 1) & 1]);
+        long long hi[8], lo[8];
+        sg::read8(tmem, (warp >> 2) * 32 + 8 * cb, hi, lo);
+        if (cb == 3) {   // every order of this warp's columns is in registers
+          tc::fence_before();
+          __syncwarp();
+          if (lane < sg::kSlices) sg::mbar_arrive(tc::smem_u32(&S.acc_empty[lane]));
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const int col = c0 + 8 * cb + c;
+          if (in && col < d.s && r >= col)
+            C[(int64_t)col * d.ld] = cv[cb & 1][c] - sg::combine(hi[c], lo[c], ea, t.b.exps[col]);
+        }
+      }
+    }
+  }
+  __syncwarp();
+  sg::teardown(S, tmem);
+}
+
+// Position of global row `key` in the sorted row structure rk[0, len).
+__device__ __forceinline__ int row_pos(const int32_t* __restrict__ rk, int len, int32_t key) {
+  int lo = 0, hi = len;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (rk[mid] < key) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
+
+// U_J tiles (lower triangle), K = all of J's columns in chunks of 128 whose
+// integer sums stay in registers. RLB: the tile is subtracted from the
+// ancestors' panels pair by pair (see k_syrk_rlb), a thread per row of the tile.
+template <bool RLB>
+__global__ void __launch_bounds__(sg::kThreads, 1)
+k_sg_syrk(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, const TileTask* __restrict__ tasks,
+          int ntasks, const unsigned char* __restrict__ slab, const int32_t* __restrict__ exps,
+          double* __restrict__ U, const int4* __restrict__ pairs, const int32_t* __restrict__ pbeg,
+          const int32_t* __restrict__ rows, double* __restrict__ L, int* err) {
+  extern __shared__ unsigned char sg_smem[];
+  __shared__ __align__(8) sg::Shared S;
+  const uint32_t base = smem_base(sg_smem);
+  const uint32_t tmem = sg::setup(S);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  auto next = [&](int i, sg::Tile& t) {
+    const int64_t q = blockIdx.x + (int64_t)i * gridDim.x;
+    if (q >= ntasks) return false;
+    const TileTask k = tasks[q];
+    const SplitDev z = sd[k.J];
+    t.a = {slab + z.soff * 64, exps + z.srow0, z.srows, k.r0};
+    t.b = {slab + z.soff * 64, exps + z.srow0, z.srows, k.c0};
+    t.nblk = z.sblk;
+    return true;
+  };
+  if (warp == sg::kEpiWarps) {
+    if (lane == 0) sg::copy_loop(S, base, next, err);
+  } else if (warp == sg::kEpiWarps + 1) {
+    if (lane == 0) sg::mma_loop(S, base, tmem, next, err);
+  } else {
+    sg::Tile t;
+    int chunk = 0;
+    bool ok = true;
+    for (int i = 0; ok && next(i, t); ++i) {
+      const TileTask k = tasks[blockIdx.x + (int64_t)i * gridDim.x];
+      const SnodeDev d = sn[k.J];
+      const int b = d.len - d.s;
+      const int r = k.r0 + (warp & 3) * 32 + lane, c0 = k.c0 + (warp >> 2) * 32;
+      const bool in = r < b;
+      const int32_t ea = in ? t.a.exps[r] : 0;
+      long long hi[32], lo[32];
+#pragma unroll
+      for (int c = 0; c < 32; ++c) hi[c] = lo[c] = 0;
+      for (int k0 = 0; ok && k0 < t.nblk; k0 += sg::kStagesPerChunk)
+        ok = sg::drain32(S, tmem, (warp >> 2) * 32, chunk++, hi, lo, err);
+      if (!ok) break;
+      if constexpr (!RLB) {
+        double* C = U + d.uoff + r;
+#pragma unroll
+        for (int c = 0; c < 32; ++c) {
+          const int col = c0 + c;
+          if (in && col < b && r >= col) C[(int64_t)col * b] = sg::combine(hi[c], lo[c], ea, t.b.exps[col]);
+        }
+      } else {
+        const int32_t* rj = rows + d.roff + d.s;
+        double v[32];
+#pragma unroll
+        for (int c = 0; c < 32; ++c)
+          v[c] = (in && c0 + c < b && r >= c0 + c) ? sg::combine(hi[c], lo[c], ea, t.b.exps[c0 + c]) : 0.0;
+        for (int p = pbeg[k.J]; p < pbeg[k.J + 1]; ++p) {
+          const int4 pr = pairs[p];   // (K, first column, end column, -)
+          if (pr.z <= c0) continue;
+          if (pr.y >= c0 + 32) break;
+          const SnodeDev dk = sn[pr.x];
+          if (!in || r < pr.y) continue;
+          double* T = L + dk.loff + row_pos(rows + dk.roff, dk.len, rj[r]);
+#pragma unroll
+          for (int c = 0; c < 32; ++c) {
+            const int cg = c0 + c;
+            if (cg < b && r >= cg && cg >= pr.y && cg < pr.z) atomicAdd(T + (int64_t)(rj[cg] - dk.f) * dk.ld, -v[c]);
+          }
+        }
+      }
+    }
+  }
+  __syncwarp();
+  sg::teardown(S, tmem);
+}
+
+}  // namespace
+
+namespace {
+
+struct SgBuffer { void** p; int64_t bytes; };
+
+std::vector<SgBuffer> sg_buffers(chol_handle* h) {
+  DeviceState* D = h->dev;
+  return {{(void**)&D->sg_slab, h->split_slab_rows * 64},
+          {(void**)&D->sg_exps, h->split_exps * 4},
+          {(void**)&D->sgt_slab[0], h->split_trows * 64},
+          {(void**)&D->sgt_slab[1], h->split_trows * 64},
+          {(void**)&D->sgt_exps[0], h->split_texps * 4},
+          {(void**)&D->sgt_exps[1], h->split_texps * 4},
+          {(void**)&D->sg_dev, (int64_t)(sizeof(SplitDev) * h->split.size())},
+          {(void**)&D->sg_split, (int64_t)(sizeof(TileTask) * h->split_tasks.size())},
+          {(void**)&D->sg_syrk, (int64_t)(sizeof(TileTask) * h->sgs_tasks.size())},
+          {(void**)&D->sg_trail, (int64_t)(sizeof(TileTask) * h->sgt_tasks.size())},
+          {(void**)&D->sg_err, 4}};
+}
+
+}  // namespace
+
+// Gives the workspaces back; later factorizations run on the binary64 pipe.
+void chol_sg_release(chol_handle* h) {
+  DeviceState* D = h->dev;
+  D->sg_ready = -1;
+  for (const SgBuffer& a : sg_buffers(h))
+    if (*a.p) {
+      cudaFree(*a.p);   // waits for the work that uses it
+      *a.p = nullptr;
+      D->bytes -= a.bytes;
+    }
+}
+
+// Workspaces and plan of the tensor-core updates, created by the first
+// factorization. D->sg_ready: 1 = in use, -1 = not: a handle with a memory cap,
+// or a device without the room, keeps the binary64 pipe's kernels, which need
+// no slices. (A later allocation that finds no room gets these back first, see
+// chol_dalloc.)
+int chol_sg_ensure(chol_handle* h) {
+  DeviceState* D = h->dev;
+  if (D->sg_ready) return CHOL_OK;
+  D->sg_ready = -1;
+  if ((h->split_tasks.empty() && h->sgt_tasks.empty()) || h->opt.device_mem_cap > 0) return CHOL_OK;
+  for (const SgBuffer& a : sg_buffers(h))
+    if (chol_dalloc(h, a.p, (size_t)a.bytes)) {
+      chol_sg_release(h);
+      return CHOL_OK;
+    }
+  CHOL_CUDA_TRY(cudaMemset(D->sg_err, 0, 4));
+  CHOL_CUDA_TRY(cudaMemcpy(D->sg_dev, h->split.data(), sizeof(SplitDev) * h->split.size(), cudaMemcpyHostToDevice));
+  auto up = [](TileTask* dst, const std::vector<TileTask>& v) {
+    return v.empty() ? cudaSuccess : cudaMemcpy(dst, v.data(), sizeof(TileTask) * v.size(), cudaMemcpyHostToDevice);
+  };
+  CHOL_CUDA_TRY(up(D->sg_split, h->split_tasks));
+  CHOL_CUDA_TRY(up(D->sg_syrk, h->sgs_tasks));
+  CHOL_CUDA_TRY(up(D->sg_trail, h->sgt_tasks));
+  const void* kernels[] = {(const void*)k_sg_trailing, (const void*)k_sg_syrk<false>, (const void*)k_sg_syrk<true>};
+  for (const void* k : kernels)
+    CHOL_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sg::kSmemBytes));
+  D->sg_ready = 1;
+  return CHOL_OK;
+}
+
+// Slices of the rows below the 64-column block of step k0 (buffer k0 / 64 mod 2).
+void chol_sg_split_block(chol_handle* h, const StepRange& s, int buf, cudaStream_t st) {
+  DeviceState* D = h->dev;
+  k_sg_split_block<<<s.sgt_next, kSplitThreads, 0, st>>>(D->sn, D->sg_dev, D->sg_trail + s.sgt_b, D->L, D->sgt_slab[buf],
+                                                        D->sgt_exps[buf]);
+}
+
+void chol_sg_trailing(chol_handle* h, const TileTask* tasks, int n, int grid, int buf, cudaStream_t st) {
+  DeviceState* D = h->dev;
+  k_sg_trailing<<<std::min(n, grid), sg::kThreads, sg::kSmemBytes, st>>>(D->sn, D->sg_dev, tasks, n, D->sgt_slab[buf],
+                                                                        D->sgt_exps[buf], D->L, D->sg_err);
+}
+
+// U_J of every blocked supernode of a level (RLB: subtracted from the ancestors).
+void chol_sg_syrk(chol_handle* h, const LevelPlan& P, cudaStream_t st) {
+  DeviceState* D = h->dev;
+  k_sg_split_rows<<<P.sgr_n, kSplitThreads, 0, st>>>(D->sn, D->sg_dev, D->sg_split + P.sgr_b, D->L, D->sg_slab,
+                                                     D->sg_exps);
+  const int grid = std::min(P.sgs_n, D->sms);
+  if (h->opt.update_mode == CHOL_UPDATE_RLB)
+    k_sg_syrk<true><<<grid, sg::kThreads, sg::kSmemBytes, st>>>(D->sn, D->sg_dev, D->sg_syrk + P.sgs_b, P.sgs_n, D->sg_slab,
+                                                                D->sg_exps, nullptr, D->rlb_pairs, D->rlb_pbeg, D->rows,
+                                                                D->L, D->sg_err);
+  else
+    k_sg_syrk<false><<<grid, sg::kThreads, sg::kSmemBytes, st>>>(D->sn, D->sg_dev, D->sg_syrk + P.sgs_b, P.sgs_n,
+                                                                 D->sg_slab, D->sg_exps, D->U, nullptr, nullptr, nullptr,
+                                                                 nullptr, D->sg_err);
+}
+
+// After a synchronized factorization: CHOL_ETIMEOUT if any tile gave up waiting.
+int chol_sg_status(chol_handle* h) {
+  DeviceState* D = h->dev;
+  if (D->sg_ready != 1 || D->status_host[3] == 0) return CHOL_OK;
+  CHOL_CUDA_TRY(cudaMemset(D->sg_err, 0, 4));
+  return CHOL_ETIMEOUT;
+}

@@ -1,0 +1,376 @@
+// split_gemm.cuh -- binary64 products on the bf16 tensor cores.
+//
+// The binary64 pipe of this part retires two FMAs per cycle and SM, the tensor
+// cores about 4,096 bf16 multiply-adds, so a binary64 product D = A B^T is
+// computed from exact pieces (the error-free splitting of Ozaki, Ogita, Oishi
+// and Rump, "Error-free transformations of matrix multiplication by using fast
+// routines of matrix multiplication", Numer. Algorithms 59, 2012):
+// - each row of an operand gets one exponent e with |x| 2^-e < 1/2 for its
+//   entries, and every entry becomes the integer Y = round(x 2^(63 - e)),
+//   written with kSlices = 7 signed base-512 digits, Y = sum_i d_i 512^(6 - i),
+//   d_i in [-256, 256]. A digit is exact in bf16.
+// - the product of slices i and j has weight 2^(ea + eb - 9 (i + j + 2)). The
+//   slice products of one order i + j = q <= 6 share one binary32 accumulator
+//   over kChunkK = 64 columns. Its integers stay at most (q + 1) 64 2^16: exact
+//   for the orders 0..3 whatever the digits; the orders 4..6 (weights of 2^-54
+//   and less) pass 2^24 only if almost all their digits are extreme and agree
+//   in sign (digits in general position give about 2^19), and then lose their
+//   last bit. Orders above 6 (2^-81 times 2^16 K at most) are left out.
+// - the seven sums are added as integers, rounded once to binary64 and scaled.
+// So an entry's error is its one rounding plus about sqrt(K) 2^-64 times the
+// two rows' largest entries, below that of K binary64 FMAs, and independent of
+// scaling the rows by powers of two. (Digits of base 256 with the same orders,
+// 2^-57, were measured too: on the irregular 36^3 Laplacian, whose solution
+// hangs on small entries of L, x was 4 times further off than with FMAs.)
+// The summation order is fixed, so results are reproducible bit for bit. A row
+// that holds an infinity or a NaN gives NaN in its row of the product.
+//
+// Slices are stored in the layout the tensor cores read from shared memory:
+// per 32-column block of K, per slice, rows of 32 bf16 (64 bytes) with the
+// 64-byte swizzle (16-byte chunk c of row r at chunk c ^ ((r >> 1) & 3)), so a
+// 128-row operand slice is one contiguous 8 KiB copy without a tensor map.
+#pragma once
+#include <cuda_bf16.h>
+
+#include <climits>
+#include <cstdint>
+
+#include "internal.h"
+#include "tc_gemm.cuh"
+
+namespace sg {
+
+constexpr int kSlices = kSplitSlices;
+constexpr int kM = 128, kN = 64;          // output tile
+constexpr int kBlockK = 32;               // K of one stage
+constexpr int kDigit = 9;                 // bits of a digit
+constexpr int kChunkK = 64;               // K per accumulator chunk (see above)
+constexpr int kStagesPerChunk = kChunkK / kBlockK;
+constexpr int kStages = 2;
+constexpr int kABytes = kM * 64, kBBytes = kN * 64;           // one slice of an operand stage
+constexpr int kStageBytes = kSlices * (kABytes + kBBytes);    // 86,016
+constexpr int kSmemBytes = kStages * kStageBytes + 1024;
+constexpr int kEpiWarps = 8;
+constexpr int kThreads = 32 * (kEpiWarps + 2);   // epilogue, copy and MMA warps
+constexpr int kTmemCols = 512;            // 7 accumulators of 64 columns
+
+constexpr int32_t kExpNaN = INT_MIN;      // exponent of a row with an infinity or a NaN
+constexpr int32_t kExpMin = -1020;        // rows of zeros and subnormals
+
+// Row exponent from the largest high word (sign cleared) of a row's entries.
+__device__ __forceinline__ int32_t row_exponent(uint32_t hi_max) {
+  const int E = (int)(hi_max >> 20);
+  if (E == 0x7ff) return kExpNaN;
+  return (E > 1 ? E : 1) - 1021;          // |x| < 2^(E - 1022), so |x| 2^-e < 1/2
+}
+
+// round(x 2^(63 - e)), |.| <= 2^62, for an entry of a row with exponent e.
+__device__ __forceinline__ long long fixed_point(double x, int32_t e) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)(u >> 52) & 0x7ff;
+  unsigned long long m = u & 0xfffffffffffffull;
+  if (ex) m |= 1ull << 52;
+  const int sh = e + 1021 - (ex ? ex : 1);          // E - ex >= 0: Y = m 2^(9 - sh), rounded
+  m <<= 9;
+  if (sh > 0) m = sh < 63 ? (m + (1ull << (sh - 1))) >> sh : 0;
+  return (u >> 63) ? -(long long)m : (long long)m;
+}
+
+// binary32 bits of a small integer (exact; the low 16 bits of the result are 0
+// for |d| <= 256 and its high 16 bits are the bf16 value)
+__device__ __forceinline__ uint32_t digit_bits(int d) {
+  return __float_as_uint(__int_as_float(0x4B400000 + d) - 12582912.0f);
+}
+
+// The digits of eight consecutive entries of a row: out[i] = the 16 bytes
+// (8 bf16) of slice i.
+__device__ __forceinline__ void digits8(const double (&x)[8], int32_t e, uint4 (&out)[kSlices]) {
+  uint32_t w[kSlices][4];
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    long long y0 = fixed_point(x[2 * p], e), y1 = fixed_point(x[2 * p + 1], e);
+#pragma unroll
+    for (int i = kSlices - 1; i >= 0; --i) {
+      // the low digit, sign-extended (the one left last is the top digit)
+      const int d0 = i ? (int)((uint32_t)y0 << (32 - kDigit)) >> (32 - kDigit) : (int)y0;
+      const int d1 = i ? (int)((uint32_t)y1 << (32 - kDigit)) >> (32 - kDigit) : (int)y1;
+      w[i][p] = __byte_perm(digit_bits(d0), digit_bits(d1), 0x7632);
+      y0 = (y0 - d0) >> kDigit;
+      y1 = (y1 - d1) >> kDigit;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < kSlices; ++i) out[i] = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
+}
+
+// Byte offset of the 16-byte chunk c (0..3) of row r inside one slice.
+__device__ __forceinline__ int64_t chunk_offset(int r, int c) {
+  return (int64_t)r * 64 + ((c ^ ((r >> 1) & 3)) << 4);
+}
+
+// m 2^e as binary64, m rounded to nearest even (once).
+__device__ __forceinline__ double scaled_int(long long m, int e) {
+  if (m == 0) return 0.0;
+  unsigned long long u = m < 0 ? (unsigned long long)(-m) : (unsigned long long)m;
+  const int lz = __clzll((long long)u);
+  u <<= lz;                                         // value = u 2^(e - lz), bit 63 set
+  const int E = 63 + 1023 + e - lz;                 // biased exponent
+  unsigned long long mant = u >> 11;
+  const uint32_t rem = (uint32_t)u & 0x7ff;
+  mant += (rem > 0x400u || (rem == 0x400u && (mant & 1))) ? 1u : 0u;
+  if (E >= 1 && E <= 2045) {
+    const unsigned long long b = ((unsigned long long)(E - 1) << 52) + mant;   // mant carries the implicit bit
+    return __longlong_as_double((long long)(b | (m < 0 ? 1ull << 63 : 0ull)));
+  }
+  return ldexp((double)m, e);
+}
+
+// The sum hi 2^-45 + lo 2^-72 times 2^(ea + eb) (hi, lo: the integer sums of
+// the orders 0..3 and 4..6). hi takes lo's carry; then the top 63 bits are rounded.
+__device__ __forceinline__ double combine(long long hi, long long lo, int32_t ea, int32_t eb) {
+  constexpr int kLow = 3 * kDigit;
+  if (ea == kExpNaN || eb == kExpNaN) return __longlong_as_double(0x7ff8000000000000ll);
+  hi += lo >> kLow;
+  const unsigned long long low = (unsigned long long)lo & ((1ull << kLow) - 1);
+  const int q = max(0, kLow + 1 - __clzll(hi ^ (hi >> 63)));   // low bits that do not fit beside hi
+  const long long m = (long long)(((unsigned long long)hi << (kLow - q)) | (low >> q));
+  return scaled_int(m, ea + eb - 8 * kDigit + q);
+}
+
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+// K-major operand, 64-byte swizzle, rows of 64 bytes, 8-row groups 512 bytes apart.
+__device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)(512 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)4 << 61;
+  return d;
+}
+
+constexpr uint32_t kIdesc =
+    (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kN >> 3) << 17) | ((uint32_t)(kM >> 4) << 24);
+
+// Bounded wait that also gives up when another role of the CTA has.
+__device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  const long long t0 = clock64();
+  for (uint32_t it = 0;; ++it) {
+    if (tc::mbar_try_wait(bar, parity)) return true;
+    if ((it & 63) == 63) {
+      if (*abort_flag) return false;
+      if (clock64() - t0 > (1ll << 31)) return false;
+    }
+  }
+}
+
+// One operand: slices of `rows` rows (K blocks of 32: [block][slice][rows][32]),
+// the tile's first row, and the rows' exponents.
+struct Operand {
+  const unsigned char* slab;
+  const int32_t* exps;
+  int64_t rows;
+  int row0;
+};
+
+struct Tile {
+  Operand a, b;
+  int nblk;      // K blocks
+};
+
+// Shared state of the CTA.
+struct Shared {
+  uint64_t full[kStages], empty[kStages], acc_full[kSlices], acc_empty[kSlices], done;
+  uint32_t tmem;
+  int abort_flag, issued;
+};
+
+__device__ __forceinline__ uint32_t setup(Shared& S) {
+  const int warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      tc::mbar_init(tc::smem_u32(&S.full[s]), 1);
+      tc::mbar_init(tc::smem_u32(&S.empty[s]), 1);
+    }
+    for (int q = 0; q < kSlices; ++q) {
+      tc::mbar_init(tc::smem_u32(&S.acc_full[q]), 1);
+      tc::mbar_init(tc::smem_u32(&S.acc_empty[q]), kEpiWarps);
+    }
+    tc::mbar_init(tc::smem_u32(&S.done), 1);
+    S.abort_flag = 0;
+    S.issued = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncwarp();
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc::smem_u32(&S.tmem)),
+                 "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  return S.tmem;
+}
+
+// Ends the CTA: after an abort, waits (bounded) for the copies in flight and
+// for the MMAs already issued; then frees the tensor memory.
+__device__ __forceinline__ void teardown(Shared& S, uint32_t tmem) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  volatile int never = 0;
+  if (warp == kEpiWarps && lane == 0 && *(volatile int*)&S.abort_flag) {
+    for (int s = 0; s < kStages && s < S.issued; ++s)
+      wait_or_abort(tc::smem_u32(&S.full[s]), (uint32_t)(((S.issued - 1 - s) / kStages) & 1), &never);
+  }
+  if (warp == kEpiWarps + 1 && lane == 0) {
+    tc::mma_commit(tc::smem_u32(&S.done));
+    wait_or_abort(tc::smem_u32(&S.done), 0, &never);
+  }
+  __syncwarp();
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+}
+
+// The copy thread's loop over the CTA's tiles: `next(i, tile)` gives the i-th tile.
+template <class Next>
+__device__ __forceinline__ void copy_loop(Shared& S, uint32_t base, Next next, int* err) {
+  int it = 0;
+  Tile t;
+  for (int i = 0; next(i, t); ++i) {
+    for (int k = 0; k < t.nblk; ++k, ++it) {
+      const int s = it % kStages, round = it / kStages;
+      if (round > 0 && !wait_or_abort(tc::smem_u32(&S.empty[s]), (uint32_t)((round - 1) & 1), &S.abort_flag)) {
+        atomicExch(err, tc::kErrTimeoutEmpty);
+        *(volatile int*)&S.abort_flag = 1;
+        S.issued = it;
+        return;
+      }
+      const uint32_t fb = tc::smem_u32(&S.full[s]);
+      tc::mbar_expect_tx(fb, (uint32_t)kStageBytes);
+      const uint32_t a0 = base + s * kStageBytes, b0 = a0 + kSlices * kABytes;
+      const unsigned char* pa = t.a.slab + ((int64_t)k * kSlices * t.a.rows + t.a.row0) * 64;
+      const unsigned char* pb = t.b.slab + ((int64_t)k * kSlices * t.b.rows + t.b.row0) * 64;
+#pragma unroll
+      for (int q = 0; q < kSlices; ++q) {
+        bulk_load(a0 + q * kABytes, pa + (int64_t)q * t.a.rows * 64, kABytes, fb);
+        bulk_load(b0 + q * kBBytes, pb + (int64_t)q * t.b.rows * 64, kBBytes, fb);
+      }
+    }
+  }
+  S.issued = it;
+}
+
+// The MMA thread's loop: per K block the 28 slice products of the orders 0..6;
+// an order's accumulator is handed to the epilogue at the end of each chunk of
+// kChunkK and taken back before its next use.
+template <class Next>
+__device__ __forceinline__ void mma_loop(Shared& S, uint32_t base, uint32_t tmem, Next next, int* err) {
+  int it = 0, chunk = 0;
+  Tile t;
+  for (int i = 0; next(i, t); ++i) {
+    for (int k = 0; k < t.nblk; ++k, ++it) {
+      const int s = it % kStages, round = it / kStages;
+      if (!wait_or_abort(tc::smem_u32(&S.full[s]), (uint32_t)(round & 1), &S.abort_flag)) {
+        atomicExch(err, tc::kErrTimeoutFull);
+        *(volatile int*)&S.abort_flag = 1;
+        return;
+      }
+      tc::fence_after();
+      const uint32_t a0 = base + s * kStageBytes;
+      const uint64_t ad = sw64_desc(a0), bd = sw64_desc(a0 + kSlices * kABytes);
+      const bool first = k % kStagesPerChunk == 0;
+      const bool last = k % kStagesPerChunk == kStagesPerChunk - 1 || k == t.nblk - 1;
+// unrolled: the descriptors become additions of constants, and the issue keeps
+      // up with the 48 cycles that a 128 x 64 x 16 product takes (operand reads)
+#pragma unroll
+      for (int q = 0; q < kSlices; ++q) {
+        if (first && chunk > 0) {
+          if (!wait_or_abort(tc::smem_u32(&S.acc_empty[q]), (uint32_t)((chunk - 1) & 1), &S.abort_flag)) {
+            atomicExch(err, tc::kErrTimeoutAccum);
+            *(volatile int*)&S.abort_flag = 1;
+            return;
+          }
+          tc::fence_after();
+        }
+        const uint32_t d = tmem + (uint32_t)(q * kN);
+#pragma unroll
+        for (int a = 0; a <= q; ++a) {
+          const uint64_t da = ad + (uint64_t)(a * (kABytes >> 4)), db = bd + (uint64_t)((q - a) * (kBBytes >> 4));
+          tc::mma<1>(d, da, db, kIdesc, (first && a == 0) ? 0u : 1u);
+          tc::mma<1>(d, da + 2, db + 2, kIdesc, 1u);
+        }
+        if (last) tc::mma_commit(tc::smem_u32(&S.acc_full[q]));
+      }
+      tc::mma_commit(tc::smem_u32(&S.empty[s]));
+      if (last) ++chunk;
+    }
+  }
+}
+
+// A whole epilogue warp waits for order q of the chunk (uniform result).
+__device__ __forceinline__ bool epi_wait(Shared& S, int q, int chunk, int* err) {
+  const bool ok = wait_or_abort(tc::smem_u32(&S.acc_full[q]), (uint32_t)(chunk & 1), &S.abort_flag);
+  if (__all_sync(0xffffffffu, ok)) return true;
+  atomicExch(err, tc::kErrTimeoutAccum);
+  *(volatile int*)&S.abort_flag = 1;
+  return false;
+}
+
+// All orders of one chunk, 32 columns (from column `col`) of the thread's row,
+// added to hi (orders 0..3) and lo (orders 4..6).
+__device__ __forceinline__ bool drain32(Shared& S, uint32_t tmem, int col, int chunk, long long (&hi)[32],
+                                        long long (&lo)[32], int* err) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col;
+#pragma unroll
+  for (int q = 0; q < kSlices; ++q) {
+    if (!epi_wait(S, q, chunk, err)) return false;
+    tc::fence_after();
+    float v[32];
+    tc::tmem_ld32(trow + (uint32_t)(q * kN), v);
+    tc::fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(tc::smem_u32(&S.acc_empty[q]));
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+      const int a = __float2int_rn(v[c]);
+      if (q < 4) hi[c] += (long long)a * (1 << (kDigit * (3 - q)));
+      else lo[c] += (long long)a * (1 << (kDigit * (6 - q)));
+    }
+  }
+  return true;
+}
+
+// The same for 8 columns of a single-chunk tile, without taking the accumulators back.
+__device__ __forceinline__ void read8(uint32_t tmem, int col, long long (&hi)[8], long long (&lo)[8]) {
+  const int warp = threadIdx.x >> 5;
+  const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) hi[c] = lo[c] = 0;
+#pragma unroll
+  for (int q = 0; q < kSlices; ++q) {
+    float v[8];
+    tc::tmem_ld8(trow + (uint32_t)(q * kN), v);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const int a = __float2int_rn(v[c]);
+      if (q < 4) hi[c] += (long long)a * (1 << (kDigit * (3 - q)));
+      else lo[c] += (long long)a * (1 << (kDigit * (6 - q)));
+    }
+  }
+}
+
+}  // namespace sg

@@ -1,0 +1,93 @@
+"""GPU parity of the binary64 updates on the tensor cores (bf16 slices).
+
+Two leaf supernodes of s columns share one separator of b rows, so that a leaf's
+panel takes trailing updates (s > 64), its update matrix has b rows and K = s,
+and the separator takes trailing updates of its own. Sizes sit at the edges of
+the 128 x 64 tiles, the 32-column blocks and the 128-column chunks.
+
+Tolerances: the slices keep every entry of a row to 2^-57 of the row's largest,
+so both this path and the oracle's FMAs are backward stable with a constant of a
+few n u; the matrices have kappa < 100 after diagonal scaling, so entries agree
+to well below the 1e-12 of the other binary64 parity tests.
+"""
+import numpy as np
+import pytest
+
+from gpu_util import check_parity, run
+from helpers import lower_csc_from_dense
+from lib_fixture import chol
+
+pytestmark = pytest.mark.gpu
+
+
+def _opts(mode=0, cap=0):
+    o = chol().chol_default_options()
+    o.small_max_cols = o.small_max_panel = 1   # everything wider than one column on the blocked path
+    o.update_mode, o.device_mem_cap = mode, cap
+    return o
+
+
+def _arrow(s, b, spread=0, seed=0):
+    """[D1 0 B1'; 0 D2 B2'; B1 B2 C], dense blocks, diagonally dominant; rows and
+    columns scaled by powers of two within 2^+-spread."""
+    rs = np.random.RandomState(1000 * s + b + seed)
+    n = 2 * s + b
+    A = rs.uniform(-1.0, 1.0, (n, n))
+    A[s:2 * s, :s] = 0.0
+    A = np.tril(A, -1) + np.tril(A, -1).T
+    A[np.diag_indices(n)] = 1.05 * np.abs(A).sum(axis=1)
+    if spread:
+        d = np.ldexp(1.0, rs.randint(-spread, spread + 1, n))
+        A = d[:, None] * A * d[None, :]
+    cp, ri, vx = lower_csc_from_dense(A)
+    return dict(n=n, colptr=cp, rowind=ri, values=vx, perm=np.arange(n, dtype=np.int32))
+
+
+SIZES = [(2, 1), (31, 63), (32, 64), (33, 65), (64, 129), (65, 128), (96, 200), (127, 127), (128, 64), (129, 191),
+         (257, 130), (300, 66)]
+
+
+@pytest.mark.parametrize("s,b", SIZES)
+@pytest.mark.parametrize("mode", [0, 1])
+def test_tiles(s, b, mode):
+    p = _arrow(s, b)
+    rhs = np.random.RandomState(1).uniform(-1, 1, (p["n"], 2))
+    got, _ = check_parity(p, rhs, _opts(mode))
+    assert got["stats"]["syrk"]["launches"] >= 2   # operand split and tiles
+
+
+@pytest.mark.parametrize("spread", [8, 200])
+def test_power_of_two_scaling(spread):
+    """Scaling rows and columns by powers of two changes no digit: L scales exactly."""
+    p, q = _arrow(130, 100), _arrow(130, 100, spread)
+    a, c = run(p, None, _opts()), run(q, None, _opts())
+    d = np.sqrt(q["values"][q["colptr"][:-1]] / p["values"][p["colptr"][:-1]])
+    lp, li, lx = a["L"]
+    assert np.array_equal(c["L"][2], lx * d[li])
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_memory_cap_keeps_the_small_workspace_path(mode):
+    p = _arrow(129, 100)
+    got, ref = check_parity(p, None, _opts(mode, cap=1 << 40))
+    assert got["stats"]["syrk"]["launches"] == 1
+    check_parity(p, None, _opts(mode), ref=ref)
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_not_finite(bad):
+    """An entry of a leaf's off-diagonal rows spoils its row of the separator."""
+    s, b = 70, 90
+    p = _arrow(s, b)
+    v = p["values"].copy()
+    t = p["colptr"][3] + (s - 3) + 40          # column 3, row 40 of the separator
+    assert p["rowind"][t] == 2 * s + 40
+    v[t] = bad
+    assert run(dict(p, values=v), None, _opts())["rc"] == 2 * s + 41
+
+
+def test_not_positive_definite():
+    p = _arrow(100, 80)
+    v = p["values"].copy()
+    v[p["colptr"][230]] = -1.0
+    assert run(dict(p, values=v), None, _opts())["rc"] == 231
