@@ -26,6 +26,7 @@ struct DeviceState {
   AsmTask* asm_tasks = nullptr;
   AsmSeg* asm_segs = nullptr;
   TriItemHost* tri = nullptr;   // solve: diagonal-triangle items
+  double* rdiag = nullptr;      // binary64 blocked path: reciprocal pivots, per column of P A P^T
   int sg_ready = 0;             // binary64 updates on the tensor cores: 1 = in use, -1 = not
   unsigned char* sg_slab = nullptr;              // slices of a level's off-diagonal rows
   int32_t* sg_exps = nullptr;                    // ... and their row exponents
@@ -205,7 +206,6 @@ int chol_dalloc(chol_handle* h, void** p, size_t bytes);
 // binary64 updates on the tensor cores (split_gemm.cu)
 int chol_sg_ensure(chol_handle* h);
 void chol_sg_release(chol_handle* h);
-void chol_sg_split_block(chol_handle* h, const StepRange& s, int buf, cudaStream_t st);
 void chol_sg_trailing(chol_handle* h, const TileTask* tasks, int n, int grid, int buf, cudaStream_t st);
 void chol_sg_syrk(chol_handle* h, const LevelPlan& P, cudaStream_t st);
 int chol_sg_status(chol_handle* h);

@@ -22,6 +22,7 @@
 #include <climits>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include <cooperative_groups.h>
 
@@ -29,6 +30,7 @@
 #include "mixed.h"
 #include "assemble.cuh"
 #include "potrf.cuh"
+#include "split_gemm.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -178,30 +180,61 @@ k_small_rlb(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list, c
 constexpr int kPotrfThreads = kPkThreads;
 __global__ void __launch_bounds__(kPotrfThreads)
 k_potrf(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list, int k0, int nb,
-        double* __restrict__ L, int* status) {
+        double* __restrict__ L, double* __restrict__ rdiag, int* status) {
   __shared__ double As[64 * kPwLd];
-  __shared__ int sok;
   const SnodeDev d = sn[list[blockIdx.x]];
   const int kb = min(nb, d.s - k0);
   double* G = L + d.loff + k0 + (int64_t)k0 * d.ld;
-  potrf_panels<double, false>(G, d.ld, kb, -INFINITY, As, &sok, status, true, d.f + k0);
+  const int r = threadIdx.x & 63, c0 = threadIdx.x >> 6;   // coalesced along a column's rows
+  double v[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const int c = c0 + 4 * i;
+    v[i] = (r < kb && c <= r) ? G[r + (int64_t)c * d.ld] : 0.0;
+  }
+#pragma unroll
+  for (int i = 0; i < 16; ++i) As[r * kPwLd + c0 + 4 * i] = r >= kb && r == c0 + 4 * i ? 1.0 : v[i];
+  potrf64_smem(kb, As, status, d.f + k0, rdiag + d.f + k0);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const int c = c0 + 4 * i;
+    if (r < kb && c <= r) G[r + (int64_t)c * d.ld] = As[r * kPwLd + c];
+  }
 }
 
-// Blocked path, step k0: rows [r0, r0 + kTrsmRows) of column block [k0, k0+kb) become
-// X = B L_kk^{-T}. Eight lanes share a row, lane q holding columns q + 8m; the
-// solved x_j is broadcast inside the 8-lane group with a shuffle and every lane
-// updates its own columns (no barriers in the substitution loop).
-constexpr int kTrsmThreads = 128;   // 8 lanes per row
-constexpr int kTrsmRows = 16;
+// Blocked path, step k0: a task's rows of column block [k0, k0+kb) become
+// X = B L_kk^{-T}. LPR lanes share a row, lane q holding columns q + LPR m; the
+// solved x_j is broadcast inside the group with a shuffle and every lane
+// updates its own columns (no barriers in the substitution loop). A warp is
+// bound by its partition's FP64 pipe (1 + 32 / LPR + 1/2 instructions of 64
+// cycles a step on average), so few rows take 16 lanes each (8 rows a CTA, the
+// shorter chain) and many rows 8 (16 rows a CTA, fewer instructions a row).
+// SPLIT: the rows' slices for the trailing update on the tensor cores are
+// written here too, where the row is on chip (split_gemm.cuh).
+constexpr int kTrsmThreads = 128;
+template <int LPR, bool SPLIT>
 __global__ void __launch_bounds__(kTrsmThreads)
-k_trsm(const SnodeDev* __restrict__ sn, const TileTask* __restrict__ tasks, int nb,
-       double* __restrict__ L) {
+k_trsm(const SnodeDev* __restrict__ sn, const TileTask* __restrict__ tasks, int nb, double* __restrict__ L,
+       const double* __restrict__ rdiag, const SplitDev* __restrict__ sd, unsigned char* __restrict__ slab,
+       int32_t* __restrict__ exps) {
+  constexpr int kRows = kTrsmThreads / LPR, kCols = 64 / LPR;
   __shared__ double Lk[64 * 65];
   __shared__ double inv[64];
-  const TileTask t = tasks[blockIdx.x];
+  const TileTask t = tasks[blockIdx.x / (kTrsmRowsHost / 2 / kRows)];
+  const int r0 = t.r0 + (blockIdx.x % (kTrsmRowsHost / 2 / kRows)) * kRows;
   const SnodeDev d = sn[t.J];
   const int kb = min(nb, d.s - t.k0);
   const double* Gd = L + d.loff + t.k0 + (int64_t)t.k0 * d.ld;
+  const int g = threadIdx.x / LPR, q = threadIdx.x & (LPR - 1);
+  const int row = r0 + g;
+  const bool live = row < d.len;
+  double* Gx = L + d.loff + row + (int64_t)t.k0 * d.ld;
+  double x[kCols];
+#pragma unroll
+  for (int m = 0; m < kCols; ++m) {
+    const int c = q + LPR * m;
+    x[m] = (live && c < kb) ? Gx[(int64_t)c * d.ld] : 0.0;
+  }
   {
     // stage the diagonal block: all loads of a thread issued before the
     // stores (column-major source: consecutive threads read consecutive rows)
@@ -209,51 +242,67 @@ k_trsm(const SnodeDev* __restrict__ sn, const TileTask* __restrict__ tasks, int 
     double v[kIt];
 #pragma unroll
     for (int i = 0; i < kIt; ++i) {
-      const int q = threadIdx.x + kTrsmThreads * i, r = q & 63, c = q >> 6;
+      const int e = threadIdx.x + kTrsmThreads * i, r = e & 63, c = e >> 6;
       v[i] = (r < kb && c < kb) ? Gd[r + (int64_t)c * d.ld] : 0.0;
     }
 #pragma unroll
     for (int i = 0; i < kIt; ++i) {
-      const int q = threadIdx.x + kTrsmThreads * i;
-      Lk[(q & 63) + (q >> 6) * 65] = v[i];
+      const int e = threadIdx.x + kTrsmThreads * i;
+      Lk[(e & 63) + (e >> 6) * 65] = v[i];
     }
+    if (threadIdx.x < 64) inv[threadIdx.x] = threadIdx.x < kb ? rdiag[d.f + t.k0 + threadIdx.x] : 0.0;
   }
   __syncthreads();
-  for (int c = threadIdx.x; c < kb; c += blockDim.x) inv[c] = 1.0 / Lk[c + c * 65];
-  __syncthreads();
-  const int g = threadIdx.x >> 3, q = threadIdx.x & 7;
-  const int row = t.r0 + g;
-  const bool live = row < d.len;
-  double* Gx = L + d.loff + row + (int64_t)t.k0 * d.ld;
-  double x[8];
 #pragma unroll
-  for (int m = 0; m < 8; ++m) {
-    const int c = q + 8 * m;
-    x[m] = (live && c < kb) ? Gx[(int64_t)c * d.ld] : 0.0;
-  }
+  for (int jm = 0; jm < kCols; ++jm) {
 #pragma unroll
-  for (int jm = 0; jm < 8; ++jm) {
-#pragma unroll
-    for (int jq = 0; jq < 8; ++jq) {
-      const int j = jm * 8 + jq;
+    for (int jq = 0; jq < LPR; ++jq) {
+      const int j = jm * LPR + jq;
       if (j < kb) {
         const double cand = x[jm] * inv[j];
-        const double xj = __shfl_sync(0xffffffffu, cand, jq, 8);
+        const double xj = __shfl_sync(0xffffffffu, cand, jq, LPR);
         if (q == jq) x[jm] = xj;
-        // columns q + 8m with m < jm are already solved: not even issued
+        // columns q + LPR m with m < jm are already solved: not even issued
 #pragma unroll
-        for (int m = jm; m < 8; ++m) {
-          const int c = q + 8 * m;
-          if (c > j && c < kb) x[m] -= xj * Lk[c + j * 65];
+        for (int m = jm; m < kCols; ++m) {
+          const int c = q + LPR * m;
+          if (c > j && c < kb) x[m] = fma(-xj, Lk[c + j * 65], x[m]);
         }
       }
     }
   }
   if (live) {
 #pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      const int c = q + 8 * m;
+    for (int m = 0; m < kCols; ++m) {
+      const int c = q + LPR * m;
       if (c < kb) Gx[(int64_t)c * d.ld] = x[m];
+    }
+  }
+  if constexpr (SPLIT) {
+    if (t.k0 + kb >= d.s) return;   // nothing right of the block (uniform across the CTA)
+    uint32_t hm = 0;
+#pragma unroll
+    for (int m = 0; m < kCols; ++m) hm = max(hm, (uint32_t)__double2hiint(x[m]) & 0x7fffffffu);
+    for (int o = LPR / 2; o > 0; o >>= 1) hm = max(hm, __shfl_xor_sync(0xffffffffu, hm, o, LPR));
+    const int32_t e = sg::row_exponent(hm);
+    __syncthreads();   // every warp is done with Lk
+    double* xs = Lk;   // row g at xs[66 g]
+#pragma unroll
+    for (int m = 0; m < kCols; ++m) xs[g * 66 + q + LPR * m] = e == sg::kExpNaN ? 0.0 : x[m];
+    const SplitDev z = sd[t.J];
+    if (live && q == 0) exps[z.trow0 + row] = e;
+    __syncwarp();      // a row's lanes are in one warp
+    if (!live) return;
+    // 8 chunks of 8 columns a row: lane q takes chunk q (LPR = 16: half the lanes)
+    if (q < 8) {
+      double y[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) y[i] = xs[g * 66 + 8 * q + i];
+      uint4 w[sg::kSlices];
+      sg::digits8(y, e, w);
+      unsigned char* out = slab + (z.toff + (int64_t)(q >> 2) * sg::kSlices * z.trows) * 64 + sg::chunk_offset(row, q & 3);
+#pragma unroll
+      for (int i = 0; i < sg::kSlices; ++i) *reinterpret_cast<uint4*>(out + (int64_t)i * z.trows * 64) = w[i];
     }
   }
 }
@@ -692,7 +741,7 @@ void chol_device_free(chol_handle* h) {
                   D->mx_diagpos, D->mx_aij, D->mx_d, D->mx_fallbacks, D->csr_ptr, D->csr_col, D->csr_src,
                   D->csr_val, D->Lbf, D->tmaps, D->tc_err, D->R, D->Z, D->Pv, D->Q, D->red, D->Y32, D->W32,
                   D->rhs_scale, D->host_vals, D->host_rhs, D->panel, D->pflags, D->dinv, D->split_part, D->split_cnt, D->hand32, D->sg_slab, D->sg_exps, D->sgt_slab[0], D->sgt_slab[1],
-                  D->sgt_exps[0], D->sgt_exps[1], D->sg_dev, D->sg_split, D->sg_syrk, D->sg_trail, D->sg_err};
+                  D->sgt_exps[0], D->sgt_exps[1], D->sg_dev, D->sg_split, D->sg_syrk, D->sg_trail, D->sg_err, D->rdiag};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (D->status_host) cudaFreeHost(D->status_host);
@@ -804,6 +853,9 @@ int chol_device_ensure(chol_handle* h) {
   if ((rc = chol_dalloc(h, (void**)&D->status, sizeof(int32_t)))) return fail(rc);
   if ((rc = chol_dalloc(h, (void**)&D->part, sizeof(double) * (size_t)std::max(h->ns, 1)))) return fail(rc);
   if ((rc = chol_dalloc(h, (void**)&D->scalar_dev, sizeof(double)))) return fail(rc);
+  if (h->opt.precision == CHOL_PREC_FP64 && h->n_large > 0 &&
+      (rc = chol_dalloc(h, (void**)&D->rdiag, sizeof(double) * (size_t)h->n)))
+    return fail(rc);
   if (cudaMallocHost((void**)&D->status_host, 4 * sizeof(int32_t)) != cudaSuccess) return fail(CHOL_ENOMEM);
   if (cudaMallocHost((void**)&D->scalar_host, sizeof(double)) != cudaSuccess) return fail(CHOL_ENOMEM);
   static bool attrs_done = false;
@@ -879,20 +931,28 @@ int enqueue_factor_fp64(chol_handle* h, const double* values, cudaStream_t st) {
       const int k0 = (int)k * nb;
       if (s.potrf_n > 0) {
         KScope ks(h, CHOL_K_POTRF, st, s.potrf_flops, 16.0 * nb * nb * s.potrf_n);
-        k_potrf<<<s.potrf_n, kPotrfThreads, 0, st>>>(D->sn, D->potrf_list + s.potrf_b, k0, nb, D->L,
+        k_potrf<<<s.potrf_n, kPotrfThreads, 0, st>>>(D->sn, D->potrf_list + s.potrf_b, k0, nb, D->L, D->rdiag,
                                                      D->status);
       }
+      const int buf = (int)(k & 1);   // step k + 2 reuses step k's slices: its rest has joined by then
       if (s.trsm_n > 0) {
-        KScope ks(h, CHOL_K_TRSM, st, s.trsm_flops, 16.0 * kTrsmRows * nb * s.trsm_n);
-        k_trsm<<<s.trsm_n, kTrsmThreads, 0, st>>>(D->sn, D->trsm + s.trsm_b, nb, D->L);
+        KScope ks(h, CHOL_K_TRSM, st, s.trsm_flops, 16.0 * (kTrsmRowsHost / 2) * nb * s.trsm_n);
+        // 8-row CTAs while they fit on the SMs two at a time
+        const bool few = s.trsm_n <= D->sms;
+        auto go = [&](auto lpr, auto split) {
+          constexpr int LPR = decltype(lpr)::value;
+          k_trsm<LPR, decltype(split)::value><<<s.trsm_n * (LPR / 8), kTrsmThreads, 0, st>>>(
+              D->sn, D->trsm + s.trsm_b, nb, D->L, D->rdiag, D->sg_dev, D->sgt_slab[buf], D->sgt_exps[buf]);
+        };
+        auto pick = [&](auto split) {
+          if (few) go(std::integral_constant<int, 16>{}, split);
+          else go(std::integral_constant<int, 8>{}, split);
+        };
+        if (sg) pick(std::true_type{});
+        else pick(std::false_type{});
       }
       const int gemm_n = sg ? s.sgt_n : s.gemm_n, gemm_next = sg ? s.sgt_next : s.gemm_next;
       const int nrest = gemm_n - gemm_next;
-      const int buf = (int)(k & 1);   // step k + 2 reuses step k's slices: its rest has joined by then
-      if (sg && gemm_n > 0) {
-        KScope ks(h, CHOL_K_GEMM, st, 0.0, 22.0 * 128.0 * nb * gemm_next);
-        chol_sg_split_block(h, s, buf, st);
-      }
       if (nrest > 0) {
         CHOL_CUDA_TRY(cudaEventRecord(D->lev[0], st));   // step k's panel is final
         CHOL_CUDA_TRY(cudaStreamWaitEvent(D->lstream, D->lev[0], 0));

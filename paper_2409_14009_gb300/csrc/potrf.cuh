@@ -38,37 +38,50 @@ __device__ __forceinline__ void pk_coord(int e, int kb, int& r, int& c) {
 // factor of the mixed modes, refined in binary64 afterwards): the hardware
 // reciprocal square root rsqrtf (a few ulps) and sqrt(d) = d rsqrt(d), which
 // keeps the pivot chain short. binary64: every FP64 instruction holds the
-// narrow FP64 pipe for about 64 cycles a warp, conversions included, and sqrt
-// plus a division expand to long dependent sequences. Instead d = m 4^k with
-// 1 <= m < 4 (exponent bits), the binary32 estimate y of 1/sqrt(m) crosses the
-// formats as integers, and one third-order step (the binomial series of
-// (1 - e)^(-1/2), e = 1 - m y^2 ~ 2^-21, cut after e^2: the next term is
-// 5/16 e^3 ~ 2^-65) gives full precision within an ulp in four dependent
-// operations (two Newton-Raphson steps and two conversions took eight). The
-// result for d 4^k is that for d scaled by 2^k, bit for bit. Subnormal pivots
-// take sqrt and a division.
+// narrow FP64 pipe for about 64 cycles a warp, conversions included, so the
+// reciprocal square root is formed with integers: d = m 4^k with 1 <= m < 4
+// (exponent bits), the binary32 estimate y of 1/sqrt(m) as a 24-bit integer,
+// e = 1 - m y^2 (|e| < 2^-20) exactly to 2^-62, and one third-order step of the
+// binomial series, y (1 + e/2 + 3/8 e^2) (the next term is 5/16 e^3 < 2^-61),
+// rounded once: within 0.57 ulp. sqrt(d) = d rsqrt(d). The result for d 4^k is
+// that for d scaled by 2^k, bit for bit. Subnormal pivots take sqrt and a
+// division.
 __device__ __forceinline__ void pivot_root(float d, bool bad, float& root, float& rroot) {
   rroot = bad ? __int_as_float(0x7fc00000) : rsqrtf(d);
   root = d * rroot;
 }
+// 1 / sqrt(d) of a positive normal d from its words, with integers (see above).
+__device__ __forceinline__ double rsqrt_bits(int hi, int lo) {
+  typedef unsigned long long u64;
+  const int E = hi >> 20, p = (E & 1) ^ 1;                   // d = m 2^(E - 1023 - p), m = 1.f 2^p
+  const unsigned fh = (unsigned)((hi & 0xfffff) | 0x100000), fl = (unsigned)lo;
+  // binary32 of m, truncated
+  const float mf = __int_as_float(((127 + p) << 23) | (int)((hi & 0xfffff) << 3 | fl >> 29));
+  float yf;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(mf));
+  yf = fmaxf(fminf(yf, 0.99999994f), 0.5f);                  // 1/2 <= y < 1
+  const unsigned y = (unsigned)((__float_as_int(yf) & 0x7fffff) | 0x800000);   // y 2^24
+  const u64 t = ((u64)y * y) << p;
+  const unsigned th = (unsigned)(t >> 32), tl = (unsigned)t;
+  // m y^2 2^64 modulo 2^64, so e 2^64 = -P
+  const u64 b = (u64)fl * th + ((u64)fh * tl + ((u64)fl * tl >> 32));
+  const long long e = -(long long)(((u64)fh * th << 28) + (b >> 4));
+  const int e50 = (int)(e >> 14);
+  // every shift rounds: a truncation here is a bias of all pivots, which adds up
+  // (1/8 of 2^-53 made x 3 to 6 times less accurate on weakly shifted Laplacians)
+  const long long c = ((e + 32) >> 6) + ((3 * (long long)__mulhi(e50, e50) + 2048) >> 12);   // (e/2 + 3/8 e^2) 2^59
+  const u64 v = ((u64)y << 38) + (u64)(((long long)(int)y * c + (1 << 20)) >> 21);           // y (1 + ...) 2^62
+  const u64 r = ((v + 256) >> 9) + (1021ull << 52);          // bit 52 is the implicit one
+  return __hiloint2double((int)(r >> 32) - ((E - 1023 - p) / 2) * (1 << 20), (int)r);
+}
 __device__ __forceinline__ void pivot_root(double d, bool bad, double& root, double& rroot) {
-  if (bad) {
+  const int hi = __double2hiint(d);
+  if (hi >= 0x00100000 && hi < 0x7ff00000) {   // positive, normal, finite
+    rroot = rsqrt_bits(hi, __double2loint(d));
+    root = d * rroot;
+  } else if (bad) {
     root = __longlong_as_double(0x7ff8000000000000LL);
     rroot = root;
-  } else if (d >= 2.2250738585072014e-308 && d < INFINITY) {
-    const int hi = __double2hiint(d), lo = __double2loint(d);
-    const int k2 = ((hi >> 20) - 1023) & ~1;               // d = m 2^k2, k2 even
-    const int mh = hi - k2 * (1 << 20);
-    const double m = __hiloint2double(mh, lo);
-    // binary32 of m, truncated: exponent rebiased, 23 bits of mantissa
-    const float mf = __int_as_float(((mh - ((1023 - 127) << 20)) << 3) | (int)((unsigned)lo >> 29));
-    const int yb = __float_as_int(rsqrtf(mf));             // 1/2 < y <= 1
-    const double y = __hiloint2double((yb >> 3) + ((1023 - 127) << 20), (int)((unsigned)yb << 29));
-    const double e = fma(-m, y * y, 1.0);
-    const double r = fma(y * e, fma(0.375, e, 0.5), y);
-    const double q = m * r;
-    rroot = __hiloint2double(__double2hiint(r) - (k2 / 2) * (1 << 20), __double2loint(r));
-    root = __hiloint2double(__double2hiint(q) + (k2 / 2) * (1 << 20), __double2loint(q));
   } else {
     root = sqrt(d);
     rroot = 1.0 / root;
@@ -320,3 +333,116 @@ __device__ __forceinline__ bool potrf_panels(T* __restrict__ G, int64_t ld, int 
   return ok;
 }
 
+// ---------------------------------------------------------------------------
+// binary64: the same panel algorithm with the panel's rows spread over up to
+// three warps. A warp-wide FP64 instruction takes one of the SM's four
+// partitions 64 cycles, whatever its active lanes, so one warp's panel (14
+// instructions a column, 7 of them for the second row of each lane) was the
+// longest chain: 56 us a block. Here warp v holds the panel's 8 diagonal rows
+// (every warp the same ones, lanes 0-7) and 24 rows below them, one row a lane:
+// 4.5 FP64 instructions a column besides the integer pivot root, each warp on
+// its own partition. The other warps subtract the previous panel's rank-8
+// product from the columns right of it, the triangle folded so that every
+// thread gets as many entries. Per entry the arithmetic and its order are
+// those of potrf_panels_smem. rdiag receives the reciprocals of the diagonal.
+constexpr int kPwRows = 24;
+
+// The panel column by column on the shared copy, one warp: any pivot, with its
+// record and poisoned column. Only reached with a pivot that is not positive,
+// normal and finite, so it is kept small.
+static __device__ __noinline__ void potrf64_panel_any(double* As, int c0, int kb, int* status, int fcol, double* rdiag) {
+  const int lane = threadIdx.x & 31;
+  for (int k = c0; k < min(c0 + 8, kb); ++k) {
+    const double dk = As[k * kPwLd + k];
+    const bool bad = !(dk > 0.0);
+    double root, rroot;
+    pivot_root(dk, bad, root, rroot);
+    __syncwarp();
+    if (lane == 0) {
+      if (bad) atomicMin(status, fcol + k + 1);
+      As[k * kPwLd + k] = root;
+      rdiag[k] = 1.0 / root;
+    }
+    for (int r = k + 1 + lane; r < kb; r += 32) As[r * kPwLd + k] *= rroot;
+    __syncwarp();
+    for (int j = k + 1; j < c0 + 8; ++j)
+      for (int r = j + lane; r < kb; r += 32) As[r * kPwLd + j] = fma(-As[r * kPwLd + k], As[j * kPwLd + k], As[r * kPwLd + j]);
+    __syncwarp();
+  }
+}
+
+// The panel [c0, c0 + 8): straight-line code, because a branch a column costs
+// 170 cycles; the pivots' range is checked at the end. False (uniform over the
+// nw warps): some pivot is not positive, normal and finite, nothing written.
+__device__ __forceinline__ bool potrf64_panel(double* __restrict__ As, int c0, int kb, int nw,
+                                              double* __restrict__ rdiag) {
+  const int lane = threadIdx.x & 31, v = threadIdx.x >> 5;
+  const int row = lane < 8 ? c0 + lane : c0 + 8 + v * kPwRows + (lane - 8);
+  double x[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) x[t] = row < 64 ? As[row * kPwLd + c0 + t] : 0.0;
+  // every warp has read the diagonal rows before warp 0 writes them back
+  asm volatile("bar.sync 1, %0;" ::"r"(32 * nw) : "memory");
+  double rd = 0.0, dg = 0.0;   // lane kk: reciprocal root and pivot of column kk
+  bool normal = true;
+#pragma unroll
+  for (int kk = 0; kk < 8; ++kk) {
+    const double dk = __shfl_sync(0xffffffffu, x[kk], kk);
+    const int dh = __double2hiint(dk);
+    normal = normal && dh >= 0x00100000 && dh < 0x7ff00000;
+    const double rroot = rsqrt_bits(dh, __double2loint(dk));
+    if (lane == kk) { rd = rroot; dg = dk; }
+    if (lane > kk) x[kk] *= rroot;
+#pragma unroll
+    for (int jj = kk + 1; jj < 8; ++jj) x[jj] = fma(-x[kk], __shfl_sync(0xffffffffu, x[kk], jj), x[jj]);
+  }
+  if (!normal) return false;
+  dg *= rd;                    // the roots
+#pragma unroll
+  for (int kk = 0; kk < 8; ++kk)
+    if (lane == kk) x[kk] = dg;
+  if (row < 64 && (lane >= 8 || v == 0)) {
+#pragma unroll
+    for (int t = 0; t < 8; ++t) As[row * kPwLd + c0 + t] = x[t];
+  }
+  // the reciprocal of the stored root, for the rows below
+  if (v == 0 && lane < 8 && c0 + lane < kb) rdiag[c0 + lane] = fma(fma(-dg, rd, 1.0), rd, rd);
+  return true;
+}
+
+// As: 64 rows of kPwLd entries, the lower triangle of the kb x kb block, zeros
+// past it but ones on the diagonal (a short last panel is then a full one).
+__device__ __forceinline__ void potrf64_smem(int kb, double* __restrict__ As, int* status, int fcol,
+                                             double* __restrict__ rdiag) {
+  const int tid = threadIdx.x, warp = tid >> 5;
+  auto panel_warps = [](int below) { return max(1, (below + kPwRows - 1) / kPwRows); };
+  __syncthreads();
+  {
+    const int nw = panel_warps(kb - 8);
+    if (warp < nw && !potrf64_panel(As, 0, kb, nw, rdiag) && warp == 0)
+      potrf64_panel_any(As, 0, kb, status, fcol, rdiag);
+  }
+  __syncthreads();
+  for (int c0 = 0; c0 + 8 < kb; c0 += 8) {
+    const int n0 = c0 + 8, wn = min(8, kb - n0), n1 = n0 + wn;   // next panel [n0, n1)
+    {
+      const int r = n0 + (tid >> 2);
+      if (r < kb)
+        for (int j = n0 + (tid & 3); j < n1 && j <= r; j += 4) potrf_rank8<double>(As, r, j, c0, 8);
+    }
+    __syncthreads();
+    const int nw = panel_warps(kb - n1);
+    if (warp < nw) {
+      if (!potrf64_panel(As, n0, kb, nw, rdiag) && warp == 0) potrf64_panel_any(As, n0, kb, status, fcol, rdiag);
+    } else {
+      // rows p and T - 1 - p of the triangle right of the next panel, T + 1 entries together
+      const int T = kb - n1, items = ((T + 1) >> 1) * (T + 1);
+      for (int q = tid - 32 * nw; q < items; q += kPkThreads - 32 * nw) {
+        const int p = q / (T + 1), o = q - p * (T + 1), p2 = T - 1 - p;
+        if (o <= p) potrf_rank8<double>(As, n1 + p, n1 + o, c0, 8);
+        else if (p2 != p) potrf_rank8<double>(As, n1 + p2, n1 + o - p - 1, c0, 8);
+      }
+    }
+    __syncthreads();
+  }
+}

@@ -3,11 +3,10 @@
 // matrices U_J = L_RJ L_RJ^T and the RLB form of the latter.
 //
 // Kernels
-//   k_sg_split_block  rows below a 64-column block of a panel, one exponent per
-//                     row of the block (the trailing update's operands)
 //   k_sg_split_rows   the off-diagonal rows L_RJ, one exponent per row over all
 //                     of J's columns (the SYRK's operands)
-//   k_sg_trailing     C -= A B^T on the panel, K = one 64-column block
+//   k_sg_trailing     C -= A B^T on the panel, K = one 64-column block (its
+//                     operands come from k_trsm, one exponent per row of the block)
 //   k_sg_syrk         U_J tiles, any K; RLB: subtracted from the ancestors
 #include "device.h"
 #include "split_gemm.cuh"
@@ -17,45 +16,6 @@ namespace {
 constexpr int kSplitThreads = 256;
 
 __device__ __forceinline__ uint32_t abs_high(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
-
-// 128 rows [r0, r0 + 128) of the column block [k0, k0 + 64): thread (r, half)
-// owns 32 columns of a row in registers (loads coalesced along the rows).
-// HBM-bound: 8 bytes read and 14 written per entry.
-__global__ void __launch_bounds__(kSplitThreads)
-k_sg_split_block(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, const TileTask* __restrict__ tasks,
-                 const double* __restrict__ L, unsigned char* __restrict__ slab, int32_t* __restrict__ exps) {
-  __shared__ uint32_t hmax[2][sg::kM];
-  const TileTask t = tasks[blockIdx.x];
-  const SnodeDev d = sn[t.J];
-  const SplitDev z = sd[t.J];
-  const int r = threadIdx.x & (sg::kM - 1), half = threadIdx.x / sg::kM;
-  const int row = t.r0 + r, c0 = t.k0 + 32 * half;
-  const double* G = L + d.loff + row;
-  double x[32];
-  uint32_t m = 0;
-#pragma unroll
-  for (int c = 0; c < 32; ++c) {
-    x[c] = (row < d.len && c0 + c < d.s) ? G[(int64_t)(c0 + c) * d.ld] : 0.0;
-    m = max(m, abs_high(x[c]));
-  }
-  hmax[half][r] = m;
-  __syncthreads();
-  const int32_t e = sg::row_exponent(max(hmax[0][r], hmax[1][r]));
-  if (row >= z.trows) return;
-  if (half == 0) exps[z.trow0 + row] = e;
-  unsigned char* out = slab + (z.toff + (int64_t)half * sg::kSlices * z.trows) * 64;
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    double y[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) y[i] = e == sg::kExpNaN ? 0.0 : x[8 * c + i];
-    uint4 w[sg::kSlices];
-    sg::digits8(y, e, w);
-#pragma unroll
-    for (int q = 0; q < sg::kSlices; ++q)
-      *reinterpret_cast<uint4*>(out + (int64_t)q * z.trows * 64 + sg::chunk_offset(row, c)) = w[q];
-  }
-}
 
 // 64 off-diagonal rows of J and all its columns: a first pass over the entries
 // for the rows' exponents, a second (from L2) for the digits; the four thread
@@ -102,9 +62,8 @@ k_sg_split_rows(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd
 
 __device__ __forceinline__ uint32_t smem_base(const unsigned char* p) { return (tc::smem_u32(p) + 1023u) & ~1023u; }
 
-// Trailing update of the panel, step k0: 128 x 64 tiles, K = 64. One chunk per
-// tile, so the epilogue reads all seven accumulators of eight columns at a
-// time; the entries of C are loaded one batch ahead.
+// Trailing update of the panel, step k0: 128 x 64 tiles, K = 64, one chunk per
+// tile. The thread's entries of C are loaded before the wait for the products.
 __global__ void __launch_bounds__(sg::kThreads, 1)
 k_sg_trailing(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, const TileTask* __restrict__ tasks,
               int ntasks, const unsigned char* __restrict__ slab, const int32_t* __restrict__ exps,
@@ -133,38 +92,21 @@ k_sg_trailing(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, 
     for (int i = 0; next(i, t); ++i) {
       const TileTask k = tasks[blockIdx.x + (int64_t)i * gridDim.x];
       const SnodeDev d = sn[k.J];
-      const int r = k.r0 + (warp & 3) * 32 + lane, c0 = k.c0 + (warp >> 2) * 32;
-      const bool in = r < d.len;
-      const int32_t ea = in ? t.a.exps[r] : 0;
-      double* C = L + d.loff + r;
-      double cv[2][8];
-      auto load = [&](int cb, double (&v)[8]) {
+      const int r = k.r0 + sg::epi_row(), c0 = k.c0 + sg::epi_col();
+      // the thread's columns c0 .. c0 + n - 1 (on or below the diagonal)
+      const int n = r < d.len ? min(sg::kCols, min(d.s, r + 1) - c0) : 0;
+      const int32_t ea = n > 0 ? t.a.exps[r] : 0;
+      double* C = L + d.loff + r + (int64_t)c0 * d.ld;
+      double cv[sg::kCols];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const int col = c0 + 8 * cb + c;
-          v[c] = (in && col < d.s && r >= col) ? C[(int64_t)col * d.ld] : 0.0;
-        }
-      };
-      load(0, cv[0]);
-      if (!sg::epi_wait(S, sg::kSlices - 1, i, err)) break;
-      tc::fence_after();
+      for (int c = 0; c < sg::kCols; ++c) cv[c] = c < n ? C[(int64_t)c * d.ld] : 0.0;
+      long long hi[sg::kCols], lo[sg::kCols];
 #pragma unroll
-      for (int cb = 0; cb < 4; ++cb) {
-        if (cb < 3) load(cb + 1, cv[(cb + 1) & 1]);
-        long long hi[8], lo[8];
-        sg::read8(tmem, (warp >> 2) * 32 + 8 * cb, hi, lo);
-        if (cb == 3) {   // every order of this warp's columns is in registers
-          tc::fence_before();
-          __syncwarp();
-          if (lane < sg::kSlices) sg::mbar_arrive(tc::smem_u32(&S.acc_empty[lane]));
-        }
+      for (int c = 0; c < sg::kCols; ++c) hi[c] = lo[c] = 0;
+      if (!sg::drain(S, tmem, i, hi, lo, err)) break;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const int col = c0 + 8 * cb + c;
-          if (in && col < d.s && r >= col)
-            C[(int64_t)col * d.ld] = cv[cb & 1][c] - sg::combine(hi[c], lo[c], ea, t.b.exps[col]);
-        }
-      }
+      for (int c = 0; c < sg::kCols; ++c)
+        if (c < n) C[(int64_t)c * d.ld] = cv[c] - sg::combine(hi[c], lo[c], ea, t.b.exps[c0 + c]);
     }
   }
   __syncwarp();
@@ -217,39 +159,36 @@ k_sg_syrk(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, cons
       const TileTask k = tasks[blockIdx.x + (int64_t)i * gridDim.x];
       const SnodeDev d = sn[k.J];
       const int b = d.len - d.s;
-      const int r = k.r0 + (warp & 3) * 32 + lane, c0 = k.c0 + (warp >> 2) * 32;
-      const bool in = r < b;
-      const int32_t ea = in ? t.a.exps[r] : 0;
-      long long hi[32], lo[32];
+      const int r = k.r0 + sg::epi_row(), c0 = k.c0 + sg::epi_col();
+      // the thread's columns c0 .. c0 + n - 1 (on or below the diagonal)
+      const int n = r < b ? min(sg::kCols, r + 1 - c0) : 0;
+      const int32_t ea = n > 0 ? t.a.exps[r] : 0;
+      long long hi[sg::kCols], lo[sg::kCols];
 #pragma unroll
-      for (int c = 0; c < 32; ++c) hi[c] = lo[c] = 0;
-      for (int k0 = 0; ok && k0 < t.nblk; k0 += sg::kStagesPerChunk)
-        ok = sg::drain32(S, tmem, (warp >> 2) * 32, chunk++, hi, lo, err);
+      for (int c = 0; c < sg::kCols; ++c) hi[c] = lo[c] = 0;
+      for (int k0 = 0; ok && k0 < t.nblk; k0 += sg::kStagesPerChunk) ok = sg::drain(S, tmem, chunk++, hi, lo, err);
       if (!ok) break;
       if constexpr (!RLB) {
-        double* C = U + d.uoff + r;
+        double* C = U + d.uoff + r + (int64_t)c0 * b;
 #pragma unroll
-        for (int c = 0; c < 32; ++c) {
-          const int col = c0 + c;
-          if (in && col < b && r >= col) C[(int64_t)col * b] = sg::combine(hi[c], lo[c], ea, t.b.exps[col]);
-        }
+        for (int c = 0; c < sg::kCols; ++c)
+          if (c < n) C[(int64_t)c * b] = sg::combine(hi[c], lo[c], ea, t.b.exps[c0 + c]);
       } else {
         const int32_t* rj = rows + d.roff + d.s;
-        double v[32];
+        double v[sg::kCols];
 #pragma unroll
-        for (int c = 0; c < 32; ++c)
-          v[c] = (in && c0 + c < b && r >= c0 + c) ? sg::combine(hi[c], lo[c], ea, t.b.exps[c0 + c]) : 0.0;
-        for (int p = pbeg[k.J]; p < pbeg[k.J + 1]; ++p) {
+        for (int c = 0; c < sg::kCols; ++c) v[c] = c < n ? sg::combine(hi[c], lo[c], ea, t.b.exps[c0 + c]) : 0.0;
+        for (int p = pbeg[k.J]; n > 0 && p < pbeg[k.J + 1]; ++p) {
           const int4 pr = pairs[p];   // (K, first column, end column, -)
           if (pr.z <= c0) continue;
-          if (pr.y >= c0 + 32) break;
+          if (pr.y >= c0 + n) break;
           const SnodeDev dk = sn[pr.x];
-          if (!in || r < pr.y) continue;
+          if (r < pr.y) break;        // the pair's rows start at its first column
           double* T = L + dk.loff + row_pos(rows + dk.roff, dk.len, rj[r]);
 #pragma unroll
-          for (int c = 0; c < 32; ++c) {
+          for (int c = 0; c < sg::kCols; ++c) {
             const int cg = c0 + c;
-            if (cg < b && r >= cg && cg >= pr.y && cg < pr.z) atomicAdd(T + (int64_t)(rj[cg] - dk.f) * dk.ld, -v[c]);
+            if (c < n && cg >= pr.y && cg < pr.z) atomicAdd(T + (int64_t)(rj[cg] - dk.f) * dk.ld, -v[c]);
           }
         }
       }
@@ -324,13 +263,7 @@ int chol_sg_ensure(chol_handle* h) {
   return CHOL_OK;
 }
 
-// Slices of the rows below the 64-column block of step k0 (buffer k0 / 64 mod 2).
-void chol_sg_split_block(chol_handle* h, const StepRange& s, int buf, cudaStream_t st) {
-  DeviceState* D = h->dev;
-  k_sg_split_block<<<s.sgt_next, kSplitThreads, 0, st>>>(D->sn, D->sg_dev, D->sg_trail + s.sgt_b, D->L, D->sgt_slab[buf],
-                                                        D->sgt_exps[buf]);
-}
-
+// Trailing tiles from the slices of parity `buf` (written by k_trsm).
 void chol_sg_trailing(chol_handle* h, const TileTask* tasks, int n, int grid, int buf, cudaStream_t st) {
   DeviceState* D = h->dev;
   k_sg_trailing<<<std::min(n, grid), sg::kThreads, sg::kSmemBytes, st>>>(D->sn, D->sg_dev, tasks, n, D->sgt_slab[buf],

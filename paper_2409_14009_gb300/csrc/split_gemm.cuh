@@ -50,7 +50,8 @@ constexpr int kStages = 2;
 constexpr int kABytes = kM * 64, kBBytes = kN * 64;           // one slice of an operand stage
 constexpr int kStageBytes = kSlices * (kABytes + kBBytes);    // 86,016
 constexpr int kSmemBytes = kStages * kStageBytes + 1024;
-constexpr int kEpiWarps = 8;
+constexpr int kEpiWarps = 16;             // four to a partition: the epilogue is integer work with short chains
+constexpr int kCols = 16;                 // columns of an epilogue thread
 constexpr int kThreads = 32 * (kEpiWarps + 2);   // epilogue, copy and MMA warps
 constexpr int kTmemCols = 512;            // 7 accumulators of 64 columns
 
@@ -126,15 +127,35 @@ __device__ __forceinline__ double scaled_int(long long m, int e) {
 }
 
 // The sum hi 2^-45 + lo 2^-72 times 2^(ea + eb) (hi, lo: the integer sums of
-// the orders 0..3 and 4..6). hi takes lo's carry; then the top 63 bits are rounded.
+// the orders 0..3 and 4..6), rounded to binary64: hi takes lo's carry, the
+// magnitude is normalised with two funnel shifts and rounded at bit 53, and the
+// exponent is put together: about 35 integer instructions and no binary64 ones. Sums below 2^-45 and exponents
+// near the limits (zero rows, NaN) take scaled_int.
 __device__ __forceinline__ double combine(long long hi, long long lo, int32_t ea, int32_t eb) {
   constexpr int kLow = 3 * kDigit;
-  if (ea == kExpNaN || eb == kExpNaN) return __longlong_as_double(0x7ff8000000000000ll);
+  const int e = ea + eb;
   hi += lo >> kLow;
-  const unsigned long long low = (unsigned long long)lo & ((1ull << kLow) - 1);
+  const uint32_t low = (uint32_t)lo & ((1u << kLow) - 1);
+  const uint32_t sgn = (uint32_t)(hi >> 63);
+  // the magnitude's three words: complement, plus one at the lowest bit
+  const uint32_t one = sgn & (1u << (32 - kLow));
+  uint32_t w0 = ((low << (32 - kLow)) ^ (sgn << (32 - kLow))) + one;
+  const unsigned long long w = ((unsigned long long)hi ^ (unsigned long long)(hi >> 63)) + (w0 < one ? 1u : 0u);
+  uint32_t w2 = (uint32_t)(w >> 32), w1 = (uint32_t)w;
+  if ((uint32_t)(e + 900) <= 1800u && ea != kExpNaN && eb != kExpNaN && (w2 | w1)) {
+    int E = 1023 + 18 - 1 + e;                     // biased exponent of bit 63 of hi, less the implicit bit's one
+    if (w2 == 0) { w2 = w1; w1 = w0; w0 = 0; E -= 32; }
+    const int lz = __clz((int)w2);
+    const uint32_t u1 = __funnelshift_l(w1, w2, lz), u0 = __funnelshift_l(w0, w1, lz);
+    // the top 53 bits, rounded (bit 52 is the implicit one and adds to the exponent field)
+    const unsigned long long m =
+        (((unsigned long long)u1 << 32 | u0) >> 11) + ((u0 >> 10) & 1u) + ((unsigned long long)(uint32_t)(E - lz) << 52);
+    return __longlong_as_double((long long)(m | (unsigned long long)(sgn & 0x80000000u) << 32));
+  }
+  if (ea == kExpNaN || eb == kExpNaN) return __longlong_as_double(0x7ff8000000000000ll);
   const int q = max(0, kLow + 1 - __clzll(hi ^ (hi >> 63)));   // low bits that do not fit beside hi
   const long long m = (long long)(((unsigned long long)hi << (kLow - q)) | (low >> q));
-  return scaled_int(m, ea + eb - 8 * kDigit + q);
+  return scaled_int(m, e - 8 * kDigit + q);
 }
 
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
@@ -189,7 +210,8 @@ struct Tile {
 
 // Shared state of the CTA.
 struct Shared {
-  uint64_t full[kStages], empty[kStages], acc_full[kSlices], acc_empty[kSlices], done;
+  // accumulators change hands in two groups: orders 0..3 and 4..6
+  uint64_t full[kStages], empty[kStages], acc_full[2], acc_empty[2], done;
   uint32_t tmem;
   int abort_flag, issued;
 };
@@ -201,7 +223,7 @@ __device__ __forceinline__ uint32_t setup(Shared& S) {
       tc::mbar_init(tc::smem_u32(&S.full[s]), 1);
       tc::mbar_init(tc::smem_u32(&S.empty[s]), 1);
     }
-    for (int q = 0; q < kSlices; ++q) {
+    for (int q = 0; q < 2; ++q) {
       tc::mbar_init(tc::smem_u32(&S.acc_full[q]), 1);
       tc::mbar_init(tc::smem_u32(&S.acc_empty[q]), kEpiWarps);
     }
@@ -273,104 +295,129 @@ __device__ __forceinline__ void copy_loop(Shared& S, uint32_t base, Next next, i
   S.issued = it;
 }
 
+// The products of the orders [Q0, Q1) of one K block; `first`: the accumulators
+// start here. Unrolled: the descriptors become additions of constants, and the
+// issue keeps up with the 48 cycles that a 128 x 64 x 16 product takes (operand
+// reads); in a loop over the slice pairs it took 112.
+template <int Q0, int Q1>
+__device__ __forceinline__ void mma_orders(uint32_t tmem, uint64_t ad, uint64_t bd, bool first) {
+#pragma unroll
+  for (int q = Q0; q < Q1; ++q) {
+    const uint32_t d = tmem + (uint32_t)(q * kN);
+#pragma unroll
+    for (int a = 0; a <= q; ++a) {
+      const uint64_t da = ad + (uint64_t)(a * (kABytes >> 4)), db = bd + (uint64_t)((q - a) * (kBBytes >> 4));
+      tc::mma<1>(d, da, db, kIdesc, (first && a == 0) ? 0u : 1u);
+      tc::mma<1>(d, da + 2, db + 2, kIdesc, 1u);
+    }
+  }
+}
+
 // The MMA thread's loop: per K block the 28 slice products of the orders 0..6;
-// an order's accumulator is handed to the epilogue at the end of each chunk of
-// kChunkK and taken back before its next use.
+// a group of orders is handed to the epilogue at the end of each chunk of
+// kChunkK and taken back before its next use, so the epilogue reads one group
+// while the other's products run.
 template <class Next>
 __device__ __forceinline__ void mma_loop(Shared& S, uint32_t base, uint32_t tmem, Next next, int* err) {
   int it = 0, chunk = 0;
   Tile t;
+  auto give_up = [&](int code) {
+    atomicExch(err, code);
+    *(volatile int*)&S.abort_flag = 1;
+  };
   for (int i = 0; next(i, t); ++i) {
     for (int k = 0; k < t.nblk; ++k, ++it) {
       const int s = it % kStages, round = it / kStages;
       if (!wait_or_abort(tc::smem_u32(&S.full[s]), (uint32_t)(round & 1), &S.abort_flag)) {
-        atomicExch(err, tc::kErrTimeoutFull);
-        *(volatile int*)&S.abort_flag = 1;
+        give_up(tc::kErrTimeoutFull);
         return;
       }
-      tc::fence_after();
       const uint32_t a0 = base + s * kStageBytes;
       const uint64_t ad = sw64_desc(a0), bd = sw64_desc(a0 + kSlices * kABytes);
       const bool first = k % kStagesPerChunk == 0;
       const bool last = k % kStagesPerChunk == kStagesPerChunk - 1 || k == t.nblk - 1;
-// unrolled: the descriptors become additions of constants, and the issue keeps
-      // up with the 48 cycles that a 128 x 64 x 16 product takes (operand reads)
-#pragma unroll
-      for (int q = 0; q < kSlices; ++q) {
-        if (first && chunk > 0) {
-          if (!wait_or_abort(tc::smem_u32(&S.acc_empty[q]), (uint32_t)((chunk - 1) & 1), &S.abort_flag)) {
-            atomicExch(err, tc::kErrTimeoutAccum);
-            *(volatile int*)&S.abort_flag = 1;
-            return;
-          }
-          tc::fence_after();
-        }
-        const uint32_t d = tmem + (uint32_t)(q * kN);
-#pragma unroll
-        for (int a = 0; a <= q; ++a) {
-          const uint64_t da = ad + (uint64_t)(a * (kABytes >> 4)), db = bd + (uint64_t)((q - a) * (kBBytes >> 4));
-          tc::mma<1>(d, da, db, kIdesc, (first && a == 0) ? 0u : 1u);
-          tc::mma<1>(d, da + 2, db + 2, kIdesc, 1u);
-        }
-        if (last) tc::mma_commit(tc::smem_u32(&S.acc_full[q]));
+      const bool take = first && chunk > 0;
+      const uint32_t par = (uint32_t)((chunk - 1) & 1);
+      if (take && !wait_or_abort(tc::smem_u32(&S.acc_empty[0]), par, &S.abort_flag)) {
+        give_up(tc::kErrTimeoutAccum);
+        return;
       }
+      tc::fence_after();
+      mma_orders<0, 4>(tmem, ad, bd, first);
+      if (last) tc::mma_commit(tc::smem_u32(&S.acc_full[0]));
+      if (take && !wait_or_abort(tc::smem_u32(&S.acc_empty[1]), par, &S.abort_flag)) {
+        give_up(tc::kErrTimeoutAccum);
+        return;
+      }
+      tc::fence_after();
+      mma_orders<4, kSlices>(tmem, ad, bd, first);
+      if (last) tc::mma_commit(tc::smem_u32(&S.acc_full[1]));
       tc::mma_commit(tc::smem_u32(&S.empty[s]));
       if (last) ++chunk;
     }
   }
 }
 
-// A whole epilogue warp waits for order q of the chunk (uniform result).
-__device__ __forceinline__ bool epi_wait(Shared& S, int q, int chunk, int* err) {
-  const bool ok = wait_or_abort(tc::smem_u32(&S.acc_full[q]), (uint32_t)(chunk & 1), &S.abort_flag);
+// A whole epilogue warp waits for group g of the chunk (uniform result).
+__device__ __forceinline__ bool epi_wait(Shared& S, int g, int chunk, int* err) {
+  const bool ok = wait_or_abort(tc::smem_u32(&S.acc_full[g]), (uint32_t)(chunk & 1), &S.abort_flag);
   if (__all_sync(0xffffffffu, ok)) return true;
   atomicExch(err, tc::kErrTimeoutAccum);
   *(volatile int*)&S.abort_flag = 1;
   return false;
 }
 
-// All orders of one chunk, 32 columns (from column `col`) of the thread's row,
-// added to hi (orders 0..3) and lo (orders 4..6).
-__device__ __forceinline__ bool drain32(Shared& S, uint32_t tmem, int col, int chunk, long long (&hi)[32],
-                                        long long (&lo)[32], int* err) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col;
-#pragma unroll
-  for (int q = 0; q < kSlices; ++q) {
-    if (!epi_wait(S, q, chunk, err)) return false;
-    tc::fence_after();
-    float v[32];
-    tc::tmem_ld32(trow + (uint32_t)(q * kN), v);
-    tc::fence_before();
-    __syncwarp();
-    if (lane == 0) mbar_arrive(tc::smem_u32(&S.acc_empty[q]));
-#pragma unroll
-    for (int c = 0; c < 32; ++c) {
-      const int a = __float2int_rn(v[c]);
-      if (q < 4) hi[c] += (long long)a * (1 << (kDigit * (3 - q)));
-      else lo[c] += (long long)a * (1 << (kDigit * (6 - q)));
-    }
-  }
-  return true;
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
 }
 
-// The same for 8 columns of a single-chunk tile, without taking the accumulators back.
-__device__ __forceinline__ void read8(uint32_t tmem, int col, long long (&hi)[8], long long (&lo)[8]) {
-  const int warp = threadIdx.x >> 5;
-  const uint32_t trow = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)col;
+// The tile rows and columns of an epilogue thread: row (its tensor memory lane)
+// 32 (warp mod 4) + lane, columns [16 (warp / 4), ... + 16).
+__device__ __forceinline__ int epi_row() { return (int)(threadIdx.x & 127); }
+__device__ __forceinline__ int epi_col() { return (int)(threadIdx.x >> 7) * kCols; }
+
+// Adds one chunk's sums of the thread's 16 entries to hi (orders 0..3) and lo
+// (orders 4..6) and gives the accumulators back. False if a wait gave up.
+__device__ __forceinline__ bool drain(Shared& S, uint32_t tmem, int chunk, long long (&hi)[kCols],
+                                      long long (&lo)[kCols], int* err) {
+  const uint32_t t0 = tmem + ((uint32_t)((threadIdx.x >> 5) & 3) << 21) + (uint32_t)epi_col();
+  if (!epi_wait(S, 0, chunk, err)) return false;
+  tc::fence_after();
 #pragma unroll
-  for (int c = 0; c < 8; ++c) hi[c] = lo[c] = 0;
+  for (int c = 0; c < kCols; c += 4) {
+    uint32_t r[4][4];
 #pragma unroll
-  for (int q = 0; q < kSlices; ++q) {
-    float v[8];
-    tc::tmem_ld8(trow + (uint32_t)(q * kN), v);
+    for (int q = 0; q < 4; ++q) tmem_ld4(t0 + (uint32_t)(q * kN + c), r[q]);
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const int a = __float2int_rn(v[c]);
-      if (q < 4) hi[c] += (long long)a * (1 << (kDigit * (3 - q)));
-      else lo[c] += (long long)a * (1 << (kDigit * (6 - q)));
-    }
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        hi[c + i] += (long long)__float2int_rn(__uint_as_float(r[q][i])) * (1 << (kDigit * (3 - q)));
   }
+  tc::fence_before();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(tc::smem_u32(&S.acc_empty[0]));
+  if (!epi_wait(S, 1, chunk, err)) return false;
+  tc::fence_after();
+#pragma unroll
+  for (int c = 0; c < kCols; c += 4) {
+    uint32_t r[3][4];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) tmem_ld4(t0 + (uint32_t)((q + 4) * kN + c), r[q]);
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        lo[c + i] += (long long)__float2int_rn(__uint_as_float(r[q][i])) * (1 << (kDigit * (2 - q)));
+  }
+  tc::fence_before();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(tc::smem_u32(&S.acc_empty[1]));
+  return true;
 }
 
 }  // namespace sg
