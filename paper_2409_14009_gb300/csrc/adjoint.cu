@@ -10,16 +10,18 @@
 // supernode by supernode from the root down, with dense blocks:
 //   T    = L_JJ^{-1}
 //   Uhat = L_RJ T
-//   Z_RJ = -Z_RR Uhat          (Z_RR gathered from the ancestors through the
-//                               relative positions, the factor's scatter in
-//                               reverse)
+//   Z_RJ = -Z_RR Uhat          (Z_RR gathered from the ancestors by the factor's
+//                               assembly tasks in reverse)
 //   Z_JJ = T^T T - Uhat^T Z_RJ
 // Z is stored in the layout of the factor's panels (binary64, column-major).
+#include <algorithm>
 #include <cstring>
 #include <vector>
 
 #include "device.h"
 #include "mixed.h"
+#include "split_gemm.cuh"
+#include "diag_inv.cuh"
 
 namespace {
 
@@ -156,109 +158,171 @@ k_gen_reduce(const GenGemm* __restrict__ descs, const GemmTile* __restrict__ til
   }
 }
 
+// ---------------------------------------------------------------------------
+// The same grouped products on the tensor cores (split_gemm.cuh): first every
+// operand of the group is split (rows of A, columns of B; one exponent a row),
+// then the 128 x 64 tiles run. The FP64 pipe kept the tiles above at 97% of its
+// 2 FMAs per cycle and SM on busy SMs; they remain for handles with a memory
+// cap and devices without room for the slices.
+struct SplitOp {          // operand rows (i, k) at p[i rs + k ks], i < rows, k < K
+  const double* p;
+  int64_t rs, ks;
+  int64_t off, exp0;      // first slice row and first exponent in the workspace
+  int32_t rows, K, prows; // prows: rows per slice, whole tiles
+  int32_t mode;           // 0 general, 1 zero for k > i, 2 symmetric (k <= i stored), 3 zero for i > k
+};
+struct SplitTask {
+  int32_t op, r0;   // first of split_rows(K) rows
+};
+struct SplitTile {
+  int32_t desc, i0, j0, kb0, kb1, pad;   // product, tile origin, range of 32-column K blocks
+};
+
+__device__ __forceinline__ double split_el(const SplitOp& o, int i, int k) {
+  if (i >= o.rows || k >= o.K) return 0.0;
+  if (o.mode == 2) return k <= i ? o.p[i * o.rs + k * o.ks] : o.p[k * o.rs + i * o.ks];
+  if ((o.mode == 1 && k > i) || (o.mode == 3 && i > k)) return 0.0;
+  return o.p[i * o.rs + k * o.ks];
+}
+
+// 16 to 64 rows of an operand: a thread takes 8 consecutive columns of a row a
+// step, with the lanes along whichever index is contiguous (a symmetric operand
+// changes at the diagonal). Two passes, the second from L2.
+constexpr int kSplitOpThreads = sg::kSplitThreads;
+__global__ void __launch_bounds__(kSplitOpThreads)
+k_split_op(const SplitOp* __restrict__ ops, const SplitTask* __restrict__ tasks, unsigned char* __restrict__ slab,
+           int32_t* __restrict__ exps) {
+  __shared__ uint32_t hmax[64];
+  const SplitTask t = tasks[blockIdx.x];
+  const SplitOp o = ops[t.op];
+  const int tid = threadIdx.x;
+  const int rsh = sg::split_rows_log2(o.K), R = 1 << rsh, csh = sg::kSplitThreadsLog2 - rsh;
+  const int step = 8 << csh;   // columns a step
+  if (tid < 64) hmax[tid] = 0;
+  __syncthreads();
+  const bool kc = o.ks == 1 && o.rs != 1;
+  // (row, first column) of the thread in the step at column k0
+  auto place = [&](int k0, int& r, int& c) {
+    const bool kfast = o.mode == 2 ? (k0 >= t.r0 + R ? o.rs == 1 : kc) : kc;
+    r = kfast ? (tid >> csh) : (tid & (R - 1));
+    c = 8 * (kfast ? (tid & ((1 << csh) - 1)) : (tid >> rsh));
+  };
+#pragma unroll 2
+  for (int k0 = 0; k0 < o.K; k0 += step) {
+    int r, c;
+    place(k0, r, c);
+    uint32_t m = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) m = max(m, (uint32_t)__double2hiint(split_el(o, t.r0 + r, k0 + c + i)) & 0x7fffffffu);
+    if (m) atomicMax(&hmax[r], m);
+  }
+  __syncthreads();
+  if (tid < R) exps[o.exp0 + t.r0 + tid] = sg::row_exponent(hmax[tid]);
+  const int kend = (o.K + 31) / 32 * 32;
+  for (int k0 = 0; k0 < kend; k0 += step) {
+    int r, c;
+    place(k0, r, c);
+    if (k0 + c >= kend) continue;
+    const int32_t e = sg::row_exponent(hmax[r]);
+    double y[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) y[i] = e == sg::kExpNaN ? 0.0 : split_el(o, t.r0 + r, k0 + c + i);
+    uint4 w[sg::kSlices];
+    sg::digits8(y, e, w);
+    const int kb = (k0 + c) >> 5;
+    unsigned char* out = slab + (o.off + (int64_t)kb * sg::kSlices * o.prows) * 64 +
+                         sg::chunk_offset(t.r0 + r, (c >> 3) & 3);
+#pragma unroll
+    for (int q = 0; q < sg::kSlices; ++q) *reinterpret_cast<uint4*>(out + (int64_t)q * o.prows * 64) = w[q];
+  }
+}
+
+// Tiles of the group's products: operand 2 desc is A, 2 desc + 1 is B.
+__global__ void __launch_bounds__(sg::kThreads, 1)
+k_split_gemm(const GenGemm* __restrict__ descs, const SplitOp* __restrict__ ops, const SplitTile* __restrict__ tiles,
+             int ntiles, const unsigned char* __restrict__ slab, const int32_t* __restrict__ exps, int* err) {
+  extern __shared__ unsigned char sg_smem[];
+  __shared__ __align__(8) sg::Shared S;
+  const uint32_t base = (tc::smem_u32(sg_smem) + 1023u) & ~1023u;
+  const uint32_t tmem = sg::setup(S);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  auto next = [&](int i, sg::Tile& t) {
+    const int64_t q = blockIdx.x + (int64_t)i * gridDim.x;
+    if (q >= ntiles) return false;
+    const SplitTile k = tiles[q];
+    const SplitOp a = ops[2 * k.desc], b = ops[2 * k.desc + 1];
+    t.a = {slab + (a.off + (int64_t)k.kb0 * sg::kSlices * a.prows) * 64, exps + a.exp0, a.prows, k.i0};
+    t.b = {slab + (b.off + (int64_t)k.kb0 * sg::kSlices * b.prows) * 64, exps + b.exp0, b.prows, k.j0};
+    t.nblk = k.kb1 - k.kb0;
+    return true;
+  };
+  if (warp == sg::kEpiWarps) {
+    if (lane == 0) sg::copy_loop(S, base, next, err);
+  } else if (warp == sg::kEpiWarps + 1) {
+    if (lane == 0) sg::mma_loop(S, base, tmem, next, err);
+  } else {
+    sg::Tile t;
+    int chunk = 0;
+    bool ok = true;
+    for (int i = 0; ok && next(i, t); ++i) {
+      const SplitTile k = tiles[blockIdx.x + (int64_t)i * gridDim.x];
+      const GenGemm g = descs[k.desc];
+      const int r = k.i0 + sg::epi_row(), c0 = k.j0 + sg::epi_col();
+      const int n = r < g.M ? min(sg::kCols, (g.lower_c ? min(g.N, r + 1) : g.N) - c0) : 0;
+      const int32_t ea = n > 0 ? t.a.exps[r] : 0;
+      long long hi[sg::kCols], lo[sg::kCols];
+#pragma unroll
+      for (int c = 0; c < sg::kCols; ++c) hi[c] = lo[c] = 0;
+      for (int k0 = 0; ok && k0 < t.nblk; k0 += sg::kStagesPerChunk) ok = sg::drain(S, tmem, chunk++, hi, lo, err);
+      if (!ok) break;
+      double* C = g.C + r * g.cr + c0 * g.cc;
+#pragma unroll
+      for (int c = 0; c < sg::kCols; ++c)
+        if (c < n) {
+          double* p = C + c * g.cc;
+          const double v = g.alpha * sg::combine(hi[c], lo[c], ea, t.b.exps[c0 + c]);
+          *p = g.beta == 0.0 ? v : g.beta * *p + v;
+        }
+    }
+  }
+  __syncwarp();
+  sg::teardown(S, tmem);
+}
+
 struct InvTask {
   const double* src;
   int64_t lds;
   double* dst;
   int64_t ldt;
+  const double* inv;   // the factor's inverse of the block (64 x 64, leading dimension 64), or null
   int32_t kb, pad;
 };
 
-// Inverse of a kb x kb (kb <= 64) lower-triangular block (column-major,
-// leading dimensions lds / ldt): thread j computes column j of the inverse by
-// forward substitution on the unit vector e_j.
-__device__ __forceinline__ void inv64_body(const double* __restrict__ Lsrc, int64_t lds, int kb,
-                                           double* __restrict__ T, int64_t ldt) {
-  __shared__ double Ls[64 * 65];
-  for (int e = threadIdx.x; e < kb * kb; e += blockDim.x) {
-    const int r = e % kb, c = e / kb;
-    Ls[r + c * 65] = r >= c ? Lsrc[r + c * lds] : 0.0;
-  }
-  __syncthreads();
-  const int j = threadIdx.x;
-  if (j >= kb) return;
-  double x[64];
-#pragma unroll
-  for (int i = 0; i < 64; ++i) x[i] = 0.0;
-  for (int i = j; i < kb; ++i) {
-    double s = (i == j) ? 1.0 : 0.0;
-    for (int k = j; k < i; ++k) s -= Ls[i + k * 65] * x[k];
-    x[i] = s / Ls[i + i * 65];
-  }
-  for (int i = 0; i < kb; ++i) T[i + j * ldt] = i >= j ? x[i] : 0.0;
-}
-
-__global__ void k_inv64_grouped(const InvTask* __restrict__ tasks) {
+// Inverses of kb x kb (kb <= 64) lower-triangular blocks into T: a copy where the
+// factor has formed the inverse for the triangle solves, else by substitution.
+__global__ void __launch_bounds__(kInvThreads)
+k_inv64_grouped(const InvTask* __restrict__ tasks) {
+  __shared__ double Lk[64 * 65], rinv[64];
   const InvTask t = tasks[blockIdx.x];
-  inv64_body(t.src, t.lds, t.kb, t.dst, t.ldt);
-}
-
-// One gather task: the part of pair (J, K) with J's off-diagonal rows
-// u in [u0, u1) (at most kGatherRows of them).
-struct LevelPair {
-  int32_t J, K, c0, c1, u0, u1;
-};
-constexpr int kGatherRows = 512;
-constexpr int kGatherUnroll = 4;
-
-// Z_RR of every supernode J of a level (lower, column-major b x b, stored in the
-// update workspace at U_J's place), gathered from the ancestors' Z panels. A
-// task covers columns [c0, c1) of J's pair with K and a chunk of rows: it
-// stages struct(K) in shared memory, finds the positions of its rows by binary
-// search, then a warp per column copies 32 rows at a time, kGatherUnroll
-// (column, row chunk) items in flight per warp. Tasks write disjoint entries.
-__global__ void __launch_bounds__(kGT)
-k_gather_zrr_level(const LevelPair* __restrict__ pairs, const SnodeDev* __restrict__ sn,
-                   const int32_t* __restrict__ rows, const double* __restrict__ Z, double* __restrict__ U) {
-  extern __shared__ int32_t gsm2[];
-  const LevelPair pr = pairs[blockIdx.x];
-  const SnodeDev dj = sn[pr.J];
-  const SnodeDev dk = sn[pr.K];
-  const int b = dj.len - dj.s;
-  double* ZRR = U + dj.uoff;
-  int32_t* sK = gsm2;
-  int32_t* pos = gsm2 + dk.len;
-  const int32_t* rk = rows + dk.roff;
-  const int32_t* rj = rows + dj.roff + dj.s;
-  for (int i = threadIdx.x; i < dk.len; i += blockDim.x) sK[i] = rk[i];
-  __syncthreads();
-  const int nu = pr.u1 - pr.u0;
-  for (int i = threadIdx.x; i < nu; i += blockDim.x) {
-    const int32_t key = rj[pr.u0 + i];
-    int lo = 0, hi = dk.len;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (sK[mid] < key) lo = mid + 1; else hi = mid;
+  const int tid = threadIdx.x;
+  if (t.inv) {
+    for (int e = tid; e < 64 * t.kb; e += kInvThreads) {
+      const int r = e & 63, c = e >> 6;
+      if (r < t.kb) t.dst[r + c * t.ldt] = t.inv[r + 64 * c];
     }
-    pos[i] = lo;
+    return;
   }
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = kGT / 32;
-  const int nch = (nu + 31) >> 5, w = pr.c1 - pr.c0;
-  const int items = w * nch;
-  for (int i0 = warp; i0 < items; i0 += nw * kGatherUnroll) {
-    double v[kGatherUnroll];
-    int64_t dst[kGatherUnroll];
+  double x[16];
+  inv64_columns(t.src, t.lds, t.kb, Lk, rinv, x);
 #pragma unroll
-    for (int q = 0; q < kGatherUnroll; ++q) {
-      const int i = i0 + q * nw;
-      dst[q] = -1;
-      if (i < items) {
-        const int cc = i / nch;
-        const int c = pr.c0 + cc;
-        const int ui = (i - cc * nch) * 32 + lane;
-        const int u = pr.u0 + ui;
-        if (ui < nu && u >= c) {
-          v[q] = Z[dk.loff + (int64_t)(rj[c] - dk.f) * dk.ld + pos[ui]];
-          dst[q] = u + (int64_t)c * b;
-        }
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < kGatherUnroll; ++q)
-      if (dst[q] >= 0) ZRR[dst[q]] = v[q];
+  for (int mm = 0; mm < 16; ++mm) {
+    const int c = (tid & 3) + 4 * mm, g = tid >> 2;
+    if (c < t.kb && g < t.kb) t.dst[c + g * t.ldt] = x[mm];
   }
 }
+
+// Longest supernode structure the selected inverse takes (else CHOL_ENOTSUP).
+constexpr int kSelinvMaxLen = 200 * 1024 / 4 - 512;
 
 // g[t] = -(xbar_r . x_c + [r != c] xbar_c . x_r) + alpha (1 + [r != c]) Z(entry t)
 __global__ void k_adj_grad(const int32_t* __restrict__ rowind, const int32_t* __restrict__ colidx,
@@ -326,6 +390,7 @@ int ensure_adjoint(chol_handle* h) {
 // ones, the output tiles of the reduction.
 struct Group {
   int32_t tb = 0, tn = 0, rb = 0, rn = 0;
+  int32_t sb = 0, sn = 0, gb = 0, gn = 0;   // tensor cores: split tasks, tiles
   double flops = 0.0;
 };
 struct SiStep {
@@ -337,7 +402,7 @@ struct SiLevel {
   int64_t t_doubles;                    // T workspace of the level (zeroed first)
   std::vector<SiStep> steps;            // the L_JJ^{-1} recurrence, batched
   Group uh, zrj, zjj1, zjj2;
-  int32_t pair_b, pair_n;
+  int32_t level;                        // of the factor's schedule (its assembly tasks gather Z_RR)
   double gemm_flops;                    // Uhat, Z_RJ and Z_JJ products
 };
 
@@ -355,13 +420,22 @@ struct SiPlan {
   std::vector<GenGemm> descs;
   std::vector<GemmTile> tiles, rtiles;
   std::vector<InvTask> invs;
-  std::vector<LevelPair> pairs;
   int64_t part_max = 0;                 // partial-tile workspace (doubles)
+  // tensor cores: two operands per product, tasks, and the workspace of the largest group
+  std::vector<SplitOp> ops;
+  std::vector<SplitTask> stasks;
+  std::vector<SplitTile> stiles;
+  int64_t slab_rows = 0, nexps = 0;
+  bool sg = false;
+  SplitOp* d_ops = nullptr;
+  SplitTask* d_stasks = nullptr;
+  SplitTile* d_stiles = nullptr;
+  unsigned char* d_slab = nullptr;
+  int32_t* d_exps = nullptr;
   GenGemm* d_descs = nullptr;
   GemmTile* d_tiles = nullptr;
   GemmTile* d_rtiles = nullptr;
   InvTask* d_invs = nullptr;
-  LevelPair* d_pairs = nullptr;
   double* d_part = nullptr;
 };
 
@@ -409,8 +483,30 @@ Group emit_group(SiPlan& pl, const std::vector<GenGemm>& gs, int sms) {
   }
   if (best < base + 0.08) ksel = 1;
   int64_t part = 0;
+  gr.sb = (int32_t)pl.stasks.size();
+  gr.gb = (int32_t)pl.stiles.size();
+  int64_t srow = 0, sexp = 0;
   for (GenGemm g : gs) {
     if (g.M <= 0 || g.N <= 0) continue;
+    {
+      const int32_t d = (int32_t)pl.descs.size();
+      auto operand = [&](const double* p, int64_t rs, int64_t ks, int rows, int mode, int extra) {
+        SplitOp o{p, rs, ks, srow, sexp, rows, g.K, (rows + 63) / 64 * 64 + extra, mode};
+        for (int r0 = 0; r0 < rows; r0 += 1 << sg::split_rows_log2(g.K)) pl.stasks.push_back({(int32_t)pl.ops.size(), r0});
+        pl.ops.push_back(o);
+        srow += (int64_t)((g.K + 31) / 32) * sg::kSlices * o.prows;
+        sexp += o.prows;
+      };
+      operand(g.A, g.ar, g.ac, g.M, g.amode, 64);               // a 128-row tile may end 64 rows past
+      operand(g.B, g.bc, g.br, g.N, g.bmode == 1 ? 3 : 0, 0);   // rows: B's columns
+      for (int j0 = 0; j0 < g.N; j0 += sg::kN)
+        for (int i0 = 0; i0 < g.M; i0 += sg::kM) {
+          if (g.lower_c && i0 + sg::kM - 1 < j0) continue;
+          const int kend = g.amode == 1 ? std::min(g.K, i0 + sg::kM) : g.K;
+          const int kb0 = g.bmode == 1 ? j0 / sg::kBlockK : 0, kb1 = (kend + sg::kBlockK - 1) / sg::kBlockK;
+          pl.stiles.push_back({d, i0, j0, std::min(kb0, kb1 - 1), kb1, 0});
+        }
+    }
     gr.flops += gemm_flops(g);
     int ks = split_of(g, ksel);
     if (ks > 1) {
@@ -431,10 +527,32 @@ Group emit_group(SiPlan& pl, const std::vector<GenGemm>& gs, int sms) {
       }
     if (ks > 1) part += (int64_t)((g.M + kGTile - 1) / kGTile) * ntj * ks * kGTile * kGTile;
   }
+  // long sums first, so that the last tiles of the launch are short ones
+  std::stable_sort(pl.stiles.begin() + gr.gb, pl.stiles.end(),
+                   [](const SplitTile& x, const SplitTile& y) { return x.kb1 - x.kb0 > y.kb1 - y.kb0; });
+  gr.sn = (int32_t)pl.stasks.size() - gr.sb;
+  gr.gn = (int32_t)pl.stiles.size() - gr.gb;
+  pl.slab_rows = std::max(pl.slab_rows, srow);
+  pl.nexps = std::max(pl.nexps, sexp);
   gr.tn = (int32_t)pl.tiles.size() - gr.tb;
   gr.rn = (int32_t)pl.rtiles.size() - gr.rb;
   pl.part_max = std::max(pl.part_max, part);
   return gr;
+}
+
+void free_si_split(chol_handle* h, SiPlan* pl) {
+  auto drop = [&](auto** p, int64_t bytes) {
+    if (*p) {
+      cudaFree(*p);
+      h->dev->bytes -= bytes;
+    }
+    *p = nullptr;
+  };
+  drop(&pl->d_ops, (int64_t)(sizeof(SplitOp) * pl->ops.size()));
+  drop(&pl->d_stasks, (int64_t)(sizeof(SplitTask) * pl->stasks.size()));
+  drop(&pl->d_stiles, (int64_t)(sizeof(SplitTile) * pl->stiles.size()));
+  drop(&pl->d_slab, pl->slab_rows * 64);
+  drop(&pl->d_exps, (int64_t)(sizeof(int32_t) * pl->nexps));
 }
 
 int build_si_plan(chol_handle* h) {
@@ -469,11 +587,12 @@ int build_si_plan(chol_handle* h) {
   if ((rc = chol_dalloc(h, (void**)&D->Tw, sizeof(double) * (size_t)std::max<int64_t>(tmax, 1)))) return rc;
   if ((rc = chol_dalloc(h, (void**)&D->Uh, sizeof(double) * (size_t)std::max<int64_t>(hmax, 1)))) return rc;
   if ((rc = chol_dalloc(h, (void**)&D->Ww, sizeof(double) * (size_t)std::max<int64_t>(wmax, 1)))) return rc;
-  std::vector<std::vector<int64_t>> pairs_of(h->ns);
-  for (size_t p = 0; p < h->rel_J.size(); ++p) pairs_of[h->rel_J[p]].push_back((int64_t)p);
+  std::vector<int32_t> fbase(h->ns, -1);   // first block of J in the solve's inverses
+  for (const TriItemHost& q : h->tri_items) fbase[q.J] = q.fbase;
   for (int lv = h->nlevels - 1; lv >= 0; --lv) {
     const LevelPlan& P = h->levels[lv];
     SiLevel sl{};
+    sl.level = lv;
     std::vector<int32_t> Js(h->level_snodes.begin() + P.snode_b, h->level_snodes.begin() + P.snode_b + P.snode_n);
     int maxnbk = 0;
     int64_t tl = 0;
@@ -495,7 +614,8 @@ int build_si_plan(chol_handle* h) {
         double* T = D->Tw + toff[J];
         for (int k0 = 0; k0 < d.s; k0 += 64) {
           const int kb = std::min(64, d.s - k0);
-          pl->invs.push_back({L + d.loff + k0 + (int64_t)k0 * d.ld, d.ld, T + k0 + (int64_t)k0 * d.s, d.s, kb, 0});
+          const double* inv = fbase[J] < 0 ? nullptr : (const double*)D->dinv + (int64_t)(fbase[J] + k0 / 64) * 4096;
+          pl->invs.push_back({L + d.loff + k0 + (int64_t)k0 * d.ld, d.ld, T + k0 + (int64_t)k0 * d.s, d.s, inv, kb, 0});
           st.flops += (double)kb * kb * kb / 3.0;
         }
       }
@@ -534,18 +654,6 @@ int build_si_plan(chol_handle* h) {
                         0.0, 0, 1, 0));
     }
     sl.uh = emit_group(*pl, gs, D->sms);
-    // Z_RR gather pairs
-    sl.pair_b = (int32_t)pl->pairs.size();
-    for (int32_t J : Js)
-      for (int64_t p : pairs_of[J]) {
-        const SnodeDev& d = h->snodes[J];
-        const int32_t b = d.len - d.s;
-        // rows u >= c0 of J are the ones in K (and later ancestors' rows are
-        // in struct(K) too); chunks of kGatherRows
-        for (int32_t u0 = h->rel_c0[p]; u0 < b; u0 += kGatherRows)
-          pl->pairs.push_back({J, h->rel_K[p], h->rel_c0[p], h->rel_c1[p], u0, std::min(b, u0 + kGatherRows)});
-      }
-    sl.pair_n = (int32_t)pl->pairs.size() - sl.pair_b;
     // Z_RJ = -Z_RR Uhat  (Z_RR at U_J's place in the update workspace)
     gs.clear();
     for (int32_t J : Js) {
@@ -584,13 +692,23 @@ int build_si_plan(chol_handle* h) {
     return CHOL_OK;
   };
   if ((rc = up(&pl->d_descs, pl->descs))) return rc;
-  if ((rc = up(&pl->d_tiles, pl->tiles))) return rc;
-  if ((rc = up(&pl->d_rtiles, pl->rtiles))) return rc;
-  if (pl->part_max > 0 && (rc = chol_dalloc(h, (void**)&pl->d_part, sizeof(double) * (size_t)pl->part_max))) return rc;
-  if ((rc = up(&pl->d_invs, pl->invs))) return rc;
-  if ((rc = up(&pl->d_pairs, pl->pairs))) return rc;
+  // the tensor-core form where its slices find room (as for the factor's updates)
   D->si_plan = pl;
-  CHOL_CUDA_TRY(cudaFuncSetAttribute(k_gather_zrr_level, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+  if (h->opt.device_mem_cap == 0 && D->sg_ready == 1 && !pl->stiles.empty()) {
+    pl->sg = up(&pl->d_ops, pl->ops) == CHOL_OK && up(&pl->d_stasks, pl->stasks) == CHOL_OK &&
+             up(&pl->d_stiles, pl->stiles) == CHOL_OK &&
+             chol_dalloc(h, (void**)&pl->d_slab, (size_t)pl->slab_rows * 64) == CHOL_OK &&
+             chol_dalloc(h, (void**)&pl->d_exps, sizeof(int32_t) * (size_t)pl->nexps) == CHOL_OK &&
+             cudaFuncSetAttribute(k_split_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, sg::kSmemBytes) ==
+                 cudaSuccess;
+    if (!pl->sg) free_si_split(h, pl);
+  }
+  if (!pl->sg) {
+    if ((rc = up(&pl->d_tiles, pl->tiles))) return rc;
+    if ((rc = up(&pl->d_rtiles, pl->rtiles))) return rc;
+    if (pl->part_max > 0 && (rc = chol_dalloc(h, (void**)&pl->d_part, sizeof(double) * (size_t)pl->part_max))) return rc;
+  }
+  if ((rc = up(&pl->d_invs, pl->invs))) return rc;
   return CHOL_OK;
 }
 
@@ -598,31 +716,37 @@ int build_si_plan(chol_handle* h) {
 // root, every supernode of a level at once.
 int selinv(chol_handle* h, cudaStream_t st) {
   if (h->selinv_valid) return CHOL_OK;
-  // the Z_RR gather stages struct(K) and the positions in shared memory
-  if ((int64_t)(h->max_len + kGatherRows) * (int64_t)sizeof(int32_t) > 200 * 1024) return CHOL_ENOTSUP;
+  if (h->max_len > kSelinvMaxLen) return CHOL_ENOTSUP;
   int rc = ensure_adjoint(h);
   if (rc) return rc;
   if ((rc = build_si_plan(h))) return rc;
   DeviceState* D = h->dev;
   SiPlan* pl = (SiPlan*)D->si_plan;
   auto launch = [&](const Group& gr) {
+    if (pl->sg) {
+      if (gr.gn == 0) return;
+      k_split_op<<<gr.sn, kSplitOpThreads, 0, st>>>(pl->d_ops, pl->d_stasks + gr.sb, pl->d_slab, pl->d_exps);
+      k_split_gemm<<<std::min(gr.gn, D->sms), sg::kThreads, sg::kSmemBytes, st>>>(
+          pl->d_descs, pl->d_ops, pl->d_stiles + gr.gb, gr.gn, pl->d_slab, pl->d_exps, D->sg_err);
+      return;
+    }
     if (gr.tn > 0) k_gen_gemm_grouped<<<gr.tn, kGT, 0, st>>>(pl->d_descs, pl->d_tiles + gr.tb, pl->d_part);
     if (gr.rn > 0) k_gen_reduce<<<gr.rn, kGT, 0, st>>>(pl->d_descs, pl->d_rtiles + gr.rb, pl->d_part);
   };
-  auto nl = [](const Group& gr) { return (gr.tn > 0) + (gr.rn > 0); };
+  auto nl = [&](const Group& gr) { return pl->sg ? 2 * (gr.gn > 0) : (gr.tn > 0) + (gr.rn > 0); };
   for (const SiLevel& sl : pl->levels) {
     CHOL_CUDA_TRY(cudaMemsetAsync(D->Tw, 0, sizeof(double) * (size_t)sl.t_doubles, st));
     for (const SiStep& q : sl.steps) {
       KScope ks(h, CHOL_K_SELINV_INV, st, q.flops, 0.0);
       ks.launches((q.inv_n > 0) + nl(q.g1) + nl(q.g2));
-      if (q.inv_n > 0) k_inv64_grouped<<<q.inv_n, 64, 0, st>>>(pl->d_invs + q.inv_b);
+      if (q.inv_n > 0) k_inv64_grouped<<<q.inv_n, kInvThreads, 0, st>>>(pl->d_invs + q.inv_b);
       launch(q.g1);
       launch(q.g2);
     }
-    if (sl.pair_n > 0) {
-      KScope ks(h, CHOL_K_SELINV_GATHER, st, 0.0, 0.0);
-      k_gather_zrr_level<<<sl.pair_n, kGT, sizeof(int32_t) * (h->max_len + kGatherRows), st>>>(pl->d_pairs + sl.pair_b, D->sn,
-                                                                                   D->rows, D->Zp, D->zrr_ws ? D->zrr_ws : D->U);
+    if (const LevelPlan& P = h->levels[sl.level]; P.asm_n + P.asmw_n > 0) {
+      KScope ks(h, CHOL_K_SELINV_GATHER, st, 0.0, 16.0 * P.asm_entries);
+      ks.launches((P.asm_n > 0) + (P.asmw_n > 0));
+      chol_gather_zrr(h, P, D->Zp, D->zrr_ws ? D->zrr_ws : D->U, st);
     }
     {
       KScope ks(h, CHOL_K_SELINV_GEMM, st, sl.gemm_flops, 0.0);
@@ -644,7 +768,8 @@ void chol_adjoint_free(chol_handle* h) {
   DeviceState* D = h->dev;
   if (!D || !D->si_plan) return;
   SiPlan* pl = (SiPlan*)D->si_plan;
-  void* ptrs[] = {pl->d_descs, pl->d_tiles, pl->d_rtiles, pl->d_invs, pl->d_pairs, pl->d_part};
+  void* ptrs[] = {pl->d_descs, pl->d_tiles, pl->d_rtiles, pl->d_invs, pl->d_part,
+                  pl->d_ops, pl->d_stasks, pl->d_stiles, pl->d_slab, pl->d_exps};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete pl;

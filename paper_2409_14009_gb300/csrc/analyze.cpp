@@ -669,7 +669,7 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
           z.srow0 = se;
           so += (int64_t)z.sblk * kSplitSlices * z.srows;
           se += z.srows;
-          for (int32_t r0 = 0; r0 < b; r0 += 64) h->split_tasks.push_back({J, 0, r0, 0});
+          for (int32_t r0 = 0; r0 < b; r0 += d.s <= 64 ? 64 : (d.s <= 128 ? 32 : 16)) h->split_tasks.push_back({J, 0, r0, 0});   // sg::split_rows_log2
           for (int32_t c0 = 0; c0 < b; c0 += kTile)
             for (int32_t r0 = c0; r0 < b; r0 += 2 * kTile) h->sgs_tasks.push_back({J, 0, r0, c0});
         }

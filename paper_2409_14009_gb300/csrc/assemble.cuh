@@ -11,6 +11,7 @@
 // fixed order, exactly as in the CTA-sized tasks.
 #pragma once
 #include <cstdint>
+#include <type_traits>
 
 #include "internal.h"
 #include "bounds.cuh"
@@ -19,13 +20,16 @@ constexpr int kAsmWarpUnroll = 4;
 
 // One warp, one task. ROWMAJOR: U_J row-major (ld = b rounded up to 8) and
 // row-major panels (the binary32 modes); else U_J column-major (ld = b) and
-// column-major panels (binary64). sK and pos: kAsmWarpPos ints each, private to
-// the warp.
-template <class T, bool ROWMAJOR>
+// column-major panels (binary64). GATHER: the other way round, U_J's entries are
+// copied from K's panel (the selected inverse's Z_RR: the same tasks cover every
+// entry of U_J once). sK and pos: kAsmWarpPos ints each, private to the warp.
+template <class T, bool ROWMAJOR, bool GATHER = false>
 __device__ __forceinline__ void assemble_warp_task(const AsmTask& t, const AsmSeg* __restrict__ segs,
                                                    const SnodeDev* __restrict__ sn,
-                                                   const int32_t* __restrict__ rows, const T* __restrict__ U,
-                                                   T* __restrict__ L, int32_t* sK, int32_t* pos) {
+                                                   const int32_t* __restrict__ rows,
+                                                   typename std::conditional<GATHER, T, const T>::type* __restrict__ U,
+                                                   typename std::conditional<GATHER, const T, T>::type* __restrict__ L,
+                                                   int32_t* sK, int32_t* pos) {
   const int lane = threadIdx.x & 31;
 #ifdef CHOL_BOUNDS_CHECK
   if (!CHOL_BC(t.K >= 0 && t.K < bc_lim.ns, kBcTaskTarget)) return;
@@ -40,7 +44,7 @@ __device__ __forceinline__ void assemble_warp_task(const AsmTask& t, const AsmSe
 #endif
   const int32_t* rk = rows + dk.roff + t.p0;
   for (int i = lane; i < np; i += 32) sK[i] = rk[i];
-  T* Lk = L + dk.loff;
+  auto* Lk = L + dk.loff;
   for (int g = t.seg_begin; g < t.seg_end; ++g) {
     const AsmSeg sg = segs[g];
 #ifdef CHOL_BOUNDS_CHECK
@@ -70,12 +74,12 @@ __device__ __forceinline__ void assemble_warp_task(const AsmTask& t, const AsmSe
 #endif
     }
     __syncwarp();
-    const T* Uj = U + dj.uoff;
+    auto* Uj = U + dj.uoff;
     const int ldu = ROWMAJOR ? ((b + 7) & ~7) : b;
     const int total = nu * w;
     for (int e0 = lane; e0 < total; e0 += 32 * kAsmWarpUnroll) {
       T v[kAsmWarpUnroll], l[kAsmWarpUnroll];
-      int64_t off[kAsmWarpUnroll];
+      int64_t off[kAsmWarpUnroll], src[kAsmWarpUnroll];
 #pragma unroll
       for (int q = 0; q < kAsmWarpUnroll; ++q) {
         const int e = e0 + 32 * q;
@@ -91,7 +95,8 @@ __device__ __forceinline__ void assemble_warp_task(const AsmTask& t, const AsmSe
             if (!CHOL_BC(col >= 0 && col < dk.s, kBcTargetCol) || pos[ui] < 0) continue;
 #endif
             off[q] = ROWMAJOR ? (int64_t)pos[ui] * dk.ld + col : col * dk.ld + pos[ui];
-            v[q] = ROWMAJOR ? Uj[(int64_t)u * ldu + c] : Uj[(int64_t)c * ldu + u];
+            src[q] = ROWMAJOR ? (int64_t)u * ldu + c : (int64_t)c * ldu + u;
+            if (!GATHER) v[q] = Uj[src[q]];
           }
         }
       }
@@ -100,20 +105,24 @@ __device__ __forceinline__ void assemble_warp_task(const AsmTask& t, const AsmSe
         if (off[q] >= 0) l[q] = Lk[off[q]];
 #pragma unroll
       for (int q = 0; q < kAsmWarpUnroll; ++q)
-        if (off[q] >= 0) Lk[off[q]] = l[q] - v[q];
+        if (off[q] >= 0) {
+          if constexpr (GATHER) Uj[src[q]] = l[q];
+          else Lk[off[q]] = l[q] - v[q];
+        }
     }
   }
 }
 
 // One launch of warp tasks: blockDim.x / 32 tasks per CTA.
-template <class T, bool ROWMAJOR>
+template <class T, bool ROWMAJOR, bool GATHER = false>
 __global__ void __launch_bounds__(256)
 k_assemble_warp(const AsmTask* __restrict__ tasks, int ntasks, const AsmSeg* __restrict__ segs,
-                const SnodeDev* __restrict__ sn, const int32_t* __restrict__ rows, const T* __restrict__ U,
-                T* __restrict__ L) {
+                const SnodeDev* __restrict__ sn, const int32_t* __restrict__ rows,
+                typename std::conditional<GATHER, T, const T>::type* __restrict__ U,
+                typename std::conditional<GATHER, const T, T>::type* __restrict__ L) {
   __shared__ int32_t wsm[8][2 * kAsmWarpPos];
   const int warp = threadIdx.x >> 5;
   const int i = blockIdx.x * (blockDim.x >> 5) + warp;
   if (i >= ntasks) return;
-  assemble_warp_task<T, ROWMAJOR>(tasks[i], segs, sn, rows, U, L, wsm[warp], wsm[warp] + kAsmWarpPos);
+  assemble_warp_task<T, ROWMAJOR, GATHER>(tasks[i], segs, sn, rows, U, L, wsm[warp], wsm[warp] + kAsmWarpPos);
 }

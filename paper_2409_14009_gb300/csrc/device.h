@@ -36,21 +36,23 @@ struct DeviceState {
   TileTask* sg_split = nullptr;
   TileTask* sg_syrk = nullptr;
   TileTask* sg_trail = nullptr;
-  int32_t* sg_err = nullptr;    // a tile gave up waiting
   int4* rlb_pairs = nullptr;    // RLB: (K, c0, c1, -) of every (J, K) pair, J-major
   int32_t* rlb_pbeg = nullptr;  // RLB: first pair of every supernode
   double* zrr_ws = nullptr;     // adjoint: Z_RR workspace when there is no update workspace (RLB)
   int32_t* tri_flags = nullptr; // solve: one flag per diagonal block and chunk column (zeroed once)
   void* dinv = nullptr;         // per 64-row diagonal block of the solve: binary64 L_ii^{-1}; mixed modes: L_ii^{-1} and two products (binary32)
   int32_t* tri_sync = nullptr;  // solve: {epoch, CTAs done} of the triangle launches
-  int32_t* sv_err = nullptr;    // solve: set when a bounded wait gave up
+  // error words beside the status word (read back together): a bounded wait of
+  // the triangle solve, or of a slice-product tile, gave up
+  int32_t* sv_err = nullptr;
+  int32_t* sg_err = nullptr;
   int32_t* ssmall = nullptr;
   TileTask* bpanel = nullptr;
   TileTask* gemv = nullptr;
   TileTask* bpart = nullptr;
   TileTask* bred = nullptr;
   int32_t* perm = nullptr;
-  int32_t* status = nullptr;    // device status word (first failing column + 1)
+  int32_t* status = nullptr;    // device words: first failing column + 1, sv_err, sg_err
   int32_t* status_host = nullptr;  // pinned
   double* part = nullptr;       // logdet partial sums (one per supernode)
   double* split_part = nullptr; // binary64 solve: partial sums of split panel products (split_slots_max x 64 x chunk)
@@ -207,5 +209,5 @@ int chol_dalloc(chol_handle* h, void** p, size_t bytes);
 int chol_sg_ensure(chol_handle* h);
 void chol_sg_release(chol_handle* h);
 void chol_sg_trailing(chol_handle* h, const TileTask* tasks, int n, int grid, int buf, cudaStream_t st);
+void chol_gather_zrr(chol_handle* h, const LevelPlan& P, const double* Z, double* ZRR, cudaStream_t st);
 void chol_sg_syrk(chol_handle* h, const LevelPlan& P, cudaStream_t st);
-int chol_sg_status(chol_handle* h);

@@ -449,11 +449,15 @@ k_syrk_rlb(const SnodeDev* __restrict__ sn, const TileTask* __restrict__ tasks, 
 // with all loads issued before the stores. Every entry of U_J hits a distinct
 // entry of K (relind is injective) and a barrier separates segments, so the
 // contributions to one entry are applied in a fixed order.
+// GATHER: U_J's entries are copied from K's panel instead (see assemble.cuh).
 constexpr int kAsmUnroll = 4;
 
+template <bool GATHER = false>
 __device__ __forceinline__ void assemble_body(const AsmTask& t, const AsmSeg* __restrict__ segs,
                                               const SnodeDev* __restrict__ sn, const int32_t* __restrict__ rows,
-                                              const double* __restrict__ U, double* __restrict__ L, int32_t* ssm) {
+                                              typename std::conditional<GATHER, double, const double>::type* __restrict__ U,
+                                              typename std::conditional<GATHER, const double, double>::type* __restrict__ L,
+                                              int32_t* ssm) {
   __shared__ int32_t tcol[kAsmCols];
 #ifdef CHOL_BOUNDS_CHECK
   if (!CHOL_BC(t.K >= 0 && t.K < bc_lim.ns, kBcTaskTarget)) return;
@@ -507,13 +511,13 @@ __device__ __forceinline__ void assemble_body(const AsmTask& t, const AsmSeg* __
 #endif
     }
     __syncthreads();
-    const double* Uj = U + dj.uoff;
-    double* Lk = L + dk.loff;
+    auto* Uj = U + dj.uoff;
+    auto* Lk = L + dk.loff;
     const int nch = (nu + 31) >> 5;
     const int items = w * nch;   // (column, 32-row chunk) pairs
     for (int i0 = warp; i0 < items; i0 += nwarps * kAsmUnroll) {
       double v[kAsmUnroll], l[kAsmUnroll];
-      int64_t off[kAsmUnroll];
+      int64_t off[kAsmUnroll], src[kAsmUnroll];
 #pragma unroll
       for (int q = 0; q < kAsmUnroll; ++q) {
         const int i = i0 + q * nwarps;
@@ -527,7 +531,8 @@ __device__ __forceinline__ void assemble_body(const AsmTask& t, const AsmSeg* __
             if (tcol[cc] < 0 || pos[u - sg.ua] < 0) continue;
 #endif
             off[q] = (int64_t)tcol[cc] * dk.ld + pos[u - sg.ua];
-            v[q] = Uj[(int64_t)c * b + u];
+            src[q] = (int64_t)c * b + u;
+            if (!GATHER) v[q] = Uj[src[q]];
           }
         }
       }
@@ -536,7 +541,10 @@ __device__ __forceinline__ void assemble_body(const AsmTask& t, const AsmSeg* __
         if (off[q] >= 0) l[q] = Lk[off[q]];
 #pragma unroll
       for (int q = 0; q < kAsmUnroll; ++q)
-        if (off[q] >= 0) Lk[off[q]] = l[q] - v[q];
+        if (off[q] >= 0) {
+          if constexpr (GATHER) Uj[src[q]] = l[q];
+          else Lk[off[q]] = l[q] - v[q];
+        }
     }
   }
 }
@@ -546,7 +554,15 @@ k_assemble(const AsmTask* __restrict__ tasks, const AsmSeg* __restrict__ segs,
            const SnodeDev* __restrict__ sn, const int32_t* __restrict__ rows,
            const double* __restrict__ U, double* __restrict__ L) {
   extern __shared__ int32_t ssm[];
-  assemble_body(tasks[blockIdx.x], segs, sn, rows, U, L, ssm);
+  assemble_body<false>(tasks[blockIdx.x], segs, sn, rows, U, L, ssm);
+}
+
+// Z_RR of a level's CTA-sized tasks (the selected inverse).
+__global__ void __launch_bounds__(kAsmThreads)
+k_gather_zrr(const AsmTask* __restrict__ tasks, const AsmSeg* __restrict__ segs, const SnodeDev* __restrict__ sn,
+             const int32_t* __restrict__ rows, double* __restrict__ ZRR, const double* __restrict__ Z) {
+  extern __shared__ int32_t ssm[];
+  assemble_body<true>(tasks[blockIdx.x], segs, sn, rows, ZRR, Z, ssm);
 }
 
 // Persistent form for problems whose supernodes all take the one-CTA kernel
@@ -571,7 +587,7 @@ k_persist_factor(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ sm
     grid.sync();
     for (int i = blockIdx.x; i < p.asm_n; i += gridDim.x) {
       __syncthreads();
-      assemble_body(tasks[p.asm_b + i], segs, sn, rows, U, L, reinterpret_cast<int32_t*>(psm));
+      assemble_body<false>(tasks[p.asm_b + i], segs, sn, rows, U, L, reinterpret_cast<int32_t*>(psm));
     }
     {
       // warp-sized tasks: one per warp of the grid, each warp in its own slice
@@ -736,12 +752,12 @@ void chol_device_free(chol_handle* h) {
   chol_adjoint_free(h);
   void* ptrs[] = {D->L, D->U, D->sn, D->rows, D->amap, D->small_list, D->potrf_list,
                   D->level_snodes, D->trsm, D->gemm, D->syrk, D->asm_tasks, D->asm_segs, D->tri, D->rlb_pairs, D->rlb_pbeg, D->zrr_ws,
-                  D->tri_flags, D->tri_sync, D->sv_err, D->bpanel, D->gemv, D->bpart, D->bred, D->P32, D->plevels, D->vals, D->sys_snode, D->sys_out,
+                  D->tri_flags, D->tri_sync, D->bpanel, D->gemv, D->bpart, D->bred, D->P32, D->plevels, D->vals, D->sys_snode, D->sys_out,
                   D->ssmall, D->Zp, D->Tw, D->Ww, D->Uh, D->a_col, D->a_row, D->adj_xb, D->perm, D->status, D->part, D->scalar_dev, D->Y, D->W,
                   D->mx_diagpos, D->mx_aij, D->mx_d, D->mx_fallbacks, D->csr_ptr, D->csr_col, D->csr_src,
                   D->csr_val, D->Lbf, D->tmaps, D->tc_err, D->R, D->Z, D->Pv, D->Q, D->red, D->Y32, D->W32,
                   D->rhs_scale, D->host_vals, D->host_rhs, D->panel, D->pflags, D->dinv, D->split_part, D->split_cnt, D->hand32, D->sg_slab, D->sg_exps, D->sgt_slab[0], D->sgt_slab[1],
-                  D->sgt_exps[0], D->sgt_exps[1], D->sg_dev, D->sg_split, D->sg_syrk, D->sg_trail, D->sg_err, D->rdiag};
+                  D->sgt_exps[0], D->sgt_exps[1], D->sg_dev, D->sg_split, D->sg_syrk, D->sg_trail, D->rdiag};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (D->status_host) cudaFreeHost(D->status_host);
@@ -838,10 +854,12 @@ int chol_device_ensure(chol_handle* h) {
     if (cudaMemset(D->split_cnt, 0, sizeof(int32_t) * slots) != cudaSuccess) return fail(CHOL_ECUDA);
   }
   if ((rc = chol_dalloc(h, (void**)&D->tri_sync, sizeof(int32_t) * 2))) return fail(rc);
-  if ((rc = chol_dalloc(h, (void**)&D->sv_err, sizeof(int32_t)))) return fail(rc);
+  if ((rc = chol_dalloc(h, (void**)&D->status, 4 * sizeof(int32_t)))) return fail(rc);
+  D->sv_err = D->status + 1;
+  D->sg_err = D->status + 2;
   if (cudaMemset(D->tri_flags, 0, sizeof(int32_t) * nflags) != cudaSuccess ||
       cudaMemset(D->tri_sync, 0, sizeof(int32_t) * 2) != cudaSuccess ||
-      cudaMemset(D->sv_err, 0, sizeof(int32_t)) != cudaSuccess)
+      cudaMemset(D->status, 0, 4 * sizeof(int32_t)) != cudaSuccess)
     return fail(CHOL_ECUDA);
   if ((rc = upload(h, &D->ssmall, h->ssmall_list))) return fail(rc);
   if ((rc = upload(h, &D->bpanel, h->bpanel_tasks))) return fail(rc);
@@ -850,13 +868,12 @@ int chol_device_ensure(chol_handle* h) {
   if ((rc = upload(h, &D->bred, h->bred_tasks))) return fail(rc);
   if ((rc = upload(h, &D->plevels, h->persist_levels))) return fail(rc);
   if ((rc = upload(h, &D->perm, h->perm))) return fail(rc);
-  if ((rc = chol_dalloc(h, (void**)&D->status, sizeof(int32_t)))) return fail(rc);
   if ((rc = chol_dalloc(h, (void**)&D->part, sizeof(double) * (size_t)std::max(h->ns, 1)))) return fail(rc);
   if ((rc = chol_dalloc(h, (void**)&D->scalar_dev, sizeof(double)))) return fail(rc);
   if (h->opt.precision == CHOL_PREC_FP64 && h->n_large > 0 &&
       (rc = chol_dalloc(h, (void**)&D->rdiag, sizeof(double) * (size_t)h->n)))
     return fail(rc);
-  if (cudaMallocHost((void**)&D->status_host, 4 * sizeof(int32_t)) != cudaSuccess) return fail(CHOL_ENOMEM);
+  if (cudaMallocHost((void**)&D->status_host, 8 * sizeof(int32_t)) != cudaSuccess) return fail(CHOL_ENOMEM);
   if (cudaMallocHost((void**)&D->scalar_host, sizeof(double)) != cudaSuccess) return fail(CHOL_ENOMEM);
   static bool attrs_done = false;
   if (!attrs_done) {
@@ -1022,6 +1039,22 @@ int enqueue_factor_fp64(chol_handle* h, const double* values, cudaStream_t st) {
   return CHOL_OK;
 }
 
+}  // namespace
+
+// Z_RR of every supernode of a level (at U_J's place in ZRR), gathered from the
+// ancestors' panels of Z.
+void chol_gather_zrr(chol_handle* h, const LevelPlan& P, const double* Z, double* ZRR, cudaStream_t st) {
+  DeviceState* D = h->dev;
+  if (P.asm_n > 0)
+    k_gather_zrr<<<P.asm_n, kAsmThreads, sizeof(int32_t) * 2 * kAsmPos, st>>>(D->asm_tasks + P.asm_b, D->asm_segs, D->sn,
+                                                                             D->rows, ZRR, Z);
+  if (P.asmw_n > 0)
+    k_assemble_warp<double, false, true><<<(P.asmw_n + 7) / 8, 256, 0, st>>>(D->asm_tasks + P.asm_b + P.asm_n, P.asmw_n,
+                                                                             D->asm_segs, D->sn, D->rows, ZRR, Z);
+}
+
+namespace {
+
 int enqueue_factor(chol_handle* h, const double* values, cudaStream_t st) {
   if (h->opt.precision == CHOL_PREC_FP64) return enqueue_factor_fp64(h, values, st);   // inverses inside
   const int rc = chol_enqueue_factor_mixed(h, values, st);
@@ -1161,15 +1194,13 @@ extern "C" int chol_factor(chol_handle* h, const double* values, void* stream) {
 int chol_finish_factor(chol_handle* h, cudaStream_t st) {
   DeviceState* D = h->dev;
   CHOL_CUDA_TRY(cudaGetLastError());
-  CHOL_CUDA_TRY(cudaMemcpyAsync(D->status_host, D->status, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+  CHOL_CUDA_TRY(cudaMemcpyAsync(D->status_host, D->status, 3 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   if (h->opt.precision != CHOL_PREC_FP64)
-    CHOL_CUDA_TRY(cudaMemcpyAsync(&D->status_host[1], D->mx_fallbacks, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-  else if (D->sg_ready == 1)
-    CHOL_CUDA_TRY(cudaMemcpyAsync(&D->status_host[3], D->sg_err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    CHOL_CUDA_TRY(cudaMemcpyAsync(&D->status_host[4], D->mx_fallbacks, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   CHOL_CUDA_TRY(cudaStreamSynchronize(st));
   if (h->opt.precision != CHOL_PREC_FP64) {
-    h->fp64_fallbacks = D->status_host[1];
-    h->perturbed_pivots = D->status_host[2];
+    h->fp64_fallbacks = D->status_host[4];
+    h->perturbed_pivots = D->status_host[5];
   }
 #ifdef CHOL_BOUNDS_CHECK
   {
@@ -1186,13 +1217,8 @@ int chol_finish_factor(chol_handle* h, cudaStream_t st) {
   if (h->opt.precision != CHOL_PREC_FP64) {
     const int rc = chol_tc_status(h);
     if (rc) return rc;
-  } else if (const int rc = chol_sg_status(h)) {
-    return rc;
   }
-  {
-    const int rc = chol_solve_status(h);
-    if (rc) return rc;
-  }
+  if (D->status_host[1] | D->status_host[2]) return chol_solve_status(h);   // clears the words
   h->factored = true;
   return CHOL_OK;
 }

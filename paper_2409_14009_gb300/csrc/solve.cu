@@ -25,6 +25,7 @@
 
 #include "device.h"
 #include "mixed.h"
+#include "diag_inv.cuh"
 
 namespace {
 
@@ -134,48 +135,17 @@ constexpr long long kTriMaxPolls = 1ll << 24;   // seconds, with the back-off be
 // (L_ii^{-1})(r, c), zero above the diagonal and past the block's width.
 constexpr int kInv64Stride = kSub * kSub;
 
-// One CTA per block: thread group g (four lanes) solves L_ii x = e_g by
-// substitution, lane q holding rows q + 4 mm, giving column g of L_ii^{-1}.
+// One CTA per block (inv64_columns).
 __global__ void __launch_bounds__(kT)
 k_diag_inv64(const SnodeDev* __restrict__ sn, const TriItem* __restrict__ items, const double* __restrict__ L,
              double* __restrict__ Dinv) {
-  __shared__ double Lk[kSub * 65];   // L_ii, column-major (ld 65), zero above the diagonal and past kb
-  __shared__ double rinv[kSub];
+  __shared__ double Lk[kSub * 65], rinv[kSub];
   const TriItem item = items[blockIdx.x];
   const SnodeDev d = sn[item.J];
-  const double* P = L + d.loff;
   const int blk = item.i, i0 = blk * kSub, kb = min(kSub, d.s - i0);
-  const int tid = threadIdx.x;
-  for (int e = tid; e < kSub * kSub; e += kT) {
-    const int rr = e & 63, cc = e >> 6;   // consecutive threads read consecutive rows of a column
-    Lk[rr + cc * 65] = (rr < kb && cc <= rr) ? P[(i0 + rr) + (int64_t)(i0 + cc) * d.ld] : 0.0;
-  }
-  __syncthreads();
-  if (tid < kSub) rinv[tid] = tid < kb ? 1.0 / Lk[tid * 66] : 0.0;
-  __syncthreads();
-  const int g = tid >> 2, q = tid & 3;
+  const int g = threadIdx.x >> 2, q = threadIdx.x & 3;
   double x[16];
-#pragma unroll
-  for (int mm = 0; mm < 16; ++mm) x[mm] = (q + 4 * mm == g) ? 1.0 : 0.0;
-  // only the first kb steps and the warps holding columns g < kb do work (a
-  // ragged block of a small supernode is often much narrower than 64)
-  if ((tid >> 5) * 8 < kb) {
-#pragma unroll
-    for (int jm = 0; jm < 16; ++jm) {
-      if (jm * 4 >= kb) break;   // uniform across the CTA
-#pragma unroll
-      for (int jq = 0; jq < 4; ++jq) {
-        const int jj = jm * 4 + jq;
-        const double xj = __shfl_sync(0xffffffffu, x[jm] * rinv[jj], jq, 4);
-        if (q == jq) x[jm] = xj;
-#pragma unroll
-        for (int mm = jm; mm < 16; ++mm) {
-          const int c = q + 4 * mm;
-          if (c > jj && 4 * mm < kb) x[mm] = fma(-xj, Lk[c + jj * 65], x[mm]);
-        }
-      }
-    }
-  }
+  inv64_columns(L + d.loff + i0 + (int64_t)i0 * d.ld, d.ld, kb, Lk, rinv, x);
   double* Di = Dinv + (int64_t)(item.fbase + blk) * kInv64Stride;
 #pragma unroll
   for (int mm = 0; mm < 16; ++mm) {
@@ -1511,15 +1481,15 @@ int chol_diag_inv(chol_handle* h, int b, int nitems, cudaStream_t st) {
   return CHOL_OK;
 }
 
-// CHOL_ETIMEOUT if a triangle launch gave up waiting since the last check
-// (for callers that have synchronized with the solves).
+// CHOL_ETIMEOUT if a triangle launch or a slice-product tile gave up waiting
+// since the last check (for callers that have synchronized with the work).
 int chol_solve_status(chol_handle* h) {
   DeviceState* D = h->dev;
   if (!D || !D->sv_err) return CHOL_OK;
-  int32_t e = 0;
-  CHOL_CUDA_TRY(cudaMemcpy(&e, D->sv_err, sizeof(int32_t), cudaMemcpyDeviceToHost));
-  if (e != 0) {
-    CHOL_CUDA_TRY(cudaMemset(D->sv_err, 0, sizeof(int32_t)));
+  int32_t e[2] = {0, 0};   // sv_err, sg_err
+  CHOL_CUDA_TRY(cudaMemcpy(e, D->sv_err, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost));
+  if (e[0] | e[1]) {
+    CHOL_CUDA_TRY(cudaMemset(D->sv_err, 0, 2 * sizeof(int32_t)));
     return CHOL_ETIMEOUT;
   }
   return CHOL_OK;

@@ -13,50 +13,48 @@
 
 namespace {
 
-constexpr int kSplitThreads = 256;
+using sg::kSplitThreads;
 
 __device__ __forceinline__ uint32_t abs_high(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
 
-// 64 off-diagonal rows of J and all its columns: a first pass over the entries
-// for the rows' exponents, a second (from L2) for the digits; the four thread
-// groups take every fourth K block.
+// 16 to 64 off-diagonal rows of J (split_rows_log2) and all its columns: a first
+// pass over the entries for the rows' exponents, a second (from L2) for the
+// digits; a thread takes 8 columns of a row a step, the lanes along the rows.
 __global__ void __launch_bounds__(kSplitThreads)
 k_sg_split_rows(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, const TileTask* __restrict__ tasks,
                 const double* __restrict__ L, unsigned char* __restrict__ slab, int32_t* __restrict__ exps) {
-  __shared__ uint32_t hmax[4][64];
+  __shared__ uint32_t hmax[64];
   const TileTask t = tasks[blockIdx.x];
   const SnodeDev d = sn[t.J];
   const SplitDev z = sd[t.J];
   const int b = d.len - d.s;
-  const int r = threadIdx.x & 63, g = threadIdx.x >> 6;
+  const int rsh = sg::split_rows_log2(d.s), R = 1 << rsh, step = 8 << (sg::kSplitThreadsLog2 - rsh);
+  const int r = threadIdx.x & (R - 1), c0 = 8 * (threadIdx.x >> rsh);
   const int row = t.r0 + r;
   const bool in = row < b;
   const double* G = L + d.loff + d.s + row;
-  uint32_t m = 0;
-  if (in) {
-#pragma unroll 8
-    for (int c = g; c < d.s; c += 4) m = max(m, abs_high(G[(int64_t)c * d.ld]));
-  }
-  hmax[g][r] = m;
+  if (threadIdx.x < 64) hmax[threadIdx.x] = 0;
   __syncthreads();
-  const int32_t e = sg::row_exponent(max(max(hmax[0][r], hmax[1][r]), max(hmax[2][r], hmax[3][r])));
-  if (g == 0) exps[z.srow0 + row] = e;
-  for (int k = g; k * sg::kBlockK < d.s; k += 4) {
-    unsigned char* out = slab + (z.soff + (int64_t)k * sg::kSlices * z.srows) * 64;
+  uint32_t m = 0;
+#pragma unroll 2
+  for (int k0 = c0; k0 < d.s; k0 += step) {
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      double y[8];
+    for (int i = 0; i < 8; ++i) m = max(m, in && k0 + i < d.s ? abs_high(G[(int64_t)(k0 + i) * d.ld]) : 0u);
+  }
+  if (m) atomicMax(&hmax[r], m);
+  __syncthreads();
+  const int32_t e = sg::row_exponent(hmax[r]);
+  if (threadIdx.x < R) exps[z.srow0 + row] = e;
+  for (int k0 = c0; k0 < z.sblk * sg::kBlockK; k0 += step) {
+    double y[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int col = k * sg::kBlockK + 8 * c + i;
-        y[i] = (in && col < d.s && e != sg::kExpNaN) ? G[(int64_t)col * d.ld] : 0.0;
-      }
-      uint4 w[sg::kSlices];
-      sg::digits8(y, e, w);
+    for (int i = 0; i < 8; ++i) y[i] = (in && k0 + i < d.s && e != sg::kExpNaN) ? G[(int64_t)(k0 + i) * d.ld] : 0.0;
+    uint4 w[sg::kSlices];
+    sg::digits8(y, e, w);
+    unsigned char* out = slab + (z.soff + (int64_t)(k0 / sg::kBlockK) * sg::kSlices * z.srows) * 64 +
+                         sg::chunk_offset(row, (k0 >> 3) & 3);
 #pragma unroll
-      for (int q = 0; q < sg::kSlices; ++q)
-        *reinterpret_cast<uint4*>(out + (int64_t)q * z.srows * 64 + sg::chunk_offset(row, c)) = w[q];
-    }
+    for (int q = 0; q < sg::kSlices; ++q) *reinterpret_cast<uint4*>(out + (int64_t)q * z.srows * 64) = w[q];
   }
 }
 
@@ -215,8 +213,7 @@ std::vector<SgBuffer> sg_buffers(chol_handle* h) {
           {(void**)&D->sg_dev, (int64_t)(sizeof(SplitDev) * h->split.size())},
           {(void**)&D->sg_split, (int64_t)(sizeof(TileTask) * h->split_tasks.size())},
           {(void**)&D->sg_syrk, (int64_t)(sizeof(TileTask) * h->sgs_tasks.size())},
-          {(void**)&D->sg_trail, (int64_t)(sizeof(TileTask) * h->sgt_tasks.size())},
-          {(void**)&D->sg_err, 4}};
+          {(void**)&D->sg_trail, (int64_t)(sizeof(TileTask) * h->sgt_tasks.size())}};
 }
 
 }  // namespace
@@ -248,7 +245,6 @@ int chol_sg_ensure(chol_handle* h) {
       chol_sg_release(h);
       return CHOL_OK;
     }
-  CHOL_CUDA_TRY(cudaMemset(D->sg_err, 0, 4));
   CHOL_CUDA_TRY(cudaMemcpy(D->sg_dev, h->split.data(), sizeof(SplitDev) * h->split.size(), cudaMemcpyHostToDevice));
   auto up = [](TileTask* dst, const std::vector<TileTask>& v) {
     return v.empty() ? cudaSuccess : cudaMemcpy(dst, v.data(), sizeof(TileTask) * v.size(), cudaMemcpyHostToDevice);
@@ -284,12 +280,4 @@ void chol_sg_syrk(chol_handle* h, const LevelPlan& P, cudaStream_t st) {
     k_sg_syrk<false><<<grid, sg::kThreads, sg::kSmemBytes, st>>>(D->sn, D->sg_dev, D->sg_syrk + P.sgs_b, P.sgs_n,
                                                                  D->sg_slab, D->sg_exps, D->U, nullptr, nullptr, nullptr,
                                                                  nullptr, D->sg_err);
-}
-
-// After a synchronized factorization: CHOL_ETIMEOUT if any tile gave up waiting.
-int chol_sg_status(chol_handle* h) {
-  DeviceState* D = h->dev;
-  if (D->sg_ready != 1 || D->status_host[3] == 0) return CHOL_OK;
-  CHOL_CUDA_TRY(cudaMemset(D->sg_err, 0, 4));
-  return CHOL_ETIMEOUT;
 }

@@ -55,6 +55,12 @@ constexpr int kCols = 16;                 // columns of an epilogue thread
 constexpr int kThreads = 32 * (kEpiWarps + 2);   // epilogue, copy and MMA warps
 constexpr int kTmemCols = 512;            // 7 accumulators of 64 columns
 
+// Operand splitting: 512 threads take R rows, 8 columns a thread, so that an
+// operand of few rows and many columns still gives enough CTAs and loads in
+// flight (64 rows and 64 columns a step took 31 us where this takes 13).
+constexpr int kSplitThreadsLog2 = 9, kSplitThreads = 1 << kSplitThreadsLog2;
+__host__ __device__ constexpr int split_rows_log2(int K) { return K <= 64 ? 6 : (K <= 128 ? 5 : 4); }
+
 constexpr int32_t kExpNaN = INT_MIN;      // exponent of a row with an infinity or a NaN
 constexpr int32_t kExpMin = -1020;        // rows of zeros and subnormals
 
