@@ -449,7 +449,7 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
   h->gemv_tasks.clear(); h->bpart_tasks.clear(); h->bred_tasks.clear();
   h->p_max = 0;
   h->split_slots_max = 0;
-  h->asm_tasks.clear(); h->asm_segs.clear();
+  h->asm_tasks.clear(); h->asm_segs.clear(); h->fasm_tasks.clear();
   h->n_small = h->n_large = 0;
   h->update_doubles = 0;
   h->update_doubles_rl = 0;
@@ -595,13 +595,24 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
         for (int32_t j = 0; j < kb; ++j) st.potrf_flops += (double)(kb - j) * (kb - j);
         const double below = (double)(d.len - k0 - kb);
         st.trsm_flops += below * (double)kb * (double)kb;   // kb divisions + 2*kb(kb-1)/2 per row
-        for (int32_t r0 = k0 + kb; r0 < d.len; r0 += trsm_rows) h->trsm_tasks.push_back({J, k0, r0, 0});
         // trailing update: 2 kb flops per entry (r, c) with c in [k0+kb, s), r in [c, len)
         const int32_t cend = d.s;
         {
           const double w = (double)(cend - k0 - kb), hgt = (double)(d.len - k0 - kb);
           st.gemm_flops += 2.0 * kb * (w * hgt - w * (w - 1.0) / 2.0);
         }
+      }
+      // the next diagonal block's rows of the supernodes that have one, then the others
+      for (int pass = 0; pass < 2; ++pass) {
+        for (int32_t J : large) {
+          const SnodeDev& d = h->snodes[J];
+          if (d.s <= k0) continue;
+          const int32_t r1 = k0 + std::min(nb, d.s - k0);
+          const int32_t rc = d.s > r1 ? std::min(d.len, r1 + nb) : r1;   // end of the first pass's rows
+          for (int32_t r0 = pass ? rc : r1; r0 < (pass ? d.len : rc); r0 += trsm_rows)
+            h->trsm_tasks.push_back({J, k0, r0, 0});
+        }
+        if (pass == 0) st.trsm_c = (int32_t)h->trsm_tasks.size() - st.trsm_b;
       }
       // the step's own trailing update covers columns [k0+kb, cend) of each
       // supernode: first column tiles of all supernodes, then the others
@@ -617,19 +628,28 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
         }
         if (pass == 0) st.gemm_next = (int32_t)h->gemm_tasks.size() - st.gemm_b;
       }
-      // the same tiles for the tensor cores, 128 rows high
+      // the same tiles for the tensor cores, 128 rows high (see StepRange)
       st.sgt_b = (int32_t)h->sgt_tasks.size();
-      for (int pass = 0; split64 && pass < 2; ++pass) {
+      for (int pass = 0; split64 && pass < 3; ++pass) {
         for (int32_t J : large) {
           const SnodeDev& d = h->snodes[J];
-          if (d.s <= k0) continue;
-          const int32_t kb = std::min(nb, d.s - k0);
-          for (int32_t c0 = k0 + kb; c0 < d.s; c0 += kTile) {
-            if ((pass == 0) != (c0 == k0 + kb)) continue;
-            for (int32_t r0 = c0; r0 < d.len; r0 += 2 * kTile) h->sgt_tasks.push_back({J, k0, r0, c0});
+          const int32_t c1 = k0 + nb, c2 = c1 + nb;   // the next two column blocks
+          if (d.s <= c1) continue;
+          auto column = [&](int32_t c0, int32_t r0) {
+            for (; r0 < d.len; r0 += 2 * kTile) h->sgt_tasks.push_back({J, 2 * kTile, r0, c0});
+          };
+          if (pass == 0) h->sgt_tasks.push_back({J, kTile, c1, c1});
+          if (pass == 1) {
+            column(c1, c1 + kTile);
+            if (c2 < d.s) h->sgt_tasks.push_back({J, kTile, c2, c2});
+          }
+          if (pass == 2) {
+            if (c2 < d.s) column(c2, c2 + kTile);
+            for (int32_t c0 = c2 + nb; c0 < d.s; c0 += kTile) column(c0, c0);
           }
         }
-        if (pass == 0) st.sgt_next = (int32_t)h->sgt_tasks.size() - st.sgt_b;
+        if (pass == 0) st.sgt_c = (int32_t)h->sgt_tasks.size() - st.sgt_b;
+        if (pass == 1) st.sgt_near = (int32_t)h->sgt_tasks.size() - st.sgt_b - st.sgt_c;
       }
       st.sgt_n = (int32_t)h->sgt_tasks.size() - st.sgt_b;
       st.potrf_n = (int32_t)h->potrf_list.size() - st.potrf_b;
@@ -851,6 +871,10 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
     P.asm_n = (int32_t)h->asm_tasks.size() - P.asm_b;
     P.asmw_n = (int32_t)warp_tasks.size();
     h->asm_tasks.insert(h->asm_tasks.end(), warp_tasks.begin(), warp_tasks.end());
+    P.fasm_b = (int32_t)h->fasm_tasks.size();
+    for (int32_t i = P.asm_b; i < (int32_t)h->asm_tasks.size(); ++i)
+      if (h->asm_tasks[i].p0 == h->asm_tasks[i].t0) h->fasm_tasks.push_back(i);
+    P.fasm_n = (int32_t)h->fasm_tasks.size() - P.fasm_b;
   }
   h->persist_levels.clear();
   h->small_panel_max = 0;

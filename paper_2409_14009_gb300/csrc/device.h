@@ -25,13 +25,14 @@ struct DeviceState {
   TileTask* syrk = nullptr;
   AsmTask* asm_tasks = nullptr;
   AsmSeg* asm_segs = nullptr;
+  int32_t* fasm = nullptr;      // solve: the assembly tasks that hold their segments' columns
   TriItemHost* tri = nullptr;   // solve: diagonal-triangle items
   double* rdiag = nullptr;      // binary64 blocked path: reciprocal pivots, per column of P A P^T
   int sg_ready = 0;             // binary64 updates on the tensor cores: 1 = in use, -1 = not
   unsigned char* sg_slab = nullptr;              // slices of a level's off-diagonal rows
   int32_t* sg_exps = nullptr;                    // ... and their row exponents
-  unsigned char* sgt_slab[2] = {nullptr, nullptr};   // slices of a 64-column block, by step parity
-  int32_t* sgt_exps[2] = {nullptr, nullptr};
+  unsigned char* sgt_slab[3] = {nullptr, nullptr, nullptr};   // slices of a 64-column block, by step mod 3
+  int32_t* sgt_exps[3] = {nullptr, nullptr, nullptr};
   SplitDev* sg_dev = nullptr;
   TileTask* sg_split = nullptr;
   TileTask* sg_syrk = nullptr;
@@ -98,7 +99,11 @@ struct DeviceState {
   cudaEvent_t gev[2] = {nullptr, nullptr};
   cudaStream_t lstream = nullptr;  // side stream of the lookahead trailing updates (lowest priority)
   cudaStream_t hstream = nullptr;  // critical path of the blocked levels (highest priority)
+  cudaStream_t mstream = nullptr;  // bulk of a step: the TRSM and next-column tiles off the diagonal chain
+  cudaStream_t sstream = nullptr;  // one-CTA supernodes of a level that also has blocked ones
+  cudaEvent_t sev[2] = {nullptr, nullptr};   // level begun / small supernodes done
   cudaEvent_t lev[3] = {nullptr, nullptr, nullptr};   // panel final / rest done / fork-join
+  cudaEvent_t mev[4] = {nullptr, nullptr, nullptr, nullptr};   // diagonal factored / its next rows solved / bulk solved / near tiles done
   cudaStream_t istream = nullptr;  // binary64: diagonal-block inverses of finished levels (lowest priority)
   cudaEvent_t iev[2] = {nullptr, nullptr};            // level factored / inverses done
   chol_kernel_stat graph_delta[CHOL_K_NCLASSES] = {};
@@ -189,6 +194,17 @@ void chol_prof_resolve(chol_handle* h);   // sum the pending event pairs
 void chol_prof_free(chol_handle* h);
 
 int chol_device_ensure(chol_handle* h);   // allocate and upload on first use
+
+// How a level's assembly tasks are launched: with few tasks (they all fit on the
+// SMs as CTAs) every task takes a CTA, whose eight warps share the chain of
+// loads; with more, the warp-sized ones take a warp each. One warp-sized task
+// alone took 25 us on a warp and takes 8 on a CTA; 12,000 of them 160 us on
+// warps.
+struct AsmSplit { int ctas, warps; };
+inline AsmSplit asm_split(const LevelPlan& P, int sms) {
+  const int all = P.asm_n + P.asmw_n;
+  return all <= 8 * sms ? AsmSplit{all, 0} : AsmSplit{P.asm_n, P.asmw_n};
+}
 
 // CHOL_ESTATE unless the handle holds a factorization on the current device.
 // Calls after chol_factor launch on whichever device is current, while the

@@ -42,37 +42,111 @@ constexpr int kAsmThreads = 256;
 
 // ---------------------------------------------------------------------------
 // dense Cholesky of the first s columns of a len x s column-major block in
-// shared memory (right-looking, one column per step). A non-positive or NaN
-// pivot records column fcol+k+1 in *status (smallest wins) and poisons the
-// column with NaN so that the failure propagates without stopping the grid.
-// ---------------------------------------------------------------------------
-__device__ void dense_chol_smem(double* P, int ld, int len, int s, int fcol, int* status) {
-  __shared__ double srk;
-  for (int k = 0; k < s; ++k) {
+// shared memory (leading dimension ld). A non-positive or NaN pivot records
+// column fcol+k+1 in *status (smallest wins) and poisons the column with NaN so
+// that the failure propagates without stopping the grid.
+//
+// Columns [c0, c0 + w) one at a time, right-looking inside the panel, one thread
+// per row: narrow panels (most supernodes of a 2D grid's lower levels) and
+// panels with a pivot that is not positive, normal and finite.
+__device__ void small_panel_columns(double* P, int ld, int len, int c0, int w, int fcol, int* status, double* srk) {
+  for (int k = c0; k < c0 + w; ++k) {
     __syncthreads();
     if (threadIdx.x == 0) {
-      // the pivot's root once, by one thread (FP64 sqrt and division are long
-      // dependent sequences on the narrow FP64 pipe)
       const double d = P[k + k * ld];
       const bool bad = !(d > 0.0);
       double dk, rk;
       pivot_root(d, bad, dk, rk);
       P[k + k * ld] = dk;
-      srk = rk;
+      *srk = rk;
       if (bad) atomicMin(status, fcol + k + 1);
     }
     __syncthreads();
-    const double inv = srk;
+    const double inv = *srk;
     for (int r = k + 1 + threadIdx.x; r < len; r += blockDim.x) P[r + k * ld] *= inv;
     __syncthreads();
-    // rank-1 update of the trailing columns, one thread per row
     for (int r = k + 1 + threadIdx.x; r < len; r += blockDim.x) {
       const double lrk = P[r + k * ld];
-      const int jmax = r < s - 1 ? r : s - 1;
+      const int jmax = min(r, c0 + w - 1);
       for (int j = k + 1; j <= jmax; ++j) P[r + j * ld] -= lrk * P[j + k * ld];
     }
   }
   __syncthreads();
+}
+
+// The panel [c0, c0 + w), 4 < w <= 8, in registers: every warp holds the panel's
+// diagonal rows (lanes 0-7, the same in all warps; identity past w) and 24 rows
+// below them a pass, and factors them in straight-line code (potrf.cuh). False
+// (uniform): some pivot is not positive, normal and finite, nothing written.
+__device__ __forceinline__ bool small_panel_warps(double* P, int ld, int len, int c0, int w) {
+  const int lane = threadIdx.x & 31, v = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int below = len - c0 - w;
+  double dg = 0.0, rd = 0.0, xd[8];
+  for (int base = 0; base == 0 || base < below; base += 24 * nw) {
+    const int row = lane < 8 ? c0 + lane : c0 + w + base + 24 * v + lane - 8;
+    const bool real = lane < 8 ? lane < w : row < len;
+    const bool idle = v > 0 && base + 24 * v >= below;   // no rows for this warp
+    bool normal = true;
+    if (!idle) {
+      double x[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) x[t] = real && t < w ? P[row + (c0 + t) * ld] : (lane == t ? 1.0 : 0.0);
+#pragma unroll
+      for (int kk = 0; kk < 8; ++kk) {
+        const double dk = __shfl_sync(0xffffffffu, x[kk], kk);
+        const int dh = __double2hiint(dk);
+        normal = normal && dh >= 0x00100000 && dh < 0x7ff00000;
+        const double rroot = rsqrt_bits(dh, __double2loint(dk));
+        if (lane == kk) { rd = rroot; dg = dk; }
+        if (lane > kk) x[kk] *= rroot;
+#pragma unroll
+        for (int jj = kk + 1; jj < 8; ++jj) x[jj] = fma(-x[kk], __shfl_sync(0xffffffffu, x[kk], jj), x[jj]);
+      }
+      if (normal && lane >= 8 && real) {
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+          if (t < w) P[row + (c0 + t) * ld] = x[t];
+      }
+#pragma unroll
+      for (int t = 0; t < 8; ++t) xd[t] = x[t];
+    }
+    // the diagonal rows are the same in every warp and pass, so the verdict is too
+    if (__syncthreads_or(!normal)) return false;
+  }
+  if (v == 0 && lane < w) {
+    dg *= rd;
+#pragma unroll
+    for (int t = 0; t < 8; ++t)
+      if (t <= lane) P[c0 + lane + (c0 + t) * ld] = t == lane ? dg : xd[t];
+  }
+  __syncthreads();
+  return true;
+}
+
+__device__ void dense_chol_smem(double* P, int ld, int len, int s, int fcol, int* status) {
+  __shared__ double srk;
+  __syncthreads();
+  for (int c0 = 0; c0 < s; c0 += 8) {
+    const int w = min(8, s - c0), n0 = c0 + w;
+    if (w <= 4 || !small_panel_warps(P, ld, len, c0, w)) small_panel_columns(P, ld, len, c0, w, fcol, status, &srk);
+    if (n0 >= s) break;
+    // the panel's rank-w product from the columns right of it, lower part: column
+    // i has R - i entries; columns p and m - 1 - p together have S
+    const int m = s - n0, R = len - n0, S = 2 * R - (m - 1), items = ((m + 1) >> 1) * S;
+    for (int q = threadIdx.x; q < items; q += blockDim.x) {
+      const int p = q / S, o = q - p * S;
+      const bool second = o >= R - p;
+      const int j = second ? m - 1 - p : p;
+      if (second && j == p) continue;   // the middle column of an odd m
+      const int r = n0 + j + (second ? o - (R - p) : o), c = n0 + j;
+      double acc = P[r + c * ld];
+#pragma unroll
+      for (int t = 0; t < 8; ++t)
+        if (t < w) acc = fma(-P[r + (c0 + t) * ld], P[c + (c0 + t) * ld], acc);
+      P[r + c * ld] = acc;
+    }
+    __syncthreads();
+  }
 }
 
 // Position of global row `key` in the sorted row structure rk[0, len).
@@ -202,57 +276,38 @@ k_potrf(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list, int k
   }
 }
 
-// Blocked path, step k0: a task's rows of column block [k0, k0+kb) become
-// X = B L_kk^{-T}. LPR lanes share a row, lane q holding columns q + LPR m; the
-// solved x_j is broadcast inside the group with a shuffle and every lane
-// updates its own columns (no barriers in the substitution loop). A warp is
-// bound by its partition's FP64 pipe (1 + 32 / LPR + 1/2 instructions of 64
-// cycles a step on average), so few rows take 16 lanes each (8 rows a CTA, the
-// shorter chain) and many rows 8 (16 rows a CTA, fewer instructions a row).
-// SPLIT: the rows' slices for the trailing update on the tensor cores are
-// written here too, where the row is on chip (split_gemm.cuh).
+// Rows of column block [k0, k0+kb) become X = B L_kk^{-T}. LPR lanes share a row,
+// lane q holding columns q + LPR m; the solved x_j is broadcast inside the group
+// with a shuffle and every lane updates its own columns (no barriers in the
+// substitution loop). A warp is bound by its partition's FP64 pipe (1 + 32 / LPR
+// + 1/2 instructions of 64 cycles a step on average).
 constexpr int kTrsmThreads = 128;
-template <int LPR, bool SPLIT>
-__global__ void __launch_bounds__(kTrsmThreads)
-k_trsm(const SnodeDev* __restrict__ sn, const TileTask* __restrict__ tasks, int nb, double* __restrict__ L,
-       const double* __restrict__ rdiag, const SplitDev* __restrict__ sd, unsigned char* __restrict__ slab,
-       int32_t* __restrict__ exps) {
-  constexpr int kRows = kTrsmThreads / LPR, kCols = 64 / LPR;
-  __shared__ double Lk[64 * 65];
-  __shared__ double inv[64];
-  const TileTask t = tasks[blockIdx.x / (kTrsmRowsHost / 2 / kRows)];
-  const int r0 = t.r0 + (blockIdx.x % (kTrsmRowsHost / 2 / kRows)) * kRows;
-  const SnodeDev d = sn[t.J];
-  const int kb = min(nb, d.s - t.k0);
-  const double* Gd = L + d.loff + t.k0 + (int64_t)t.k0 * d.ld;
-  const int g = threadIdx.x / LPR, q = threadIdx.x & (LPR - 1);
-  const int row = r0 + g;
-  const bool live = row < d.len;
-  double* Gx = L + d.loff + row + (int64_t)t.k0 * d.ld;
-  double x[kCols];
+
+// Stage L_kk (column-major, leading dimension 65) and the reciprocal pivots: all
+// loads of a thread issued before the stores (consecutive threads read
+// consecutive rows). NT threads.
+template <int NT>
+__device__ __forceinline__ void stage_diag(const double* __restrict__ Gd, int64_t ld, int kb,
+                                           const double* __restrict__ rdiag, double* Lk, double* inv) {
+  constexpr int kIt = 64 * 64 / NT;
+  double v[kIt];
 #pragma unroll
-  for (int m = 0; m < kCols; ++m) {
-    const int c = q + LPR * m;
-    x[m] = (live && c < kb) ? Gx[(int64_t)c * d.ld] : 0.0;
+  for (int i = 0; i < kIt; ++i) {
+    const int e = threadIdx.x + NT * i, r = e & 63, c = e >> 6;
+    v[i] = (r < kb && c < kb) ? Gd[r + (int64_t)c * ld] : 0.0;
   }
-  {
-    // stage the diagonal block: all loads of a thread issued before the
-    // stores (column-major source: consecutive threads read consecutive rows)
-    constexpr int kIt = 64 * 64 / kTrsmThreads;
-    double v[kIt];
 #pragma unroll
-    for (int i = 0; i < kIt; ++i) {
-      const int e = threadIdx.x + kTrsmThreads * i, r = e & 63, c = e >> 6;
-      v[i] = (r < kb && c < kb) ? Gd[r + (int64_t)c * d.ld] : 0.0;
-    }
-#pragma unroll
-    for (int i = 0; i < kIt; ++i) {
-      const int e = threadIdx.x + kTrsmThreads * i;
-      Lk[(e & 63) + (e >> 6) * 65] = v[i];
-    }
-    if (threadIdx.x < 64) inv[threadIdx.x] = threadIdx.x < kb ? rdiag[d.f + t.k0 + threadIdx.x] : 0.0;
+  for (int i = 0; i < kIt; ++i) {
+    const int e = threadIdx.x + NT * i;
+    Lk[(e & 63) + (e >> 6) * 65] = v[i];
   }
-  __syncthreads();
+  if (threadIdx.x < 64) inv[threadIdx.x] = threadIdx.x < kb ? rdiag[threadIdx.x] : 0.0;
+}
+
+template <int LPR>
+__device__ __forceinline__ void trsm_rows(double (&x)[64 / LPR], int kb, const double* Lk, const double* inv) {
+  constexpr int kCols = 64 / LPR;
+  const int q = threadIdx.x & (LPR - 1);
 #pragma unroll
   for (int jm = 0; jm < kCols; ++jm) {
 #pragma unroll
@@ -271,6 +326,65 @@ k_trsm(const SnodeDev* __restrict__ sn, const TileTask* __restrict__ tasks, int 
       }
     }
   }
+}
+
+// The slices of a solved row (its lanes in one warp) for the trailing update on
+// the tensor cores, written where the row is on chip (split_gemm.cuh). xs: 64
+// doubles of shared memory private to the row, which receive the row.
+template <int LPR>
+__device__ __forceinline__ void slice_row(const double (&x)[64 / LPR], bool live, int row, const SplitDev& z, double* xs,
+                                          unsigned char* __restrict__ slab, int32_t* __restrict__ exps) {
+  constexpr int kCols = 64 / LPR;
+  const int q = threadIdx.x & (LPR - 1);
+  uint32_t hm = 0;
+#pragma unroll
+  for (int m = 0; m < kCols; ++m) hm = max(hm, (uint32_t)__double2hiint(x[m]) & 0x7fffffffu);
+  for (int o = LPR / 2; o > 0; o >>= 1) hm = max(hm, __shfl_xor_sync(0xffffffffu, hm, o, LPR));
+  const int32_t e = sg::row_exponent(hm);
+#pragma unroll
+  for (int m = 0; m < kCols; ++m) xs[q + LPR * m] = x[m];
+  if (live && q == 0) exps[z.trow0 + row] = e;
+  __syncwarp();
+  // 8 chunks of 8 columns a row: lane q takes chunk q (LPR = 16: half the lanes)
+  if (live && q < 8) {
+    double y[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) y[i] = e == sg::kExpNaN ? 0.0 : xs[8 * q + i];
+    uint4 w[sg::kSlices];
+    sg::digits8(y, e, w);
+    unsigned char* out = slab + (z.toff + (int64_t)(q >> 2) * sg::kSlices * z.trows) * 64 + sg::chunk_offset(row, q & 3);
+#pragma unroll
+    for (int i = 0; i < sg::kSlices; ++i) *reinterpret_cast<uint4*>(out + (int64_t)i * z.trows * 64) = w[i];
+  }
+}
+
+// One task's rows; few rows take 16 lanes each (8 rows a CTA, the shorter chain)
+// and many rows 8 (16 rows a CTA, fewer instructions a row).
+template <int LPR, bool SPLIT>
+__global__ void __launch_bounds__(kTrsmThreads)
+k_trsm(const SnodeDev* __restrict__ sn, const TileTask* __restrict__ tasks, int nb, double* __restrict__ L,
+       const double* __restrict__ rdiag, const SplitDev* __restrict__ sd, unsigned char* __restrict__ slab,
+       int32_t* __restrict__ exps) {
+  constexpr int kRows = kTrsmThreads / LPR, kCols = 64 / LPR;
+  __shared__ double Lk[64 * 65];
+  __shared__ double inv[64];
+  const TileTask t = tasks[blockIdx.x / (kTrsmRowsHost / 2 / kRows)];
+  const int r0 = t.r0 + (blockIdx.x % (kTrsmRowsHost / 2 / kRows)) * kRows;
+  const SnodeDev d = sn[t.J];
+  const int kb = min(nb, d.s - t.k0);
+  const int g = threadIdx.x / LPR, q = threadIdx.x & (LPR - 1);
+  const int row = r0 + g;
+  const bool live = row < d.len;
+  double* Gx = L + d.loff + row + (int64_t)t.k0 * d.ld;
+  double x[kCols];
+#pragma unroll
+  for (int m = 0; m < kCols; ++m) {
+    const int c = q + LPR * m;
+    x[m] = (live && c < kb) ? Gx[(int64_t)c * d.ld] : 0.0;
+  }
+  stage_diag<kTrsmThreads>(L + d.loff + t.k0 + (int64_t)t.k0 * d.ld, d.ld, kb, rdiag + d.f + t.k0, Lk, inv);
+  __syncthreads();
+  trsm_rows<LPR>(x, kb, Lk, inv);
   if (live) {
 #pragma unroll
     for (int m = 0; m < kCols; ++m) {
@@ -280,31 +394,85 @@ k_trsm(const SnodeDev* __restrict__ sn, const TileTask* __restrict__ tasks, int 
   }
   if constexpr (SPLIT) {
     if (t.k0 + kb >= d.s) return;   // nothing right of the block (uniform across the CTA)
-    uint32_t hm = 0;
-#pragma unroll
-    for (int m = 0; m < kCols; ++m) hm = max(hm, (uint32_t)__double2hiint(x[m]) & 0x7fffffffu);
-    for (int o = LPR / 2; o > 0; o >>= 1) hm = max(hm, __shfl_xor_sync(0xffffffffu, hm, o, LPR));
-    const int32_t e = sg::row_exponent(hm);
     __syncthreads();   // every warp is done with Lk
-    double* xs = Lk;   // row g at xs[66 g]
-#pragma unroll
-    for (int m = 0; m < kCols; ++m) xs[g * 66 + q + LPR * m] = e == sg::kExpNaN ? 0.0 : x[m];
-    const SplitDev z = sd[t.J];
-    if (live && q == 0) exps[z.trow0 + row] = e;
-    __syncwarp();      // a row's lanes are in one warp
-    if (!live) return;
-    // 8 chunks of 8 columns a row: lane q takes chunk q (LPR = 16: half the lanes)
-    if (q < 8) {
-      double y[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) y[i] = xs[g * 66 + 8 * q + i];
-      uint4 w[sg::kSlices];
-      sg::digits8(y, e, w);
-      unsigned char* out = slab + (z.toff + (int64_t)(q >> 2) * sg::kSlices * z.trows) * 64 + sg::chunk_offset(row, q & 3);
-#pragma unroll
-      for (int i = 0; i < sg::kSlices; ++i) *reinterpret_cast<uint4*>(out + (int64_t)i * z.trows * 64) = w[i];
-    }
+    slice_row<LPR>(x, live, row, sd[t.J], Lk + 66 * g, slab, exps);
   }
+}
+
+// The link of the diagonal chain between two POTRFs, one cluster of eight CTAs per
+// supernode with a next diagonal block: the TRSM of its (at most) 64 rows, eight
+// a CTA, then its update C -= X X^T (lower triangle), every CTA gathering the 64
+// solved rows through distributed shared memory, a thread per entry. One launch
+// of about 14 us in place of two (17 + 15): on 64 rows the FP64 pipes of eight
+// SMs (4 us each part) beat the latency of a tensor-core tile.
+constexpr int kLinkCtas = 8;
+constexpr int kLinkThreads = 256;
+__global__ void __cluster_dims__(kLinkCtas, 1, 1) __launch_bounds__(kLinkThreads)
+k_link(const SnodeDev* __restrict__ sn, const TileTask* __restrict__ tasks, double* __restrict__ L,
+       const double* __restrict__ rdiag, const SplitDev* __restrict__ sd, unsigned char* __restrict__ slab,
+       int32_t* __restrict__ exps) {
+  __shared__ double Lk[64 * 65];        // L_kk, then the 64 solved rows (row r at 65 r)
+  __shared__ double inv[64];
+  __shared__ double xs[8][66];          // this CTA's solved rows
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank();
+  const TileTask t = tasks[blockIdx.x / kLinkCtas];   // the next diagonal block: r0 = c0 = its first row
+  const SnodeDev d = sn[t.J];
+  const int r1 = t.c0, k0 = r1 - 64;
+  const int nr = min(64, d.len - r1), nc = min(64, d.s - r1);
+  constexpr int LPR = 16, kCols = 4;
+  const int g = threadIdx.x / LPR, q = threadIdx.x & (LPR - 1);
+  const int row = r1 + 8 * rank + g;
+  const bool live = g < 8 && row < d.len;
+  double* Gx = L + d.loff + row + (int64_t)k0 * d.ld;
+  double x[kCols];
+#pragma unroll
+  for (int m = 0; m < kCols; ++m) x[m] = live ? Gx[(int64_t)(q + LPR * m) * d.ld] : 0.0;
+  stage_diag<kLinkThreads>(L + d.loff + k0 + (int64_t)k0 * d.ld, d.ld, 64, rdiag + d.f + k0, Lk, inv);
+  // entry e of the 64 x 64 lower triangle: rows p and 63 - p together hold 65 entries
+  auto entry = [](int e, int& r, int& c) {
+    const int p = e / 65, o = e - 65 * p;
+    r = o <= p ? p : 63 - p;
+    c = o <= p ? o : o - p - 1;
+  };
+  const int e0 = rank * kLinkThreads + threadIdx.x;
+  int er, ec;
+  entry(e0, er, ec);
+  double* C = L + d.loff + r1 + (int64_t)r1 * d.ld;
+  const bool mine = er < nr && ec < nc;
+  const double c0 = mine ? C[er + (int64_t)ec * d.ld] : 0.0;
+  __syncthreads();
+  if (threadIdx.x < 128) {              // one warp a partition, two rows each
+    trsm_rows<LPR>(x, 64, Lk, inv);
+    if (live) {
+#pragma unroll
+      for (int m = 0; m < kCols; ++m) Gx[(int64_t)(q + LPR * m) * d.ld] = x[m];
+    }
+    slice_row<LPR>(x, live, row, sd[t.J], xs[g], slab, exps);
+  }
+  cl.sync();                            // every CTA's rows are in its xs
+#pragma unroll
+  for (int i = 0; i < 64 * 64 / kLinkThreads; ++i) {
+    const int e = threadIdx.x + kLinkThreads * i, r = e >> 6, k = e & 63;
+    Lk[r * 65 + k] = *cl.map_shared_rank(&xs[r & 7][k], r >> 3);
+  }
+  __syncthreads();
+  auto dot = [&](int r, int c) {
+    double acc[2] = {0.0, 0.0};         // even and odd columns
+#pragma unroll 8
+    for (int k = 0; k < 64; k += 2) {
+      acc[0] = fma(Lk[r * 65 + k], Lk[c * 65 + k], acc[0]);
+      acc[1] = fma(Lk[r * 65 + k + 1], Lk[c * 65 + k + 1], acc[1]);
+    }
+    return acc[0] + acc[1];
+  };
+  if (mine) C[er + (int64_t)ec * d.ld] = c0 - dot(er, ec);
+  // 64 * 65 / 2 = 2080 entries on 2048 threads: the last 32
+  if (rank == 0 && threadIdx.x >= kLinkThreads - 32) {
+    entry(2048 + threadIdx.x - (kLinkThreads - 32), er, ec);
+    if (er < nr && ec < nc) C[er + (int64_t)ec * d.ld] -= dot(er, ec);
+  }
+  cl.sync();                            // no CTA ends while others read its xs
 }
 
 // ---------------------------------------------------------------------------
@@ -602,20 +770,40 @@ k_persist_factor(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ sm
   }
 }
 
-// log det: per-supernode partial sums, then one fixed-order reduction.
-__global__ void k_logdet_part(const SnodeDev* __restrict__ sn, const double* __restrict__ L,
-                              double* __restrict__ part) {
-  __shared__ double red[128];
-  const SnodeDev d = sn[blockIdx.x];
-  double acc = 0.0;
-  for (int c = threadIdx.x; c < d.s; c += blockDim.x) acc += log(L[d.loff + c + (int64_t)c * d.ld]);
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+// log det: per-supernode partial sums, then one fixed-order reduction. A group
+// of G lanes multiplies the supernode's diagonal (mantissas, with the exponents
+// counted apart, so nothing over- or underflows) and takes one logarithm: a
+// binary64 logarithm is dozens of instructions of the narrow FP64 pipe, and one
+// per column on a CTA per supernode took 1.5 ms of a batch's 16.
+template <int G>
+__global__ void __launch_bounds__(256)
+k_logdet_part(const SnodeDev* __restrict__ sn, int ns, const double* __restrict__ L, double* __restrict__ part) {
+  const int J = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G), q = threadIdx.x & (G - 1);
+  if (J >= ns) return;   // whole groups
+  const SnodeDev d = sn[J];
+  double m = 1.0;        // product 1 <= |m| < 2 after every step
+  int e = 0;
+  auto times = [&](double v, int ev) {
+    m *= v;
+    const int hi = __double2hiint(m), x = (hi >> 20) - 1023;
+    e += x + ev;
+    m = __hiloint2double(hi - x * (1 << 20), __double2loint(m));
+  };
+#pragma unroll 4
+  for (int c = q; c < d.s; c += G) {
+    double v = L[d.loff + c + (int64_t)c * d.ld];
+    int ev = 0;
+    if (v < 2.2250738585072014e-308) { v *= 18014398509481984.0; ev = -54; }   // subnormal: times 2^54
+    const int hi = __double2hiint(v), x = (hi >> 20) - 1023;
+    times(__hiloint2double(hi - x * (1 << 20), __double2loint(v)), x + ev);
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = red[0];
+  const unsigned mask = G == 32 ? 0xffffffffu : ((1u << G) - 1) << ((threadIdx.x & 31) & ~(G - 1));
+  for (int o = G / 2; o > 0; o >>= 1) {
+    const double mo = __shfl_xor_sync(mask, m, o, G);
+    const int eo = __shfl_xor_sync(mask, e, o, G);
+    times(mo, eo);
+  }
+  if (q == 0) part[J] = log(m) + (double)e * 0.693147180559945309417;
 }
 
 // log det of every system: 2 x the supernode partials of its range, in order.
@@ -756,8 +944,8 @@ void chol_device_free(chol_handle* h) {
                   D->ssmall, D->Zp, D->Tw, D->Ww, D->Uh, D->a_col, D->a_row, D->adj_xb, D->perm, D->status, D->part, D->scalar_dev, D->Y, D->W,
                   D->mx_diagpos, D->mx_aij, D->mx_d, D->mx_fallbacks, D->csr_ptr, D->csr_col, D->csr_src,
                   D->csr_val, D->Lbf, D->tmaps, D->tc_err, D->R, D->Z, D->Pv, D->Q, D->red, D->Y32, D->W32,
-                  D->rhs_scale, D->host_vals, D->host_rhs, D->panel, D->pflags, D->dinv, D->split_part, D->split_cnt, D->hand32, D->sg_slab, D->sg_exps, D->sgt_slab[0], D->sgt_slab[1],
-                  D->sgt_exps[0], D->sgt_exps[1], D->sg_dev, D->sg_split, D->sg_syrk, D->sg_trail, D->rdiag};
+                  D->rhs_scale, D->host_vals, D->host_rhs, D->panel, D->pflags, D->dinv, D->split_part, D->split_cnt, D->hand32, D->sg_slab, D->sg_exps, D->sgt_slab[0], D->sgt_slab[1], D->sgt_slab[2],
+                  D->sgt_exps[0], D->sgt_exps[1], D->sgt_exps[2], D->sg_dev, D->sg_split, D->sg_syrk, D->sg_trail, D->rdiag, D->fasm};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (D->status_host) cudaFreeHost(D->status_host);
@@ -768,6 +956,12 @@ void chol_device_free(chol_handle* h) {
   if (D->lstream) cudaStreamDestroy(D->lstream);
   if (D->hstream) cudaStreamDestroy(D->hstream);
   if (D->istream) cudaStreamDestroy(D->istream);
+  if (D->mstream) cudaStreamDestroy(D->mstream);
+  if (D->sstream) cudaStreamDestroy(D->sstream);
+  for (cudaEvent_t e : D->sev)
+    if (e) cudaEventDestroy(e);
+  for (cudaEvent_t e : D->mev)
+    if (e) cudaEventDestroy(e);
   for (cudaEvent_t e : D->lev)
     if (e) cudaEventDestroy(e);
   for (cudaEvent_t e : D->iev)
@@ -802,6 +996,14 @@ int chol_device_ensure(chol_handle* h) {
         cudaStreamCreateWithPriority(&D->hstream, cudaStreamNonBlocking, hi) != cudaSuccess ||
         cudaStreamCreateWithPriority(&D->lstream, cudaStreamNonBlocking, lo) != cudaSuccess ||
         cudaStreamCreateWithPriority(&D->istream, cudaStreamNonBlocking, lo) != cudaSuccess ||
+        cudaStreamCreateWithPriority(&D->mstream, cudaStreamNonBlocking, (lo + hi) / 2) != cudaSuccess ||
+        cudaStreamCreateWithPriority(&D->sstream, cudaStreamNonBlocking, (lo + hi) / 2) != cudaSuccess ||
+        cudaEventCreateWithFlags(&D->sev[0], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&D->sev[1], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&D->mev[0], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&D->mev[1], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&D->mev[2], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&D->mev[3], cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&D->iev[0], cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&D->iev[1], cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&D->lev[0], cudaEventDisableTiming) != cudaSuccess ||
@@ -835,6 +1037,7 @@ int chol_device_ensure(chol_handle* h) {
   if ((rc = upload(h, &D->syrk, h->syrk_tasks))) return fail(rc);
   if ((rc = upload(h, &D->asm_tasks, h->asm_tasks))) return fail(rc);
   if ((rc = upload(h, &D->asm_segs, h->asm_segs))) return fail(rc);
+  if ((rc = upload(h, &D->fasm, h->fasm_tasks))) return fail(rc);
   if ((rc = upload(h, &D->tri, h->tri_items))) return fail(rc);
   if (h->opt.update_mode == CHOL_UPDATE_RLB) {
     std::vector<int4> pr(h->rel_J.size());
@@ -890,10 +1093,151 @@ int chol_device_ensure(chol_handle* h) {
 
 namespace {
 
+// TRSM tasks [b, b + n) of the step; `few`: 8-row CTAs while they fit on the SMs
+// two at a time. split: the rows' slices go to buffer buf.
+void launch_trsm(chol_handle* h, const StepRange& s, int b, int n, bool split, int buf, cudaStream_t st) {
+  if (n <= 0) return;
+  DeviceState* D = h->dev;
+  KScope ks(h, CHOL_K_TRSM, st, s.trsm_flops * n / s.trsm_n, 16.0 * (kTrsmRowsHost / 2) * h->opt.block_cols * n);
+  auto go = [&](auto lpr, auto sp) {
+    constexpr int LPR = decltype(lpr)::value;
+    k_trsm<LPR, decltype(sp)::value><<<n * (LPR / 8), kTrsmThreads, 0, st>>>(
+        D->sn, D->trsm + s.trsm_b + b, h->opt.block_cols, D->L, D->rdiag, D->sg_dev, D->sgt_slab[buf], D->sgt_exps[buf]);
+  };
+  auto pick = [&](auto sp) {
+    if (n <= D->sms) go(std::integral_constant<int, 16>{}, sp);
+    else go(std::integral_constant<int, 8>{}, sp);
+  };
+  if (split) pick(std::true_type{});
+  else pick(std::false_type{});
+}
+
+void launch_potrf(chol_handle* h, const StepRange& s, int k0, cudaStream_t st) {
+  if (s.potrf_n <= 0) return;
+  DeviceState* D = h->dev;
+  const int nb = h->opt.block_cols;
+  KScope ks(h, CHOL_K_POTRF, st, s.potrf_flops, 16.0 * nb * nb * s.potrf_n);
+  k_potrf<<<s.potrf_n, kPotrfThreads, 0, st>>>(D->sn, D->potrf_list + s.potrf_b, k0, nb, D->L, D->rdiag, D->status);
+}
+
+// The column steps of a level's blocked supernodes, updates on the tensor cores.
+// The chain from one diagonal block to the next is POTRF and the link kernel (the
+// TRSM of the next block's 64 rows and that block's update); everything else of
+// a step runs beside it:
+// - main stream (highest priority): the chain;
+// - bulk stream: the other rows' TRSM, then the rest of the next column block
+//   and the diagonal block after it (near tiles): what the chain needs a step
+//   later;
+// - side stream (lowest priority): the other trailing tiles.
+// The chain waits for the near tiles of the step before (its TRSM's rows), the
+// near tiles for the side stream's tiles of the step before (they share
+// columns). Every tile receives its updates in step order. The slices of step k
+// are last read by its side tiles, which are done when step k + 3 writes the
+// same buffer (its TRSM follows near(k + 1), which waited for side(k)).
+// With the whole step on the chain a step of the 37x29x23 grid took 77 us.
+int enqueue_steps_sg(chol_handle* h, const LevelPlan& P, cudaStream_t st) {
+  DeviceState* D = h->dev;
+  const cudaStream_t ms = D->mstream, ls = D->lstream;
+  const int nb = h->opt.block_cols;
+  enum { kFactored = 0, kNextRows = 1, kBulk = 2, kNear = 3 };
+  bool near_pending = false, rest_pending = false;
+  for (size_t k = 0; k < P.steps.size(); ++k) {
+    const StepRange& s = P.steps[k];
+    const int buf = (int)(k % 3);
+    launch_potrf(h, s, (int)k * nb, st);
+    if (s.sgt_n > 0) {
+      CHOL_CUDA_TRY(cudaEventRecord(D->mev[kFactored], st));
+      CHOL_CUDA_TRY(cudaStreamWaitEvent(ms, D->mev[kFactored], 0));
+    }
+    if (near_pending) {
+      CHOL_CUDA_TRY(cudaStreamWaitEvent(st, D->mev[kNear], 0));
+      near_pending = false;
+    }
+    if (s.sgt_n == 0) {   // no supernode goes on past this step
+      launch_trsm(h, s, 0, s.trsm_n, false, 0, st);
+      continue;
+    }
+    const int nrest = s.sgt_n - s.sgt_c - s.sgt_near;
+    const TileTask* tiles = D->sg_trail + s.sgt_b;
+    auto flops = [&](int n) { return s.gemm_flops * n / s.sgt_n; };
+    {
+      KScope ks(h, CHOL_K_GEMM, st, flops(s.sgt_c), 16.0 * kTile * kTile * s.sgt_c);
+      k_link<<<s.sgt_c * kLinkCtas, kLinkThreads, 0, st>>>(D->sn, tiles, D->L, D->rdiag, D->sg_dev, D->sgt_slab[buf],
+                                                           D->sgt_exps[buf]);
+    }
+    CHOL_CUDA_TRY(cudaEventRecord(D->mev[kNextRows], st));
+    launch_trsm(h, s, s.trsm_c, s.trsm_n - s.trsm_c, true, buf, ms);
+    CHOL_CUDA_TRY(cudaStreamWaitEvent(ms, D->mev[kNextRows], 0));
+    if (nrest > 0) {
+      CHOL_CUDA_TRY(cudaEventRecord(D->mev[kBulk], ms));
+      CHOL_CUDA_TRY(cudaStreamWaitEvent(ls, D->mev[kBulk], 0));
+    }
+    if (rest_pending) {
+      CHOL_CUDA_TRY(cudaStreamWaitEvent(ms, D->lev[1], 0));
+      rest_pending = false;
+    }
+    if (s.sgt_near > 0) {
+      KScope ks(h, CHOL_K_GEMM, ms, flops(s.sgt_near), 32.0 * kTile * kTile * s.sgt_near);
+      chol_sg_trailing(h, tiles + s.sgt_c, s.sgt_near, INT_MAX, buf, ms);
+    }
+    CHOL_CUDA_TRY(cudaEventRecord(D->mev[kNear], ms));
+    near_pending = true;
+    if (nrest > 0) {
+      KScope ks(h, CHOL_K_GEMM, ls, flops(nrest), 32.0 * kTile * kTile * nrest);
+      chol_sg_trailing(h, tiles + s.sgt_c + s.sgt_near, nrest, INT_MAX, buf, ls);
+      CHOL_CUDA_TRY(cudaEventRecord(D->lev[1], ls));
+      rest_pending = true;
+    }
+  }
+  if (near_pending) CHOL_CUDA_TRY(cudaStreamWaitEvent(st, D->mev[kNear], 0));
+  if (rest_pending) CHOL_CUDA_TRY(cudaStreamWaitEvent(st, D->lev[1], 0));
+  return CHOL_OK;
+}
+
+// The same steps on the binary64 pipe. One-step lookahead: the trailing tiles of
+// step k other than the next block column ("rest") run on the side stream,
+// beside the POTRF and TRSM of step k + 1 on the main stream. Before step k +
+// 1's own trailing tiles, the main stream waits for step k's rest (they share
+// tiles); the side stream keeps the rests in order. Each tile still receives its
+// updates in step order, so the result is the same as without lookahead.
+int enqueue_steps(chol_handle* h, const LevelPlan& P, cudaStream_t st) {
+  DeviceState* D = h->dev;
+  const int nb = h->opt.block_cols;
+  bool rest_pending = false;
+  for (size_t k = 0; k < P.steps.size(); ++k) {
+    const StepRange& s = P.steps[k];
+    launch_potrf(h, s, (int)k * nb, st);
+    launch_trsm(h, s, 0, s.trsm_n, false, 0, st);
+    const int nrest = s.gemm_n - s.gemm_next;
+    if (nrest > 0) {
+      CHOL_CUDA_TRY(cudaEventRecord(D->lev[0], st));   // step k's panel is final
+      CHOL_CUDA_TRY(cudaStreamWaitEvent(D->lstream, D->lev[0], 0));
+    }
+    if (rest_pending) {
+      CHOL_CUDA_TRY(cudaStreamWaitEvent(st, D->lev[1], 0));   // step k-1's rest
+      rest_pending = false;
+    }
+    if (s.gemm_n > 0) {
+      const double frac = (double)s.gemm_next / s.gemm_n;
+      if (s.gemm_next > 0) {
+        KScope ks(h, CHOL_K_GEMM, st, s.gemm_flops * frac, 16.0 * kTile * kTile * s.gemm_next);
+        k_gemm_trailing<<<s.gemm_next, kGemmThreads, 0, st>>>(D->sn, D->gemm + s.gemm_b, nb, D->L);
+      }
+      if (nrest > 0) {
+        KScope ks(h, CHOL_K_GEMM, D->lstream, s.gemm_flops * (1.0 - frac), 16.0 * kTile * kTile * nrest);
+        k_gemm_trailing<<<nrest, kGemmThreads, 0, D->lstream>>>(D->sn, D->gemm + s.gemm_b + s.gemm_next, nb, D->L);
+        CHOL_CUDA_TRY(cudaEventRecord(D->lev[1], D->lstream));
+        rest_pending = true;
+      }
+    }
+  }
+  if (rest_pending) CHOL_CUDA_TRY(cudaStreamWaitEvent(st, D->lev[1], 0));   // join before SYRK
+  return CHOL_OK;
+}
+
 // Enqueue the binary64 factorization (no synchronization).
 int enqueue_factor_fp64(chol_handle* h, const double* values, cudaStream_t st) {
   DeviceState* D = h->dev;
-  const int nb = h->opt.block_cols;
   k_status_init<<<1, 1, 0, st>>>(D->status);
   CHOL_CUDA_TRY(cudaMemsetAsync(D->L, 0, sizeof(double) * (size_t)h->panel_doubles, st));
   if (h->nnz_a > 0) {
@@ -927,76 +1271,27 @@ int enqueue_factor_fp64(chol_handle* h, const double* values, cudaStream_t st) {
   for (const LevelPlan& P : h->levels) {
     NvtxRange nvtx_level("level", (long long)(&P - h->levels.data()));
     const bool rlb = h->opt.update_mode == CHOL_UPDATE_RLB;
+    // one-CTA supernodes, beside the blocked ones of the level if it has both
+    bool small_pending = false;
     if (P.small_n > 0) {
-      KScope ks(h, CHOL_K_SMALL, st, P.small_flops, P.small_bytes);
+      small_pending = !P.steps.empty();
+      const cudaStream_t ss = small_pending ? D->sstream : st;
+      if (small_pending) {
+        CHOL_CUDA_TRY(cudaEventRecord(D->sev[0], st));
+        CHOL_CUDA_TRY(cudaStreamWaitEvent(ss, D->sev[0], 0));
+      }
+      KScope ks(h, CHOL_K_SMALL, ss, P.small_flops, P.small_bytes);
       if (rlb)
-        k_small_rlb<<<P.small_n, kSmallThreads, sizeof(double) * P.small_max_panel, st>>>(
+        k_small_rlb<<<P.small_n, kSmallThreads, sizeof(double) * P.small_max_panel, ss>>>(
             D->sn, D->small_list + P.small_b, D->rlb_pairs, D->rlb_pbeg, D->rows, D->L, D->status);
       else
-        k_small<<<P.small_n, kSmallThreads, sizeof(double) * P.small_max_panel, st>>>(
+        k_small<<<P.small_n, kSmallThreads, sizeof(double) * P.small_max_panel, ss>>>(
             D->sn, D->small_list + P.small_b, D->L, D->U, D->status);
     }
-    // One-step lookahead: the trailing tiles of step k other than the next
-    // block column ("rest") run on the side stream, beside the POTRF and TRSM
-    // of step k + 1 on the main stream. Before step k + 1's own trailing tiles,
-    // the main stream waits for step k's rest (they share tiles); the side
-    // stream keeps the rests in order. Each tile still receives its updates in
-    // step order, so the result is the same as without lookahead.
-    bool rest_pending = false;
-    for (size_t k = 0; k < P.steps.size(); ++k) {
-      const StepRange& s = P.steps[k];
-      const int k0 = (int)k * nb;
-      if (s.potrf_n > 0) {
-        KScope ks(h, CHOL_K_POTRF, st, s.potrf_flops, 16.0 * nb * nb * s.potrf_n);
-        k_potrf<<<s.potrf_n, kPotrfThreads, 0, st>>>(D->sn, D->potrf_list + s.potrf_b, k0, nb, D->L, D->rdiag,
-                                                     D->status);
-      }
-      const int buf = (int)(k & 1);   // step k + 2 reuses step k's slices: its rest has joined by then
-      if (s.trsm_n > 0) {
-        KScope ks(h, CHOL_K_TRSM, st, s.trsm_flops, 16.0 * (kTrsmRowsHost / 2) * nb * s.trsm_n);
-        // 8-row CTAs while they fit on the SMs two at a time
-        const bool few = s.trsm_n <= D->sms;
-        auto go = [&](auto lpr, auto split) {
-          constexpr int LPR = decltype(lpr)::value;
-          k_trsm<LPR, decltype(split)::value><<<s.trsm_n * (LPR / 8), kTrsmThreads, 0, st>>>(
-              D->sn, D->trsm + s.trsm_b, nb, D->L, D->rdiag, D->sg_dev, D->sgt_slab[buf], D->sgt_exps[buf]);
-        };
-        auto pick = [&](auto split) {
-          if (few) go(std::integral_constant<int, 16>{}, split);
-          else go(std::integral_constant<int, 8>{}, split);
-        };
-        if (sg) pick(std::true_type{});
-        else pick(std::false_type{});
-      }
-      const int gemm_n = sg ? s.sgt_n : s.gemm_n, gemm_next = sg ? s.sgt_next : s.gemm_next;
-      const int nrest = gemm_n - gemm_next;
-      if (nrest > 0) {
-        CHOL_CUDA_TRY(cudaEventRecord(D->lev[0], st));   // step k's panel is final
-        CHOL_CUDA_TRY(cudaStreamWaitEvent(D->lstream, D->lev[0], 0));
-      }
-      if (rest_pending) {
-        CHOL_CUDA_TRY(cudaStreamWaitEvent(st, D->lev[1], 0));   // step k-1's rest
-        rest_pending = false;
-      }
-      if (gemm_n > 0) {
-        const double frac = (double)gemm_next / gemm_n;
-        const double tile_bytes = 16.0 * kTile * kTile * (sg ? 2 : 1);
-        if (gemm_next > 0) {
-          KScope ks(h, CHOL_K_GEMM, st, s.gemm_flops * frac, tile_bytes * gemm_next);
-          if (sg) chol_sg_trailing(h, D->sg_trail + s.sgt_b, gemm_next, D->sms, buf, st);
-          else k_gemm_trailing<<<gemm_next, kGemmThreads, 0, st>>>(D->sn, D->gemm + s.gemm_b, nb, D->L);
-        }
-        if (nrest > 0) {
-          KScope ks(h, CHOL_K_GEMM, D->lstream, s.gemm_flops * (1.0 - frac), tile_bytes * nrest);
-          if (sg) chol_sg_trailing(h, D->sg_trail + s.sgt_b + gemm_next, nrest, INT_MAX, buf, D->lstream);
-          else
-            k_gemm_trailing<<<nrest, kGemmThreads, 0, D->lstream>>>(D->sn, D->gemm + s.gemm_b + gemm_next, nb, D->L);
-          CHOL_CUDA_TRY(cudaEventRecord(D->lev[1], D->lstream));
-          rest_pending = true;
-        }
-      }
-    }
-    if (rest_pending) CHOL_CUDA_TRY(cudaStreamWaitEvent(st, D->lev[1], 0));   // join before SYRK
+    if (small_pending) CHOL_CUDA_TRY(cudaEventRecord(D->sev[1], D->sstream));
+    if (int rc = sg ? enqueue_steps_sg(h, P, st) : enqueue_steps(h, P, st)) return rc;
+    // (a level's small supernodes may have triangle items too)
+    if (small_pending) CHOL_CUDA_TRY(cudaStreamWaitEvent(st, D->sev[1], 0));
     // the level's diagonal blocks are final: their inverses (for the triangle
     // solves) on a side stream, beside the SYRK, the assembly and later levels
     if (P.tri_n > 0) {
@@ -1018,13 +1313,14 @@ int enqueue_factor_fp64(chol_handle* h, const double* values, cudaStream_t st) {
     }
     if (!rlb && P.asm_n + P.asmw_n > 0) {
       KScope ks(h, CHOL_K_ASSEMBLE, st, P.asm_entries, 24.0 * P.asm_entries);
-      ks.launches((P.asm_n > 0) + (P.asmw_n > 0));
-      if (P.asm_n > 0)
-        k_assemble<<<P.asm_n, kAsmThreads, sizeof(int32_t) * 2 * kAsmPos, st>>>(
+      const AsmSplit a = asm_split(P, D->sms);
+      ks.launches((a.ctas > 0) + (a.warps > 0));
+      if (a.ctas > 0)
+        k_assemble<<<a.ctas, kAsmThreads, sizeof(int32_t) * 2 * kAsmPos, st>>>(
             D->asm_tasks + P.asm_b, D->asm_segs, D->sn, D->rows, D->U, D->L);
-      if (P.asmw_n > 0)
-        k_assemble_warp<double, false><<<(P.asmw_n + 7) / 8, 256, 0, st>>>(
-            D->asm_tasks + P.asm_b + P.asm_n, P.asmw_n, D->asm_segs, D->sn, D->rows, D->U, D->L);
+      if (a.warps > 0)
+        k_assemble_warp<double, false><<<(a.warps + 7) / 8, 256, 0, st>>>(
+            D->asm_tasks + P.asm_b + a.ctas, a.warps, D->asm_segs, D->sn, D->rows, D->U, D->L);
     }
   }
   if (inv_pending) {   // the inverses join the factor's stream before it ends
@@ -1045,11 +1341,12 @@ int enqueue_factor_fp64(chol_handle* h, const double* values, cudaStream_t st) {
 // ancestors' panels of Z.
 void chol_gather_zrr(chol_handle* h, const LevelPlan& P, const double* Z, double* ZRR, cudaStream_t st) {
   DeviceState* D = h->dev;
-  if (P.asm_n > 0)
-    k_gather_zrr<<<P.asm_n, kAsmThreads, sizeof(int32_t) * 2 * kAsmPos, st>>>(D->asm_tasks + P.asm_b, D->asm_segs, D->sn,
+  const AsmSplit a = asm_split(P, D->sms);
+  if (a.ctas > 0)
+    k_gather_zrr<<<a.ctas, kAsmThreads, sizeof(int32_t) * 2 * kAsmPos, st>>>(D->asm_tasks + P.asm_b, D->asm_segs, D->sn,
                                                                              D->rows, ZRR, Z);
-  if (P.asmw_n > 0)
-    k_assemble_warp<double, false, true><<<(P.asmw_n + 7) / 8, 256, 0, st>>>(D->asm_tasks + P.asm_b + P.asm_n, P.asmw_n,
+  if (a.warps > 0)
+    k_assemble_warp<double, false, true><<<(a.warps + 7) / 8, 256, 0, st>>>(D->asm_tasks + P.asm_b + a.ctas, a.warps,
                                                                              D->asm_segs, D->sn, D->rows, ZRR, Z);
 }
 
@@ -1316,6 +1613,14 @@ extern "C" int chol_autotune(chol_handle* h, const double* values, void* stream)
   return chol_factor(h, values, stream);
 }
 
+// A warp per supernode; 8 lanes for the tens of thousands of a batch (8 columns
+// on average).
+static void logdet_parts(chol_handle* h, cudaStream_t st) {
+  DeviceState* D = h->dev;
+  if (h->ns > 32768) k_logdet_part<8><<<(h->ns + 31) / 32, 256, 0, st>>>(D->sn, h->ns, D->L, D->part);
+  else k_logdet_part<32><<<(h->ns + 7) / 8, 256, 0, st>>>(D->sn, h->ns, D->L, D->part);
+}
+
 extern "C" int chol_logdet_batch(chol_handle* h, double* out, void* stream) {
   if (!h) return -1;
   if (!out) return -2;
@@ -1331,7 +1636,7 @@ extern "C" int chol_logdet_batch(chol_handle* h, double* out, void* stream) {
   }
   if (h->ns > 0) {
     if (h->opt.precision == CHOL_PREC_FP64)
-      k_logdet_part<<<h->ns, 128, 0, st>>>(D->sn, D->L, D->part);
+      logdet_parts(h, st);
     else if ((rc = chol_logdet_parts_mixed(h, st)))
       return rc;
   }
@@ -1351,7 +1656,7 @@ extern "C" int chol_logdet(chol_handle* h, double* out, void* stream) {
   if (h->opt.precision != CHOL_PREC_FP64) return chol_logdet_mixed(h, out, st);
   if (h->ns > 0) {
     KScope ks(h, CHOL_K_LOGDET, st, (double)h->n, 8.0 * h->n);
-    k_logdet_part<<<h->ns, 128, 0, st>>>(D->sn, D->L, D->part);
+    logdet_parts(h, st);
     k_logdet_reduce<<<1, 1024, 0, st>>>(D->part, h->ns, D->scalar_dev);
   } else {
     CHOL_CUDA_TRY(cudaMemsetAsync(D->scalar_dev, 0, sizeof(double), st));

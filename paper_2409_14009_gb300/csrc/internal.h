@@ -85,7 +85,11 @@ struct AsmSeg {
 struct StepRange {
   int32_t potrf_b, potrf_n, trsm_b, trsm_n, gemm_b, gemm_n, ogemm_b, ogemm_n, ok0, okb;
   int32_t gemm_next, ogemm_next;
-  int32_t sgt_b, sgt_n, sgt_next;   // binary64 on the tensor cores: 128 x 64 trailing tiles (in sgt_tasks), next column first
+  // binary64 on the tensor cores: trailing tiles (in sgt_tasks; TileTask.k0 = rows,
+  // 64 or 128), first the next diagonal blocks (sgt_c), then the rest of the next
+  // column block and the diagonal block after it (sgt_near), then the others; and
+  // the TRSM tasks with the next diagonal blocks' rows first (trsm_c)
+  int32_t sgt_b, sgt_n, sgt_c, sgt_near, trsm_c;
   int32_t panel_b, panel_n, panel_ticket, join_rest;
   double potrf_flops, trsm_flops, gemm_flops, ogemm_flops, panel_flops;
 };
@@ -118,6 +122,7 @@ struct LevelPlan {
   int32_t sgr_b, sgr_n;       // ... and the 64-row tasks that split their operands (in split_tasks)
   int32_t asm_b, asm_n;       // assembly tasks, one CTA each
   int32_t asmw_n;             // then (from asm_b + asm_n) small tasks, one warp each
+  int32_t fasm_b, fasm_n;     // the first position chunks among the tasks (in fasm_tasks): the forward solve's assembly
   int32_t tri_b, tri_n;       // diagonal-triangle solve items (in tri_items), dependency order
   int32_t ssmall_b, ssmall_n; // supernodes solved by one warp each (in ssmall_list),
   int32_t ssmall8_n;          // the first ssmall8_n of them with s <= 8
@@ -197,6 +202,7 @@ struct chol_handle {
   int32_t panel_nflags = 0, panel_ntickets = 0; // progress flags and work counters of all panel launches
   std::vector<AsmTask> asm_tasks;
   std::vector<AsmSeg> asm_segs;
+  std::vector<int32_t> fasm_tasks;              // indices into asm_tasks
   int32_t n_small = 0, n_large = 0;
   // batches and launch configuration
   std::vector<int32_t> sys_ptr;       // count+1 column offsets of the systems

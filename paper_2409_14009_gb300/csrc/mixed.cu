@@ -881,13 +881,14 @@ int chol_enqueue_factor_mixed(chol_handle* h, const double* values, cudaStream_t
     }
     if (P.asm_n + P.asmw_n > 0) {
       KScope ks(h, CHOL_K_ASSEMBLE, st, P.asm_entries, 12.0 * P.asm_entries);
-      ks.launches((P.asm_n > 0) + (P.asmw_n > 0));
-      if (P.asm_n > 0)
-        k_mx_assemble<<<P.asm_n, kMxThreads, sizeof(int32_t) * 2 * kAsmPos, st>>>(
+      const AsmSplit a = asm_split(P, D->sms);
+      ks.launches((a.ctas > 0) + (a.warps > 0));
+      if (a.ctas > 0)
+        k_mx_assemble<<<a.ctas, kMxThreads, sizeof(int32_t) * 2 * kAsmPos, st>>>(
             D->asm_tasks + P.asm_b, D->asm_segs, D->sn, D->rows, U, L);
-      if (P.asmw_n > 0)
-        k_assemble_warp<float, true><<<(P.asmw_n + 7) / 8, 256, 0, st>>>(
-            D->asm_tasks + P.asm_b + P.asm_n, P.asmw_n, D->asm_segs, D->sn, D->rows, U, L);
+      if (a.warps > 0)
+        k_assemble_warp<float, true><<<(a.warps + 7) / 8, 256, 0, st>>>(
+            D->asm_tasks + P.asm_b + a.ctas, a.warps, D->asm_segs, D->sn, D->rows, U, L);
     }
   }
   if (st != caller) {

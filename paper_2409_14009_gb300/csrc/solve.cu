@@ -483,18 +483,27 @@ k_sv_gemv(const SnodeDev* __restrict__ sn, const TileTask* __restrict__ tasks, c
 }
 
 // y[targets] -= w_J through the relind task lists (pull-ordered), one warp per
-// task: only the first position chunk of a column tile holds the segments'
-// columns; segments are applied in order (the same y entries can appear in
-// several), so each entry receives its contributions in a fixed order.
+// task (the first position chunk of a column tile holds the segments' columns);
+// segments are applied in order (the same y entries can appear in several), so
+// each entry receives its contributions in a fixed order. Two forms of the same
+// arithmetic:
+// - k_sv_fasm_many, for the tens of thousands of tasks of a batch (a few short
+//   segments each): straight to y, other warps hide the loads;
+// - k_sv_fasm, when the tasks do not fill the GPU and the cost is the chain of
+//   loads: the lanes fetch 32 segments' descriptors at once, the values of four
+//   segments are in flight together, and the tile of y stays in shared memory, so
+//   a segment waits for no load of the one before it.
+// Batch of 1,000: 0.42 ms a solve with the first, 0.67 with the second; 2D 64^2:
+// 0.26 and 0.20.
+constexpr int kFasmMany = 16384;   // tasks from which a level takes the first form
 template <class T>
 __global__ void __launch_bounds__(kT)
-k_sv_fasm(const AsmTask* __restrict__ tasks, int ntasks, const AsmSeg* __restrict__ segs,
-          const SnodeDev* __restrict__ sn, const int32_t* __restrict__ rows, const T* __restrict__ W,
-          T* __restrict__ Y, int n, int nrhs) {
+k_sv_fasm_many(const int32_t* __restrict__ list, int ntasks, const AsmTask* __restrict__ tasks,
+               const AsmSeg* __restrict__ segs, const SnodeDev* __restrict__ sn, const int32_t* __restrict__ rows,
+               const T* __restrict__ W, T* __restrict__ Y, int n, int nrhs) {
   const int i = blockIdx.x * (kT / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= ntasks) return;
-  const AsmTask t = tasks[i];
-  if (t.p0 != t.t0) return;
+  const AsmTask t = tasks[list[i]];
   for (int g = t.seg_begin; g < t.seg_end; ++g) {
     const AsmSeg sg = segs[g];
     const SnodeDev dj = sn[sg.J];
@@ -508,6 +517,71 @@ k_sv_fasm(const AsmTask* __restrict__ tasks, int ntasks, const AsmSeg* __restric
     }
     __syncwarp();
   }
+}
+
+template <class T>
+__global__ void __launch_bounds__(kT)
+k_sv_fasm(const int32_t* __restrict__ list, int ntasks, const AsmTask* __restrict__ tasks,
+          const AsmSeg* __restrict__ segs, const SnodeDev* __restrict__ sn, const int32_t* __restrict__ rows,
+          const T* __restrict__ W, T* __restrict__ Y, int n, int nrhs) {
+  extern __shared__ __align__(16) unsigned char fasm_smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int i = blockIdx.x * (kT / 32) + warp;
+  if (i >= ntasks) return;
+  T* acc = reinterpret_cast<T*>(fasm_smem) + warp * kAsmCols * nrhs;   // tile column c, right-hand side r: acc[c + 32 r]
+  const AsmTask t = tasks[list[i]];
+  const int y0 = sn[t.K].f + t.t0, nc = t.t1 - t.t0;
+  for (int r = 0; r < nrhs; ++r)
+    if (lane < nc) acc[lane + kAsmCols * r] = Y[y0 + lane + (int64_t)r * n];
+  constexpr int kFly = 4;   // segments in flight
+  for (int g0 = t.seg_begin; g0 < t.seg_end; g0 += 32) {
+    const int ng = min(32, t.seg_end - g0);
+    AsmSeg sg{};
+    int b = 0, ncol = 0;
+    int64_t ro = 0, wo = 0;
+    if (lane < ng) {
+      sg = segs[g0 + lane];
+      const SnodeDev dj = sn[sg.J];
+      b = dj.len - dj.s;
+      ncol = sg.cb - sg.ca;
+      ro = dj.roff + dj.s + sg.ca;
+      wo = dj.wpre * nrhs + sg.ca;
+    }
+    for (int g = 0; g < ng; g += kFly) {
+      T v[kFly];
+      int pos[kFly], nq[kFly], nk[kFly], bk[kFly];
+      int64_t rk[kFly], wk[kFly];
+#pragma unroll
+      for (int k = 0; k < kFly; ++k) {
+        pos[k] = -1;
+        nq[k] = 0;
+        if (g + k >= ng) continue;   // uniform
+        nk[k] = __shfl_sync(0xffffffffu, ncol, g + k);
+        bk[k] = __shfl_sync(0xffffffffu, b, g + k);
+        rk[k] = __shfl_sync(0xffffffffu, ro, g + k);
+        wk[k] = __shfl_sync(0xffffffffu, wo, g + k);
+        nq[k] = nk[k] * nrhs;
+        if (lane < nq[k]) {
+          const int r = nrhs == 1 ? 0 : lane / nk[k], c = lane - r * nk[k];
+          v[k] = W[wk[k] + c + (int64_t)r * bk[k]];
+          pos[k] = rows[rk[k] + c] - y0 + kAsmCols * r;
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < kFly; ++k) {
+        if (g + k >= ng) continue;
+        __syncwarp();   // the previous segment is in the tile
+        if (pos[k] >= 0) acc[pos[k]] -= v[k];
+        for (int q = lane + 32; q < nq[k]; q += 32) {
+          const int r = q / nk[k], c = q - r * nk[k];
+          acc[rows[rk[k] + c] - y0 + kAsmCols * r] -= W[wk[k] + c + (int64_t)r * bk[k]];
+        }
+      }
+    }
+  }
+  __syncwarp();
+  for (int r = 0; r < nrhs; ++r)
+    if (lane < nc) Y[y0 + lane + (int64_t)r * n] = acc[lane + kAsmCols * r];
 }
 
 // Backward panel: y_J[c] -= sum_u L(s+u, c) x[rows[s+u]] for the columns of a task.
@@ -1304,12 +1378,15 @@ int solve_levels(chol_handle* h, const T* L, T* Y, T* W, T* part, int nr, cudaSt
       });
       delete ks;
     }
-    if (P.asm_n + P.asmw_n > 0) {
-      // the CTA-sized and the warp-sized assembly tasks of the level, contiguous
+    if (P.fasm_n > 0) {
       KScope* ks = scope(CHOL_K_SOLVE_FASM);
-      const int nt = P.asm_n + P.asmw_n;
-      k_sv_fasm<T><<<(nt + kT / 32 - 1) / (kT / 32), kT, 0, st>>>(D->asm_tasks + P.asm_b, nt, D->asm_segs, D->sn,
-                                                                  D->rows, W, Y, n, nr);
+      const int grid = (P.fasm_n + kT / 32 - 1) / (kT / 32);
+      if (P.fasm_n >= kFasmMany)
+        k_sv_fasm_many<T><<<grid, kT, 0, st>>>(D->fasm + P.fasm_b, P.fasm_n, D->asm_tasks, D->asm_segs, D->sn, D->rows, W,
+                                               Y, n, nr);
+      else
+        k_sv_fasm<T><<<grid, kT, sizeof(T) * (kT / 32) * kAsmCols * nr, st>>>(
+            D->fasm + P.fasm_b, P.fasm_n, D->asm_tasks, D->asm_segs, D->sn, D->rows, W, Y, n, nr);
       delete ks;
     }
   }

@@ -60,8 +60,8 @@ k_sg_split_rows(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd
 
 __device__ __forceinline__ uint32_t smem_base(const unsigned char* p) { return (tc::smem_u32(p) + 1023u) & ~1023u; }
 
-// Trailing update of the panel, step k0: 128 x 64 tiles, K = 64, one chunk per
-// tile. The thread's entries of C are loaded before the wait for the products.
+// Trailing update of the panel: tiles of 64 columns and 128 (or only 64) rows,
+// K = 64, one chunk per tile. The thread's entries of C are loaded before the wait for the products.
 __global__ void __launch_bounds__(sg::kThreads, 1)
 k_sg_trailing(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, const TileTask* __restrict__ tasks,
               int ntasks, const unsigned char* __restrict__ slab, const int32_t* __restrict__ exps,
@@ -92,7 +92,7 @@ k_sg_trailing(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, 
       const SnodeDev d = sn[k.J];
       const int r = k.r0 + sg::epi_row(), c0 = k.c0 + sg::epi_col();
       // the thread's columns c0 .. c0 + n - 1 (on or below the diagonal)
-      const int n = r < d.len ? min(sg::kCols, min(d.s, r + 1) - c0) : 0;
+      const int n = r < min(d.len, k.r0 + k.k0) ? min(sg::kCols, min(d.s, r + 1) - c0) : 0;
       const int32_t ea = n > 0 ? t.a.exps[r] : 0;
       double* C = L + d.loff + r + (int64_t)c0 * d.ld;
       double cv[sg::kCols];
@@ -208,8 +208,10 @@ std::vector<SgBuffer> sg_buffers(chol_handle* h) {
           {(void**)&D->sg_exps, h->split_exps * 4},
           {(void**)&D->sgt_slab[0], h->split_trows * 64},
           {(void**)&D->sgt_slab[1], h->split_trows * 64},
+          {(void**)&D->sgt_slab[2], h->split_trows * 64},
           {(void**)&D->sgt_exps[0], h->split_texps * 4},
           {(void**)&D->sgt_exps[1], h->split_texps * 4},
+          {(void**)&D->sgt_exps[2], h->split_texps * 4},
           {(void**)&D->sg_dev, (int64_t)(sizeof(SplitDev) * h->split.size())},
           {(void**)&D->sg_split, (int64_t)(sizeof(TileTask) * h->split_tasks.size())},
           {(void**)&D->sg_syrk, (int64_t)(sizeof(TileTask) * h->sgs_tasks.size())},
@@ -259,7 +261,7 @@ int chol_sg_ensure(chol_handle* h) {
   return CHOL_OK;
 }
 
-// Trailing tiles from the slices of parity `buf` (written by k_trsm).
+// Trailing tiles from the slices in buffer `buf` (written by k_trsm).
 void chol_sg_trailing(chol_handle* h, const TileTask* tasks, int n, int grid, int buf, cudaStream_t st) {
   DeviceState* D = h->dev;
   k_sg_trailing<<<std::min(n, grid), sg::kThreads, sg::kSmemBytes, st>>>(D->sn, D->sg_dev, tasks, n, D->sgt_slab[buf],
