@@ -719,7 +719,10 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
       if (warp_solved(J) && h->snodes[J].s <= 8) h->ssmall_list.push_back(J);
     P.ssmall8_n = (int32_t)h->ssmall_list.size() - P.ssmall_b;
     for (int32_t J : Js)
-      if (warp_solved(J) && h->snodes[J].s > 8) h->ssmall_list.push_back(J);
+      if (warp_solved(J) && h->snodes[J].s > 8 && h->snodes[J].s <= 16) h->ssmall_list.push_back(J);
+    P.ssmall16_n = (int32_t)h->ssmall_list.size() - P.ssmall_b - P.ssmall8_n;
+    for (int32_t J : Js)
+      if (warp_solved(J) && h->snodes[J].s > 16) h->ssmall_list.push_back(J);
     P.ssmall_n = (int32_t)h->ssmall_list.size() - P.ssmall_b;
     P.tri_b = (int32_t)h->tri_items.size();
     for (int32_t J : Js) {

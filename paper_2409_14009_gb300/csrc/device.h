@@ -27,7 +27,7 @@ struct DeviceState {
   AsmSeg* asm_segs = nullptr;
   int32_t* fasm = nullptr;      // solve: the assembly tasks that hold their segments' columns
   TriItemHost* tri = nullptr;   // solve: diagonal-triangle items
-  double* rdiag = nullptr;      // binary64 blocked path: reciprocal pivots, per column of P A P^T
+  double* rdiag = nullptr;      // binary64: reciprocals of diag(L), per column of P A P^T
   int sg_ready = 0;             // binary64 updates on the tensor cores: 1 = in use, -1 = not
   unsigned char* sg_slab = nullptr;              // slices of a level's off-diagonal rows
   int32_t* sg_exps = nullptr;                    // ... and their row exponents

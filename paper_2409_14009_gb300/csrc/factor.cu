@@ -49,7 +49,8 @@ constexpr int kAsmThreads = 256;
 // Columns [c0, c0 + w) one at a time, right-looking inside the panel, one thread
 // per row: narrow panels (most supernodes of a 2D grid's lower levels) and
 // panels with a pivot that is not positive, normal and finite.
-__device__ void small_panel_columns(double* P, int ld, int len, int c0, int w, int fcol, int* status, double* srk) {
+__device__ void small_panel_columns(double* P, int ld, int len, int c0, int w, int fcol, int* status, double* srk,
+                                    double* __restrict__ rdiag) {
   for (int k = c0; k < c0 + w; ++k) {
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -60,6 +61,7 @@ __device__ void small_panel_columns(double* P, int ld, int len, int c0, int w, i
       P[k + k * ld] = dk;
       *srk = rk;
       if (bad) atomicMin(status, fcol + k + 1);
+      rdiag[k] = fma(fma(-dk, rk, 1.0), rk, rk);
     }
     __syncthreads();
     const double inv = *srk;
@@ -78,7 +80,7 @@ __device__ void small_panel_columns(double* P, int ld, int len, int c0, int w, i
 // diagonal rows (lanes 0-7, the same in all warps; identity past w) and 24 rows
 // below them a pass, and factors them in straight-line code (potrf.cuh). False
 // (uniform): some pivot is not positive, normal and finite, nothing written.
-__device__ __forceinline__ bool small_panel_warps(double* P, int ld, int len, int c0, int w) {
+__device__ __forceinline__ bool small_panel_warps(double* P, int ld, int len, int c0, int w, double* __restrict__ rdiag) {
   const int lane = threadIdx.x & 31, v = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int below = len - c0 - w;
   double dg = 0.0, rd = 0.0, xd[8];
@@ -118,17 +120,20 @@ __device__ __forceinline__ bool small_panel_warps(double* P, int ld, int len, in
 #pragma unroll
     for (int t = 0; t < 8; ++t)
       if (t <= lane) P[c0 + lane + (c0 + t) * ld] = t == lane ? dg : xd[t];
+    rdiag[c0 + lane] = fma(fma(-dg, rd, 1.0), rd, rd);
   }
   __syncthreads();
   return true;
 }
 
-__device__ void dense_chol_smem(double* P, int ld, int len, int s, int fcol, int* status) {
+// rdiag: receives the reciprocals of the s diagonal entries.
+__device__ void dense_chol_smem(double* P, int ld, int len, int s, int fcol, int* status, double* __restrict__ rdiag) {
   __shared__ double srk;
   __syncthreads();
   for (int c0 = 0; c0 < s; c0 += 8) {
     const int w = min(8, s - c0), n0 = c0 + w;
-    if (w <= 4 || !small_panel_warps(P, ld, len, c0, w)) small_panel_columns(P, ld, len, c0, w, fcol, status, &srk);
+    if (w <= 4 || !small_panel_warps(P, ld, len, c0, w, rdiag))
+      small_panel_columns(P, ld, len, c0, w, fcol, status, &srk, rdiag);
     if (n0 >= s) break;
     // the panel's rank-w product from the columns right of it, lower part: column
     // i has R - i entries; columns p and m - 1 - p together have S
@@ -174,12 +179,12 @@ __global__ void k_scatter(const double* __restrict__ vals, const int64_t* __rest
 
 // One CTA per small supernode: the whole len x s panel lives in shared memory.
 __device__ __forceinline__ void small_body(const SnodeDev& d, double* __restrict__ L, double* __restrict__ U,
-                                           int* status, double* P) {
+                                           int* status, double* P, double* __restrict__ rdiag) {
   const int len = d.len, s = d.s, b = len - s;
   double* G = L + d.loff;
   for (int c = 0; c < s; ++c)
     for (int r = threadIdx.x; r < len; r += blockDim.x) P[r + c * len] = G[r + (int64_t)c * d.ld];
-  dense_chol_smem(P, len, len, s, d.f, status);
+  dense_chol_smem(P, len, len, s, d.f, status, rdiag + d.f);
   for (int c = 0; c < s; ++c)
     for (int r = c + threadIdx.x; r < len; r += blockDim.x) G[r + (int64_t)c * d.ld] = P[r + c * len];
   if (b <= 0) return;
@@ -201,9 +206,9 @@ __device__ __forceinline__ void small_body(const SnodeDev& d, double* __restrict
 
 __global__ void __launch_bounds__(kSmallThreads)
 k_small(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list, double* __restrict__ L,
-        double* __restrict__ U, int* status) {
+        double* __restrict__ U, int* status, double* __restrict__ rdiag) {
   extern __shared__ double P[];
-  small_body(sn[list[blockIdx.x]], L, U, status, P);
+  small_body(sn[list[blockIdx.x]], L, U, status, P, rdiag);
 }
 
 // RLB form of the one-CTA kernel: after the factorization in shared memory,
@@ -212,7 +217,7 @@ k_small(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list, doubl
 __global__ void __launch_bounds__(kSmallThreads)
 k_small_rlb(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list, const int4* __restrict__ pairs,
             const int32_t* __restrict__ pbeg, const int32_t* __restrict__ rows, double* __restrict__ L,
-            int* status) {
+            int* status, double* __restrict__ rdiag) {
   extern __shared__ double P[];
   __shared__ int32_t pos[kRlbSmallRows];
   const int32_t J = list[blockIdx.x];
@@ -221,7 +226,7 @@ k_small_rlb(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list, c
   double* G = L + d.loff;
   for (int c = 0; c < s; ++c)
     for (int r = threadIdx.x; r < len; r += blockDim.x) P[r + c * len] = G[r + (int64_t)c * d.ld];
-  dense_chol_smem(P, len, len, s, d.f, status);
+  dense_chol_smem(P, len, len, s, d.f, status, rdiag + d.f);
   for (int c = 0; c < s; ++c)
     for (int r = c + threadIdx.x; r < len; r += blockDim.x) G[r + (int64_t)c * d.ld] = P[r + c * len];
   if (b <= 0) return;
@@ -743,14 +748,14 @@ __global__ void __launch_bounds__(NT)
 k_persist_factor(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ small_list,
                  const AsmTask* __restrict__ tasks, const AsmSeg* __restrict__ segs,
                  const int32_t* __restrict__ rows, const PersistLevel* __restrict__ lv, int nlevels,
-                 double* __restrict__ L, double* __restrict__ U, int* status) {
+                 double* __restrict__ L, double* __restrict__ U, int* status, double* __restrict__ rdiag) {
   extern __shared__ double psm[];
   cg::grid_group grid = cg::this_grid();
   for (int l = 0; l < nlevels; ++l) {
     const PersistLevel p = lv[l];
     for (int i = blockIdx.x; i < p.small_n; i += gridDim.x) {
       __syncthreads();
-      small_body(sn[small_list[p.small_b + i]], L, U, status, psm);
+      small_body(sn[small_list[p.small_b + i]], L, U, status, psm, rdiag);
     }
     grid.sync();
     for (int i = blockIdx.x; i < p.asm_n; i += gridDim.x) {
@@ -1073,8 +1078,8 @@ int chol_device_ensure(chol_handle* h) {
   if ((rc = upload(h, &D->perm, h->perm))) return fail(rc);
   if ((rc = chol_dalloc(h, (void**)&D->part, sizeof(double) * (size_t)std::max(h->ns, 1)))) return fail(rc);
   if ((rc = chol_dalloc(h, (void**)&D->scalar_dev, sizeof(double)))) return fail(rc);
-  if (h->opt.precision == CHOL_PREC_FP64 && h->n_large > 0 &&
-      (rc = chol_dalloc(h, (void**)&D->rdiag, sizeof(double) * (size_t)h->n)))
+  if (h->opt.precision == CHOL_PREC_FP64 &&
+      (rc = chol_dalloc(h, (void**)&D->rdiag, sizeof(double) * (size_t)std::max(h->n, 1))))
     return fail(rc);
   if (cudaMallocHost((void**)&D->status_host, 8 * sizeof(int32_t)) != cudaSuccess) return fail(CHOL_ENOMEM);
   if (cudaMallocHost((void**)&D->scalar_host, sizeof(double)) != cudaSuccess) return fail(CHOL_ENOMEM);
@@ -1283,10 +1288,10 @@ int enqueue_factor_fp64(chol_handle* h, const double* values, cudaStream_t st) {
       KScope ks(h, CHOL_K_SMALL, ss, P.small_flops, P.small_bytes);
       if (rlb)
         k_small_rlb<<<P.small_n, kSmallThreads, sizeof(double) * P.small_max_panel, ss>>>(
-            D->sn, D->small_list + P.small_b, D->rlb_pairs, D->rlb_pbeg, D->rows, D->L, D->status);
+            D->sn, D->small_list + P.small_b, D->rlb_pairs, D->rlb_pbeg, D->rows, D->L, D->status, D->rdiag);
       else
         k_small<<<P.small_n, kSmallThreads, sizeof(double) * P.small_max_panel, ss>>>(
-            D->sn, D->small_list + P.small_b, D->L, D->U, D->status);
+            D->sn, D->small_list + P.small_b, D->L, D->U, D->status, D->rdiag);
     }
     if (small_pending) CHOL_CUDA_TRY(cudaEventRecord(D->sev[1], D->sstream));
     if (int rc = sg ? enqueue_steps_sg(h, P, st) : enqueue_steps(h, P, st)) return rc;
@@ -1389,6 +1394,9 @@ int chol_launch_persistent(chol_handle* h, void* L, void* U, cudaStream_t st) {
   const int grid = per_sm * sms;
   int nlevels = h->nlevels;
   D->mx_spiv = h->opt.static_pivot ? (float)h->opt.pivot_tau : 0.f;
+  // the kernels of the two precisions share all but the last arguments
+  void* args64[] = {(void*)&D->sn, (void*)&D->small_list, (void*)&D->asm_tasks, (void*)&D->asm_segs, (void*)&D->rows,
+                    (void*)&D->plevels, (void*)&nlevels, (void*)&L, (void*)&U, (void*)&D->status, (void*)&D->rdiag};
   void* args[] = {(void*)&D->sn, (void*)&D->small_list, (void*)&D->asm_tasks, (void*)&D->asm_segs,
                   (void*)&D->rows, (void*)&D->plevels, (void*)&nlevels, (void*)&L, (void*)&U,
                   (void*)&D->status, (void*)&D->mx_spiv, (void*)&D->mx_fallbacks};
@@ -1402,7 +1410,7 @@ int chol_launch_persistent(chol_handle* h, void* L, void* U, cudaStream_t st) {
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  CHOL_CUDA_TRY(cudaLaunchKernelExC(&cfg, fn, args));
+  CHOL_CUDA_TRY(cudaLaunchKernelExC(&cfg, fn, fp64 ? args64 : args));
   return CHOL_OK;
 }
 

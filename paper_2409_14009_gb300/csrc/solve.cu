@@ -782,74 +782,173 @@ k_sv_bred(const SnodeDev* __restrict__ sn, const TileTask* __restrict__ tasks, c
   }
 }
 
-// Small supernodes (s <= 32, len <= 256), one warp each. Lane i holds row i of
-// the diagonal block in registers (loaded once, with the reciprocal pivots), so
-// the substitution chain is shuffles and FMAs only. Forward: the solved entry
-// is broadcast by shuffle; then w_J = L_RJ y_J with lanes along the
-// off-diagonal rows. S bounds s (8 or 32), which sizes the register copy of
-// the row.
-template <class T, bool RM, int S>
+// Small supernodes (s <= 32, len <= 256): a group of G = 8, 16 or 32 lanes each
+// (s <= G), so that a warp holds four, two or one. A warp-wide FP64 instruction
+// takes its partition 64 cycles whatever its active lanes, and a batch's
+// supernodes have 8 columns on average: one a warp left three quarters of the
+// pipe, and of the loads in flight, unused (batch of 1,000: 3.4 ms a solve).
+// Lane i of a group holds row i of the diagonal block in registers (binary64:
+// scaled by the reciprocal pivot, so a substitution step is a shuffle and one
+// FMA; binary32 keeps the unscaled rows, which rounds once less per entry).
+// Forward: substitution by shuffles, then w_J = L_RJ y_J, a lane per row of a
+// G-row group with all s entries loaded at once.
+template <int G>
+__device__ __forceinline__ unsigned group_mask() {
+  return G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u) << ((threadIdx.x & 31) & ~(G - 1));
+}
+
+template <class T>
+__device__ __forceinline__ T pivot_recip(const T* __restrict__ P, const SnodeDev& d, int i, bool rm,
+                                         const double* __restrict__ rdiag) {
+  if constexpr (sizeof(T) == 8) return rdiag[d.f + i];
+  else return T(1) / P[(int64_t)i * d.ld + i];
+}
+
+template <class T, bool RM, int G>
 __global__ void __launch_bounds__(kT)
 k_sv_small_fwd(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list, int count,
-               const T* __restrict__ L, T* __restrict__ Y, int n, T* __restrict__ W, int nrhs) {
-  __shared__ T ysh[kT / 32][S];
-  const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (wid >= count) return;
-  const SnodeDev d = sn[list[wid]];
+               const T* __restrict__ L, const double* __restrict__ rdiag, T* __restrict__ Y, int n, T* __restrict__ W,
+               int nrhs) {
+  const int gid = (blockIdx.x * blockDim.x + threadIdx.x) / G, g = threadIdx.x & (G - 1);
+  if (gid >= count) return;   // whole groups
+  const unsigned mask = group_mask<G>();
+  const SnodeDev d = sn[list[gid]];
   const T* P = L + d.loff;
   const int b = d.len - d.s;
   T* Wj = W + d.wpre * nrhs;
-  // binary64: lane i holds row i of the block scaled by 1 / L(i, i), y_i =
-  // b_i / L(i, i) - sum_k (L(i, k) / L(i, i)) y_k, so a step of the substitution
-  // chain is a shuffle and one FMA (a binary64 multiply on the chain costs ~65
-  // cycles). binary32 (4-cycle multiplies) keeps the unscaled rows and divides
-  // on the chain, which rounds once less per entry.
   constexpr bool kScaled = sizeof(T) == 8;
-  const T rdiag = lane < d.s ? T(1) / lval<T, RM>(P, d, lane, lane) : T(0);
-  T lrow[S];   // L(lane, k) (binary64: / L(lane, lane)), k < lane (s <= S)
+  const T rd = g < d.s ? pivot_recip<T>(P, d, g, RM, rdiag) : T(0);
+  T lrow[G];   // L(g, k) (binary64: / L(g, g)), k < g < s, else 0
+#pragma unroll
+  for (int k = 0; k < G; ++k) lrow[k] = (k < g && g < d.s) ? lval<T, RM>(P, d, g, k) * (kScaled ? rd : T(1)) : T(0);
+  for (int r = 0; r < nrhs; ++r) {
+    T y = g < d.s ? Y[d.f + g + (int64_t)r * n] * (kScaled ? rd : T(1)) : T(0);
+    T ya[G];   // y_J, every lane
+#pragma unroll
+    for (int k = 0; k < G; ++k) {   // past s: no lane g > k is a row
+      ya[k] = __shfl_sync(mask, kScaled ? y : y * rd, k, G);
+      if (!kScaled && g == k) y = ya[k];
+      if (g > k) y -= lrow[k] * ya[k];
+    }
+    if (g < d.s) Y[d.f + g + (int64_t)r * n] = y;
+    for (int u = g; u < b; u += G) {
+      T lv[G], a4[4] = {T(0), T(0), T(0), T(0)};
+#pragma unroll
+      for (int k = 0; k < G; ++k) lv[k] = k < d.s ? lval<T, RM>(P, d, d.s + u, k) : T(0);
+#pragma unroll
+      for (int k = 0; k < G; ++k)
+        if (k < d.s) a4[kScaled ? (k & 3) : 0] += lv[k] * ya[k];
+      Wj[u + (int64_t)r * b] = (a4[0] + a4[1]) + (a4[2] + a4[3]);
+    }
+  }
+}
+
+// Backward for the same supernodes: t_k = sum_u L(s+u, k) x[rows[s+u]] (ancestor
+// rows are final), a lane per row u of a G-row group, the lanes' sums combined in
+// a fixed tree that leaves t_g on lane g; then the transposed diagonal solve with
+// shuffles, lane i holding column i of the block.
+template <class T, bool RM, int G>
+__global__ void __launch_bounds__(kT)
+k_sv_small_bwd(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list, int count,
+               const int32_t* __restrict__ rows, const T* __restrict__ L, const double* __restrict__ rdiag,
+               T* __restrict__ Y, int n, int nrhs) {
+  const int gid = (blockIdx.x * blockDim.x + threadIdx.x) / G, g = threadIdx.x & (G - 1);
+  if (gid >= count) return;   // whole groups
+  const unsigned mask = group_mask<G>();
+  const SnodeDev d = sn[list[gid]];
+  const T* P = L + d.loff;
+  const int b = d.len - d.s;
+  const int32_t* rj = rows + d.roff + d.s;
+  constexpr bool kScaled = sizeof(T) == 8;
+  const T rd = g < d.s ? pivot_recip<T>(P, d, g, RM, rdiag) : T(0);
+  T lcol[G];   // L(k, g) (binary64: / L(g, g)), g < k < s, else 0
+#pragma unroll
+  for (int k = 0; k < G; ++k) lcol[k] = (k > g && k < d.s) ? lval<T, RM>(P, d, k, g) * (kScaled ? rd : T(1)) : T(0);
+  for (int r = 0; r < nrhs; ++r) {
+    T acc[G];
+#pragma unroll
+    for (int k = 0; k < G; ++k) acc[k] = T(0);
+    for (int u = g; u < b; u += G) {
+      const T x = Y[rj[u] + (int64_t)r * n];
+#pragma unroll
+      for (int k = 0; k < G; ++k)
+        if (k < d.s) acc[k] += lval<T, RM>(P, d, d.s + u, k) * x;
+    }
+#pragma unroll
+    for (int h = G / 2; h > 0; h >>= 1) {
+#pragma unroll
+      for (int i = 0; i < h; ++i) {
+        const T send = (g & h) ? acc[i] : acc[i + h], keep = (g & h) ? acc[i + h] : acc[i];
+        acc[i] = keep + __shfl_xor_sync(mask, send, h, G);
+      }
+    }
+    T y = g < d.s ? (Y[d.f + g + (int64_t)r * n] - acc[0]) * (kScaled ? rd : T(1)) : T(0);
+#pragma unroll
+    for (int k = G - 1; k >= 0; --k) {
+      const T xk = __shfl_sync(mask, kScaled ? y : y * rd, k, G);
+      if (k < d.s) {
+        if (!kScaled && g == k) y = xk;
+        if (g < k) y -= lcol[k] * xk;
+      }
+    }
+    if (g < d.s) Y[d.f + g + (int64_t)r * n] = y;
+  }
+}
+
+// The same supernodes in binary64, one warp each (S = 8 or 32 bounds s): fewer
+// FP64 instructions a supernode than the lane groups where they hold few of its
+// rows or columns, and the shorter chain where a level has few supernodes. Used
+// for s > 16 and for levels below kPackedMin.
+constexpr int kPackedMin = 4096;
+template <int S>
+__global__ void __launch_bounds__(kT)
+k_sv_wide_fwd(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list, int count,
+               const double* __restrict__ L, const double* __restrict__ rdiag, double* __restrict__ Y, int n, double* __restrict__ W, int nrhs) {
+  __shared__ double ysh[kT / 32][S];
+  const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (wid >= count) return;
+  const SnodeDev d = sn[list[wid]];
+  const double* P = L + d.loff;
+  const int b = d.len - d.s;
+  double* Wj = W + d.wpre * nrhs;
+  const double rd = lane < d.s ? rdiag[d.f + lane] : 0.0;
+  double lrow[S];   // L(lane, k) (binary64: / L(lane, lane)), k < lane (s <= S)
 #pragma unroll
   for (int k = 0; k < S; ++k)
-    lrow[k] = (k < lane && lane < d.s) ? lval<T, RM>(P, d, lane, k) * (kScaled ? rdiag : T(1)) : T(0);
+    lrow[k] = (k < lane && lane < d.s) ? P[lane + (int64_t)k * d.ld] * rd : 0.0;
   for (int r = 0; r < nrhs; ++r) {
-    T y = lane < d.s ? Y[d.f + lane + (int64_t)r * n] * (kScaled ? rdiag : T(1)) : T(0);
+    double y = lane < d.s ? Y[d.f + lane + (int64_t)r * n] * rd : 0.0;
 #pragma unroll
     for (int k = 0; k < S; ++k) {
       if (k < d.s) {   // uniform across the warp
-        if constexpr (kScaled) {
-          const T yk = __shfl_sync(0xffffffffu, y, k);
-          if (lane > k) y -= lrow[k] * yk;
-        } else {
-          const T yk = __shfl_sync(0xffffffffu, y * rdiag, k);
-          if (lane == k) y = yk;
-          if (lane > k) y -= lrow[k] * yk;
-        }
+        const double yk = __shfl_sync(0xffffffffu, y, k);
+        if (lane > k) y -= lrow[k] * yk;
       }
     }
     if (lane < d.s) Y[d.f + lane + (int64_t)r * n] = y;
     // w_J = L_RJ y_J, lane u holding rows u, u + 32, ...: per 32-row group all
     // s entries of the lane's row are loaded at once (one memory round trip per
-    // group), then multiplied with y_J from shared memory; binary64 keeps four
-    // partial sums (k mod 4, added pairwise) to shorten its FMA chain, binary32
-    // one, in k order
-    T* yk = ysh[threadIdx.x >> 5];   // y_J of this warp's supernode (broadcast reads)
+    // group), then multiplied with y_J from shared memory into four partial sums
+    // (k mod 4, added pairwise), which shortens the FMA chain
+    double* yk = ysh[threadIdx.x >> 5];   // y_J of this warp's supernode (broadcast reads)
     if (lane < S) yk[lane] = y;
     __syncwarp();
     for (int c = 0; c < kSolveSmallRows / 32; ++c) {
       if (32 * c >= b) break;   // uniform across the warp
       const int u = lane + 32 * c;
-      // binary64 with S = 32: two halves of 16 loads (the row copy of the
-      // block stays in registers for every right-hand side)
-      constexpr int KH = (sizeof(T) == 8 && S > 16) ? 16 : S;
-      T a4[4] = {T(0), T(0), T(0), T(0)};
+      // S = 32: two halves of 16 loads (the row copy of the block stays in
+      // registers for every right-hand side)
+      constexpr int KH = S > 16 ? 16 : S;
+      double a4[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 1
       for (int k0 = 0; k0 < S; k0 += KH) {
         if (k0 >= d.s) break;   // uniform across the warp
-        T lv[KH];
+        double lv[KH];
 #pragma unroll
         for (int kk = 0; kk < KH; ++kk)
-          lv[kk] = (k0 + kk < d.s && u < b) ? lval<T, RM>(P, d, d.s + u, k0 + kk) : T(0);
+          lv[kk] = (k0 + kk < d.s && u < b) ? P[d.s + u + (int64_t)(k0 + kk) * d.ld] : 0.0;
 #pragma unroll
-        for (int kk = 0; kk < KH; ++kk) a4[kScaled ? (kk & 3) : 0] += lv[kk] * yk[k0 + kk];
+        for (int kk = 0; kk < KH; ++kk) a4[kk & 3] += lv[kk] * yk[k0 + kk];
       }
       if (u < b) Wj[u + (int64_t)r * b] = (a4[0] + a4[1]) + (a4[2] + a4[3]);
     }
@@ -860,55 +959,45 @@ k_sv_small_fwd(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list
 // Backward for the same supernodes: lane k gathers t_k = sum_u L(s+u, k) x[rows[s+u]]
 // (ancestor rows are final; four rows' loads in flight), then the transposed
 // diagonal solve with shuffles, lane i holding column i of the block.
-template <class T, bool RM, int S>
+template <int S>
 __global__ void __launch_bounds__(kT)
-k_sv_small_bwd(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list, int count,
-               const int32_t* __restrict__ rows, const T* __restrict__ L, T* __restrict__ Y, int n, int nrhs) {
+k_sv_wide_bwd(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list, int count,
+               const int32_t* __restrict__ rows, const double* __restrict__ L, const double* __restrict__ rdiag, double* __restrict__ Y, int n, int nrhs) {
   const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (wid >= count) return;
   const SnodeDev d = sn[list[wid]];
-  const T* P = L + d.loff;
+  const double* P = L + d.loff;
   const int b = d.len - d.s;
   const int32_t* rj = rows + d.roff + d.s;
-  // lane i holds column i of the block (binary64: scaled by 1 / L(i, i), as in
-  // the forward kernel)
-  constexpr bool kScaled = sizeof(T) == 8;
-  const T rdiag = lane < d.s ? T(1) / lval<T, RM>(P, d, lane, lane) : T(0);
-  T lcol[S];   // L(k, lane) (binary64: / L(lane, lane)), k > lane (s <= S)
+  const double rd = lane < d.s ? rdiag[d.f + lane] : 0.0;
+  double lcol[S];   // L(k, lane) (binary64: / L(lane, lane)), k > lane (s <= S)
 #pragma unroll
   for (int k = 0; k < S; ++k)
-    lcol[k] = (k > lane && k < d.s) ? lval<T, RM>(P, d, k, lane) * (kScaled ? rdiag : T(1)) : T(0);
+    lcol[k] = (k > lane && k < d.s) ? P[k + (int64_t)lane * d.ld] * rd : 0.0;
   for (int r = 0; r < nrhs; ++r) {
-    // binary64: four partial sums (u mod 4), added pairwise, a chain of b/4
-    // dependent FMAs; binary32: one, in u order (16 rows' loads in flight per
-    // round)
-    T t4[4] = {T(0), T(0), T(0), T(0)};
+    // four partial sums (u mod 4), added pairwise: a chain of b/4 dependent FMAs;
+    // 16 rows' loads in flight per round
+    double t4[4] = {0.0, 0.0, 0.0, 0.0};
     if (lane < d.s) {
       for (int u0 = 0; u0 < b; u0 += 16) {
-        T lv[16], xv[16];
+        double lv[16], xv[16];
 #pragma unroll
         for (int uu = 0; uu < 16; ++uu) {
           const int u = u0 + uu;
-          lv[uu] = u < b ? lval<T, RM>(P, d, d.s + u, lane) : T(0);
-          xv[uu] = u < b ? Y[rj[u] + (int64_t)r * n] : T(0);
+          lv[uu] = u < b ? P[d.s + u + (int64_t)lane * d.ld] : 0.0;
+          xv[uu] = u < b ? Y[rj[u] + (int64_t)r * n] : 0.0;
         }
 #pragma unroll
-        for (int uu = 0; uu < 16; ++uu) t4[kScaled ? (uu & 3) : 0] += lv[uu] * xv[uu];
+        for (int uu = 0; uu < 16; ++uu) t4[uu & 3] += lv[uu] * xv[uu];
       }
     }
-    const T t = (t4[0] + t4[1]) + (t4[2] + t4[3]);
-    T y = lane < d.s ? (Y[d.f + lane + (int64_t)r * n] - t) * (kScaled ? rdiag : T(1)) : T(0);
+    const double t = (t4[0] + t4[1]) + (t4[2] + t4[3]);
+    double y = lane < d.s ? (Y[d.f + lane + (int64_t)r * n] - t) * rd : 0.0;
 #pragma unroll
     for (int k = S - 1; k >= 0; --k) {
       if (k < d.s) {   // uniform across the warp
-        if constexpr (kScaled) {
-          const T xk = __shfl_sync(0xffffffffu, y, k);
-          if (lane < k) y -= lcol[k] * xk;
-        } else {
-          const T xk = __shfl_sync(0xffffffffu, y * rdiag, k);
-          if (lane == k) y = xk;
-          if (lane < k) y -= lcol[k] * xk;
-        }
+        const double xk = __shfl_sync(0xffffffffu, y, k);
+        if (lane < k) y -= lcol[k] * xk;
       }
     }
     if (lane < d.s) Y[d.f + lane + (int64_t)r * n] = y;
@@ -1345,6 +1434,25 @@ int launch_tri(chol_handle* h, const LevelPlan& P, const T* L, T* Y, int nr, cud
   return CHOL_OK;
 }
 
+// Calls f for the level's small supernodes by class: lanes a supernode, and
+// whether the one-warp form is taken (binary64 where it is the better one).
+// Measured: batch of 600, binary32, 9.5 -> 7.6 ms with the lane groups; 3D 40^3,
+// 16 right-hand sides, binary64, 7.0 ms a solve on warps, 10.8 on groups.
+template <class T, class F>
+int small_groups(const LevelPlan& P, F&& f) {
+  const int n8 = P.ssmall8_n, n16 = P.ssmall16_n, n32 = P.ssmall_n - n8 - n16, b = P.ssmall_b;
+  using std::integral_constant;
+  if (sizeof(T) == 8 && n8 + n16 < kPackedMin) {
+    if (n8 > 0) f(integral_constant<int, 8>{}, std::true_type{}, b, n8);
+    if (n16 + n32 > 0) f(integral_constant<int, 32>{}, std::true_type{}, b + n8, n16 + n32);
+    return (n8 > 0) + (n16 + n32 > 0);
+  }
+  if (n8 > 0) f(integral_constant<int, 8>{}, std::false_type{}, b, n8);
+  if (n16 > 0) f(integral_constant<int, 16>{}, std::false_type{}, b + n8, n16);
+  if (n32 > 0) f(integral_constant<int, 32>{}, std::bool_constant<sizeof(T) == 8>{}, b + n8 + n16, n32);
+  return (n8 > 0) + (n16 > 0) + (n32 > 0);
+}
+
 template <class T, bool RM>
 int solve_levels(chol_handle* h, const T* L, T* Y, T* W, T* part, int nr, cudaStream_t st, bool prof) {
   DeviceState* D = h->dev;
@@ -1354,14 +1462,16 @@ int solve_levels(chol_handle* h, const T* L, T* Y, T* W, T* part, int nr, cudaSt
   NvtxRange nvtx_forward("forward");
   for (const LevelPlan& P : h->levels) {
     if (P.ssmall_n > 0) {
-      // supernodes with s <= 8 first, then the wider ones
       KScope* ks = scope(CHOL_K_SOLVE_DIAG);
-      const int n8 = P.ssmall8_n, nw = P.ssmall_n - P.ssmall8_n;
-      if (n8 > 0)
-        k_sv_small_fwd<T, RM, 8><<<(n8 + 7) / 8, kT, 0, st>>>(D->sn, D->ssmall + P.ssmall_b, n8, L, Y, n, W, nr);
-      if (nw > 0)
-        k_sv_small_fwd<T, RM, 32><<<(nw + 7) / 8, kT, 0, st>>>(D->sn, D->ssmall + P.ssmall_b + n8, nw, L, Y, n, W, nr);
-      if (ks) ks->launches((n8 > 0) + (nw > 0));
+      const int nk = small_groups<T>(P, [&](auto G, auto wide, int b, int cnt) {
+        constexpr int kG = decltype(G)::value;
+        if constexpr (decltype(wide)::value && !RM)
+          k_sv_wide_fwd<kG><<<(cnt + 7) / 8, kT, 0, st>>>(D->sn, D->ssmall + b, cnt, L, D->rdiag, Y, n, W, nr);
+        else
+          k_sv_small_fwd<T, RM, kG><<<(cnt * kG + kT - 1) / kT, kT, 0, st>>>(D->sn, D->ssmall + b, cnt, L, D->rdiag, Y, n,
+                                                                            W, nr);
+      });
+      if (ks) ks->launches(nk);
       delete ks;
     }
     if (P.tri_n > 0) {
@@ -1414,13 +1524,15 @@ int solve_levels(chol_handle* h, const T* L, T* Y, T* W, T* part, int nr, cudaSt
     }
     if (P.ssmall_n > 0) {
       KScope* ks = scope(CHOL_K_SOLVE_DIAG);
-      const int n8 = P.ssmall8_n, nw = P.ssmall_n - P.ssmall8_n;
-      if (n8 > 0)
-        k_sv_small_bwd<T, RM, 8><<<(n8 + 7) / 8, kT, 0, st>>>(D->sn, D->ssmall + P.ssmall_b, n8, D->rows, L, Y, n, nr);
-      if (nw > 0)
-        k_sv_small_bwd<T, RM, 32><<<(nw + 7) / 8, kT, 0, st>>>(D->sn, D->ssmall + P.ssmall_b + n8, nw, D->rows, L, Y,
-                                                                n, nr);
-      if (ks) ks->launches((n8 > 0) + (nw > 0));
+      const int nk = small_groups<T>(P, [&](auto G, auto wide, int b, int cnt) {
+        constexpr int kG = decltype(G)::value;
+        if constexpr (decltype(wide)::value && !RM)
+          k_sv_wide_bwd<kG><<<(cnt + 7) / 8, kT, 0, st>>>(D->sn, D->ssmall + b, cnt, D->rows, L, D->rdiag, Y, n, nr);
+        else
+          k_sv_small_bwd<T, RM, kG><<<(cnt * kG + kT - 1) / kT, kT, 0, st>>>(D->sn, D->ssmall + b, cnt, D->rows, L,
+                                                                            D->rdiag, Y, n, nr);
+      });
+      if (ks) ks->launches(nk);
       delete ks;
     }
     if (P.tri_n > 0) {
