@@ -454,6 +454,19 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
   h->update_doubles = 0;
   h->update_doubles_rl = 0;
   h->w_rows_max = 0;
+  // the one-CTA class of the options
+  auto one_cta = [&](int32_t J) {
+    const SnodeDev& d = h->snodes[J];
+    return d.s <= h->opt.small_max_cols && (int64_t)d.len * d.s <= h->opt.small_max_panel && d.len <= h->opt.small_max_rows;
+  };
+  // Binary64 problems that have blocked supernodes anyway (so they never run as
+  // one persistent launch): of the one-CTA class, those wider than this are
+  // factored by the blocked kernels too. One SM's FP64 pipe needs 175 us for a
+  // dense block of 128 columns; the 304 roots of a batch of 1,000 took 1.2 ms
+  // on a CTA each and take 0.3 on the blocked path.
+  constexpr int32_t kBlockedCols = 64;
+  bool any_large = false;
+  for (int32_t J = 0; J < ns && !any_large; ++J) any_large = !one_cta(J);
   for (int32_t lv = 0; lv < h->nlevels; ++lv) {
     LevelPlan& P = h->levels[lv];
     const auto& Js = by_level[lv];
@@ -463,6 +476,8 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
     std::vector<int32_t> large;
     P.small_b = (int32_t)h->small_list.size();
     P.small_max_panel = 0;
+    std::vector<int32_t> by_class[4];   // warp (s <= 8, s <= 16), CTA, blocked
+    P.cta_max_panel = 0;
     int64_t uo = 0, wo = 0;
     for (int32_t J : Js) {
       SnodeDev& d = h->snodes[J];
@@ -471,19 +486,25 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
       uo += (int64_t)b * (h->opt.precision == CHOL_PREC_FP64 ? b : ((b + 7) & ~7));
       d.wpre = wo;
       wo += b;
-      bool small = d.s <= h->opt.small_max_cols && (int64_t)d.len * d.s <= h->opt.small_max_panel &&
-                   d.len <= h->opt.small_max_rows;
-      if (small) {
+      if (one_cta(J)) {
         for (int32_t j = d.f; j < d.f + d.s; ++j) P.small_flops += (double)h->colcount[j] * h->colcount[j];
         P.small_bytes += 16.0 * (double)d.len * d.s + 8.0 * (double)b * (b + 1) / 2.0;
-        h->small_list.push_back(J);
         P.small_max_panel = std::max(P.small_max_panel, d.len * d.s);
         h->n_small++;
+        const int cls = mixed ? 2 : (d.len <= 32 && d.s <= 8) ? 0 : (d.len <= 32 && d.s <= 16) ? 1
+                        : (any_large && split64 && d.s > kBlockedCols) ? 3 : 2;
+        by_class[cls].push_back(J);
+        if (cls == 2) P.cta_max_panel = std::max(P.cta_max_panel, d.len * d.s);
+        if (cls == 3) large.push_back(J);
       } else {
         large.push_back(J);
         h->n_large++;
       }
     }
+    for (const auto& c : by_class) h->small_list.insert(h->small_list.end(), c.begin(), c.end());
+    P.tiny8_n = (int32_t)by_class[0].size();
+    P.tiny16_n = (int32_t)by_class[1].size();
+    P.small_k = P.tiny8_n + P.tiny16_n + (int32_t)by_class[2].size();
     P.small_n = (int32_t)h->small_list.size() - P.small_b;
     P.u_doubles = uo;
     P.w_rows = wo;
