@@ -787,12 +787,140 @@ __device__ __forceinline__ void assemble_body(const AsmTask& t, const AsmSeg* __
   }
 }
 
+// The same task with its tile of K (at most 64 positions x 32 columns) in shared
+// memory, eight segments a round: warp w fetches segment w's descriptors and
+// finds its positions, then the first entries of all eight are loaded together
+// and subtracted in segment order. A segment then waits for no global load of
+// the one before it; with the tile in global memory a task of a 2D 64^2 grid
+// spent about 2 us a segment on that chain. Same operations per entry and order.
+constexpr int kAsmFly = kAsmThreads / 32;
 __global__ void __launch_bounds__(kAsmThreads)
 k_assemble(const AsmTask* __restrict__ tasks, const AsmSeg* __restrict__ segs,
            const SnodeDev* __restrict__ sn, const int32_t* __restrict__ rows,
            const double* __restrict__ U, double* __restrict__ L) {
-  extern __shared__ int32_t ssm[];
-  assemble_body<false>(tasks[blockIdx.x], segs, sn, rows, U, L, ssm);
+  constexpr int kLd = kAsmPos + 1;
+  __shared__ double tile[kAsmCols * kLd];           // entry (position p, column c) at c kLd + p
+  __shared__ int32_t sK[kAsmPos];
+  __shared__ int32_t spos[kAsmFly][kAsmPos], scol[kAsmFly][kAsmCols];
+  __shared__ int64_t sbase[kAsmFly];                // U entry (ua, ca)
+  __shared__ int32_t sb[kAsmFly], snu[kAsmFly], sw[kAsmFly], slow[kAsmFly];
+  const AsmTask t = tasks[blockIdx.x];
+#ifdef CHOL_BOUNDS_CHECK
+  if (!CHOL_BC(t.K >= 0 && t.K < bc_lim.ns, kBcTaskTarget)) return;
+#endif
+  const SnodeDev dk = sn[t.K];
+  const int np = t.p1 - t.p0, nc = t.t1 - t.t0;
+#ifdef CHOL_BOUNDS_CHECK
+  if (!CHOL_BC(t.p0 >= 0 && np >= 0 && t.p1 <= dk.len && np <= kAsmPos && t.t0 >= 0 && nc <= kAsmCols &&
+                   t.t1 <= dk.s && t.seg_begin >= 0 && t.seg_begin <= t.seg_end && t.seg_end <= bc_lim.nsegs,
+               kBcTaskPositions))
+    return;
+#endif
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  static_assert(kAsmPos == 64 && kAsmThreads == 256 && kAsmCols == 32, "thread map: row tid mod 64, columns tid / 64 + 4 i");
+  const int u = tid & 63, c0 = tid >> 6;
+  double* Lt = L + dk.loff + t.p0 + (int64_t)t.t0 * dk.ld;
+  {
+    double v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = (u < np && c0 + 4 * i < nc) ? Lt[u + (int64_t)(c0 + 4 * i) * dk.ld] : 0.0;
+    if (tid < np) sK[tid] = rows[dk.roff + t.p0 + tid];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) tile[(c0 + 4 * i) * kLd + u] = v[i];
+  }
+  for (int g0 = t.seg_begin; g0 < t.seg_end; g0 += kAsmFly) {
+    const int ng = min(kAsmFly, t.seg_end - g0);
+    __syncthreads();   // sK and the tile are staged, the round before is applied
+    if (warp < ng) {
+      const AsmSeg sg = segs[g0 + warp];
+      bool ok = true;
+#ifdef CHOL_BOUNDS_CHECK
+      ok = CHOL_BC(sg.J >= 0 && sg.J < bc_lim.ns, kBcSegSource);
+#endif
+      int nu = 0, w = 0;
+      if (ok) {
+        const SnodeDev dj = sn[sg.J];
+        const int b = dj.len - dj.s;
+        const int32_t* rj = rows + dj.roff + dj.s;
+        nu = sg.ub - sg.ua;
+        w = sg.cb - sg.ca;
+#ifdef CHOL_BOUNDS_CHECK
+        if (!CHOL_BC(sg.ua >= 0 && sg.ua <= sg.ub && sg.ub <= b && sg.ca >= 0 && sg.ca <= sg.cb && sg.cb <= b &&
+                         nu <= kAsmPos && w <= kAsmCols,
+                     kBcSegRange))
+          nu = w = 0;
+#endif
+        for (int i = lane; i < nu; i += 32) {
+          const int32_t key = rj[sg.ua + i];
+          int lo = 0, hi = np;
+          while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (sK[mid] < key) lo = mid + 1; else hi = mid;
+          }
+#ifdef CHOL_BOUNDS_CHECK
+          if (!CHOL_BC(lo < np && sK[lo] == key, kBcTargetRow)) lo = -1;
+#endif
+          spos[warp][i] = lo;
+        }
+        for (int c = lane; c < w; c += 32) {
+          int col = rj[sg.ca + c] - dk.f - t.t0;
+#ifdef CHOL_BOUNDS_CHECK
+          if (!CHOL_BC(col >= 0 && col < nc, kBcTargetCol)) col = -1;
+#endif
+          scol[warp][c] = col;
+        }
+        if (lane == 0) {
+          sbase[warp] = dj.uoff + (int64_t)sg.ca * b + sg.ua;
+          sb[warp] = b;
+          slow[warp] = sg.ca - sg.ua;   // entry (u, c) is in the lower triangle iff u >= c + slow
+        }
+      }
+      if (lane == 0) {
+        snu[warp] = nu;
+        sw[warp] = w;
+      }
+    }
+    __syncthreads();
+    // the tile entry of (u, c) of segment k, or -1
+    auto target = [&](int k, int c) {
+      if (u >= snu[k] || c >= sw[k] || u < c + slow[k]) return -1;
+      const int p = spos[k][u], col = scol[k][c];
+#ifdef CHOL_BOUNDS_CHECK
+      if (p < 0 || col < 0) return -1;
+#endif
+      return col * kLd + p;
+    };
+    double v[kAsmFly];
+    int off[kAsmFly];
+#pragma unroll
+    for (int k = 0; k < kAsmFly; ++k) {
+      off[k] = k < ng ? target(k, c0) : -1;
+      if (off[k] >= 0) v[k] = U[sbase[k] + (int64_t)c0 * sb[k] + u];
+    }
+#pragma unroll
+    for (int k = 0; k < kAsmFly; ++k) {
+      if (k >= ng) break;   // uniform
+      if (off[k] >= 0) tile[off[k]] -= v[k];
+      if (sw[k] > 4) {      // the columns past the first four
+        double z[7];
+        int oz[7];
+#pragma unroll
+        for (int i = 0; i < 7; ++i) {
+          const int c = c0 + 4 * (i + 1);
+          oz[i] = target(k, c);
+          if (oz[i] >= 0) z[i] = U[sbase[k] + (int64_t)c * sb[k] + u];
+        }
+#pragma unroll
+        for (int i = 0; i < 7; ++i)
+          if (oz[i] >= 0) tile[oz[i]] -= z[i];
+      }
+      if (k + 1 < ng) __syncthreads();   // the next segment may meet the same entries
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if (u < np && c0 + 4 * i < nc) Lt[u + (int64_t)(c0 + 4 * i) * dk.ld] = tile[(c0 + 4 * i) * kLd + u];
 }
 
 // Z_RR of a level's CTA-sized tasks (the selected inverse).
@@ -1150,8 +1278,6 @@ int chol_device_ensure(chol_handle* h) {
   if (cudaMallocHost((void**)&D->scalar_host, sizeof(double)) != cudaSuccess) return fail(CHOL_ENOMEM);
   static bool attrs_done = false;
   if (!attrs_done) {
-    if (cudaFuncSetAttribute(k_assemble, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess)
-      return fail(CHOL_ECUDA);
     if (cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 24576 * 8) != cudaSuccess)
       return fail(CHOL_ECUDA);
     if (cudaFuncSetAttribute(k_small_rlb, cudaFuncAttributeMaxDynamicSharedMemorySize, 24576 * 8) != cudaSuccess)
@@ -1395,8 +1521,7 @@ int enqueue_factor_fp64(chol_handle* h, const double* values, cudaStream_t st) {
       const AsmSplit a = asm_split(P, D->sms);
       ks.launches((a.ctas > 0) + (a.warps > 0));
       if (a.ctas > 0)
-        k_assemble<<<a.ctas, kAsmThreads, sizeof(int32_t) * 2 * kAsmPos, st>>>(
-            D->asm_tasks + P.asm_b, D->asm_segs, D->sn, D->rows, D->U, D->L);
+        k_assemble<<<a.ctas, kAsmThreads, 0, st>>>(D->asm_tasks + P.asm_b, D->asm_segs, D->sn, D->rows, D->U, D->L);
       if (a.warps > 0)
         k_assemble_warp<double, false><<<(a.warps + 7) / 8, 256, 0, st>>>(
             D->asm_tasks + P.asm_b + a.ctas, a.warps, D->asm_segs, D->sn, D->rows, D->U, D->L);
