@@ -20,7 +20,7 @@
 
 #include "device.h"
 #include "mixed.h"
-#include "split_gemm.cuh"
+#include "split_op.cuh"
 #include "diag_inv.cuh"
 
 namespace {
@@ -164,78 +164,9 @@ k_gen_reduce(const GenGemm* __restrict__ descs, const GemmTile* __restrict__ til
 // then the 128 x 64 tiles run. The FP64 pipe kept the tiles above at 97% of its
 // 2 FMAs per cycle and SM on busy SMs; they remain for handles with a memory
 // cap and devices without room for the slices.
-struct SplitOp {          // operand rows (i, k) at p[i rs + k ks], i < rows, k < K
-  const double* p;
-  int64_t rs, ks;
-  int64_t off, exp0;      // first slice row and first exponent in the workspace
-  int32_t rows, K, prows; // prows: rows per slice, whole tiles
-  int32_t mode;           // 0 general, 1 zero for k > i, 2 symmetric (k <= i stored), 3 zero for i > k
-};
-struct SplitTask {
-  int32_t op, r0;   // first of split_rows(K) rows
-};
 struct SplitTile {
   int32_t desc, i0, j0, kb0, kb1, pad;   // product, tile origin, range of 32-column K blocks
 };
-
-__device__ __forceinline__ double split_el(const SplitOp& o, int i, int k) {
-  if (i >= o.rows || k >= o.K) return 0.0;
-  if (o.mode == 2) return k <= i ? o.p[i * o.rs + k * o.ks] : o.p[k * o.rs + i * o.ks];
-  if ((o.mode == 1 && k > i) || (o.mode == 3 && i > k)) return 0.0;
-  return o.p[i * o.rs + k * o.ks];
-}
-
-// 16 to 64 rows of an operand: a thread takes 8 consecutive columns of a row a
-// step, with the lanes along whichever index is contiguous (a symmetric operand
-// changes at the diagonal). Two passes, the second from L2.
-constexpr int kSplitOpThreads = sg::kSplitThreads;
-__global__ void __launch_bounds__(kSplitOpThreads)
-k_split_op(const SplitOp* __restrict__ ops, const SplitTask* __restrict__ tasks, unsigned char* __restrict__ slab,
-           int32_t* __restrict__ exps) {
-  __shared__ uint32_t hmax[64];
-  const SplitTask t = tasks[blockIdx.x];
-  const SplitOp o = ops[t.op];
-  const int tid = threadIdx.x;
-  const int rsh = sg::split_rows_log2(o.K), R = 1 << rsh, csh = sg::kSplitThreadsLog2 - rsh;
-  const int step = 8 << csh;   // columns a step
-  if (tid < 64) hmax[tid] = 0;
-  __syncthreads();
-  const bool kc = o.ks == 1 && o.rs != 1;
-  // (row, first column) of the thread in the step at column k0
-  auto place = [&](int k0, int& r, int& c) {
-    const bool kfast = o.mode == 2 ? (k0 >= t.r0 + R ? o.rs == 1 : kc) : kc;
-    r = kfast ? (tid >> csh) : (tid & (R - 1));
-    c = 8 * (kfast ? (tid & ((1 << csh) - 1)) : (tid >> rsh));
-  };
-#pragma unroll 2
-  for (int k0 = 0; k0 < o.K; k0 += step) {
-    int r, c;
-    place(k0, r, c);
-    uint32_t m = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) m = max(m, (uint32_t)__double2hiint(split_el(o, t.r0 + r, k0 + c + i)) & 0x7fffffffu);
-    if (m) atomicMax(&hmax[r], m);
-  }
-  __syncthreads();
-  if (tid < R) exps[o.exp0 + t.r0 + tid] = sg::row_exponent(hmax[tid]);
-  const int kend = (o.K + 31) / 32 * 32;
-  for (int k0 = 0; k0 < kend; k0 += step) {
-    int r, c;
-    place(k0, r, c);
-    if (k0 + c >= kend) continue;
-    const int32_t e = sg::row_exponent(hmax[r]);
-    double y[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) y[i] = e == sg::kExpNaN ? 0.0 : split_el(o, t.r0 + r, k0 + c + i);
-    uint4 w[sg::kSlices];
-    sg::digits8(y, e, w);
-    const int kb = (k0 + c) >> 5;
-    unsigned char* out = slab + (o.off + (int64_t)kb * sg::kSlices * o.prows) * 64 +
-                         sg::chunk_offset(t.r0 + r, (c >> 3) & 3);
-#pragma unroll
-    for (int q = 0; q < sg::kSlices; ++q) *reinterpret_cast<uint4*>(out + (int64_t)q * o.prows * 64) = w[q];
-  }
-}
 
 // Tiles of the group's products: operand 2 desc is A, 2 desc + 1 is B.
 __global__ void __launch_bounds__(sg::kThreads, 1)
@@ -425,9 +356,10 @@ struct SiPlan {
   std::vector<SplitOp> ops;
   std::vector<SplitTask> stasks;
   std::vector<SplitTile> stiles;
-  int64_t slab_rows = 0, nexps = 0;
+  int64_t slab_rows = 0, nexps = 0, nkexps = 0;
   bool sg = false;
   SplitOp* d_ops = nullptr;
+  int32_t* d_kexps = nullptr;
   SplitTask* d_stasks = nullptr;
   SplitTile* d_stiles = nullptr;
   unsigned char* d_slab = nullptr;
@@ -449,7 +381,10 @@ struct SiPlan {
 // two waves are split, and a split must gain at least 8% of fill to pay for
 // its partial tiles.
 constexpr int kGenCtasPerSm = 3;   // __launch_bounds__ of k_gen_gemm_grouped
-Group emit_group(SiPlan& pl, const std::vector<GenGemm>& gs, int sms) {
+// kx: place of x_k of each product (SplitOp), or empty; ksgn: A's sign, 0: A's row
+// exponents are the x_k of products to come.
+Group emit_group(SiPlan& pl, const std::vector<GenGemm>& gs, int sms, const std::vector<int64_t>& kx = {},
+                 int16_t ksgn = 0) {
   Group gr;
   gr.tb = (int32_t)pl.tiles.size();
   gr.rb = (int32_t)pl.rtiles.size();
@@ -486,19 +421,21 @@ Group emit_group(SiPlan& pl, const std::vector<GenGemm>& gs, int sms) {
   gr.sb = (int32_t)pl.stasks.size();
   gr.gb = (int32_t)pl.stiles.size();
   int64_t srow = 0, sexp = 0;
-  for (GenGemm g : gs) {
+  for (size_t gi = 0; gi < gs.size(); ++gi) {
+    GenGemm g = gs[gi];
     if (g.M <= 0 || g.N <= 0) continue;
     {
       const int32_t d = (int32_t)pl.descs.size();
-      auto operand = [&](const double* p, int64_t rs, int64_t ks, int rows, int mode, int extra) {
-        SplitOp o{p, rs, ks, srow, sexp, rows, g.K, (rows + 63) / 64 * 64 + extra, mode};
-        for (int r0 = 0; r0 < rows; r0 += 1 << sg::split_rows_log2(g.K)) pl.stasks.push_back({(int32_t)pl.ops.size(), r0});
+      auto operand = [&](const double* p, int64_t rs, int64_t ks, int rows, int16_t mode, int extra, int16_t ksgn,
+                         bool has_kx) {
+        SplitOp o{p, rs, ks, srow, sexp, has_kx && !kx.empty() ? kx[gi] : -1, rows, g.K, (rows + 63) / 64 * 64 + extra, mode, ksgn};
+        for (int r0 = 0; r0 < rows; r0 += 1 << SPLIT_ROWS_LOG2(g.K)) pl.stasks.push_back({(int32_t)pl.ops.size(), r0});
         pl.ops.push_back(o);
         srow += (int64_t)((g.K + 31) / 32) * sg::kSlices * o.prows;
         sexp += o.prows;
       };
-      operand(g.A, g.ar, g.ac, g.M, g.amode, 64);               // a 128-row tile may end 64 rows past
-      operand(g.B, g.bc, g.br, g.N, g.bmode == 1 ? 3 : 0, 0);   // rows: B's columns
+      operand(g.A, g.ar, g.ac, g.M, (int16_t)g.amode, 64, ksgn, true);               // a 128-row tile may end 64 rows past
+      operand(g.B, g.bc, g.br, g.N, g.bmode == 1 ? 3 : 0, 0, (int16_t)-ksgn, ksgn != 0);   // rows: B's columns
       for (int j0 = 0; j0 < g.N; j0 += sg::kN)
         for (int i0 = 0; i0 < g.M; i0 += sg::kM) {
           if (g.lower_c && i0 + sg::kM - 1 < j0) continue;
@@ -553,6 +490,7 @@ void free_si_split(chol_handle* h, SiPlan* pl) {
   drop(&pl->d_stiles, (int64_t)(sizeof(SplitTile) * pl->stiles.size()));
   drop(&pl->d_slab, pl->slab_rows * 64);
   drop(&pl->d_exps, (int64_t)(sizeof(int32_t) * pl->nexps));
+  drop(&pl->d_kexps, (int64_t)(sizeof(int32_t) * std::max<int64_t>(pl->nkexps, 1)));
 }
 
 int build_si_plan(chol_handle* h) {
@@ -626,6 +564,8 @@ int build_si_plan(chol_handle* h) {
       SiStep st{};
       st.inv_b = (int32_t)pl->invs.size();
       std::vector<GenGemm> g1s, g2s;
+      std::vector<int64_t> kx;
+      int64_t xoff = 0;
       for (int32_t J : Js) {
         const SnodeDev& d = h->snodes[J];
         double* T = D->Tw + toff[J];
@@ -636,24 +576,33 @@ int build_si_plan(chol_handle* h) {
                            mc, bs, bs, 1.0, 0.0, 0, 1, 0));
           g2s.push_back(mk(T + c0 + (int64_t)c0 * d.s, 1, d.s, Wp, 1, mc, T + c0 + (int64_t)i0 * d.s, 1, d.s, mc, bs, mc,
                            -1.0, 0.0, 1, 0, 0));
+          kx.push_back(xoff);
+          xoff += mc;
           Wp += (int64_t)mc * bs;
         }
       }
-      st.g1 = emit_group(*pl, g1s, D->sms);
-      st.g2 = emit_group(*pl, g2s, D->sms);
+      pl->nkexps = std::max(pl->nkexps, xoff);
+      st.g1 = emit_group(*pl, g1s, D->sms, kx, 0);
+      st.g2 = emit_group(*pl, g2s, D->sms, kx, 1);
       st.flops = st.g1.flops + st.g2.flops;
       sl.steps.push_back(st);
     }
     // Uhat = L_RJ T
     std::vector<GenGemm> gs;
+    std::vector<int64_t> kx;   // row exponents of L_RJ
+    int64_t xoff = 0;
     for (int32_t J : Js) {
       const SnodeDev& d = h->snodes[J];
       const int b = d.len - d.s;
-      if (b > 0)
+      if (b > 0) {
         gs.push_back(mk(L + d.loff + d.s, 1, d.ld, D->Tw + toff[J], 1, d.s, D->Uh + hoff[J], 1, b, b, d.s, d.s, 1.0,
                         0.0, 0, 1, 0));
+        kx.push_back(xoff);
+        xoff += b;
+      }
     }
-    sl.uh = emit_group(*pl, gs, D->sms);
+    pl->nkexps = std::max(pl->nkexps, xoff);
+    sl.uh = emit_group(*pl, gs, D->sms, kx, 0);
     // Z_RJ = -Z_RR Uhat  (Z_RR at U_J's place in the update workspace)
     gs.clear();
     for (int32_t J : Js) {
@@ -663,7 +612,7 @@ int build_si_plan(chol_handle* h) {
         gs.push_back(mk(ZRR + d.uoff, 1, b, D->Uh + hoff[J], 1, b, Z + d.loff + d.s, 1, d.ld, b, d.s, b, -1.0, 0.0, 2,
                         0, 0));
     }
-    sl.zrj = emit_group(*pl, gs, D->sms);
+    sl.zrj = emit_group(*pl, gs, D->sms, kx, 1);
     // Z_JJ = T^T T, then -= Uhat^T Z_RJ
     gs.clear();
     for (int32_t J : Js) {
@@ -680,7 +629,7 @@ int build_si_plan(chol_handle* h) {
         gs.push_back(mk(D->Uh + hoff[J], b, 1, Z + d.loff + d.s, 1, d.ld, Z + d.loff, 1, d.ld, d.s, d.s, b, -1.0, 1.0, 0,
                         0, 1));
     }
-    sl.zjj2 = emit_group(*pl, gs, D->sms);
+    sl.zjj2 = emit_group(*pl, gs, D->sms, kx, -1);
     sl.gemm_flops = sl.uh.flops + sl.zrj.flops + sl.zjj1.flops + sl.zjj2.flops;
     pl->levels.push_back(std::move(sl));
   }
@@ -698,6 +647,7 @@ int build_si_plan(chol_handle* h) {
     pl->sg = up(&pl->d_ops, pl->ops) == CHOL_OK && up(&pl->d_stasks, pl->stasks) == CHOL_OK &&
              up(&pl->d_stiles, pl->stiles) == CHOL_OK &&
              chol_dalloc(h, (void**)&pl->d_slab, (size_t)pl->slab_rows * 64) == CHOL_OK &&
+             chol_dalloc(h, (void**)&pl->d_kexps, sizeof(int32_t) * (size_t)std::max<int64_t>(pl->nkexps, 1)) == CHOL_OK &&
              chol_dalloc(h, (void**)&pl->d_exps, sizeof(int32_t) * (size_t)pl->nexps) == CHOL_OK &&
              cudaFuncSetAttribute(k_split_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, sg::kSmemBytes) ==
                  cudaSuccess;
@@ -725,7 +675,7 @@ int selinv(chol_handle* h, cudaStream_t st) {
   auto launch = [&](const Group& gr) {
     if (pl->sg) {
       if (gr.gn == 0) return;
-      k_split_op<<<gr.sn, kSplitOpThreads, 0, st>>>(pl->d_ops, pl->d_stasks + gr.sb, pl->d_slab, pl->d_exps);
+      k_split_op<<<gr.sn, kSplitOpThreads, 0, st>>>(pl->d_ops, pl->d_stasks + gr.sb, pl->d_slab, pl->d_exps, pl->d_kexps);
       k_split_gemm<<<std::min(gr.gn, D->sms), sg::kThreads, sg::kSmemBytes, st>>>(
           pl->d_descs, pl->d_ops, pl->d_stiles + gr.gb, gr.gn, pl->d_slab, pl->d_exps, D->sg_err);
       return;
@@ -769,7 +719,7 @@ void chol_adjoint_free(chol_handle* h) {
   if (!D || !D->si_plan) return;
   SiPlan* pl = (SiPlan*)D->si_plan;
   void* ptrs[] = {pl->d_descs, pl->d_tiles, pl->d_rtiles, pl->d_invs, pl->d_part,
-                  pl->d_ops, pl->d_stasks, pl->d_stiles, pl->d_slab, pl->d_exps};
+                  pl->d_ops, pl->d_stasks, pl->d_stiles, pl->d_slab, pl->d_exps, pl->d_kexps};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete pl;

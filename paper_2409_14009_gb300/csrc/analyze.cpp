@@ -429,6 +429,10 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
   // binary64 updates on the tensor cores: their operand blocks are 64 columns wide
   const bool split64 = !mixed && nb == 64;
   h->split.assign(split64 ? ns : 0, SplitDev{});
+  h->vs_dev.assign(split64 ? ns : 0, SolveSplitDev{});
+  h->vs_list.clear(); h->vs_tasks.clear(); h->vs_tiles.clear();
+  h->vs_work = 0.0;
+  h->vs_slab_rows = h->vs_exps = h->vs_rslab_rows = h->vs_rexps = h->vs_slots = h->vs_fexps = 0;
   h->sgt_tasks.clear(); h->sgs_tasks.clear(); h->split_tasks.clear();
   h->split_slab_rows = h->split_exps = h->split_trows = h->split_texps = 0;
   const int tg = tc_modes ? kTileTC : kTile;
@@ -710,7 +714,7 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
           z.srow0 = se;
           so += (int64_t)z.sblk * kSplitSlices * z.srows;
           se += z.srows;
-          for (int32_t r0 = 0; r0 < b; r0 += d.s <= 64 ? 64 : (d.s <= 128 ? 32 : 16)) h->split_tasks.push_back({J, 0, r0, 0});   // sg::split_rows_log2
+          for (int32_t r0 = 0; r0 < b; r0 += 1 << SPLIT_ROWS_LOG2(d.s)) h->split_tasks.push_back({J, 0, r0, 0});
           for (int32_t c0 = 0; c0 < b; c0 += kTile)
             for (int32_t r0 = c0; r0 < b; r0 += 2 * kTile) h->sgs_tasks.push_back({J, 0, r0, c0});
         }
@@ -795,6 +799,63 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
       }
     }
     h->split_slots_max = std::max<int64_t>(h->split_slots_max, std::max(gemv_slots, bpanel_slots));
+    // the same products for several right-hand sides, on the tensor cores
+    P.vs_b = (int32_t)h->vs_list.size();
+    P.vs_entries = 0.0;
+    if (split64) {
+      int64_t fo = 0, bo = 0, ro = 0, be = 0, re = 0;
+      int64_t& fe = h->vs_fexps;
+      int64_t tiles[2] = {0, 0};
+      for (int32_t J : Js) {
+        const SnodeDev& d = h->snodes[J];
+        const int32_t b = d.len - d.s;
+        if (b <= 0 || warp_solved(J)) continue;
+        SolveSplitDev& z = h->vs_dev[J];
+        z.frows = (b + 127) / 128 * 128;
+        z.brows = (d.s + 127) / 128 * 128;
+        z.foff = fo; z.boff = bo; z.roff = ro;
+        z.fexp = fe; z.bexp = be; z.rexp = re;
+        fo += (int64_t)((d.s + 31) / 32) * kSplitSlices * z.frows;
+        bo += (int64_t)((b + 31) / 32) * kSplitSlices * z.brows;
+        ro += (int64_t)((std::max(d.s, b) + 31) / 32) * kSplitSlices * 16;
+        fe += z.frows; be += z.brows; re += 16;
+        tiles[0] += z.frows / 128;
+        tiles[1] += z.brows / 128;
+        P.vs_entries += (double)b * d.s;
+        h->vs_list.push_back(J);
+      }
+      P.vs_n = (int32_t)h->vs_list.size() - P.vs_b;
+      h->vs_work = std::max(h->vs_work, P.vs_entries);
+      h->vs_slab_rows = std::max(h->vs_slab_rows, std::max(fo, bo));
+      h->vs_exps = std::max(h->vs_exps, be);
+      h->vs_rslab_rows = std::max(h->vs_rslab_rows, ro);
+      h->vs_rexps = std::max(h->vs_rexps, re);
+      for (int dir = 0; dir < 2; ++dir) {
+        P.vs_task_b[dir] = (int32_t)h->vs_tasks.size();
+        P.vs_tile_b[dir] = (int32_t)h->vs_tiles.size();
+        int64_t slots = 0;
+        for (int32_t q = 0; q < P.vs_n; ++q) {
+          const int32_t J = h->vs_list[P.vs_b + q];
+          const SnodeDev& d = h->snodes[J];
+          const int32_t rows = dir ? d.s : d.len - d.s, K = dir ? d.len - d.s : d.s;
+          for (int32_t r0 = 0; r0 < rows; r0 += 1 << SPLIT_ROWS_LOG2(K))
+            h->vs_tasks.push_back({2 * (P.vs_b + q) + dir, r0});
+          // parts of at least 8 K blocks, two tiles an SM
+          const int32_t nblk = (K + 31) / 32;
+          const int32_t parts = (int32_t)std::max<int64_t>(
+              1, std::min<int64_t>(nblk / 8, (304 + tiles[dir] - 1) / std::max<int64_t>(tiles[dir], 1)));
+          for (int32_t r0 = 0; r0 < rows; r0 += 128) {
+            for (int32_t p = 0; p < parts; ++p)
+              h->vs_tiles.push_back({J, r0, (int32_t)((int64_t)nblk * p / parts), (int32_t)((int64_t)nblk * (p + 1) / parts),
+                                     (int32_t)slots, p, parts, 0});
+            if (parts > 1) slots += parts;
+          }
+        }
+        h->vs_slots = std::max(h->vs_slots, slots);
+        P.vs_task_n[dir] = (int32_t)h->vs_tasks.size() - P.vs_task_b[dir];
+        P.vs_tile_n[dir] = (int32_t)h->vs_tiles.size() - P.vs_tile_b[dir];
+      }
+    }
     P.gemv_n = (int32_t)h->gemv_tasks.size() - P.gemv_b;
     // row-major backward panel: 64-row chunks x 256-column tiles, then a reduction
     P.bpart_b = (int32_t)h->bpart_tasks.size();
@@ -900,6 +961,8 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
       if (h->asm_tasks[i].p0 == h->asm_tasks[i].t0) h->fasm_tasks.push_back(i);
     P.fasm_n = (int32_t)h->fasm_tasks.size() - P.fasm_b;
   }
+  for (int32_t J : h->vs_list) h->vs_dev[J].bexp += h->vs_fexps;
+  h->vs_exps += h->vs_fexps;
   h->persist_levels.clear();
   h->small_panel_max = 0;
   for (const LevelPlan& P : h->levels) {

@@ -25,6 +25,19 @@ struct DeviceState {
   TileTask* syrk = nullptr;
   AsmTask* asm_tasks = nullptr;
   AsmSeg* asm_segs = nullptr;
+  int vs_ready = 0;             // solve products on the tensor cores: 1 = planned, -1 = not available
+  bool vs_pinned = false;       // a captured solve holds the buffers' addresses
+  unsigned char* vs_slab = nullptr;   // slices of a level's off-diagonal blocks, and their exponents
+  int32_t* vs_exps = nullptr;
+  unsigned char* vs_rslab = nullptr;  // slices of the right-hand sides
+  int32_t* vs_rexps = nullptr;
+  double* vs_part = nullptr;          // partial tiles and arrival counters
+  int32_t* vs_cnt = nullptr;
+  SolveSplitDev* vs_dev = nullptr;
+  void* vs_ops = nullptr;
+  int32_t* vs_list = nullptr;
+  void* vs_tasks = nullptr;
+  SolveTile* vs_tiles = nullptr;
   int32_t* fasm = nullptr;      // solve: the assembly tasks that hold their segments' columns
   TriItemHost* tri = nullptr;   // solve: diagonal-triangle items
   double* rdiag = nullptr;      // binary64: reciprocals of diag(L), per column of P A P^T
@@ -223,6 +236,9 @@ int chol_dalloc(chol_handle* h, void** p, size_t bytes);
 
 // binary64 updates on the tensor cores (split_gemm.cu)
 int chol_sg_ensure(chol_handle* h);
+int chol_vs_ensure(chol_handle* h, cudaStream_t st);   // 1: available
+void chol_vs_release(chol_handle* h);
+void chol_vs_products(chol_handle* h, const LevelPlan& P, bool trans, double* Y, double* W, int nr, cudaStream_t st);
 void chol_sg_release(chol_handle* h);
 void chol_sg_trailing(chol_handle* h, const TileTask* tasks, int n, int grid, int buf, cudaStream_t st);
 void chol_gather_zrr(chol_handle* h, const LevelPlan& P, const double* Z, double* ZRR, cudaStream_t st);

@@ -1109,8 +1109,14 @@ int chol_dalloc(chol_handle* h, void** p, size_t bytes) {
   if (bytes == 0) return CHOL_OK;
   if (h->opt.device_mem_cap > 0 && D->bytes + (int64_t)bytes > h->opt.device_mem_cap) return CHOL_ENOMEM;
   cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && D->vs_ready == 1 && !D->vs_pinned) {
+    // first the slices of the solves' products, then those of the updates: the
+    // parts that can be done without
+    cudaGetLastError();
+    chol_vs_release(h);
+    e = cudaMalloc(p, bytes);
+  }
   if (e == cudaErrorMemoryAllocation && D->sg_ready == 1) {
-    // the tensor-core updates' workspaces are the part that can be done without
     cudaGetLastError();
     if (D->graph_exec) {   // captured with them
       cudaGraphExecDestroy(D->graph_exec);
@@ -1143,7 +1149,8 @@ void chol_device_free(chol_handle* h) {
                   D->mx_diagpos, D->mx_aij, D->mx_d, D->mx_fallbacks, D->csr_ptr, D->csr_col, D->csr_src,
                   D->csr_val, D->Lbf, D->tmaps, D->tc_err, D->R, D->Z, D->Pv, D->Q, D->red, D->Y32, D->W32,
                   D->rhs_scale, D->host_vals, D->host_rhs, D->panel, D->pflags, D->dinv, D->split_part, D->split_cnt, D->hand32, D->sg_slab, D->sg_exps, D->sgt_slab[0], D->sgt_slab[1], D->sgt_slab[2],
-                  D->sgt_exps[0], D->sgt_exps[1], D->sgt_exps[2], D->sg_dev, D->sg_split, D->sg_syrk, D->sg_trail, D->rdiag, D->fasm};
+                  D->sgt_exps[0], D->sgt_exps[1], D->sgt_exps[2], D->sg_dev, D->sg_split, D->sg_syrk, D->sg_trail, D->rdiag, D->fasm, D->vs_slab, D->vs_exps, D->vs_rslab, D->vs_rexps,
+                  D->vs_part, D->vs_cnt, D->vs_dev, D->vs_ops, D->vs_list, D->vs_tasks, D->vs_tiles};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (D->status_host) cudaFreeHost(D->status_host);

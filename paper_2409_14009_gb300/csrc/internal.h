@@ -1,5 +1,6 @@
 // internal.h -- handle layout shared by the host analysis and the CUDA driver.
 #pragma once
+#include <array>
 #include <cstdint>
 #include <vector>
 
@@ -45,6 +46,27 @@ struct SplitDev {
   int64_t srow0, trow0;  // first exponent
   int32_t srows, trows;  // rows per slice (a multiple of 64, at least 64 past the last row's tile)
   int32_t sblk, pad;     // 32-column blocks of the SYRK operand
+};
+
+// log2 of the rows that one CTA splits into slices (512 threads, 8 columns each):
+// an operand of K > 1024 columns takes 4 rows, so that operands of few rows still
+// give enough CTAs and a row's two passes are few steps long.
+#define SPLIT_ROWS_LOG2(K) ((K) <= 64 ? 6 : (K) <= 128 ? 5 : (K) <= 512 ? 4 : (K) <= 1024 ? 3 : 2)
+
+// The solves' panel products on the tensor cores (solve_split.cu): slices of L_RJ
+// by rows (f*, forward) and by columns (b*, backward), and of the right-hand
+// sides (r*, 16 rows; K = s or b, laid out for the larger). Offsets within a level,
+// those of the exponents fexp, which the backward pass reads too, and bexp behind
+// them within the plan.
+struct SolveSplitDev {
+  int64_t foff, boff, roff;      // first slice row (64 bytes each)
+  int64_t fexp, bexp, rexp;      // first exponent
+  int32_t frows, brows;          // rows per slice, whole 128-row tiles
+};
+// Tile rows [r0, r0 + 128), K blocks [kb0, kb1); parts > 1: part `part` of a sum
+// whose partial tiles lie at slots [slot, slot + parts).
+struct SolveTile {
+  int32_t J, r0, kb0, kb1, slot, part, parts, pad;
 };
 
 // Blocked large-supernode task: supernode J, column step k0, tile origin (r0, c0).
@@ -130,6 +152,10 @@ struct LevelPlan {
   int32_t tri_b, tri_n;       // diagonal-triangle solve items (in tri_items), dependency order
   int32_t ssmall_b, ssmall_n; // supernodes solved by one warp each (in ssmall_list),
   int32_t ssmall8_n, ssmall16_n; // the first ssmall8_n of them with s <= 8, the next ssmall16_n with s <= 16
+  // several right-hand sides: supernodes (vs_list), splitting tasks and tiles of the
+  // forward [0] and backward [1] products, panel entries
+  int32_t vs_b, vs_n, vs_task_b[2], vs_task_n[2], vs_tile_b[2], vs_tile_n[2];
+  double vs_entries;
   int32_t gemv_b, gemv_n;     // forward-solve panel products (TileTask: J, r0)
   int32_t bpart_b, bpart_n;   // row-major backward panel, stage 1 (J, chunk, u0, c0)
   int32_t bred_b, bred_n;     // row-major backward panel, stage 2 (J, c0)
@@ -198,6 +224,12 @@ struct chol_handle {
   std::vector<TriItemHost> tri_items;          // solve: diagonal-triangle blocks per level
   int32_t tri_nflags = 0;                      // solve: one flag per 64-row diagonal block
   std::vector<int32_t> ssmall_list;            // solve: one-warp supernodes per level
+  std::vector<int32_t> vs_list;                 // solve products on the tensor cores (binary64)
+  std::vector<SolveSplitDev> vs_dev;
+  std::vector<std::array<int32_t, 2>> vs_tasks; // (operand 2 i + direction of vs_list[i], first row)
+  std::vector<SolveTile> vs_tiles;
+  double vs_work = 0.0;                         // largest level's panel entries
+  int64_t vs_slab_rows = 0, vs_exps = 0, vs_rslab_rows = 0, vs_rexps = 0, vs_slots = 0, vs_fexps = 0;
   std::vector<TileTask> gemv_tasks;             // solve: (J, r0) off-diagonal row tiles
   std::vector<TileTask> bpart_tasks, bred_tasks; // solve: row-major backward panel stages
   int64_t p_max = 0;                            // largest per-level partial-sum rows

@@ -1453,11 +1453,24 @@ int small_groups(const LevelPlan& P, F&& f) {
   return (n8 > 0) + (n16 > 0) + (n32 > 0);
 }
 
+// Levels whose panel products go to the tensor cores (solve_split.cu): at least 9
+// right-hand sides, and 8e6 products of panel entry and right-hand side. The
+// splitting costs the same for any number of right-hand sides: 3D 48^3, a solve
+// with 4, 8 and 16 of them takes 4.4, 5.7 and 7.9 ms there and 3.6, 5.6 and 11.3 ms
+// on the FP64 pipe. The three launches take about 45 us (forward) and 65 us
+// (backward) where a level is small: a line at 2e7 gave 8.07 ms, at 5e7 8.55.
+constexpr int kVsMinRhs = 9;
+constexpr double kVsMinWork = 8e6;
+
 template <class T, bool RM>
 int solve_levels(chol_handle* h, const T* L, T* Y, T* W, T* part, int nr, cudaStream_t st, bool prof) {
   DeviceState* D = h->dev;
   const int n = h->n;
   auto scope = [&](int cls) { return prof ? new KScope(h, cls, st, 0.0, 0.0) : nullptr; };
+  // binary64 with several right-hand sides: levels of enough work go to the tensor
+  // cores (prof: not the entry point that must not allocate)
+  const bool tc = sizeof(T) == 8 && prof && nr >= kVsMinRhs && h->vs_work * nr >= kVsMinWork && chol_vs_ensure(h, st) == 1;
+  auto products_on_tc = [&](const LevelPlan& P) { return tc && P.vs_entries * nr >= kVsMinWork; };
   {   // forward pass (an NVTX range over the scope; early returns pop it)
   NvtxRange nvtx_forward("forward");
   for (const LevelPlan& P : h->levels) {
@@ -1480,7 +1493,14 @@ int solve_levels(chol_handle* h, const T* L, T* Y, T* W, T* part, int nr, cudaSt
       delete ks;
       if (rc) return rc;
     }
-    if (P.gemv_n > 0) {
+    if (products_on_tc(P)) {
+      if constexpr (sizeof(T) == 8) {
+        KScope* ks = scope(CHOL_K_SOLVE_GEMV);
+        if (ks) ks->launches(3);
+        chol_vs_products(h, P, false, Y, W, nr, st);
+        delete ks;
+      }
+    } else if (P.gemv_n > 0) {
       KScope* ks = scope(CHOL_K_SOLVE_GEMV);
       with_nr(nr, [&](auto c) {
         k_sv_gemv<T, RM, decltype(c)::value><<<P.gemv_n, kT, 0, st>>>(D->sn, D->gemv + P.gemv_b, L, Y, n, W, nr,
@@ -1512,6 +1532,13 @@ int solve_levels(chol_handle* h, const T* L, T* Y, T* W, T* part, int nr, cudaSt
                                                                       part, h->p_max, nr);
         });
         k_sv_bred<T><<<P.bred_n, kT, 0, st>>>(D->sn, D->bred + P.bred_b, part, h->p_max, Y, n, nr);
+        delete ks;
+      }
+    } else if (products_on_tc(P)) {
+      if constexpr (sizeof(T) == 8) {
+        KScope* ks = scope(CHOL_K_SOLVE_BPANEL);
+        if (ks) ks->launches(3);
+        chol_vs_products(h, P, true, Y, W, nr, st);
         delete ks;
       }
     } else if (P.bpanel_n > 0) {
@@ -1679,6 +1706,7 @@ int chol_solve_status(chol_handle* h) {
   CHOL_CUDA_TRY(cudaMemcpy(e, D->sv_err, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost));
   if (e[0] | e[1]) {
     CHOL_CUDA_TRY(cudaMemset(D->sv_err, 0, 2 * sizeof(int32_t)));
+    if (D->vs_cnt) CHOL_CUDA_TRY(cudaMemset(D->vs_cnt, 0, sizeof(int32_t) * (size_t)h->vs_slots));
     return CHOL_ETIMEOUT;
   }
   return CHOL_OK;

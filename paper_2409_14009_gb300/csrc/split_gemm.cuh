@@ -41,25 +41,34 @@
 namespace sg {
 
 constexpr int kSlices = kSplitSlices;
-constexpr int kM = 128, kN = 64;          // output tile
+constexpr int kM = 128, kN = 64;          // output tile (kN: of the updates; Cfg<N>)
 constexpr int kBlockK = 32;               // K of one stage
 constexpr int kDigit = 9;                 // bits of a digit
 constexpr int kChunkK = 64;               // K per accumulator chunk (see above)
 constexpr int kStagesPerChunk = kChunkK / kBlockK;
-constexpr int kStages = 2;
-constexpr int kABytes = kM * 64, kBBytes = kN * 64;           // one slice of an operand stage
-constexpr int kStageBytes = kSlices * (kABytes + kBBytes);    // 86,016
-constexpr int kSmemBytes = kStages * kStageBytes + 1024;
-constexpr int kEpiWarps = 16;             // four to a partition: the epilogue is integer work with short chains
+constexpr int kABytes = kM * 64;          // one slice of an operand stage
 constexpr int kCols = 16;                 // columns of an epilogue thread
-constexpr int kThreads = 32 * (kEpiWarps + 2);   // epilogue, copy and MMA warps
-constexpr int kTmemCols = 512;            // 7 accumulators of 64 columns
+// A kernel with tiles of N columns: 64 (updates, one stage of 86 KB) or 16 (the
+// products with right-hand sides, 64 KB).
+template <int N>
+struct Cfg {
+  static constexpr int kBBytes = N * 64;
+  static constexpr int kStageBytes = kSlices * (kABytes + kBBytes);
+  static constexpr int kStages = N == 64 ? 2 : 3;
+  static constexpr int kSmemBytes = kStages * kStageBytes + 1024;
+  static constexpr int kEpiWarps = 4 * (N / kCols);   // 16 or 4: the epilogue is integer work with short chains
+  static constexpr int kThreads = 32 * (kEpiWarps + 2);   // epilogue, copy and MMA warps
+  static constexpr int kTmemCols = N == 64 ? 512 : 128;   // 7 accumulators of N columns
+  static constexpr uint32_t kIdesc =
+      (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kM >> 4) << 24);
+};
+constexpr int kEpiWarps = Cfg<kN>::kEpiWarps, kThreads = Cfg<kN>::kThreads, kSmemBytes = Cfg<kN>::kSmemBytes;
 
 // Operand splitting: 512 threads take R rows, 8 columns a thread, so that an
 // operand of few rows and many columns still gives enough CTAs and loads in
 // flight (64 rows and 64 columns a step took 31 us where this takes 13).
 constexpr int kSplitThreadsLog2 = 9, kSplitThreads = 1 << kSplitThreadsLog2;
-__host__ __device__ constexpr int split_rows_log2(int K) { return K <= 64 ? 6 : (K <= 128 ? 5 : 4); }
+__device__ __forceinline__ int split_rows_log2(int K) { return SPLIT_ROWS_LOG2(K); }
 
 constexpr int32_t kExpNaN = INT_MIN;      // exponent of a row with an infinity or a NaN
 constexpr int32_t kExpMin = -1020;        // rows of zeros and subnormals
@@ -89,13 +98,13 @@ __device__ __forceinline__ uint32_t digit_bits(int d) {
   return __float_as_uint(__int_as_float(0x4B400000 + d) - 12582912.0f);
 }
 
-// The digits of eight consecutive entries of a row: out[i] = the 16 bytes
-// (8 bf16) of slice i.
-__device__ __forceinline__ void digits8(const double (&x)[8], int32_t e, uint4 (&out)[kSlices]) {
+// The digits of eight consecutive entries of a row (e: exponent of each): out[i] =
+// the 16 bytes (8 bf16) of slice i.
+__device__ __forceinline__ void digits8(const double (&x)[8], const int32_t (&e)[8], uint4 (&out)[kSlices]) {
   uint32_t w[kSlices][4];
 #pragma unroll
   for (int p = 0; p < 4; ++p) {
-    long long y0 = fixed_point(x[2 * p], e), y1 = fixed_point(x[2 * p + 1], e);
+    long long y0 = fixed_point(x[2 * p], e[2 * p]), y1 = fixed_point(x[2 * p + 1], e[2 * p + 1]);
 #pragma unroll
     for (int i = kSlices - 1; i >= 0; --i) {
       // the low digit, sign-extended (the one left last is the top digit)
@@ -108,6 +117,11 @@ __device__ __forceinline__ void digits8(const double (&x)[8], int32_t e, uint4 (
   }
 #pragma unroll
   for (int i = 0; i < kSlices; ++i) out[i] = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
+}
+
+__device__ __forceinline__ void digits8(const double (&x)[8], int32_t e, uint4 (&out)[kSlices]) {
+  const int32_t ee[8] = {e, e, e, e, e, e, e, e};
+  digits8(x, ee, out);
 }
 
 // Byte offset of the 16-byte chunk c (0..3) of row r inside one slice.
@@ -185,9 +199,6 @@ __device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
   return d;
 }
 
-constexpr uint32_t kIdesc =
-    (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kN >> 3) << 17) | ((uint32_t)(kM >> 4) << 24);
-
 // Bounded wait that also gives up when another role of the CTA has.
 __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
   const long long t0 = clock64();
@@ -215,23 +226,25 @@ struct Tile {
 };
 
 // Shared state of the CTA.
+constexpr int kMaxStages = 3;
 struct Shared {
   // accumulators change hands in two groups: orders 0..3 and 4..6
-  uint64_t full[kStages], empty[kStages], acc_full[2], acc_empty[2], done;
+  uint64_t full[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2], done;
   uint32_t tmem;
   int abort_flag, issued;
 };
 
+template <int N = kN>
 __device__ __forceinline__ uint32_t setup(Shared& S) {
   const int warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
+    for (int s = 0; s < Cfg<N>::kStages; ++s) {
       tc::mbar_init(tc::smem_u32(&S.full[s]), 1);
       tc::mbar_init(tc::smem_u32(&S.empty[s]), 1);
     }
     for (int q = 0; q < 2; ++q) {
       tc::mbar_init(tc::smem_u32(&S.acc_full[q]), 1);
-      tc::mbar_init(tc::smem_u32(&S.acc_empty[q]), kEpiWarps);
+      tc::mbar_init(tc::smem_u32(&S.acc_empty[q]), Cfg<N>::kEpiWarps);
     }
     tc::mbar_init(tc::smem_u32(&S.done), 1);
     S.abort_flag = 0;
@@ -241,7 +254,7 @@ __device__ __forceinline__ uint32_t setup(Shared& S) {
   __syncwarp();
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc::smem_u32(&S.tmem)),
-                 "r"(kTmemCols)
+                 "r"(Cfg<N>::kTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -253,14 +266,15 @@ __device__ __forceinline__ uint32_t setup(Shared& S) {
 
 // Ends the CTA: after an abort, waits (bounded) for the copies in flight and
 // for the MMAs already issued; then frees the tensor memory.
+template <int N = kN>
 __device__ __forceinline__ void teardown(Shared& S, uint32_t tmem) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int never = 0;
-  if (warp == kEpiWarps && lane == 0 && *(volatile int*)&S.abort_flag) {
-    for (int s = 0; s < kStages && s < S.issued; ++s)
-      wait_or_abort(tc::smem_u32(&S.full[s]), (uint32_t)(((S.issued - 1 - s) / kStages) & 1), &never);
+  if (warp == Cfg<N>::kEpiWarps && lane == 0 && *(volatile int*)&S.abort_flag) {
+    for (int s = 0; s < Cfg<N>::kStages && s < S.issued; ++s)
+      wait_or_abort(tc::smem_u32(&S.full[s]), (uint32_t)(((S.issued - 1 - s) / Cfg<N>::kStages) & 1), &never);
   }
-  if (warp == kEpiWarps + 1 && lane == 0) {
+  if (warp == Cfg<N>::kEpiWarps + 1 && lane == 0) {
     tc::mma_commit(tc::smem_u32(&S.done));
     wait_or_abort(tc::smem_u32(&S.done), 0, &never);
   }
@@ -269,17 +283,17 @@ __device__ __forceinline__ void teardown(Shared& S, uint32_t tmem) {
   __syncthreads();
   tc::fence_after();
   if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Cfg<N>::kTmemCols) : "memory");
 }
 
 // The copy thread's loop over the CTA's tiles: `next(i, tile)` gives the i-th tile.
-template <class Next>
+template <int N = kN, class Next>
 __device__ __forceinline__ void copy_loop(Shared& S, uint32_t base, Next next, int* err) {
   int it = 0;
   Tile t;
   for (int i = 0; next(i, t); ++i) {
     for (int k = 0; k < t.nblk; ++k, ++it) {
-      const int s = it % kStages, round = it / kStages;
+      const int s = it % Cfg<N>::kStages, round = it / Cfg<N>::kStages;
       if (round > 0 && !wait_or_abort(tc::smem_u32(&S.empty[s]), (uint32_t)((round - 1) & 1), &S.abort_flag)) {
         atomicExch(err, tc::kErrTimeoutEmpty);
         *(volatile int*)&S.abort_flag = 1;
@@ -287,14 +301,14 @@ __device__ __forceinline__ void copy_loop(Shared& S, uint32_t base, Next next, i
         return;
       }
       const uint32_t fb = tc::smem_u32(&S.full[s]);
-      tc::mbar_expect_tx(fb, (uint32_t)kStageBytes);
-      const uint32_t a0 = base + s * kStageBytes, b0 = a0 + kSlices * kABytes;
+      tc::mbar_expect_tx(fb, (uint32_t)Cfg<N>::kStageBytes);
+      const uint32_t a0 = base + s * Cfg<N>::kStageBytes, b0 = a0 + kSlices * kABytes;
       const unsigned char* pa = t.a.slab + ((int64_t)k * kSlices * t.a.rows + t.a.row0) * 64;
       const unsigned char* pb = t.b.slab + ((int64_t)k * kSlices * t.b.rows + t.b.row0) * 64;
 #pragma unroll
       for (int q = 0; q < kSlices; ++q) {
         bulk_load(a0 + q * kABytes, pa + (int64_t)q * t.a.rows * 64, kABytes, fb);
-        bulk_load(b0 + q * kBBytes, pb + (int64_t)q * t.b.rows * 64, kBBytes, fb);
+        bulk_load(b0 + q * Cfg<N>::kBBytes, pb + (int64_t)q * t.b.rows * 64, Cfg<N>::kBBytes, fb);
       }
     }
   }
@@ -305,16 +319,16 @@ __device__ __forceinline__ void copy_loop(Shared& S, uint32_t base, Next next, i
 // start here. Unrolled: the descriptors become additions of constants, and the
 // issue keeps up with the 48 cycles that a 128 x 64 x 16 product takes (operand
 // reads); in a loop over the slice pairs it took 112.
-template <int Q0, int Q1>
+template <int N, int Q0, int Q1>
 __device__ __forceinline__ void mma_orders(uint32_t tmem, uint64_t ad, uint64_t bd, bool first) {
 #pragma unroll
   for (int q = Q0; q < Q1; ++q) {
-    const uint32_t d = tmem + (uint32_t)(q * kN);
+    const uint32_t d = tmem + (uint32_t)(q * N);
 #pragma unroll
     for (int a = 0; a <= q; ++a) {
-      const uint64_t da = ad + (uint64_t)(a * (kABytes >> 4)), db = bd + (uint64_t)((q - a) * (kBBytes >> 4));
-      tc::mma<1>(d, da, db, kIdesc, (first && a == 0) ? 0u : 1u);
-      tc::mma<1>(d, da + 2, db + 2, kIdesc, 1u);
+      const uint64_t da = ad + (uint64_t)(a * (kABytes >> 4)), db = bd + (uint64_t)((q - a) * (Cfg<N>::kBBytes >> 4));
+      tc::mma<1>(d, da, db, Cfg<N>::kIdesc, (first && a == 0) ? 0u : 1u);
+      tc::mma<1>(d, da + 2, db + 2, Cfg<N>::kIdesc, 1u);
     }
   }
 }
@@ -323,7 +337,7 @@ __device__ __forceinline__ void mma_orders(uint32_t tmem, uint64_t ad, uint64_t 
 // a group of orders is handed to the epilogue at the end of each chunk of
 // kChunkK and taken back before its next use, so the epilogue reads one group
 // while the other's products run.
-template <class Next>
+template <int N = kN, class Next>
 __device__ __forceinline__ void mma_loop(Shared& S, uint32_t base, uint32_t tmem, Next next, int* err) {
   int it = 0, chunk = 0;
   Tile t;
@@ -333,12 +347,12 @@ __device__ __forceinline__ void mma_loop(Shared& S, uint32_t base, uint32_t tmem
   };
   for (int i = 0; next(i, t); ++i) {
     for (int k = 0; k < t.nblk; ++k, ++it) {
-      const int s = it % kStages, round = it / kStages;
+      const int s = it % Cfg<N>::kStages, round = it / Cfg<N>::kStages;
       if (!wait_or_abort(tc::smem_u32(&S.full[s]), (uint32_t)(round & 1), &S.abort_flag)) {
         give_up(tc::kErrTimeoutFull);
         return;
       }
-      const uint32_t a0 = base + s * kStageBytes;
+      const uint32_t a0 = base + s * Cfg<N>::kStageBytes;
       const uint64_t ad = sw64_desc(a0), bd = sw64_desc(a0 + kSlices * kABytes);
       const bool first = k % kStagesPerChunk == 0;
       const bool last = k % kStagesPerChunk == kStagesPerChunk - 1 || k == t.nblk - 1;
@@ -349,14 +363,14 @@ __device__ __forceinline__ void mma_loop(Shared& S, uint32_t base, uint32_t tmem
         return;
       }
       tc::fence_after();
-      mma_orders<0, 4>(tmem, ad, bd, first);
+      mma_orders<N, 0, 4>(tmem, ad, bd, first);
       if (last) tc::mma_commit(tc::smem_u32(&S.acc_full[0]));
       if (take && !wait_or_abort(tc::smem_u32(&S.acc_empty[1]), par, &S.abort_flag)) {
         give_up(tc::kErrTimeoutAccum);
         return;
       }
       tc::fence_after();
-      mma_orders<4, kSlices>(tmem, ad, bd, first);
+      mma_orders<N, 4, kSlices>(tmem, ad, bd, first);
       if (last) tc::mma_commit(tc::smem_u32(&S.acc_full[1]));
       tc::mma_commit(tc::smem_u32(&S.empty[s]));
       if (last) ++chunk;
@@ -386,6 +400,7 @@ __device__ __forceinline__ int epi_col() { return (int)(threadIdx.x >> 7) * kCol
 
 // Adds one chunk's sums of the thread's 16 entries to hi (orders 0..3) and lo
 // (orders 4..6) and gives the accumulators back. False if a wait gave up.
+template <int N = kN>
 __device__ __forceinline__ bool drain(Shared& S, uint32_t tmem, int chunk, long long (&hi)[kCols],
                                       long long (&lo)[kCols], int* err) {
   const uint32_t t0 = tmem + ((uint32_t)((threadIdx.x >> 5) & 3) << 21) + (uint32_t)epi_col();
@@ -395,7 +410,7 @@ __device__ __forceinline__ bool drain(Shared& S, uint32_t tmem, int chunk, long 
   for (int c = 0; c < kCols; c += 4) {
     uint32_t r[4][4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) tmem_ld4(t0 + (uint32_t)(q * kN + c), r[q]);
+    for (int q = 0; q < 4; ++q) tmem_ld4(t0 + (uint32_t)(q * N + c), r[q]);
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -412,7 +427,7 @@ __device__ __forceinline__ bool drain(Shared& S, uint32_t tmem, int chunk, long 
   for (int c = 0; c < kCols; c += 4) {
     uint32_t r[3][4];
 #pragma unroll
-    for (int q = 0; q < 3; ++q) tmem_ld4(t0 + (uint32_t)((q + 4) * kN + c), r[q]);
+    for (int q = 0; q < 3; ++q) tmem_ld4(t0 + (uint32_t)((q + 4) * N + c), r[q]);
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < 4; ++i)

@@ -115,3 +115,57 @@ def test_selected_inverse(s, b, mode):
     A = np.tril(A) + np.tril(A, -1).T
     ref = np.linalg.inv(A)[p["rowind"], cols]
     assert np.max(np.abs(z.cpu().numpy() - ref)) <= 1e-11 * np.max(np.abs(ref))
+
+
+def test_selected_inverse_scaling():
+    """Z scales exactly too: the K index of Z_RR U and U^T Z_RJ is balanced."""
+    import torch
+    P = chol()
+    p = _arrow(130, 100)
+    zs = []
+    for q in (p, _arrow(130, 100, 60)):
+        rc, h = P.chol_analyze(q["n"], q["colptr"], q["rowind"], q["perm"], _opts())
+        v = torch.as_tensor(q["values"], device="cuda")
+        z = torch.empty_like(v)
+        assert rc == 0 and P.chol_factor(h, v) == 0 and P.chol_selected_inverse(h, z) == 0
+        assert P.chol_check_waits(h) == 0
+        P.chol_destroy(h)
+        zs.append(z.cpu().numpy())
+    d = np.sqrt(q["values"][q["colptr"][:-1]] / p["values"][p["colptr"][:-1]])
+    cols = np.repeat(np.arange(p["n"]), np.diff(p["colptr"]))
+    assert np.array_equal(zs[1], zs[0] / d[cols] / d[p["rowind"]])
+
+
+# a level's panel entries times right-hand sides, 2 s b nrhs >= 8e6, nrhs >= 9, takes
+# the tensor cores; 17 = a chunk of 16 and one right-hand side on the other path
+@pytest.mark.parametrize("s,b,nrhs", [(300, 905, 16), (129, 2000, 17), (601, 1399, 9), (1030, 1030, 12)])
+def test_solve_products(s, b, nrhs):
+    """Solves of a system and of its scaling by powers of two, which is exactly the
+    scaled solution; a column of NaN stays alone. n <= 3100, kappa < 100 after
+    scaling: within n u kappa < 4e-11 of the largest entry."""
+    import torch
+    P = chol()
+    rs = np.random.RandomState(7)
+    x = rs.uniform(-1, 1, (2 * s + b, nrhs))
+    got = []
+    for spread in (0, 60):
+        p = _arrow(s, b, spread)
+        n, cols = p["n"], np.repeat(np.arange(p["n"]), np.diff(p["colptr"]))
+        d = np.ones(n)
+        if spread:
+            d = np.sqrt(p["values"][p["colptr"][:-1]] / diag)
+        diag = p["values"][p["colptr"][:-1]]
+        if not spread:
+            A = np.zeros((n, n))
+            A[p["rowind"], cols] = p["values"]
+            rhs = A @ x + np.tril(A, -1).T @ x
+            rhs[:, nrhs - 1 if nrhs <= 16 else 3] = np.nan
+        rc, h = P.chol_analyze(n, p["colptr"], p["rowind"], p["perm"], _opts())
+        assert rc == 0 and P.chol_factor(h, torch.as_tensor(p["values"], device="cuda")) == 0
+        y = torch.as_tensor(np.ascontiguousarray((rhs * d[:, None]).T), device="cuda")
+        assert P.chol_solve(h, y, nrhs) == 0 and P.chol_check_waits(h) == 0
+        P.chol_destroy(h)
+        got.append(y.cpu().numpy().T * d[:, None])
+    ok = ~np.isnan(rhs[0])
+    assert np.max(np.abs(got[0][:, ok] - x[:, ok])) <= 4e-11
+    assert np.isnan(got[0][:, ~ok]).all() and np.array_equal(got[0][:, ok], got[1][:, ok])
