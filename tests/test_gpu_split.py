@@ -169,3 +169,36 @@ def test_solve_products(s, b, nrhs):
     ok = ~np.isnan(rhs[0])
     assert np.max(np.abs(got[0][:, ok] - x[:, ok])) <= 4e-11
     assert np.isnan(got[0][:, ~ok]).all() and np.array_equal(got[0][:, ok], got[1][:, ok])
+
+
+def test_solve_products_captured():
+    """A solve captured before any other takes the binary64 kernels, one captured
+    after a plain solve the tensor cores; both replay to the plain solve's x."""
+    import torch
+    P = chol()
+    p = _arrow(300, 905)
+    n, nrhs = p["n"], 16
+    rc, h = P.chol_analyze(n, p["colptr"], p["rowind"], p["perm"], _opts())
+    assert rc == 0 and P.chol_factor(h, torch.as_tensor(p["values"], device="cuda")) == 0
+    b = torch.as_tensor(np.random.RandomState(2).uniform(-1, 1, (nrhs, n)), device="cuda")
+    st = torch.cuda.Stream()
+    got = []
+    with torch.cuda.stream(st):
+        one = b[0].clone()
+        assert P.chol_solve(h, one, 1, st) == 0     # the workspaces every solve needs
+        st.synchronize()
+        for k in range(2):
+            y = b.clone()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=st, capture_error_mode="thread_local"):
+                assert P.chol_solve(h, y, nrhs, st) == 0
+            for _ in range(2):
+                y.copy_(b)
+                g.replay()
+            st.synchronize()
+            got.append(y.clone())
+            x = b.clone()
+            assert P.chol_solve(h, x, nrhs, st) == 0 and P.chol_check_waits(h, st) == 0
+    P.chol_destroy(h)
+    assert torch.equal(got[1], x)
+    assert (got[0] - x).abs().max() <= 6e-11 * x.abs().max()
