@@ -33,10 +33,13 @@ WORKLOAD = "3D 7-point var-coef Laplacian 64^3 (n=262144), FP64 factor + 8-RHS s
 NRHS = 8
 # FP64 peak derived from unit counts: 152 SMs x 2 FP64 FMA/clk/SM x 2 flop x 2.07 GHz
 FP64_PEAK_GFLOPS = 152 * 2 * 2 * 2.07
-# DRAM bytes (read + write) per k_syrk launch on this workload, from the ncu
-# capture summarised in profiles/k_syrk_fp64_3d64_traffic.md (18 launches of one
-# factorization: 1.228 GB read + 2.780 GB written)
-K_SYRK_TRAFFIC_PER_LAUNCH = 4.0074e9 / 18
+# binary64 products run as 28 bf16 slice products on the tensor cores
+# (csrc/split_gemm.cuh); cuBLAS bf16 under the power cap where it was measured
+SLICE_PRODUCTS = 28
+BF16_SUSTAINED_TFLOPS = 1700.0
+# DRAM bytes (read + write) per launch of the SYRK class on this workload, from
+# the ncu capture summarised in profiles/k_sg_syrk_fp64_3d64_traffic.md
+SYRK_TRAFFIC_PER_LAUNCH = 8.246e9 / 36
 
 
 def _env_int(k, d):
@@ -98,6 +101,14 @@ class ClockSampler:
             return {"sm_mhz": None, "sm_max_mhz": None, "reasons": ["unsampled"]}
         return {"sm_mhz": float(np.median(sm)), "sm_max_mhz": mx, "reasons": sorted(reasons),
                 "samples": len(sm)}
+
+
+def bf16_sustained_tflops():
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            return float(json.load(f)["bf16_tflops_sustained"])
+    except (OSError, KeyError, ValueError):
+        return BF16_SUSTAINED_TFLOPS
 
 
 def max_over_ranks(dist, values, device):
@@ -546,9 +557,9 @@ def run_ours(args, rank, world, local_rank):
     for _ in range(max(args.warmup, 0)):
         step()
     torch.cuda.synchronize()
-    # time the dominant kernel (the SYRK class: 62% of the serialised factor
-    # time in the ncu launch list, the trailing GEMM class 30%) inside the timed
-    # region; per-launch events on one class only keep the step's overhead small
+    # time the SYRK class (the most flops of a class, and alone on the GPU while it
+    # runs) inside the timed region; per-launch events on one class only keep the
+    # step's overhead small
     P.chol_profile(S.h, 1 << P.KERNEL_CLASSES.index("syrk"))
     P.chol_get_stats(S.h, reset=True)
     e0 = torch.cuda.Event(enable_timing=True)
@@ -606,22 +617,28 @@ def run_ours(args, rank, world, local_rank):
                                            S.info.update_doubles)
     ms, e2e_ms = max_over_ranks(dist, [ms, e2e_ms], dev)
     if rank == 0:
-        dom = "syrk"
-        ds = stats[dom]
+        ds = stats["syrk"]
         achieved = ds["flops"] / (ds["ms"] * 1e-3) / 1e9 if ds["ms"] > 0 else None
         stored_ratio = S.info.flops_stored / flops
         rc_p, dfma, dfma_ghz = P.chol_probe_fp64(0, 3)
         rc_q, dmma, dmma_ghz = P.chol_probe_fp64(1, 3)
-        roof = {"bound": "alu", "kernel": "k_gemm_trailing" if dom == "gemm" else "k_syrk",
-                "achieved": achieved, "peak": FP64_PEAK_GFLOPS, "unit": "GFLOP/s",
-                "frac": (achieved / FP64_PEAK_GFLOPS) if achieved else None,
+        tensor = achieved is not None and achieved > FP64_PEAK_GFLOPS   # else the binary64 pipe's kernel ran
+        peak = bf16_sustained_tflops() * 1e3 if tensor else FP64_PEAK_GFLOPS
+        done = achieved * SLICE_PRODUCTS if tensor else achieved
+        roof = {"bound": "tensor" if tensor else "alu",
+                "kernel": "k_sg_split_rows + k_sg_syrk" if tensor else "k_syrk",
+                # tensor: bf16 flops of the slice products, splitting included in the time
+                "achieved": done, "peak": peak, "unit": "GFLOP/s",
+                "frac": (done / peak) if done else None,
+                "fp64_gflops": achieved, "fp64_pipe_peak": FP64_PEAK_GFLOPS,
                 # the kernel's flops count the explicit zeros of relaxed merging;
                 # the method's own share scales by the symbolic / stored ratio
-                "frac_symbolic": (achieved / FP64_PEAK_GFLOPS / stored_ratio) if achieved else None,
-                "traffic": K_SYRK_TRAFFIC_PER_LAUNCH if dom == "syrk" else None,
-                "traffic_source": "profiles/k_syrk_fp64_3d64_traffic.md (ncu dram__bytes_read/write.sum of the "
-                                  "18 k_syrk launches of one 64^3 factorization, per launch)",
-                "peak_source": "derived: 152 SMs x 2 FP64 FMA/clk x 2.07 GHz (FP64 DFMA pipe); measured beside it "
+                "frac_symbolic": (done / peak / stored_ratio) if done else None,
+                "traffic": SYRK_TRAFFIC_PER_LAUNCH if tensor else None,
+                "traffic_source": "profiles/k_sg_syrk_fp64_3d64_traffic.md (ncu dram__bytes_read/write.sum of the "
+                                  "SYRK class of one 64^3 factorization, per launch)",
+                "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained (cuBLAS bf16)" if tensor else
+                               "derived: 152 SMs x 2 FP64 FMA/clk x 2.07 GHz (FP64 DFMA pipe); measured beside it "
                                "by chol_probe_fp64 (profiles/fp64_peak_probe.md)",
                 "peak_measured": {"dfma": dfma if rc_p == 0 else None, "dfma_sm_ghz": dfma_ghz,
                                   "dmma": dmma if rc_q == 0 else None, "dmma_sm_ghz": dmma_ghz,
