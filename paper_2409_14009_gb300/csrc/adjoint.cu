@@ -304,15 +304,17 @@ int upload_v(chol_handle* h, T** dst, const std::vector<T>& v) {
 
 int ensure_adjoint(chol_handle* h) {
   DeviceState* D = h->dev;
-  if (D->Zp) return CHOL_OK;
+  if (D->Zp && D->a_col && D->a_row) return CHOL_OK;   // an earlier call may have found room for some of them only
   int rc;
-  if ((rc = chol_dalloc(h, (void**)&D->Zp, sizeof(double) * (size_t)std::max<int64_t>(h->panel_doubles, 1)))) return rc;
+  if (!D->Zp &&
+      (rc = chol_dalloc(h, (void**)&D->Zp, sizeof(double) * (size_t)std::max<int64_t>(h->panel_doubles, 1))))
+    return rc;
   // column index of every stored entry of A (original ordering)
   std::vector<int32_t> colidx(h->nnz_a), rowidx(h->nnz_a);
   for (int32_t c = 0; c < h->n; ++c)
     for (int64_t t = h->a_colptr[c]; t < h->a_colptr[c + 1]; ++t) colidx[t] = c;
-  if ((rc = upload_v(h, &D->a_col, colidx))) return rc;
-  if ((rc = upload_v(h, &D->a_row, h->a_rowind))) return rc;
+  if (!D->a_col && (rc = upload_v(h, &D->a_col, colidx))) return rc;
+  if (!D->a_row && (rc = upload_v(h, &D->a_row, h->a_rowind))) return rc;
   return CHOL_OK;
 }
 
@@ -358,6 +360,7 @@ struct SiPlan {
   std::vector<SplitTile> stiles;
   int64_t slab_rows = 0, nexps = 0, nkexps = 0;
   bool sg = false;
+  bool pinned = false;   // a captured selected inverse holds the plan's addresses
   SplitOp* d_ops = nullptr;
   int32_t* d_kexps = nullptr;
   SplitTask* d_stasks = nullptr;
@@ -477,14 +480,17 @@ Group emit_group(SiPlan& pl, const std::vector<GenGemm>& gs, int sms, const std:
   return gr;
 }
 
+template <class T>
+void si_drop(chol_handle* h, T** p, int64_t bytes) {
+  if (*p) {
+    cudaFree(*p);   // waits for the work that uses it
+    h->dev->bytes -= bytes;
+  }
+  *p = nullptr;
+}
+
 void free_si_split(chol_handle* h, SiPlan* pl) {
-  auto drop = [&](auto** p, int64_t bytes) {
-    if (*p) {
-      cudaFree(*p);
-      h->dev->bytes -= bytes;
-    }
-    *p = nullptr;
-  };
+  auto drop = [&](auto** p, int64_t bytes) { si_drop(h, p, bytes); };
   drop(&pl->d_ops, (int64_t)(sizeof(SplitOp) * pl->ops.size()));
   drop(&pl->d_stasks, (int64_t)(sizeof(SplitTask) * pl->stasks.size()));
   drop(&pl->d_stiles, (int64_t)(sizeof(SplitTile) * pl->stiles.size()));
@@ -493,16 +499,30 @@ void free_si_split(chol_handle* h, SiPlan* pl) {
   drop(&pl->d_kexps, (int64_t)(sizeof(int32_t) * std::max<int64_t>(pl->nkexps, 1)));
 }
 
+void free_si_plan(chol_handle* h, SiPlan* pl) {
+  free_si_split(h, pl);
+  si_drop(h, &pl->d_descs, (int64_t)(sizeof(GenGemm) * pl->descs.size()));
+  si_drop(h, &pl->d_tiles, (int64_t)(sizeof(GemmTile) * pl->tiles.size()));
+  si_drop(h, &pl->d_rtiles, (int64_t)(sizeof(GemmTile) * pl->rtiles.size()));
+  si_drop(h, &pl->d_invs, (int64_t)(sizeof(InvTask) * pl->invs.size()));
+  si_drop(h, &pl->d_part, (int64_t)sizeof(double) * pl->part_max);
+  delete pl;
+}
+
 int build_si_plan(chol_handle* h) {
   DeviceState* D = h->dev;
   if (D->si_plan) return CHOL_OK;
   SiPlan* pl = new SiPlan();
+  auto fail = [&](int rc) {
+    free_si_plan(h, pl);
+    return rc;
+  };
   const double* L = D->L;
   // Z_RR of a level lives in the update workspace, at U_J's place; an RLB
   // handle has none, so it gets its own
   if (h->update_doubles < h->update_doubles_rl && !D->zrr_ws) {
     const int rz = chol_dalloc(h, (void**)&D->zrr_ws, sizeof(double) * (size_t)h->update_doubles_rl);
-    if (rz) { delete pl; return rz; }
+    if (rz) return fail(rz);
   }
   double* ZRR = D->zrr_ws ? D->zrr_ws : D->U;
   double* Z = D->Zp;
@@ -522,9 +542,10 @@ int build_si_plan(chol_handle* h) {
     tmax = std::max(tmax, t); hmax = std::max(hmax, u); wmax = std::max(wmax, w);
   }
   int rc;
-  if ((rc = chol_dalloc(h, (void**)&D->Tw, sizeof(double) * (size_t)std::max<int64_t>(tmax, 1)))) return rc;
-  if ((rc = chol_dalloc(h, (void**)&D->Uh, sizeof(double) * (size_t)std::max<int64_t>(hmax, 1)))) return rc;
-  if ((rc = chol_dalloc(h, (void**)&D->Ww, sizeof(double) * (size_t)std::max<int64_t>(wmax, 1)))) return rc;
+  auto work = [&](double** p, int64_t n) {   // kept by a build that found no room further on
+    return *p ? CHOL_OK : chol_dalloc(h, (void**)p, sizeof(double) * (size_t)std::max<int64_t>(n, 1));
+  };
+  if ((rc = work(&D->Tw, tmax)) || (rc = work(&D->Uh, hmax)) || (rc = work(&D->Ww, wmax))) return fail(rc);
   std::vector<int32_t> fbase(h->ns, -1);   // first block of J in the solve's inverses
   for (const TriItemHost& q : h->tri_items) fbase[q.J] = q.fbase;
   for (int lv = h->nlevels - 1; lv >= 0; --lv) {
@@ -640,9 +661,8 @@ int build_si_plan(chol_handle* h) {
     CHOL_CUDA_TRY(cudaMemcpy(*dst, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice));
     return CHOL_OK;
   };
-  if ((rc = up(&pl->d_descs, pl->descs))) return rc;
+  if ((rc = up(&pl->d_descs, pl->descs))) return fail(rc);
   // the tensor-core form where its slices find room (as for the factor's updates)
-  D->si_plan = pl;
   if (h->opt.device_mem_cap == 0 && D->sg_ready == 1 && !pl->stiles.empty()) {
     pl->sg = up(&pl->d_ops, pl->ops) == CHOL_OK && up(&pl->d_stasks, pl->stasks) == CHOL_OK &&
              up(&pl->d_stiles, pl->stiles) == CHOL_OK &&
@@ -654,11 +674,14 @@ int build_si_plan(chol_handle* h) {
     if (!pl->sg) free_si_split(h, pl);
   }
   if (!pl->sg) {
-    if ((rc = up(&pl->d_tiles, pl->tiles))) return rc;
-    if ((rc = up(&pl->d_rtiles, pl->rtiles))) return rc;
-    if (pl->part_max > 0 && (rc = chol_dalloc(h, (void**)&pl->d_part, sizeof(double) * (size_t)pl->part_max))) return rc;
+    if ((rc = up(&pl->d_tiles, pl->tiles))) return fail(rc);
+    if ((rc = up(&pl->d_rtiles, pl->rtiles))) return fail(rc);
+    if (pl->part_max > 0 && (rc = chol_dalloc(h, (void**)&pl->d_part, sizeof(double) * (size_t)pl->part_max)))
+      return fail(rc);
   }
-  if ((rc = up(&pl->d_invs, pl->invs))) return rc;
+  if ((rc = up(&pl->d_invs, pl->invs))) return fail(rc);
+  if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) return fail(CHOL_ECUDA);   // the copies
+  D->si_plan = pl;
   return CHOL_OK;
 }
 
@@ -672,6 +695,9 @@ int selinv(chol_handle* h, cudaStream_t st) {
   if ((rc = build_si_plan(h))) return rc;
   DeviceState* D = h->dev;
   SiPlan* pl = (SiPlan*)D->si_plan;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  CHOL_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
+  if (cap != cudaStreamCaptureStatusNone) pl->pinned = true;
   auto launch = [&](const Group& gr) {
     if (pl->sg) {
       if (gr.gn == 0) return;
@@ -717,13 +743,16 @@ int selinv(chol_handle* h, cudaStream_t st) {
 void chol_adjoint_free(chol_handle* h) {
   DeviceState* D = h->dev;
   if (!D || !D->si_plan) return;
-  SiPlan* pl = (SiPlan*)D->si_plan;
-  void* ptrs[] = {pl->d_descs, pl->d_tiles, pl->d_rtiles, pl->d_invs, pl->d_part,
-                  pl->d_ops, pl->d_stasks, pl->d_stiles, pl->d_slab, pl->d_exps, pl->d_kexps};
-  for (void* p : ptrs)
-    if (p) cudaFree(p);
-  delete pl;
+  free_si_plan(h, (SiPlan*)D->si_plan);
   D->si_plan = nullptr;
+}
+
+// Gives back a plan that holds slices (the next call builds one without them).
+bool chol_adjoint_release(chol_handle* h) {
+  const SiPlan* pl = (const SiPlan*)h->dev->si_plan;
+  if (!pl || !pl->sg || pl->pinned) return false;
+  chol_adjoint_free(h);
+  return true;
 }
 
 extern "C" int chol_selected_inverse(chol_handle* h, double* zvals, void* stream) {

@@ -11,10 +11,13 @@
 // Kernel classes
 //   k_scatter        A's values into the zeroed panels (HBM-bound gather/scatter)
 //   k_small          one CTA per small supernode: POTRF + TRSM + SYRK in shared memory
+//   k_small_warp     one warp per tiny supernode, in levels of thousands
 //   k_potrf          blocked path, diagonal block of one column step
-//   k_trsm           blocked path, row tiles below the diagonal block
-//   k_gemm_trailing  blocked path, trailing update of the panel (FP64 DFMA tiles)
-//   k_syrk           blocked path, U_J tiles (lower triangle only)
+//   k_link           blocked path, the rows and the update of the next diagonal block
+//   k_trsm           blocked path, the other rows below the diagonal block
+//   k_sg_trailing, k_sg_split_rows, k_sg_syrk (split_gemm.cu)   trailing updates and
+//                    U_J on the tensor cores
+//   k_gemm_trailing, k_syrk   the same on the FP64 pipe: handles without slices
 //   k_assemble       relind scatter-add, pull-ordered: each task owns target
 //                    columns and applies its contributors in a fixed order, so
 //                    no atomics and a bitwise-deterministic result
@@ -473,7 +476,7 @@ k_trsm(const SnodeDev* __restrict__ sn, const TileTask* __restrict__ tasks, int 
 // supernode with a next diagonal block: the TRSM of its (at most) 64 rows, eight
 // a CTA, then its update C -= X X^T (lower triangle), every CTA gathering the 64
 // solved rows through distributed shared memory, a thread per entry. One launch
-// of about 14 us in place of two (17 + 15): on 64 rows the FP64 pipes of eight
+// of about 19 us in place of two (17 + 15): on 64 rows the FP64 pipes of eight
 // SMs (4 us each part) beat the latency of a tensor-core tile.
 constexpr int kLinkCtas = 8;
 constexpr int kLinkThreads = 256;
@@ -1125,6 +1128,10 @@ int chol_dalloc(chol_handle* h, void** p, size_t bytes) {
     chol_sg_release(h);
     e = cudaMalloc(p, bytes);
   }
+  if (e == cudaErrorMemoryAllocation && chol_adjoint_release(h)) {
+    cudaGetLastError();
+    e = cudaMalloc(p, bytes);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
@@ -1337,7 +1344,9 @@ void launch_potrf(chol_handle* h, const StepRange& s, int k0, cudaStream_t st) {
 // columns). Every tile receives its updates in step order. The slices of step k
 // are last read by its side tiles, which are done when step k + 3 writes the
 // same buffer (its TRSM follows near(k + 1), which waited for side(k)).
-// With the whole step on the chain a step of the 37x29x23 grid took 77 us.
+// A step of the 37x29x23 grid takes 65 us; with the whole step on the chain 77.
+// (Several trailing tiles a CTA, a persistent grid, and 128 x 32 tiles with two
+// CTAs an SM were measured at 3D 64^3: 49 to 50.5 ms against 50.)
 int enqueue_steps_sg(chol_handle* h, const LevelPlan& P, cudaStream_t st) {
   DeviceState* D = h->dev;
   const cudaStream_t ms = D->mstream, ls = D->lstream;

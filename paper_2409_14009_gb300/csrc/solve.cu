@@ -9,15 +9,18 @@
 //
 // Forward, levels leaves -> root, for every supernode J of the level:
 //   - the diagonal triangle, as 64-row blocks in one cooperative launch per
-//     level (k_sv_tri): a block accumulates the products with the blocks
-//     already solved as their flags are published, then substitutes.
-//   - one panel product w_J = L_RJ y_J for the off-diagonal rows (k_sv_gemv).
+//     level (k_sv_tri64, k_sv_tri32): a block accumulates the products with the
+//     blocks already solved as they are published, then multiplies by its inverse.
+//   - one panel product w_J = L_RJ y_J for the off-diagonal rows (k_sv_gemv; with
+//     many right-hand sides in binary64 on the tensor cores, solve_split.cu).
 //   - w_J is scatter-subtracted into the ancestors' rows of y through the
 //     factor's pull-ordered relind task lists (k_sv_fasm).
-//   Supernodes with s <= 32 and len <= 256 take one warp each instead.
+//   Supernodes with s <= 32 and len <= 256 take one warp each instead, or 8 or 16
+//   lanes where there are thousands of them.
 // Backward, levels root -> leaves:
-//   - y_J -= L_RJ^T x_R, a gather of the already final ancestor rows (k_sv_bpanel).
-//   - the transposed diagonal triangle, blocks last to first (k_sv_tri).
+//   - y_J -= L_RJ^T x_R, a gather of the already final ancestor rows (k_sv_bpanel
+//     or solve_split.cu).
+//   - the transposed diagonal triangle, blocks last to first.
 // Every output entry is written by exactly one thread per launch and every
 // reduction runs in a fixed order, so the solve is deterministic.
 #include <mutex>
@@ -1738,6 +1741,7 @@ int chol_solve_status(chol_handle* h) {
   if (e[0] | e[1]) {
     CHOL_CUDA_TRY(cudaMemset(D->sv_err, 0, 2 * sizeof(int32_t)));
     if (D->vs_cnt) CHOL_CUDA_TRY(cudaMemset(D->vs_cnt, 0, sizeof(int32_t) * (size_t)h->vs_slots));
+    CHOL_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));
     return CHOL_ETIMEOUT;
   }
   return CHOL_OK;

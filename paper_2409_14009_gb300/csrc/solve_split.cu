@@ -239,7 +239,9 @@ int chol_vs_ensure(chol_handle* h, cudaStream_t st) {
     up(D->vs_tasks, h->vs_tasks.data(), sizeof(SplitTask) * h->vs_tasks.size());
     up(D->vs_tiles, h->vs_tiles.data(), sizeof(SolveTile) * h->vs_tiles.size());
   }
+  // the copies and the memset run on the legacy stream, which non-blocking streams do not wait for
   ok = ok && (h->vs_slots == 0 || cudaMemset(D->vs_cnt, 0, h->vs_slots * 4) == cudaSuccess) &&
+       cudaStreamSynchronize(cudaStreamLegacy) == cudaSuccess &&
        cudaFuncSetAttribute(k_vs_tile<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes) == cudaSuccess &&
        cudaFuncSetAttribute(k_vs_tile<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes) == cudaSuccess;
   if (!ok) {

@@ -121,7 +121,7 @@ __device__ __forceinline__ int row_pos(const int32_t* __restrict__ rk, int len, 
   return lo;
 }
 
-// U_J tiles (lower triangle), K = all of J's columns in chunks of 128 whose
+// U_J tiles (lower triangle), K = all of J's columns in chunks of 64 whose
 // integer sums stay in registers. RLB: the tile is subtracted from the
 // ancestors' panels pair by pair (see k_syrk_rlb), a thread per row of the tile.
 template <bool RLB>
@@ -254,6 +254,7 @@ int chol_sg_ensure(chol_handle* h) {
   CHOL_CUDA_TRY(up(D->sg_split, h->split_tasks));
   CHOL_CUDA_TRY(up(D->sg_syrk, h->sgs_tasks));
   CHOL_CUDA_TRY(up(D->sg_trail, h->sgt_tasks));
+  CHOL_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));   // non-blocking streams do not wait for the copies
   const void* kernels[] = {(const void*)k_sg_trailing, (const void*)k_sg_syrk<false>, (const void*)k_sg_syrk<true>};
   for (const void* k : kernels)
     CHOL_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sg::kSmemBytes));

@@ -3,9 +3,9 @@
 Two leaf supernodes of s columns share one separator of b rows, so that a leaf's
 panel takes trailing updates (s > 64), its update matrix has b rows and K = s,
 and the separator takes trailing updates of its own. Sizes sit at the edges of
-the 128 x 64 tiles, the 32-column blocks and the 128-column chunks.
+the 128 x 64 tiles, the 32-column blocks and the 64-column chunks.
 
-Tolerances: the slices keep every entry of a row to 2^-57 of the row's largest,
+Tolerances: the slices keep every entry of a row to 2^-64 of the row's largest,
 so both this path and the oracle's FMAs are backward stable with a constant of a
 few n u; the matrices have kappa < 100 after diagonal scaling, so entries agree
 to well below the 1e-12 of the other binary64 parity tests.
@@ -202,3 +202,50 @@ def test_solve_products_captured():
     P.chol_destroy(h)
     assert torch.equal(got[1], x)
     assert (got[0] - x).abs().max() <= 6e-11 * x.abs().max()
+
+
+def test_selected_inverse_out_of_room():
+    """A selected inverse that a memory cap refuses is refused again, wherever its
+    allocations stop, and one that fits comes out as without a cap."""
+    import torch
+    P = chol()
+    p = _arrow(130, 190)
+    v = torch.as_tensor(p["values"], device="cuda")
+
+    def attempt(cap):
+        rc, h = P.chol_analyze(p["n"], p["colptr"], p["rowind"], p["perm"], _opts(cap=cap))
+        assert rc == 0
+        rcs, z = [P.chol_factor(h, v)], torch.empty_like(v)
+        if rcs[0] == 0:
+            rcs = [P.chol_selected_inverse(h, z) for _ in range(2)]
+            assert P.chol_check_waits(h) == 0
+        P.chol_destroy(h)
+        return rcs, z
+    want = attempt(1 << 40)
+    assert want[0] == [0, 0]
+    seen = set()
+    for cap in np.linspace(1 << 18, 1 << 26, 256).astype(np.int64):
+        rcs, z = attempt(int(cap))
+        assert len(set(rcs)) == 1 and rcs[0] in (0, -1001)
+        seen.add((len(rcs), rcs[0]))
+        if rcs == [0, 0]:
+            assert torch.equal(z, want[1])
+    assert seen == {(1, -1001), (2, -1001), (2, 0)}
+
+
+def test_factor_from_a_graph():
+    """Blocked levels captured (the chain, bulk, side and small streams) and replayed."""
+    p = _arrow(257, 130)
+    o = _opts()
+    o.use_graph = 1
+    o.small_max_cols, o.small_max_panel = 64, 4096
+    a, c = run(p, None, o), run(p, None, _opts())
+    assert np.allclose(a["L"][2], c["L"][2], rtol=0, atol=1e-12 * np.abs(c["L"][2]).max())
+    import torch
+    P = chol()
+    rc, h = P.chol_analyze(p["n"], p["colptr"], p["rowind"], p["perm"], o)
+    v = torch.as_tensor(p["values"], device="cuda")
+    for _ in range(3):
+        assert P.chol_factor(h, v) == 0
+    assert np.array_equal(P.chol_get_factor(h)[2], a["L"][2])
+    P.chol_destroy(h)
