@@ -77,7 +77,9 @@ typedef struct chol_options {
   int32_t block_cols;      /* column block of the blocked large-supernode path  */
                            /* (POTRF/TRSM/update step); default 64               */
   int64_t device_mem_cap;  /* refuse device allocations above this many bytes;  */
-                           /* 0 = no cap (for testing the ENOMEM path)          */
+                           /* 0 = no cap (for testing the ENOMEM path). With a  */
+                           /* cap, binary64 products stay on the FP64 pipe,      */
+                           /* which needs no slice workspaces                    */
   double merge_growth;     /* relaxed supernode merging budget (Sec. IV setup): */
                            /* merge adjacent (J, parent(J)) pairs, fewest added */
                            /* explicit zeros first (ties: smaller J), while the */
@@ -177,10 +179,16 @@ int chol_analyze(int32_t n, const int64_t* colptr, const int32_t* rowind,
  * U_J into the ancestors (pull-ordered, atomic-free, deterministic). It ends
  * by inverting the 64x64 diagonal blocks the triangle solves multiply by
  * (binary64: the inverse; mixed modes: also the last-dependency products).
+ * Binary64 products run on the tensor cores as exact bf16 slices (an entry's
+ * error is below that of binary64 FMAs); their workspaces belong to the handle,
+ * are created by the first call, given back when a later allocation of the
+ * handle finds no room, and left out on a device without room or under
+ * device_mem_cap, where the FP64 pipe does the products.
  *   values  device, colptr[n] doubles in the order of the analyzed rowind
  *   stream  cudaStream_t as void*
  * Returns CHOL_OK, +j (not positive definite at column j of P A P^T), or an
- * error. Synchronizes `stream` once at the end to read the status word.
+ * error (CHOL_ETIMEOUT: a bounded device wait of a product ran out).
+ * Synchronizes `stream` once at the end to read the status word.
  */
 int chol_factor(chol_handle* h, const double* values, void* stream);
 
@@ -195,7 +203,10 @@ int chol_factor(chol_handle* h, const double* values, void* stream);
  * blocks of a triangle wait (bounded, chol_options.wait_polls) for the blocks
  * they depend on; a wait that runs out leaves X invalid and is reported as
  * CHOL_ETIMEOUT by chol_check_waits, or by the next chol_factor or
- * chol_solve_refine on the handle. Calls on one handle must not overlap on the
+ * chol_solve_refine on the handle. In binary64 with 9 and more right-hand sides
+ * the panel products of large levels run on the tensor cores (bounded waits
+ * too); the first such call creates their workspaces, and one that is captured
+ * before that, or finds no room, keeps the FP64 pipe's kernels. Calls on one handle must not overlap on the
  * GPU (they share workspaces). CHOL_ESTATE if the current device is not the
  * one the handle was factored on.
  */
@@ -205,8 +216,8 @@ int chol_solve(chol_handle* h, double* b, int32_t nrhs, void* stream);
  * Report the bounded waits of the solves enqueued so far on this handle
  * (chol_solve, chol_solve_batch, chol_solve_noalloc, and the solves inside
  * chol_solve_refine). Synchronizes `stream` (the stream the solves ran on),
- * then returns CHOL_ETIMEOUT if any wait of a diagonal-triangle block gave up
- * since the last check (the solutions of those calls are invalid) and clears
+ * then returns CHOL_ETIMEOUT if any wait of a diagonal-triangle block or of a
+ * tensor-core product gave up since the last check (the solutions of those calls are invalid) and clears
  * the record; CHOL_OK otherwise. CHOL_ESTATE without a factorization on the
  * current device. The paper's solves are host-driven library calls with no
  * device-side waits; this check belongs to the cooperative triangle kernel.
@@ -218,7 +229,8 @@ int chol_check_waits(chol_handle* h, void* stream);
  * exists for callers that cannot call cudaMalloc once they are set up (a
  * process whose memory pool already owns the GPU, or a latency-bound loop in
  * which an allocation could stall on device-wide synchronization). Arguments,
- * layout and result are those of chol_solve; the handle must hold a factor.
+ * layout and result (to rounding: no tensor-core products here) are those of
+ * chol_solve; the handle must hold a factor.
  * Its workspaces live in one fixed device array of 2^21 doubles (16 MiB) that
  * every GPU loading the library keeps until the process exits; a problem needs
  * n + (largest per-level sum of off-diagonal supernode rows) doubles per
@@ -290,7 +302,8 @@ int chol_solve_refine(chol_handle* h, const double* b, double* x, int32_t nrhs, 
  * Uhat = L_RJ T, Z_RJ = -Z_RR Uhat with Z_RR gathered from the ancestors
  * through the relative positions, Z_JJ = T^T T - Uhat^T Z_RJ). The first call
  * builds the level plan and its workspaces (largest level's sum of s^2,
- * b s and 64 s doubles). CHOL_PREC_FP64 handles only (else CHOL_ENOTSUP).
+ * b s and s^2 / 2 doubles, and the slices of its largest group of products, which
+ * run on the tensor cores where chol_factor's do). CHOL_PREC_FP64 handles only (else CHOL_ENOTSUP).
  * Asynchronous.
  */
 int chol_selected_inverse(chol_handle* h, double* zvals, void* stream);
@@ -514,8 +527,8 @@ int chol_get_stats(chol_handle* h, chol_kernel_stat* out, int32_t reset);
 
 /*
  * Measured binary64 throughput of the current GPU (the paper has no
- * counterpart; a measurement aid for the roofline of the binary64 factor,
- * whose dense updates run on the FP64 FMA pipe). kind 0: DFMA, independent
+ * counterpart; a measurement aid for the roofline of the binary64 kernels that
+ * run on the FP64 FMA pipe). kind 0: DFMA, independent
  * fused multiply-add chains on every SM; kind 1: DMMA, mma.sync m8n8k4 f64.
  * Tries 8 and 16 independent chains per thread and 2, 4 and 6 CTAs of 256
  * threads per SM, each shape with reps + 1 timed launches of a few
