@@ -855,7 +855,7 @@ k_sv_small_fwd(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list
   T lrow[G];   // L(g, k) (binary64: / L(g, g)), k < g < s, else 0
 #pragma unroll
   for (int k = 0; k < G; ++k) lrow[k] = (k < g && g < d.s) ? lval<T, RM>(P, d, g, k) * (kScaled ? rd : T(1)) : T(0);
-  for (int r = 0; r < nrhs; ++r) {
+  for (int r = blockIdx.y; r < nrhs; r += gridDim.y) {
     T y = g < d.s ? Y[d.f + g + (int64_t)r * n] * (kScaled ? rd : T(1)) : T(0);
     T ya[G];   // y_J, every lane
 #pragma unroll
@@ -898,7 +898,7 @@ k_sv_small_bwd(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list
   T lcol[G];   // L(k, g) (binary64: / L(g, g)), g < k < s, else 0
 #pragma unroll
   for (int k = 0; k < G; ++k) lcol[k] = (k > g && k < d.s) ? lval<T, RM>(P, d, k, g) * (kScaled ? rd : T(1)) : T(0);
-  for (int r = 0; r < nrhs; ++r) {
+  for (int r = blockIdx.y; r < nrhs; r += gridDim.y) {
     T acc[G];
 #pragma unroll
     for (int k = 0; k < G; ++k) acc[k] = T(0);
@@ -950,7 +950,7 @@ k_sv_wide_fwd(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list,
 #pragma unroll
   for (int k = 0; k < S; ++k)
     lrow[k] = (k < lane && lane < d.s) ? P[lane + (int64_t)k * d.ld] * rd : 0.0;
-  for (int r = 0; r < nrhs; ++r) {
+  for (int r = blockIdx.y; r < nrhs; r += gridDim.y) {
     double y = lane < d.s ? Y[d.f + lane + (int64_t)r * n] * rd : 0.0;
 #pragma unroll
     for (int k = 0; k < S; ++k) {
@@ -1008,7 +1008,7 @@ k_sv_wide_bwd(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list,
 #pragma unroll
   for (int k = 0; k < S; ++k)
     lcol[k] = (k > lane && k < d.s) ? P[k + (int64_t)lane * d.ld] * rd : 0.0;
-  for (int r = 0; r < nrhs; ++r) {
+  for (int r = blockIdx.y; r < nrhs; r += gridDim.y) {
     // four partial sums (u mod 4), added pairwise: a chain of b/4 dependent FMAs;
     // 16 rows' loads in flight per round
     double t4[4] = {0.0, 0.0, 0.0, 0.0};
@@ -1487,6 +1487,16 @@ int small_groups(const LevelPlan& P, F&& f) {
   return (n8 > 0) + (n16 > 0) + (n32 > 0);
 }
 
+// Grid of a small-supernode launch of `ctas` CTAs (8 warps each): the right-hand
+// sides, independent of one another, are dealt over blockIdx.y while that leaves
+// at most 4 CTAs an SM. One warp after another on them was a chain of nrhs times
+// substitution and gather: 16 of them, level 0 of 3D 48^3, 430 us backward. Solve
+// 7.9 -> 6.1 ms; binary32 refinement with 8 (3D 51x49x50) 18.4 -> 16.1. 8 CTAs an SM
+// measured the same.
+dim3 small_grid(const DeviceState* D, int ctas, int nr) {
+  return dim3(ctas, std::max(1, std::min(nr, 4 * D->sms / std::max(ctas, 1))));
+}
+
 // Levels whose panel products go to the tensor cores (solve_split.cu): at least 9
 // right-hand sides, and 8e6 products of panel entry and right-hand side. The
 // splitting costs the same for any number of right-hand sides: 3D 48^3, a solve
@@ -1513,9 +1523,9 @@ int solve_levels(chol_handle* h, const T* L, T* Y, T* W, T* part, int nr, cudaSt
       const int nk = small_groups<T>(P, [&](auto G, auto wide, int b, int cnt) {
         constexpr int kG = decltype(G)::value;
         if constexpr (decltype(wide)::value && !RM)
-          k_sv_wide_fwd<kG><<<(cnt + 7) / 8, kT, 0, st>>>(D->sn, D->ssmall + b, cnt, L, D->rdiag, Y, n, W, nr);
+          k_sv_wide_fwd<kG><<<small_grid(D, (cnt + 7) / 8, nr), kT, 0, st>>>(D->sn, D->ssmall + b, cnt, L, D->rdiag, Y, n, W, nr);
         else
-          k_sv_small_fwd<T, RM, kG><<<(cnt * kG + kT - 1) / kT, kT, 0, st>>>(D->sn, D->ssmall + b, cnt, L, D->rdiag, Y, n,
+          k_sv_small_fwd<T, RM, kG><<<small_grid(D, (cnt * kG + kT - 1) / kT, nr), kT, 0, st>>>(D->sn, D->ssmall + b, cnt, L, D->rdiag, Y, n,
                                                                             W, nr);
       });
       if (ks) ks->launches(nk);
@@ -1588,9 +1598,9 @@ int solve_levels(chol_handle* h, const T* L, T* Y, T* W, T* part, int nr, cudaSt
       const int nk = small_groups<T>(P, [&](auto G, auto wide, int b, int cnt) {
         constexpr int kG = decltype(G)::value;
         if constexpr (decltype(wide)::value && !RM)
-          k_sv_wide_bwd<kG><<<(cnt + 7) / 8, kT, 0, st>>>(D->sn, D->ssmall + b, cnt, D->rows, L, D->rdiag, Y, n, nr);
+          k_sv_wide_bwd<kG><<<small_grid(D, (cnt + 7) / 8, nr), kT, 0, st>>>(D->sn, D->ssmall + b, cnt, D->rows, L, D->rdiag, Y, n, nr);
         else
-          k_sv_small_bwd<T, RM, kG><<<(cnt * kG + kT - 1) / kT, kT, 0, st>>>(D->sn, D->ssmall + b, cnt, D->rows, L,
+          k_sv_small_bwd<T, RM, kG><<<small_grid(D, (cnt * kG + kT - 1) / kT, nr), kT, 0, st>>>(D->sn, D->ssmall + b, cnt, D->rows, L,
                                                                             D->rdiag, Y, n, nr);
       });
       if (ks) ks->launches(nk);
