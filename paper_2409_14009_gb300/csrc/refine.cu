@@ -24,39 +24,61 @@ inline unsigned grid1d(int64_t n, int threads) {
   return (unsigned)(g > 0 ? g : 1);
 }
 
+// *out = max(*out, the CTA's values): one atomic a CTA (one a warp or a row on the
+// same word kept the others waiting).
+__device__ __forceinline__ void block_max(unsigned long long v, unsigned long long* out) {
+  __shared__ unsigned long long top[kT / 32];
+  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  __syncthreads();   // top is free
+  if ((threadIdx.x & 31) == 0) top[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kT / 32; ++w) v = max(v, top[w]);
+    atomicMax(out, v);
+  }
+}
+
 // per right-hand side: out[r] = max_i |b_ir| (ordering of non-negative doubles)
 __global__ void k_maxabs_cols(const double* __restrict__ b, int n, int nr, unsigned long long* __restrict__ out) {
-  for (int r = 0; r < nr; ++r) {
+  for (int r = blockIdx.y; r < nr; r += gridDim.y) {
     double m = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
       m = fmax(m, fabs(b[i + (int64_t)r * n]));
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(out + r, (unsigned long long)__double_as_longlong(m));
+    block_max((unsigned long long)__double_as_longlong(m), out + r);
   }
 }
 
 // ---- binary64 vector kernels for refinement -----------------------------------
 
-// R = B - A X (full CSR, warp per row, fixed-order lane reduction); also
-// rmax[r] = max_i |R_ir| via the ordering of non-negative doubles.
+// R = B - A X (full CSR, G = 8 or 32 lanes per row, fixed-order lane reduction);
+// also rmax[r] = max_i |R_ir| via the ordering of non-negative doubles, reduced
+// per CTA. A warp per row took eight FP64 instructions of 64 cycles for the 81
+// entries of an elasticity row where 8 lanes take 3.5 a row, and an atomic per row
+// on one word: 411 us for 331,776 rows, now 94.
+template <int G>
 __global__ void __launch_bounds__(kT)
 k_residual(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci, const double* __restrict__ av,
            const double* __restrict__ X, const double* __restrict__ B, int n, int nrhs, double* __restrict__ R,
            unsigned long long* __restrict__ rmax) {
-  const int lane = threadIdx.x & 31;
-  const int warps = (gridDim.x * blockDim.x) >> 5;
-  for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += warps) {
-    for (int r = 0; r < nrhs; ++r) {
-      const double* x = X + (int64_t)r * n;
+  const int lane = threadIdx.x & (G - 1);
+  const int groups = gridDim.x * (kT / G);
+  const int rounds = (n + groups - 1) / groups;   // uniform: the shuffles take whole warps
+  for (int r = blockIdx.y; r < nrhs; r += gridDim.y) {
+    const double* x = X + (int64_t)r * n;
+    unsigned long long m = 0;
+    for (int q = 0; q < rounds; ++q) {
+      const int64_t i = (int64_t)q * groups + (blockIdx.x * kT + threadIdx.x) / G;
       double s = 0.0;
-      for (int64_t t = rp[i] + lane; t < rp[i + 1]; t += 32) s = fma(av[t], x[ci[t]], s);
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) {
+      if (i < n)
+        for (int64_t t = rp[i] + lane; t < rp[i + 1]; t += G) s = fma(av[t], x[ci[t]], s);
+      for (int o = G / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0 && i < n) {
         const double v = B[i + (int64_t)r * n] - s;
         R[i + (int64_t)r * n] = v;
-        atomicMax(rmax + r, (unsigned long long)__double_as_longlong(fabs(v)));
+        m = max(m, (unsigned long long)__double_as_longlong(fabs(v)));
       }
     }
+    block_max(m, rmax + r);
   }
 }
 
@@ -67,7 +89,7 @@ __global__ void __launch_bounds__(kT)
 k_residual_rows(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci, const double* __restrict__ av,
                 const double* __restrict__ X, const double* __restrict__ B, int n, int nrhs,
                 double* __restrict__ R, unsigned long long* __restrict__ rmax) {
-  for (int r = 0; r < nrhs; ++r) {
+  for (int r = blockIdx.y; r < nrhs; r += gridDim.y) {
     const double* x = X + (int64_t)r * n;
     double m = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -77,8 +99,7 @@ k_residual_rows(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci, 
       R[i + (int64_t)r * n] = v;
       m = fmax(m, fabs(v));
     }
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(rmax + r, (unsigned long long)__double_as_longlong(m));
+    block_max((unsigned long long)__double_as_longlong(m), rmax + r);
   }
 }
 
@@ -232,11 +253,17 @@ extern "C" int chol_solve_refine(chol_handle* h, const double* b, double* x, int
   const unsigned gsp = grid1d((int64_t)n * 32, kT);
   // a warp per row wastes most lanes on rows of a few entries
   const bool few_per_row = h->csr_ptr[n] <= 16 * (int64_t)n;
+  const bool many_per_row = h->csr_ptr[n] > 256 * (int64_t)n;
+  const auto k_res = many_per_row ? k_residual<32> : k_residual<8>;
+  const unsigned gres = grid1d((int64_t)n * (many_per_row ? 32 : 8), kT);
 
   // ||A||_inf and ||b||_inf
   CHOL_CUDA_TRY(cudaMemsetAsync(red, 0, sizeof(double) * (3 * nrhs + 1), st));
   k_anorm<<<grid1d(n, 256), 256, 0, st>>>(D->csr_ptr, D->csr_val, n, anorm);
-  k_maxabs_cols<<<grid1d(n, 256), 256, 0, st>>>(b, n, nrhs, bmax);
+  // the right-hand sides side by side (they took turns: 3D 51x49x50 with 8, 40 us a
+  // residual; with an atomic a warp 26 us a maximum)
+  const unsigned ry = (unsigned)std::min(nrhs, 64);
+  k_maxabs_cols<<<dim3(grid1d(n, 256), ry), 256, 0, st>>>(b, n, nrhs, bmax);
   // x0 = solve(b)
   CHOL_CUDA_TRY(cudaMemcpyAsync(x, b, nb, cudaMemcpyDeviceToDevice, st));
   if ((rc = correction_solve(h, x, nrhs, st))) return rc;
@@ -247,10 +274,10 @@ extern "C" int chol_solve_refine(chol_handle* h, const double* b, double* x, int
     // R = b - A x; eta = ||R|| / (||A|| ||x|| + ||b||)
     CHOL_CUDA_TRY(cudaMemsetAsync(rmax, 0, sizeof(double) * 2 * nrhs, st));
     if (few_per_row)
-      k_residual_rows<<<grid1d(n, kT), kT, 0, st>>>(D->csr_ptr, D->csr_col, D->csr_val, x, b, n, nrhs, D->R, rmax);
+      k_residual_rows<<<dim3(grid1d(n, kT), ry), kT, 0, st>>>(D->csr_ptr, D->csr_col, D->csr_val, x, b, n, nrhs, D->R, rmax);
     else
-      k_residual<<<gsp, kT, 0, st>>>(D->csr_ptr, D->csr_col, D->csr_val, x, b, n, nrhs, D->R, rmax);
-    k_maxabs_cols<<<grid1d(n, 256), 256, 0, st>>>(x, n, nrhs, xmax);
+      k_res<<<dim3(gres, ry), kT, 0, st>>>(D->csr_ptr, D->csr_col, D->csr_val, x, b, n, nrhs, D->R, rmax);
+    k_maxabs_cols<<<dim3(grid1d(n, 256), ry), 256, 0, st>>>(x, n, nrhs, xmax);
     CHOL_CUDA_TRY(cudaMemcpyAsync(D->red_host, red, sizeof(double) * (3 * nrhs + 1), cudaMemcpyDeviceToHost, st));
     CHOL_CUDA_TRY(cudaStreamSynchronize(st));
     const unsigned long long* hb = (const unsigned long long*)D->red_host;

@@ -82,12 +82,19 @@ __global__ void k_sv_permute_out(const T* __restrict__ Y, const int32_t* __restr
 
 // per right-hand side: out[r] = max_i |b_ir| (ordering of non-negative doubles)
 __global__ void k_sv_maxabs(const double* __restrict__ b, int n, int nr, unsigned long long* __restrict__ out) {
-  for (int r = 0; r < nr; ++r) {
+  __shared__ double top[kT / 32];
+  for (int r = blockIdx.y; r < nr; r += gridDim.y) {
     double m = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
       m = fmax(m, fabs(b[i + (int64_t)r * n]));
     for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(out + r, (unsigned long long)__double_as_longlong(m));
+    __syncthreads();   // top is free
+    if ((threadIdx.x & 31) == 0) top[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {   // one atomic a CTA
+      for (int w = 1; w < kT / 32; ++w) m = fmax(m, top[w]);
+      atomicMax(out + r, (unsigned long long)__double_as_longlong(m));
+    }
   }
 }
 
@@ -802,18 +809,27 @@ k_sv_bpart(const SnodeDev* __restrict__ sn, const TileTask* __restrict__ tasks, 
 template <class T>
 __global__ void __launch_bounds__(kT)
 k_sv_bred(const SnodeDev* __restrict__ sn, const TileTask* __restrict__ tasks, const T* __restrict__ part,
-          int64_t pstride, T* __restrict__ Y, int n, int nrhs) {
+          int64_t pstride, T* __restrict__ Y, int n) {
   const TileTask t = tasks[blockIdx.x];
   const SnodeDev d = sn[t.J];
   const int c = t.c0 + threadIdx.x;
   if (c >= d.s) return;
   const int nchunks = (d.len - d.s + kSub - 1) / kSub;
-  for (int r = 0; r < nrhs; ++r) {
-    const T* p = part + r * pstride + d.ppre + c;
-    T acc = T(0);
-    for (int ch = 0; ch < nchunks; ++ch) acc += p[(int64_t)ch * d.s];
-    Y[d.f + c + (int64_t)r * n] -= acc;
+  // a right-hand side per blockIdx.y, 16 partials in flight, added in chunk order
+  // (8 right-hand sides one after another took 36 us near the root)
+  const int r = blockIdx.y;
+  const T* p = part + r * pstride + d.ppre + c;
+  T* y = Y + d.f + c + (int64_t)r * n;
+  const T y0 = *y;
+  T acc = T(0);
+  for (int c0 = 0; c0 < nchunks; c0 += 16) {
+    T v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = p[(int64_t)min(c0 + i, nchunks - 1) * d.s];   // unconditional: all in flight
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc = c0 + i < nchunks ? acc + v[i] : acc;
   }
+  *y = y0 - acc;
 }
 
 // Small supernodes (s <= 32, len <= 256): a group of G = 8, 16 or 32 lanes each
@@ -1575,7 +1591,7 @@ int solve_levels(chol_handle* h, const T* L, T* Y, T* W, T* part, int nr, cudaSt
           k_sv_bpart<T, decltype(c)::value><<<P.bpart_n, kT, 0, st>>>(D->sn, D->bpart + P.bpart_b, D->rows, L, Y, n,
                                                                       part, h->p_max, nr);
         });
-        k_sv_bred<T><<<P.bred_n, kT, 0, st>>>(D->sn, D->bred + P.bred_b, part, h->p_max, Y, n, nr);
+        k_sv_bred<T><<<dim3(P.bred_n, nr), kT, 0, st>>>(D->sn, D->bred + P.bred_b, part, h->p_max, Y, n);
         delete ks;
       }
     } else if (products_on_tc(P)) {
@@ -1705,7 +1721,7 @@ int chol_solve_mixed(chol_handle* h, double* b, int32_t nrhs, cudaStream_t st) {
     CHOL_CUDA_TRY(cudaMemsetAsync(sc, 0, sizeof(double) * kSolveChunk, st));
     {
       KScope ks(h, CHOL_K_PERMUTE, st, 0.0, 12.0 * n * nr);
-      k_sv_maxabs<<<grid1d(n, 256), 256, 0, st>>>(B, n, nr, sc);
+      k_sv_maxabs<<<dim3(grid1d(n, kT), nr), kT, 0, st>>>(B, n, nr, sc);
       k_sv_permute_in<float><<<grid1d((int64_t)n * nr, 256), 256, 0, st>>>(B, D->perm, D->mx_d, sc, n, nr, D->Y32);
     }
     if ((rc = solve_levels<float, true>(h, (const float*)D->L, D->Y32, D->W32, D->P32, nr, st, true))) return rc;
