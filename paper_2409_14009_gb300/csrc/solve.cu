@@ -1285,12 +1285,24 @@ k_sv_tri32(const SnodeDev* __restrict__ sn, const TriItem* __restrict__ items, i
         const int j = TRANS ? item.nb - 1 - q : q;
         const int j0 = j * kSub, jb = min(kSub, d.s - j0);
         const int row = i0 + r;
+        const bool in = q < ndep && r < kb;
+        if constexpr (TRANS) {
 #pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-          const int k = ka + kk;
-          lv[t][kk] = (q < ndep && r < kb && k < jb)
-                          ? (TRANS ? P[(int64_t)(j0 + k) * d.ld + row] : P[(int64_t)row * d.ld + j0 + k])
-                          : 0.f;
+          for (int kk = 0; kk < 16; ++kk)
+            lv[t][kk] = in && ka + kk < jb ? P[(int64_t)(j0 + ka + kk) * d.ld + row] : 0.f;
+        } else {
+          // lanes along the rows, so 16-byte loads (rows start 32-byte aligned, and
+          // ld is a multiple of 8): single words were 32 lines a load each (elasticity
+          // 48^3, one right-hand side: 72 us a launch, now 50)
+#pragma unroll
+          for (int kk = 0; kk < 16; kk += 4) {
+            float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (in && ka + kk < jb) w = *reinterpret_cast<const float4*>(P + (int64_t)row * d.ld + j0 + ka + kk);
+            lv[t][kk] = w.x;   // ka + kk < jb or zero
+            lv[t][kk + 1] = ka + kk + 1 < jb ? w.y : 0.f;
+            lv[t][kk + 2] = ka + kk + 2 < jb ? w.z : 0.f;
+            lv[t][kk + 3] = ka + kk + 3 < jb ? w.w : 0.f;
+          }
         }
       }
       __syncthreads();   // the previous round is done with ys
