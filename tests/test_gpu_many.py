@@ -84,3 +84,31 @@ def test_wide_one_cta_beside_blocked(s, mode):
     o.small_max_cols, o.small_max_panel, o.small_max_rows, o.update_mode = 128, 20000, 512, mode
     p = dict(n=n, colptr=cp, rowind=ri, values=vx, perm=np.arange(n, dtype=np.int32))
     check_parity(p, rs.uniform(-1, 1, (n, 2)), o)
+
+
+# rows of about 30, 240 and 1,200 entries (8 lanes; a warp a row); 66 right-hand
+# sides pass the 64 that run side by side; 1,100 rows are 18 chunks of partials
+@pytest.mark.parametrize("s,b,nrhs", [(15, 12, 1), (15, 11, 66), (120, 90, 3), (70, 1100, 3)])
+def test_refinement_of_long_rows(s, b, nrhs):
+    """Refined to a backward error of 1e-12 with kappa < 100 after scaling: x within 1e-9."""
+    import torch
+    P = chol()
+    rs = np.random.RandomState(s + b)
+    n = 2 * s + b
+    A = np.tril(rs.uniform(-1.0, 1.0, (n, n)), -1)
+    A[s:2 * s, :s] = 0.0
+    A = A + A.T
+    A[np.diag_indices(n)] = 1.05 * np.abs(A).sum(axis=1)
+    cp, ri, vx = lower_csc_from_dense(A)
+    o = P.chol_default_options()
+    o.precision = P.CHOL_PREC_FP32
+    o.small_max_cols = o.small_max_panel = 1
+    rc, h = P.chol_analyze(n, cp, ri, np.arange(n, dtype=np.int32), o)
+    assert rc == 0 and P.chol_factor(h, to_dev(vx)) == 0
+    x = rs.uniform(-1, 1, (n, nrhs))
+    X = colmajor(np.zeros((n, nrhs)))
+    rc, iters, berr = P.chol_solve_refine(h, colmajor(A @ x), X, nrhs, 1e-12, 50)
+    torch.cuda.synchronize()
+    P.chol_destroy(h)
+    assert rc == 0 and np.max(berr) <= 1e-12
+    assert np.max(np.abs(X.cpu().numpy().reshape((n, nrhs), order="F") - x)) <= 1e-9
