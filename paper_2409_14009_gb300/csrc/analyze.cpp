@@ -627,13 +627,16 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
           st.gemm_flops += 2.0 * kb * (w * hgt - w * (w - 1.0) / 2.0);
         }
       }
-      // the next diagonal block's rows of the supernodes that have one, then the others
+      // tensor-core updates: the next diagonal block's rows of the supernodes that
+      // have one, then the others (a task has no end of its own, so the first pass
+      // must end on a task's last row); otherwise all rows at once
+      static_assert(kTile % (kTrsmRowsHost / 2) == 0, "the next diagonal block is whole tasks");
       for (int pass = 0; pass < 2; ++pass) {
         for (int32_t J : large) {
           const SnodeDev& d = h->snodes[J];
           if (d.s <= k0) continue;
           const int32_t r1 = k0 + std::min(nb, d.s - k0);
-          const int32_t rc = d.s > r1 ? std::min(d.len, r1 + nb) : r1;   // end of the first pass's rows
+          const int32_t rc = split64 && d.s > r1 ? std::min(d.len, r1 + nb) : r1;   // end of the first pass's rows
           for (int32_t r0 = pass ? rc : r1; r0 < (pass ? d.len : rc); r0 += trsm_rows)
             h->trsm_tasks.push_back({J, k0, r0, 0});
         }
