@@ -171,7 +171,7 @@ struct SplitTile {
 // Tiles of the group's products: operand 2 desc is A, 2 desc + 1 is B.
 __global__ void __launch_bounds__(sg::kThreads, 1)
 k_split_gemm(const GenGemm* __restrict__ descs, const SplitOp* __restrict__ ops, const SplitTile* __restrict__ tiles,
-             int ntiles, const unsigned char* __restrict__ slab, const int32_t* __restrict__ exps, int* err) {
+             int ntiles, const unsigned char* __restrict__ slab, const int32_t* __restrict__ exps, sg::Waits waits) {
   extern __shared__ unsigned char sg_smem[];
   __shared__ __align__(8) sg::Shared S;
   const uint32_t base = (tc::smem_u32(sg_smem) + 1023u) & ~1023u;
@@ -188,9 +188,9 @@ k_split_gemm(const GenGemm* __restrict__ descs, const SplitOp* __restrict__ ops,
     return true;
   };
   if (warp == sg::kEpiWarps) {
-    if (lane == 0) sg::copy_loop(S, base, next, err);
+    if (lane == 0) sg::copy_loop(S, base, next, waits);
   } else if (warp == sg::kEpiWarps + 1) {
-    if (lane == 0) sg::mma_loop(S, base, tmem, next, err);
+    if (lane == 0) sg::mma_loop(S, base, tmem, next, waits);
   } else {
     sg::Tile t;
     int chunk = 0;
@@ -204,7 +204,7 @@ k_split_gemm(const GenGemm* __restrict__ descs, const SplitOp* __restrict__ ops,
       long long hi[sg::kCols], lo[sg::kCols];
 #pragma unroll
       for (int c = 0; c < sg::kCols; ++c) hi[c] = lo[c] = 0;
-      for (int k0 = 0; ok && k0 < t.nblk; k0 += sg::kStagesPerChunk) ok = sg::drain(S, tmem, chunk++, hi, lo, err);
+      for (int k0 = 0; ok && k0 < t.nblk; k0 += sg::kStagesPerChunk) ok = sg::drain(S, tmem, chunk++, hi, lo, waits);
       if (!ok) break;
       double* C = g.C + r * g.cr + c0 * g.cc;
 #pragma unroll
@@ -703,7 +703,8 @@ int selinv(chol_handle* h, cudaStream_t st) {
       if (gr.gn == 0) return;
       k_split_op<<<gr.sn, kSplitOpThreads, 0, st>>>(pl->d_ops, pl->d_stasks + gr.sb, pl->d_slab, pl->d_exps, pl->d_kexps);
       k_split_gemm<<<std::min(gr.gn, D->sms), sg::kThreads, sg::kSmemBytes, st>>>(
-          pl->d_descs, pl->d_ops, pl->d_stiles + gr.gb, gr.gn, pl->d_slab, pl->d_exps, D->sg_err);
+          pl->d_descs, pl->d_ops, pl->d_stiles + gr.gb, gr.gn, pl->d_slab, pl->d_exps,
+          sg::Waits{D->sg_err, chol_test_wait(h, kTestWaitSelinv)});
       return;
     }
     if (gr.tn > 0) k_gen_gemm_grouped<<<gr.tn, kGT, 0, st>>>(pl->d_descs, pl->d_tiles + gr.tb, pl->d_part);

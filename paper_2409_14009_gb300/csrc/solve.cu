@@ -1471,7 +1471,7 @@ int launch_tri(chol_handle* h, const LevelPlan& P, const T* L, T* Y, int nr, cud
   const TriItem* items = reinterpret_cast<const TriItem*>(D->tri) + P.tri_b;
   int nitems = P.tri_n, n = h->n;
   long long max_polls = h->opt.wait_polls > 0 ? (long long)h->opt.wait_polls : kTriMaxPolls;
-  int skew = h->opt.test_unreachable_flags ? 1 : 0;
+  int skew = h->opt.test_unreachable_flags & kTestWaitTriangle ? 1 : 0;
   cudaError_t e;
   if constexpr (f32) {
     const float* Dinv = reinterpret_cast<const float*>(D->dinv);

@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1)
 k_vs_tile(const SnodeDev* __restrict__ sn, const SolveSplitDev* __restrict__ vd, const SolveTile* __restrict__ tiles,
           int ntiles, const unsigned char* __restrict__ lslab, const int32_t* __restrict__ lexps,
           const unsigned char* __restrict__ rslab, const int32_t* __restrict__ rexps, double* __restrict__ Y,
-          double* __restrict__ W, int n, int nr, double* __restrict__ part, int* __restrict__ cnt, int* err) {
+          double* __restrict__ W, int n, int nr, double* __restrict__ part, int* __restrict__ cnt, sg::Waits waits) {
   extern __shared__ unsigned char sg_smem[];
   __shared__ __align__(8) sg::Shared S;
   __shared__ int s_last;
@@ -94,9 +94,9 @@ k_vs_tile(const SnodeDev* __restrict__ sn, const SolveSplitDev* __restrict__ vd,
     return true;
   };
   if (warp == Cfg::kEpiWarps) {
-    if (lane == 0) sg::copy_loop<kN>(S, base, next, err);
+    if (lane == 0) sg::copy_loop<kN>(S, base, next, waits);
   } else if (warp == Cfg::kEpiWarps + 1) {
-    if (lane == 0) sg::mma_loop<kN>(S, base, tmem, next, err);
+    if (lane == 0) sg::mma_loop<kN>(S, base, tmem, next, waits);
   } else {
     sg::Tile t;
     int chunk = 0;
@@ -111,7 +111,7 @@ k_vs_tile(const SnodeDev* __restrict__ sn, const SolveSplitDev* __restrict__ vd,
       long long hi[sg::kCols], lo[sg::kCols];
 #pragma unroll
       for (int c = 0; c < sg::kCols; ++c) hi[c] = lo[c] = 0;
-      for (int k0 = 0; ok && k0 < t.nblk; k0 += sg::kStagesPerChunk) ok = sg::drain<kN>(S, tmem, chunk++, hi, lo, err);
+      for (int k0 = 0; ok && k0 < t.nblk; k0 += sg::kStagesPerChunk) ok = sg::drain<kN>(S, tmem, chunk++, hi, lo, waits);
       if (!ok) break;
       double v[sg::kCols];
 #pragma unroll
@@ -260,17 +260,18 @@ void chol_vs_products(chol_handle* h, const LevelPlan& P, bool trans, double* Y,
                                                          D->vs_slab, D->vs_exps, D->vs_exps);
   const SolveTile* tiles = D->vs_tiles + P.vs_tile_b[t];
   const int nt = P.vs_tile_n[t], grid = std::min(nt, D->sms);
+  const sg::Waits waits{D->sg_err, -1};
   if (trans) {
     k_vs_rhs<true><<<dim3(P.vs_n, nr), kRhsThreads, 0, st>>>(D->sn, D->vs_dev, D->vs_list + P.vs_b, D->rows, Y, n, D->vs_exps,
                                                D->vs_rslab, D->vs_rexps);
     k_vs_tile<true><<<grid, Cfg::kThreads, Cfg::kSmemBytes, st>>>(D->sn, D->vs_dev, tiles, nt, D->vs_slab, D->vs_exps,
                                                                   D->vs_rslab, D->vs_rexps, Y, W, n, nr, D->vs_part,
-                                                                  D->vs_cnt, D->sg_err);
+                                                                  D->vs_cnt, waits);
   } else {
     k_vs_rhs<false><<<dim3(P.vs_n, nr), kRhsThreads, 0, st>>>(D->sn, D->vs_dev, D->vs_list + P.vs_b, D->rows, Y, n, D->vs_exps,
                                                 D->vs_rslab, D->vs_rexps);
     k_vs_tile<false><<<grid, Cfg::kThreads, Cfg::kSmemBytes, st>>>(D->sn, D->vs_dev, tiles, nt, D->vs_slab, D->vs_exps,
                                                                    D->vs_rslab, D->vs_rexps, Y, W, n, nr, D->vs_part,
-                                                                   D->vs_cnt, D->sg_err);
+                                                                   D->vs_cnt, waits);
   }
 }

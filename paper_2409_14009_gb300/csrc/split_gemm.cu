@@ -65,7 +65,7 @@ __device__ __forceinline__ uint32_t smem_base(const unsigned char* p) { return (
 __global__ void __launch_bounds__(sg::kThreads, 1)
 k_sg_trailing(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, const TileTask* __restrict__ tasks,
               int ntasks, const unsigned char* __restrict__ slab, const int32_t* __restrict__ exps,
-              double* __restrict__ L, int* err) {
+              double* __restrict__ L, sg::Waits waits) {
   extern __shared__ unsigned char sg_smem[];
   __shared__ __align__(8) sg::Shared S;
   const uint32_t base = smem_base(sg_smem);
@@ -82,9 +82,9 @@ k_sg_trailing(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, 
     return true;
   };
   if (warp == sg::kEpiWarps) {
-    if (lane == 0) sg::copy_loop(S, base, next, err);
+    if (lane == 0) sg::copy_loop(S, base, next, waits);
   } else if (warp == sg::kEpiWarps + 1) {
-    if (lane == 0) sg::mma_loop(S, base, tmem, next, err);
+    if (lane == 0) sg::mma_loop(S, base, tmem, next, waits);
   } else {
     sg::Tile t;
     for (int i = 0; next(i, t); ++i) {
@@ -101,7 +101,7 @@ k_sg_trailing(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, 
       long long hi[sg::kCols], lo[sg::kCols];
 #pragma unroll
       for (int c = 0; c < sg::kCols; ++c) hi[c] = lo[c] = 0;
-      if (!sg::drain(S, tmem, i, hi, lo, err)) break;
+      if (!sg::drain(S, tmem, i, hi, lo, waits)) break;
 #pragma unroll
       for (int c = 0; c < sg::kCols; ++c)
         if (c < n) C[(int64_t)c * d.ld] = cv[c] - sg::combine(hi[c], lo[c], ea, t.b.exps[c0 + c]);
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(sg::kThreads, 1)
 k_sg_syrk(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, const TileTask* __restrict__ tasks,
           int ntasks, const unsigned char* __restrict__ slab, const int32_t* __restrict__ exps,
           double* __restrict__ U, const int4* __restrict__ pairs, const int32_t* __restrict__ pbeg,
-          const int32_t* __restrict__ rows, double* __restrict__ L, int* err) {
+          const int32_t* __restrict__ rows, double* __restrict__ L, sg::Waits waits) {
   extern __shared__ unsigned char sg_smem[];
   __shared__ __align__(8) sg::Shared S;
   const uint32_t base = smem_base(sg_smem);
@@ -146,9 +146,9 @@ k_sg_syrk(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, cons
     return true;
   };
   if (warp == sg::kEpiWarps) {
-    if (lane == 0) sg::copy_loop(S, base, next, err);
+    if (lane == 0) sg::copy_loop(S, base, next, waits);
   } else if (warp == sg::kEpiWarps + 1) {
-    if (lane == 0) sg::mma_loop(S, base, tmem, next, err);
+    if (lane == 0) sg::mma_loop(S, base, tmem, next, waits);
   } else {
     sg::Tile t;
     int chunk = 0;
@@ -164,7 +164,7 @@ k_sg_syrk(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, cons
       long long hi[sg::kCols], lo[sg::kCols];
 #pragma unroll
       for (int c = 0; c < sg::kCols; ++c) hi[c] = lo[c] = 0;
-      for (int k0 = 0; ok && k0 < t.nblk; k0 += sg::kStagesPerChunk) ok = sg::drain(S, tmem, chunk++, hi, lo, err);
+      for (int k0 = 0; ok && k0 < t.nblk; k0 += sg::kStagesPerChunk) ok = sg::drain(S, tmem, chunk++, hi, lo, waits);
       if (!ok) break;
       if constexpr (!RLB) {
         double* C = U + d.uoff + r + (int64_t)c0 * b;
@@ -266,7 +266,8 @@ int chol_sg_ensure(chol_handle* h) {
 void chol_sg_trailing(chol_handle* h, const TileTask* tasks, int n, int grid, int buf, cudaStream_t st) {
   DeviceState* D = h->dev;
   k_sg_trailing<<<std::min(n, grid), sg::kThreads, sg::kSmemBytes, st>>>(D->sn, D->sg_dev, tasks, n, D->sgt_slab[buf],
-                                                                        D->sgt_exps[buf], D->L, D->sg_err);
+                                                                        D->sgt_exps[buf], D->L,
+                                                                        sg::Waits{D->sg_err, chol_test_wait(h, kTestWaitFactor)});
 }
 
 // U_J of every blocked supernode of a level (RLB: subtracted from the ancestors).
@@ -275,12 +276,13 @@ void chol_sg_syrk(chol_handle* h, const LevelPlan& P, cudaStream_t st) {
   k_sg_split_rows<<<P.sgr_n, kSplitThreads, 0, st>>>(D->sn, D->sg_dev, D->sg_split + P.sgr_b, D->L, D->sg_slab,
                                                      D->sg_exps);
   const int grid = std::min(P.sgs_n, D->sms);
+  const sg::Waits waits{D->sg_err, chol_test_wait(h, kTestWaitFactor)};
   if (h->opt.update_mode == CHOL_UPDATE_RLB)
     k_sg_syrk<true><<<grid, sg::kThreads, sg::kSmemBytes, st>>>(D->sn, D->sg_dev, D->sg_syrk + P.sgs_b, P.sgs_n, D->sg_slab,
                                                                 D->sg_exps, nullptr, D->rlb_pairs, D->rlb_pbeg, D->rows,
-                                                                D->L, D->sg_err);
+                                                                D->L, waits);
   else
     k_sg_syrk<false><<<grid, sg::kThreads, sg::kSmemBytes, st>>>(D->sn, D->sg_dev, D->sg_syrk + P.sgs_b, P.sgs_n,
                                                                  D->sg_slab, D->sg_exps, D->U, nullptr, nullptr, nullptr,
-                                                                 nullptr, D->sg_err);
+                                                                 nullptr, waits);
 }

@@ -225,6 +225,13 @@ struct Tile {
   int nblk;      // K blocks
 };
 
+// Where a wait that gave up is recorded. fail (testing the failure path only,
+// else -1): the epilogue warp whose waits count as run out at once.
+struct Waits {
+  int* err;
+  int fail;
+};
+
 // Shared state of the CTA.
 constexpr int kMaxStages = 3;
 struct Shared {
@@ -264,13 +271,15 @@ __device__ __forceinline__ uint32_t setup(Shared& S) {
   return S.tmem;
 }
 
-// Ends the CTA: after an abort, waits (bounded) for the copies in flight and
-// for the MMAs already issued; then frees the tensor memory.
+// Ends the CTA: waits (bounded) for the last copy issued into each stage and for the
+// MMAs already issued; then frees the tensor memory. The copies are waited for
+// whether a wait has given up or not: one that gives up later, after the copy
+// thread has got here, may leave copies that no MMA has waited for.
 template <int N = kN>
 __device__ __forceinline__ void teardown(Shared& S, uint32_t tmem) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int never = 0;
-  if (warp == Cfg<N>::kEpiWarps && lane == 0 && *(volatile int*)&S.abort_flag) {
+  if (warp == Cfg<N>::kEpiWarps && lane == 0) {
     for (int s = 0; s < Cfg<N>::kStages && s < S.issued; ++s)
       wait_or_abort(tc::smem_u32(&S.full[s]), (uint32_t)(((S.issued - 1 - s) / Cfg<N>::kStages) & 1), &never);
   }
@@ -288,14 +297,14 @@ __device__ __forceinline__ void teardown(Shared& S, uint32_t tmem) {
 
 // The copy thread's loop over the CTA's tiles: `next(i, tile)` gives the i-th tile.
 template <int N = kN, class Next>
-__device__ __forceinline__ void copy_loop(Shared& S, uint32_t base, Next next, int* err) {
+__device__ __forceinline__ void copy_loop(Shared& S, uint32_t base, Next next, Waits w) {
   int it = 0;
   Tile t;
   for (int i = 0; next(i, t); ++i) {
     for (int k = 0; k < t.nblk; ++k, ++it) {
       const int s = it % Cfg<N>::kStages, round = it / Cfg<N>::kStages;
       if (round > 0 && !wait_or_abort(tc::smem_u32(&S.empty[s]), (uint32_t)((round - 1) & 1), &S.abort_flag)) {
-        atomicExch(err, tc::kErrTimeoutEmpty);
+        atomicExch(w.err, tc::kErrTimeoutEmpty);
         *(volatile int*)&S.abort_flag = 1;
         S.issued = it;
         return;
@@ -338,11 +347,11 @@ __device__ __forceinline__ void mma_orders(uint32_t tmem, uint64_t ad, uint64_t 
 // kChunkK and taken back before its next use, so the epilogue reads one group
 // while the other's products run.
 template <int N = kN, class Next>
-__device__ __forceinline__ void mma_loop(Shared& S, uint32_t base, uint32_t tmem, Next next, int* err) {
+__device__ __forceinline__ void mma_loop(Shared& S, uint32_t base, uint32_t tmem, Next next, Waits w) {
   int it = 0, chunk = 0;
   Tile t;
   auto give_up = [&](int code) {
-    atomicExch(err, code);
+    atomicExch(w.err, code);
     *(volatile int*)&S.abort_flag = 1;
   };
   for (int i = 0; next(i, t); ++i) {
@@ -379,10 +388,11 @@ __device__ __forceinline__ void mma_loop(Shared& S, uint32_t base, uint32_t tmem
 }
 
 // A whole epilogue warp waits for group g of the chunk (uniform result).
-__device__ __forceinline__ bool epi_wait(Shared& S, int g, int chunk, int* err) {
-  const bool ok = wait_or_abort(tc::smem_u32(&S.acc_full[g]), (uint32_t)(chunk & 1), &S.abort_flag);
+__device__ __forceinline__ bool epi_wait(Shared& S, int g, int chunk, Waits w) {
+  const bool ok = (int)(threadIdx.x >> 5) != w.fail &&
+                  wait_or_abort(tc::smem_u32(&S.acc_full[g]), (uint32_t)(chunk & 1), &S.abort_flag);
   if (__all_sync(0xffffffffu, ok)) return true;
-  atomicExch(err, tc::kErrTimeoutAccum);
+  atomicExch(w.err, tc::kErrTimeoutAccum);
   *(volatile int*)&S.abort_flag = 1;
   return false;
 }
@@ -402,9 +412,9 @@ __device__ __forceinline__ int epi_col() { return (int)(threadIdx.x >> 7) * kCol
 // (orders 4..6) and gives the accumulators back. False if a wait gave up.
 template <int N = kN>
 __device__ __forceinline__ bool drain(Shared& S, uint32_t tmem, int chunk, long long (&hi)[kCols],
-                                      long long (&lo)[kCols], int* err) {
+                                      long long (&lo)[kCols], Waits w) {
   const uint32_t t0 = tmem + ((uint32_t)((threadIdx.x >> 5) & 3) << 21) + (uint32_t)epi_col();
-  if (!epi_wait(S, 0, chunk, err)) return false;
+  if (!epi_wait(S, 0, chunk, w)) return false;
   tc::fence_after();
 #pragma unroll
   for (int c = 0; c < kCols; c += 4) {
@@ -421,7 +431,7 @@ __device__ __forceinline__ bool drain(Shared& S, uint32_t tmem, int chunk, long 
   tc::fence_before();
   __syncwarp();
   if ((threadIdx.x & 31) == 0) mbar_arrive(tc::smem_u32(&S.acc_empty[0]));
-  if (!epi_wait(S, 1, chunk, err)) return false;
+  if (!epi_wait(S, 1, chunk, w)) return false;
   tc::fence_after();
 #pragma unroll
   for (int c = 0; c < kCols; c += 4) {
