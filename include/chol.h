@@ -120,10 +120,10 @@ typedef struct chol_options {
   int32_t test_unreachable_flags; /* testing the failure path only (bits): 1 =  */
                            /* the triangle solve's dependent blocks wait for a   */
                            /* flag value that no block publishes, so every such  */
-                           /* wait runs out after wait_polls polls; 2, 8 = one   */
-                           /* warp's waits of every tensor-core tile count as    */
-                           /* run out (chol_factor; the selected inverse);       */
-                           /* 0 = off (default)                                  */
+                           /* wait runs out after wait_polls polls; 2, 4, 8 =    */
+                           /* one warp's waits of every tensor-core tile count   */
+                           /* as run out (chol_factor; the solves' panel         */
+                           /* products; the selected inverse); 0 = off (default) */
   int32_t reserved_opt;
 } chol_options;
 

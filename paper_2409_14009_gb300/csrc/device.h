@@ -235,8 +235,8 @@ inline int chol_factored_here(const chol_handle* h) {
 int chol_dalloc(chol_handle* h, void** p, size_t bytes);
 
 // Bits of chol_options.test_unreachable_flags, and the epilogue warp whose waits
-// count as run out under one of the last two (-1: none).
-enum { kTestWaitTriangle = 1, kTestWaitFactor = 2, kTestWaitSelinv = 8 };
+// count as run out under one of the last three (-1: none).
+enum { kTestWaitTriangle = 1, kTestWaitFactor = 2, kTestWaitSolve = 4, kTestWaitSelinv = 8 };
 inline int chol_test_wait(const chol_handle* h, int bit) { return h->opt.test_unreachable_flags & bit ? 0 : -1; }
 
 // binary64 updates on the tensor cores (split_gemm.cu)

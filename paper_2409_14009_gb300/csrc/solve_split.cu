@@ -112,6 +112,9 @@ k_vs_tile(const SnodeDev* __restrict__ sn, const SolveSplitDev* __restrict__ vd,
 #pragma unroll
       for (int c = 0; c < sg::kCols; ++c) hi[c] = lo[c] = 0;
       for (int k0 = 0; ok && k0 < t.nblk; k0 += sg::kStagesPerChunk) ok = sg::drain<kN>(S, tmem, chunk++, hi, lo, waits);
+      // one verdict for the four warps, which meet at barriers below: a warp whose wait
+      // gave up and one whose wait was met just after it leave together
+      ok = sg::epi_vote<kN>(ok);
       if (!ok) break;
       double v[sg::kCols];
 #pragma unroll
@@ -260,7 +263,7 @@ void chol_vs_products(chol_handle* h, const LevelPlan& P, bool trans, double* Y,
                                                          D->vs_slab, D->vs_exps, D->vs_exps);
   const SolveTile* tiles = D->vs_tiles + P.vs_tile_b[t];
   const int nt = P.vs_tile_n[t], grid = std::min(nt, D->sms);
-  const sg::Waits waits{D->sg_err, -1};
+  const sg::Waits waits{D->sg_err, chol_test_wait(h, kTestWaitSolve)};
   if (trans) {
     k_vs_rhs<true><<<dim3(P.vs_n, nr), kRhsThreads, 0, st>>>(D->sn, D->vs_dev, D->vs_list + P.vs_b, D->rows, Y, n, D->vs_exps,
                                                D->vs_rslab, D->vs_rexps);

@@ -387,7 +387,8 @@ __device__ __forceinline__ void mma_loop(Shared& S, uint32_t base, uint32_t tmem
   }
 }
 
-// A whole epilogue warp waits for group g of the chunk (uniform result).
+// A whole epilogue warp waits for group g of the chunk (uniform over the warp; other
+// warps may see the same wait met, so a barrier among them needs epi_vote first).
 __device__ __forceinline__ bool epi_wait(Shared& S, int g, int chunk, Waits w) {
   const bool ok = (int)(threadIdx.x >> 5) != w.fail &&
                   wait_or_abort(tc::smem_u32(&S.acc_full[g]), (uint32_t)(chunk & 1), &S.abort_flag);
@@ -395,6 +396,19 @@ __device__ __forceinline__ bool epi_wait(Shared& S, int g, int chunk, Waits w) {
   atomicExch(w.err, tc::kErrTimeoutAccum);
   *(volatile int*)&S.abort_flag = 1;
   return false;
+}
+
+// True in every epilogue warp if `ok` is true in all of them: a barrier (named
+// barrier 1) that each of them passes once a tile, whether its waits were met or not.
+template <int N = kN>
+__device__ __forceinline__ bool epi_vote(bool ok) {
+  int all;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %1, 0;\n bar.red.and.pred q, 1, %2, p;\n selp.s32 %0, 1, 0, q;\n}\n"
+      : "=r"(all)
+      : "r"((int)ok), "n"(32 * Cfg<N>::kEpiWarps)
+      : "memory");
+  return all != 0;
 }
 
 __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {

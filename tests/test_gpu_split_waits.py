@@ -57,3 +57,31 @@ def test_selected_inverse(s, b):
         assert P.chol_factor(h, v) == 0
     finally:
         P.chol_destroy(h)
+
+
+# (the second leaf is one supernode with the separator: s b nrhs products in level 0)
+@pytest.mark.parametrize("s,b,nrhs", [(600, 1000, 16), (1030, 1030, 12)])
+def test_solve_products(s, b, nrhs):
+    """The tiles whose sums are cut in parts have barriers among the epilogue warps: the
+    warps whose waits were met must not stay behind at one. The arrival counters are
+    clean again afterwards: the next solves report the same, one column is right."""
+    p = _arrow(s, b)
+    P, h = _handle(p, 4)
+    n = p["n"]
+    x = np.random.RandomState(3).uniform(-1, 1, (nrhs, n))
+    try:
+        assert P.chol_factor(h, to_dev(p["values"])) == 0
+        for _ in range(2):
+            assert P.chol_solve(h, to_dev(x), nrhs) == 0                # asynchronous
+            assert P.chol_check_waits(h) == P.CHOL_ETIMEOUT
+            assert P.chol_check_waits(h) == 0
+        y = to_dev(x[0])
+        assert P.chol_solve(h, y, 1) == 0 and P.chol_check_waits(h) == 0
+        cols = np.repeat(np.arange(n), np.diff(p["colptr"]))
+        A = np.zeros((n, n))
+        A[p["rowind"], cols] = p["values"]
+        A = np.tril(A) + np.tril(A, -1).T
+        r = A @ y.cpu().numpy() - x[0]
+        assert np.max(np.abs(r)) <= 1e-12 * np.max(np.abs(A).sum(axis=1))   # |x| < 1
+    finally:
+        P.chol_destroy(h)
