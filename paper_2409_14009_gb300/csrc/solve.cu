@@ -1778,6 +1778,7 @@ int chol_solve_status(chol_handle* h) {
   CHOL_CUDA_TRY(cudaMemcpy(e, D->sv_err, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost));
   if (e[0] | e[1]) {
     CHOL_CUDA_TRY(cudaMemset(D->sv_err, 0, 2 * sizeof(int32_t)));
+    if (e[1]) h->selinv_valid = false;   // its products may be the ones: computed again by the next call
     if (D->vs_cnt) CHOL_CUDA_TRY(cudaMemset(D->vs_cnt, 0, sizeof(int32_t) * (size_t)h->vs_slots));
     CHOL_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));
     return CHOL_ETIMEOUT;

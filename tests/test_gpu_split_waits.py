@@ -54,6 +54,11 @@ def test_selected_inverse(s, b):
         assert P.chol_selected_inverse(h, torch.empty_like(v)) == 0    # asynchronous
         assert P.chol_check_waits(h) == P.CHOL_ETIMEOUT
         assert P.chol_check_waits(h) == 0                              # the record was cleared
+        # the broken Z is not kept: the next calls compute it again (and lose again)
+        for call in (lambda: P.chol_selected_inverse(h, torch.empty_like(v)),
+                     lambda: P.chol_adjoint(h, None, None, 0, 1.0, None, torch.empty_like(v))):
+            assert call() == 0
+            assert P.chol_check_waits(h) == P.CHOL_ETIMEOUT
         assert P.chol_factor(h, v) == 0
     finally:
         P.chol_destroy(h)
