@@ -307,7 +307,8 @@ int chol_solve_refine(chol_handle* h, const double* b, double* x, int32_t nrhs, 
  * builds the level plan and its workspaces (largest level's sum of s^2,
  * b s and s^2 / 2 doubles, and the slices of its largest group of products, which
  * run on the tensor cores where chol_factor's do). CHOL_PREC_FP64 handles only (else CHOL_ENOTSUP).
- * Asynchronous.
+ * A call captured in a CUDA graph (after a plain one, which builds the plan) computes
+ * at each of the graph's replays, from the factor of that moment. Asynchronous.
  */
 int chol_selected_inverse(chol_handle* h, double* zvals, void* stream);
 

@@ -688,16 +688,18 @@ int build_si_plan(chol_handle* h) {
 // Selected inverse into D->Zp (once per factorization), level by level from the
 // root, every supernode of a level at once.
 int selinv(chol_handle* h, cudaStream_t st) {
-  if (h->selinv_valid) return CHOL_OK;
+  // a captured call computes whether Z is there or not: its replays may follow another factor
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  CHOL_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
+  const bool capturing = cap != cudaStreamCaptureStatusNone;
+  if (h->selinv_valid && !capturing) return CHOL_OK;
   if (h->max_len > kSelinvMaxLen) return CHOL_ENOTSUP;
   int rc = ensure_adjoint(h);
   if (rc) return rc;
   if ((rc = build_si_plan(h))) return rc;
   DeviceState* D = h->dev;
   SiPlan* pl = (SiPlan*)D->si_plan;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  CHOL_CUDA_TRY(cudaStreamIsCapturing(st, &cap));
-  if (cap != cudaStreamCaptureStatusNone) pl->pinned = true;
+  if (capturing) pl->pinned = true;
   auto launch = [&](const Group& gr) {
     if (pl->sg) {
       if (gr.gn == 0) return;
@@ -735,7 +737,7 @@ int selinv(chol_handle* h, cudaStream_t st) {
     }
   }
   CHOL_CUDA_TRY(cudaGetLastError());
-  h->selinv_valid = true;
+  if (!capturing) h->selinv_valid = true;
   return CHOL_OK;
 }
 
