@@ -65,7 +65,7 @@ __device__ void small_panel_columns(double* P, int ld, int len, int c0, int w, i
       P[k + k * ld] = dk;
       *srk = rk;
       if (bad) atomicMin(status, fcol + k + 1);
-      rdiag[k] = fma(fma(-dk, rk, 1.0), rk, rk);
+      rdiag[k] = root_recip(dk, rk);
     }
     __syncthreads();
     const double inv = *srk;
@@ -247,7 +247,7 @@ k_small_warp(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list, 
       if (bad && lane == 0) atomicMin(status, d.f + k + 1);
       double root, rroot;
       pivot_root(dk, bad, root, rroot);
-      if (lane == k) rd = fma(fma(-root, rroot, 1.0), rroot, rroot);
+      if (lane == k) rd = root_recip(root, rroot);
       x[k] = lane == k ? root : x[k] * rroot;
 #pragma unroll
       for (int j = k + 1; j < S; ++j)

@@ -74,6 +74,7 @@ __device__ __forceinline__ double rsqrt_bits(int hi, int lo) {
   const u64 r = ((v + 256) >> 9) + (1021ull << 52);          // bit 52 is the implicit one
   return __hiloint2double((int)(r >> 32) - ((E - 1023 - p) / 2) * (1 << 20), (int)r);
 }
+// 1 / root from the root and its reciprocal of the line above, rounded nearly
 __device__ __forceinline__ void pivot_root(double d, bool bad, double& root, double& rroot) {
   const int hi = __double2hiint(d);
   if (hi >= 0x00100000 && hi < 0x7ff00000) {   // positive, normal, finite
@@ -86,6 +87,13 @@ __device__ __forceinline__ void pivot_root(double d, bool bad, double& root, dou
     root = sqrt(d);
     rroot = 1.0 / root;
   }
+}
+// 1 / root from a root and its reciprocal rounded twice (rsqrt): one correction. Of an
+// infinite root (an infinite pivot) and of NaN it is the reciprocal itself, 0 and NaN:
+// the correction would be NaN for both.
+__device__ __forceinline__ double root_recip(double root, double rroot) {
+  const bool finite = (__double2hiint(root) & 0x7ff00000) != 0x7ff00000;
+  return finite ? fma(fma(-root, rroot, 1.0), rroot, rroot) : rroot;
 }
 
 // Factor the block at G (row-major with leading dimension ld if RM, else
