@@ -984,6 +984,7 @@ k_logdet_part(const SnodeDev* __restrict__ sn, int ns, const double* __restrict_
   const SnodeDev d = sn[J];
   double m = 1.0;        // product 1 <= |m| < 2 after every step
   int e = 0;
+  int odd = 0;           // 1: an entry is infinite (its pivot was), 2: one is NaN
   auto times = [&](double v, int ev) {
     m *= v;
     const int hi = __double2hiint(m), x = (hi >> 20) - 1023;
@@ -993,6 +994,10 @@ k_logdet_part(const SnodeDev* __restrict__ sn, int ns, const double* __restrict_
 #pragma unroll 4
   for (int c = q; c < d.s; c += G) {
     double v = L[d.loff + c + (int64_t)c * d.ld];
+    if ((__double2hiint(v) & 0x7ff00000) == 0x7ff00000) {
+      odd |= v > 0.0 ? 1 : 2;
+      continue;
+    }
     int ev = 0;
     if (v < 2.2250738585072014e-308) { v *= 18014398509481984.0; ev = -54; }   // subnormal: times 2^54
     const int hi = __double2hiint(v), x = (hi >> 20) - 1023;
@@ -1002,9 +1007,12 @@ k_logdet_part(const SnodeDev* __restrict__ sn, int ns, const double* __restrict_
   for (int o = G / 2; o > 0; o >>= 1) {
     const double mo = __shfl_xor_sync(mask, m, o, G);
     const int eo = __shfl_xor_sync(mask, e, o, G);
+    odd |= __shfl_xor_sync(mask, odd, o, G);
     times(mo, eo);
   }
-  if (q == 0) part[J] = log(m) + (double)e * 0.693147180559945309417;
+  if (q == 0)
+    part[J] = odd ? __longlong_as_double(odd > 1 ? 0x7ff8000000000000ll : 0x7ff0000000000000ll)
+                  : log(m) + (double)e * 0.693147180559945309417;
 }
 
 // log det of every system: 2 x the supernode partials of its range, in order.

@@ -1,7 +1,7 @@
 """Infinite diagonal entries (nodes pinned by an infinite penalty): the pivot's root
 is infinite and its reciprocal zero, so the column of L below it is zero, x is zero
-there and elsewhere that of the system without the node, and the selected inverse
-is zero in its row.
+there and elsewhere that of the system without the node, the selected inverse is
+zero in its row, and log det is infinite (of its own system only in a batch).
 
 The remaining systems have n <= 400 and kappa < 1e4: n u kappa < 5e-10; 1e-10 of
 the largest entry as in the other tests of such grids.
@@ -64,6 +64,9 @@ def test_pinned_nodes(mode, nrhs):
             got.append(X.cpu().numpy().reshape(n, nrhs))
         z = torch.empty_like(v)
         assert P.chol_selected_inverse(h, z) == 0 and P.chol_check_waits(h) == 0
+        rc, ld = P.chol_logdet(h)
+        rcb, ldb = P.chol_logdet_batch(h, 1)
+        assert rc == 0 and rcb == 0
     finally:
         P.chol_destroy(h)
     A = _dense(p)[np.ix_(keep, keep)]
@@ -76,6 +79,7 @@ def test_pinned_nodes(mode, nrhs):
     Z[np.ix_(keep, keep)] = np.linalg.inv(A)
     zr = Z[p["rowind"], np.repeat(np.arange(n), np.diff(p["colptr"]))]
     assert np.max(np.abs(z.cpu().numpy() - zr)) <= TOL * np.max(np.abs(zr))
+    assert ld == np.inf and ldb[0] == np.inf
 
 
 def test_pinned_node_of_a_batch():
@@ -100,13 +104,17 @@ def test_pinned_node_of_a_batch():
             assert P.chol_factor_batch(h, to_dev(np.tile(vals, copies))) == 0
             X = colmajor(np.tile(b, (copies, 1)))
             assert P.chol_solve_batch(h, X, 1) == 0 and P.chol_check_waits(h) == 0
-            out.append(X.cpu().numpy().reshape(copies, one.n))
+            rc, ld = P.chol_logdet_batch(h, len(offs) - 1)
+            assert rc == 0
+            out.append((X.cpu().numpy().reshape(copies, one.n), np.asarray(ld).reshape(copies, 7)))
         finally:
             P.chol_destroy(h)
-    x0, x1 = out
+    (x0, ld0), (x1, ld1) = out
     other = np.ones(one.n, bool)
     other[offs1[q]:offs1[q + 1]] = False
     assert np.array_equal(x1[:, other], x0[:, other])
+    rest = np.arange(7) != q
+    assert np.array_equal(ld1[:, rest], ld0[:, rest]) and (ld1[:, q] == np.inf).all()
     keep = np.setdiff1d(np.arange(n3), local)
     A = _dense(probs[q])[np.ix_(keep, keep)]
     ref = np.zeros(n3)
