@@ -1010,6 +1010,12 @@ k_logdet_part(const SnodeDev* __restrict__ sn, int ns, const double* __restrict_
     odd |= __shfl_xor_sync(mask, odd, o, G);
     times(mo, eo);
   }
+  // a product a little below a power of two counts from above it: next to 1 the
+  // logarithm alone keeps its relative accuracy, log(2 - d) - log(2) would not
+  if (m > 1.4142135623730951) {
+    m *= 0.5;
+    ++e;
+  }
   if (q == 0)
     part[J] = odd ? __longlong_as_double(odd > 1 ? 0x7ff8000000000000ll : 0x7ff0000000000000ll)
                   : log(m) + (double)e * 0.693147180559945309417;
