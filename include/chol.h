@@ -341,7 +341,7 @@ typedef struct chol_info {
   int64_t panel_doubles;   /* device storage of the supernodal panels */
   int64_t update_doubles;  /* update-matrix workspace (largest level) */
   double flops;            /* sum_j c_j^2, c_j = nnz(L_{*,j}) incl. diagonal */
-  int32_t n_small;         /* supernodes on the one-CTA kernel */
+  int32_t n_small;         /* supernodes on the one-CTA (one-warp) kernels */
   int32_t n_large;         /* supernodes on the blocked path */
   int32_t nsuper_storage;  /* supernodes after relaxed merging (= nsuper if off) */
   int32_t reserved;

@@ -480,7 +480,7 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
     std::vector<int32_t> large;
     P.small_b = (int32_t)h->small_list.size();
     P.small_max_panel = 0;
-    std::vector<int32_t> by_class[4];   // warp (s <= 8, s <= 16), CTA, blocked
+    std::vector<int32_t> by_class[3];   // warp (s <= 8, s <= 16), CTA
     P.cta_max_panel = 0;
     int64_t uo = 0, wo = 0;
     for (int32_t J : Js) {
@@ -490,25 +490,22 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
       uo += (int64_t)b * (h->opt.precision == CHOL_PREC_FP64 ? b : ((b + 7) & ~7));
       d.wpre = wo;
       wo += b;
-      if (one_cta(J)) {
-        for (int32_t j = d.f; j < d.f + d.s; ++j) P.small_flops += (double)h->colcount[j] * h->colcount[j];
-        P.small_bytes += 16.0 * (double)d.len * d.s + 8.0 * (double)b * (b + 1) / 2.0;
-        P.small_max_panel = std::max(P.small_max_panel, d.len * d.s);
-        h->n_small++;
-        const int cls = mixed ? 2 : (d.len <= 32 && d.s <= 8) ? 0 : (d.len <= 32 && d.s <= 16) ? 1
-                        : (any_large && split64 && d.s > kBlockedCols) ? 3 : 2;
-        by_class[cls].push_back(J);
-        if (cls == 2) P.cta_max_panel = std::max(P.cta_max_panel, d.len * d.s);
-        if (cls == 3) large.push_back(J);
-      } else {
+      if (!one_cta(J) || (any_large && split64 && d.s > kBlockedCols)) {
         large.push_back(J);
         h->n_large++;
+        continue;
       }
+      for (int32_t j = d.f; j < d.f + d.s; ++j) P.small_flops += (double)h->colcount[j] * h->colcount[j];
+      P.small_bytes += 16.0 * (double)d.len * d.s + 8.0 * (double)b * (b + 1) / 2.0;
+      P.small_max_panel = std::max(P.small_max_panel, d.len * d.s);
+      h->n_small++;
+      const int cls = mixed ? 2 : (d.len <= 32 && d.s <= 8) ? 0 : (d.len <= 32 && d.s <= 16) ? 1 : 2;
+      by_class[cls].push_back(J);
+      if (cls == 2) P.cta_max_panel = std::max(P.cta_max_panel, d.len * d.s);
     }
     for (const auto& c : by_class) h->small_list.insert(h->small_list.end(), c.begin(), c.end());
     P.tiny8_n = (int32_t)by_class[0].size();
     P.tiny16_n = (int32_t)by_class[1].size();
-    P.small_k = P.tiny8_n + P.tiny16_n + (int32_t)by_class[2].size();
     P.small_n = (int32_t)h->small_list.size() - P.small_b;
     P.u_doubles = uo;
     P.w_rows = wo;

@@ -1500,7 +1500,7 @@ int enqueue_factor_fp64(chol_handle* h, const double* values, cudaStream_t st) {
     const bool rlb = h->opt.update_mode == CHOL_UPDATE_RLB;
     // one-CTA supernodes, beside the blocked ones of the level if it has both
     bool small_pending = false;
-    if (P.small_k > 0) {
+    if (P.small_n > 0) {
       small_pending = !P.steps.empty();
       const cudaStream_t ss = small_pending ? D->sstream : st;
       if (small_pending) {
@@ -1509,11 +1509,11 @@ int enqueue_factor_fp64(chol_handle* h, const double* values, cudaStream_t st) {
       }
       KScope ks(h, CHOL_K_SMALL, ss, P.small_flops, P.small_bytes);
       if (rlb)
-        k_small_rlb<<<P.small_k, kSmallThreads, sizeof(double) * P.small_max_panel, ss>>>(
+        k_small_rlb<<<P.small_n, kSmallThreads, sizeof(double) * P.small_max_panel, ss>>>(
             D->sn, D->small_list + P.small_b, D->rlb_pairs, D->rlb_pbeg, D->rows, D->L, D->status, D->rdiag);
       else {
         const bool warps = P.tiny8_n + P.tiny16_n >= kTinyMin;
-        const int n8 = warps ? P.tiny8_n : 0, n16 = warps ? P.tiny16_n : 0, nc = P.small_k - n8 - n16;
+        const int n8 = warps ? P.tiny8_n : 0, n16 = warps ? P.tiny16_n : 0, nc = P.small_n - n8 - n16;
         const int32_t* list = D->small_list + P.small_b;
         ks.launches((n8 > 0) + (n16 > 0) + (nc > 0));
         if (nc > 0)

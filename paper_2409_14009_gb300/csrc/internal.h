@@ -139,9 +139,9 @@ struct LevelPlan {
   int32_t small_b, small_n;   // one-CTA supernodes (in small_list)
   int32_t small_max_panel;    // largest len*s among them (shared memory sizing)
   // binary64, level by level: the first tiny8_n (s <= 8) and tiny16_n (s <= 16), of at
-  // most 32 rows, take a warp each; up to small_k a CTA each (cta_max_panel: their
-  // largest len*s); those after small_k take the blocked path
-  int32_t tiny8_n, tiny16_n, small_k, cta_max_panel;
+  // most 32 rows, take a warp each, the others a CTA each (cta_max_panel: their
+  // largest len*s)
+  int32_t tiny8_n, tiny16_n, cta_max_panel;
   std::vector<StepRange> steps;
   int32_t syrk_b, syrk_n;     // U tiles (in syrk_tasks)
   int32_t sgs_b, sgs_n;       // binary64 on the tensor cores: U tiles of 128 x 64 (in sgs_tasks)
