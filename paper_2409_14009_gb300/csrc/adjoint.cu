@@ -724,7 +724,8 @@ int selinv(chol_handle* h, cudaStream_t st) {
     }
     if (const LevelPlan& P = h->levels[sl.level]; P.asm_n + P.asmw_n > 0) {
       KScope ks(h, CHOL_K_SELINV_GATHER, st, 0.0, 16.0 * P.asm_entries);
-      ks.launches((P.asm_n > 0) + (P.asmw_n > 0));
+      const AsmSplit a = asm_split(P, D->sms);
+      ks.launches((a.ctas > 0) + (a.warps > 0));
       chol_gather_zrr(h, P, D->Zp, D->zrr_ws ? D->zrr_ws : D->U, st);
     }
     {

@@ -3,7 +3,7 @@ factor it."""
 import gridgen
 import pytest
 
-from gpu_util import run
+from gpu_util import run, to_dev
 from lib_fixture import chol
 
 pytestmark = pytest.mark.gpu
@@ -29,3 +29,20 @@ def test_wide_one_cta_supernodes_beside_blocked_ones():
     assert info.n_small + info.n_large == info.nsuper_storage
     assert (info.n_small, info.n_large) == (ref_info.n_small, ref_info.n_large)
     assert ref_info.n_large > 2 and got == ref
+
+
+def test_gather_launches():
+    """The selected inverse gathers by the factor's assembly tasks, level by level in the
+    same launches (one level has CTA-sized and warp-sized tasks, few enough for one)."""
+    P = chol()
+    p = gridgen.elasticity_27pt(10)
+    rc, h = P.chol_analyze(p.n, p["colptr"], p["rowind"], p["perm"])
+    assert rc == 0
+    try:
+        v = to_dev(p["values"])
+        assert P.chol_factor(h, v) == 0 and P.chol_selected_inverse(h, to_dev(p["values"])) == 0
+        assert P.chol_check_waits(h) == 0
+        st = P.chol_get_stats(h)
+    finally:
+        P.chol_destroy(h)
+    assert st["selinv_gather"]["launches"] == st["assemble"]["launches"] > 0
