@@ -124,7 +124,13 @@ typedef struct chol_options {
                            /* one warp's waits of every tensor-core tile count   */
                            /* as run out (chol_factor; the solves' panel         */
                            /* products; the selected inverse); 0 = off (default) */
-  int32_t reserved_opt;
+  int32_t fp64_products;   /* binary64 products of chol_factor, of solves with    */
+                           /* many right-hand sides and of the selected inverse: */
+                           /* 0 = on the tensor cores, errors relative to the    */
+                           /* largest entries of the rows multiplied (see        */
+                           /* chol_factor; default); nonzero = FMAs on the FP64  */
+                           /* pipe, errors relative to the terms of each entry's */
+                           /* own sum, and no slice workspaces                   */
 } chol_options;
 
 enum { CHOL_UPDATE_RL = 0, CHOL_UPDATE_RLB = 1 };
@@ -182,11 +188,23 @@ int chol_analyze(int32_t n, const int64_t* colptr, const int32_t* rowind,
  * U_J into the ancestors (pull-ordered, atomic-free, deterministic). It ends
  * by inverting the 64x64 diagonal blocks the triangle solves multiply by
  * (binary64: the inverse; mixed modes: also the last-dependency products).
- * Binary64 products run on the tensor cores as exact bf16 slices (an entry's
- * error is below that of binary64 FMAs); their workspaces belong to the handle,
- * are created by the first call, given back when a later allocation of the
- * handle finds no room, and left out on a device without room or under
- * device_mem_cap, where the FP64 pipe does the products.
+ * Binary64 products of blocked supernodes (block_cols = 64) run on the tensor
+ * cores as bf16 slices of the operands. The error of an entry sum_k a_k b_k, k < K,
+ * is one rounding plus at most about K 2^-60 max|a| max|b| (sqrt(K) 2^-62 in
+ * general): normwise less than that of K FMAs, and unchanged when rows are scaled
+ * by powers of two. FMAs are within K 2^-53 of sum |a_k| |b_k|, which is far
+ * smaller where the large entries of each row meet small ones of the other
+ * (rows graded over many powers of two, as of a strongly decaying inverse): there
+ * an entry below 2^-10 of its row's largest enters with fewer than 53 bits, one
+ * below 2^-63 with none, and small entries of L and of x lose relative (not
+ * absolute) accuracy. chol_options.fp64_products keeps FMAs for such matrices.
+ * The slices' workspaces belong to the handle: 14 bytes per entry of the level
+ * with the most entries in L_RJ of its blocked supernodes, and three blocks of 14
+ * bytes per entry of 64 columns of the level with the most rows in supernodes
+ * wider than 64. They are created by the first call, given back when a later
+ * allocation of the handle finds no room (not when another user of the GPU does),
+ * and left out on a device without room or under device_mem_cap, where the FP64
+ * pipe does the products.
  *   values  device, colptr[n] doubles in the order of the analyzed rowind
  *   stream  cudaStream_t as void*
  * Returns CHOL_OK, +j (not positive definite at column j of P A P^T), or an

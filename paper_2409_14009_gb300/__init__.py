@@ -50,7 +50,7 @@ class chol_options(C.Structure):
                 ("device_mem_cap", C.c_int64), ("merge_growth", C.c_double),
                 ("small_max_rows", C.c_int32), ("persistent", C.c_int32), ("pivot_tau", C.c_double),
                 ("static_pivot", C.c_int32), ("use_graph", C.c_int32), ("update_mode", C.c_int32),
-                ("wait_polls", C.c_int64), ("test_unreachable_flags", C.c_int32), ("reserved_opt", C.c_int32)]
+                ("wait_polls", C.c_int64), ("test_unreachable_flags", C.c_int32), ("fp64_products", C.c_int32)]
 
 
 class chol_info(C.Structure):

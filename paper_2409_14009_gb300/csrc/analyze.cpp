@@ -35,6 +35,7 @@ extern "C" void chol_default_options(chol_options* opt) {
   opt->update_mode = CHOL_UPDATE_RL;
   opt->wait_polls = 0;
   opt->test_unreachable_flags = 0;
+  opt->fp64_products = 0;
 }
 
 namespace {
@@ -427,7 +428,7 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
   const bool tc_modes = h->opt.precision == CHOL_PREC_TF32 || h->opt.precision == CHOL_PREC_BF16;
   const bool mixed = h->opt.precision != CHOL_PREC_FP64;
   // binary64 updates on the tensor cores: their operand blocks are 64 columns wide
-  const bool split64 = !mixed && nb == 64;
+  const bool split64 = !mixed && nb == 64 && !h->opt.fp64_products;
   h->split.assign(split64 ? ns : 0, SplitDev{});
   h->vs_dev.assign(split64 ? ns : 0, SolveSplitDev{});
   h->vs_list.clear(); h->vs_tasks.clear(); h->vs_tiles.clear();

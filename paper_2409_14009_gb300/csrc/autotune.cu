@@ -68,6 +68,7 @@ extern "C" int chol_tune_batch(int32_t count, const int32_t* sys_ptr, const int6
   if (perm) key = fnv1a(key, perm, sizeof(int32_t) * (size_t)n);
   key = fnv1a(key, &b0.precision, sizeof(b0.precision));
   key = fnv1a(key, &b0.update_mode, sizeof(b0.update_mode));
+  if (b0.fp64_products) key = fnv1a(key, "fp64 products", 13);   // other kernels, other best choice
   key = fnv1a(key, prop.name, std::strlen(prop.name));
   key = fnv1a(key, &prop.multiProcessorCount, sizeof(int));
   char keystr[32];

@@ -17,9 +17,15 @@
 //   in sign (digits in general position give about 2^19), and then lose their
 //   last bit. Orders above 6 (2^-81 times 2^16 K at most) are left out.
 // - the seven sums are added as integers, rounded once to binary64 and scaled.
-// So an entry's error is its one rounding plus about sqrt(K) 2^-64 times the
-// two rows' largest entries, below that of K binary64 FMAs, and independent of
-// scaling the rows by powers of two. (Digits of base 256 with the same orders,
+// So an entry's error is its one rounding plus about sqrt(K) 2^-62, at most about
+// K 2^-60 (equal entries), times the product of the two rows' largest entries.
+// Normwise that is less than the error of K binary64 FMAs (K 2^-53), and it does
+// not change when rows are scaled by powers of two. It is not relative to the sum's
+// own terms, as the FMAs' is: an entry below 2^-10 of its row's largest keeps fewer
+// than 53 bits and one below 2^-63 none, so where every large entry of one row
+// meets a small one of the other (graded rows), the result has fewer correct
+// bits than FMAs give it (chol_options.fp64_products).
+// (Digits of base 256 with the same orders,
 // 2^-57, were measured too: on the irregular 36^3 Laplacian, whose solution
 // hangs on small entries of L, x was 4 times further off than with FMAs.)
 // The summation order is fixed, so results are reproducible bit for bit. A row
