@@ -226,10 +226,15 @@ int chol_factor(chol_handle* h, const double* values, void* stream);
  * CHOL_ETIMEOUT by chol_check_waits, or by the next chol_factor or
  * chol_solve_refine on the handle. In binary64 with 9 and more right-hand sides
  * the panel products of large levels run on the tensor cores (bounded waits
- * too); the first such call creates their workspaces, and one that is captured
- * before that, or finds no room, keeps the FP64 pipe's kernels. Calls on one handle must not overlap on the
- * GPU (they share workspaces). CHOL_ESTATE if the current device is not the
- * one the handle was factored on.
+ * too; accuracy as for chol_factor's products), so a column's last bits may differ
+ * between calls with fewer and with more columns beside it. The first such call
+ * creates their workspaces (14 bytes per entry of the level with the most entries
+ * in off-diagonal blocks of supernodes that take a CTA or more), also when it is
+ * captured in a CUDA graph after another solve; if it finds no room, the handle
+ * stays with the FP64 pipe's kernels. The same call on the same route gives the
+ * same bits; chol_info.tc_products says which route that is. Calls on one handle
+ * must not overlap on the GPU (they share workspaces). CHOL_ESTATE if the current
+ * device is not the one the handle was factored on.
  */
 int chol_solve(chol_handle* h, double* b, int32_t nrhs, void* stream);
 
@@ -362,7 +367,11 @@ typedef struct chol_info {
   int32_t n_small;         /* supernodes on the one-CTA (one-warp) kernels */
   int32_t n_large;         /* supernodes on the blocked path */
   int32_t nsuper_storage;  /* supernodes after relaxed merging (= nsuper if off) */
-  int32_t reserved;
+  int32_t tc_products;     /* binary64 products that run on the tensor cores:     */
+                           /* bit 0 = chol_factor, bit 1 = solves with 9 and     */
+                           /* more right-hand sides, bit 2 = the selected        */
+                           /* inverse; each set by the first such call, cleared  */
+                           /* if the workspaces are given back for want of room  */
   int64_t nnz_stored;      /* stored factor entries incl. explicit zeros of merging */
   double flops_stored;     /* sum over stored columns of their stored count^2 */
   int32_t precision;       /* CHOL_PREC_* of the handle */

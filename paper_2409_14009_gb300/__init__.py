@@ -59,7 +59,7 @@ class chol_info(C.Structure):
                 ("n_relind_pairs", C.c_int64), ("relind_len", C.c_int64),
                 ("panel_doubles", C.c_int64), ("update_doubles", C.c_int64),
                 ("flops", C.c_double), ("n_small", C.c_int32), ("n_large", C.c_int32),
-                ("nsuper_storage", C.c_int32), ("reserved", C.c_int32), ("nnz_stored", C.c_int64),
+                ("nsuper_storage", C.c_int32), ("tc_products", C.c_int32), ("nnz_stored", C.c_int64),
                 ("flops_stored", C.c_double), ("precision", C.c_int32), ("fp64_fallbacks", C.c_int32),
                 ("perturbed_pivots", C.c_int32), ("nsys", C.c_int32), ("persistent_ok", C.c_int32),
                 ("persistent_threads", C.c_int32), ("persistent_ctas_per_sm", C.c_int32),

@@ -751,6 +751,11 @@ void chol_adjoint_free(chol_handle* h) {
   D->si_plan = nullptr;
 }
 
+bool chol_adjoint_split(const chol_handle* h) {
+  const SiPlan* pl = (const SiPlan*)h->dev->si_plan;
+  return pl && pl->sg;
+}
+
 // Gives back a plan that holds slices (the next call builds one without them).
 bool chol_adjoint_release(chol_handle* h) {
   const SiPlan* pl = (const SiPlan*)h->dev->si_plan;

@@ -1096,6 +1096,7 @@ extern "C" int chol_get_info(const chol_handle* h, chol_info* info) {
     }
     info->relind_len = tot;
   }
+  info->tc_products = chol_tc_products(h);
   info->panel_doubles = h->panel_doubles;
   info->update_doubles = h->update_doubles;
   info->flops = h->flops;

@@ -271,3 +271,4 @@ constexpr int kSplitMin = 128;        // ... of at least this many columns (gemv
 constexpr int kRlbSmallRows = 1024;   // RLB: rows of a supernode on the one-CTA kernel (small_max_rows cap)
 
 void chol_device_free(chol_handle* h);  // CUDA side
+int32_t chol_tc_products(const chol_handle* h);   // chol_info.tc_products

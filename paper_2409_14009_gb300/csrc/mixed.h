@@ -23,6 +23,7 @@ int chol_tc_syrk(chol_handle* h, const TileTask* tasks, int n, cudaStream_t st);
 int chol_tc_status(chol_handle* h);
 void chol_adjoint_free(chol_handle* h);
 bool chol_adjoint_release(chol_handle* h);
+bool chol_adjoint_split(const chol_handle* h);   // a selected-inverse plan with slices
 int chol_solve_status(chol_handle* h);
 int chol_diag_inv(chol_handle* h, int b, int nitems, cudaStream_t st);
 int chol_bc_begin_mixed(const chol_handle* h);

@@ -22,7 +22,9 @@
 //     or solve_split.cu).
 //   - the transposed diagonal triangle, blocks last to first.
 // Every output entry is written by exactly one thread per launch and every
-// reduction runs in a fixed order, so the solve is deterministic.
+// reduction runs in a fixed order, so the solve is deterministic on its route (which
+// levels' products go to the tensor cores: by the number of right-hand sides, and by
+// room for their workspaces).
 #include <mutex>
 #include <type_traits>
 

@@ -194,24 +194,14 @@ void chol_vs_release(chol_handle* h) {
     }
 }
 
-// Plan and workspaces, created by the first solve that can use them (not while
-// `st` is being captured: that solve keeps the binary64 pipe's kernels). Handles
-// without the factor's slices (a memory cap, a device without room) go without,
-// and a later allocation that finds no room gets these back first, unless a
-// captured solve holds their addresses.
-int chol_vs_ensure(chol_handle* h, cudaStream_t st) {
+// Creates the plan and its workspaces: while the caller's stream is being captured
+// too, so that whether a solve takes the tensor cores does not depend on what was
+// called before it. For that the thread's captures do not restrict the calls made
+// here (relaxed mode), none of them goes to the stream under capture or to the
+// legacy stream, and what they do is done once, not at the replays.
+static int vs_create(chol_handle* h) {
   DeviceState* D = h->dev;
-  if (D->vs_ready == -1 || D->sg_ready != 1 || h->vs_list.empty()) return -1;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
-    cudaGetLastError();
-    return -1;
-  }
-  if (D->vs_ready == 1) {
-    if (cap != cudaStreamCaptureStatusNone) D->vs_pinned = true;
-    return 1;
-  }
-  if (cap != cudaStreamCaptureStatusNone) return -1;
+  const cudaStream_t ps = D->lstream;
   // the panel operands of both directions
   std::vector<SplitOp> ops;
   ops.reserve(2 * h->vs_list.size());
@@ -233,7 +223,7 @@ int chol_vs_ensure(chol_handle* h, cudaStream_t st) {
     D->bytes += b.bytes;
   }
   auto up = [&](void* dst, const void* src, size_t bytes) {
-    ok = ok && cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
+    ok = ok && cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, ps) == cudaSuccess;
   };
   if (ok) {
     up(D->vs_dev, h->vs_dev.data(), sizeof(SolveSplitDev) * h->vs_dev.size());
@@ -242,9 +232,8 @@ int chol_vs_ensure(chol_handle* h, cudaStream_t st) {
     up(D->vs_tasks, h->vs_tasks.data(), sizeof(SplitTask) * h->vs_tasks.size());
     up(D->vs_tiles, h->vs_tiles.data(), sizeof(SolveTile) * h->vs_tiles.size());
   }
-  // the copies and the memset run on the legacy stream, which non-blocking streams do not wait for
-  ok = ok && (h->vs_slots == 0 || cudaMemset(D->vs_cnt, 0, h->vs_slots * 4) == cudaSuccess) &&
-       cudaStreamSynchronize(cudaStreamLegacy) == cudaSuccess &&
+  ok = ok && (h->vs_slots == 0 || cudaMemsetAsync(D->vs_cnt, 0, h->vs_slots * 4, ps) == cudaSuccess) &&
+       cudaStreamSynchronize(ps) == cudaSuccess &&
        cudaFuncSetAttribute(k_vs_tile<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes) == cudaSuccess &&
        cudaFuncSetAttribute(k_vs_tile<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes) == cudaSuccess;
   if (!ok) {
@@ -253,6 +242,31 @@ int chol_vs_ensure(chol_handle* h, cudaStream_t st) {
     return -1;
   }
   return D->vs_ready = 1;
+}
+
+// Plan and workspaces, created by the first solve that can use them. Handles
+// without the factor's slices (a memory cap, a device without room) go without,
+// and a later allocation that finds no room gets these back first, unless a
+// captured solve holds their addresses.
+int chol_vs_ensure(chol_handle* h, cudaStream_t st) {
+  DeviceState* D = h->dev;
+  if (D->vs_ready == -1 || D->sg_ready != 1 || h->vs_list.empty()) return -1;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return -1;
+  }
+  if (D->vs_ready == 0) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) {
+      cudaGetLastError();
+      return -1;
+    }
+    vs_create(h);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+  }
+  if (D->vs_ready == 1 && cap != cudaStreamCaptureStatusNone) D->vs_pinned = true;
+  return D->vs_ready;
 }
 
 // The level's panel products of one direction for nr <= 16 right-hand sides.

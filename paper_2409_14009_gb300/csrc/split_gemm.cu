@@ -9,6 +9,7 @@
 //                     operands come from k_trsm, one exponent per row of the block)
 //   k_sg_syrk         U_J tiles, any K; RLB: subtracted from the ancestors
 #include "device.h"
+#include "mixed.h"
 #include "split_gemm.cuh"
 
 namespace {
@@ -219,6 +220,13 @@ std::vector<SgBuffer> sg_buffers(chol_handle* h) {
 }
 
 }  // namespace
+
+int32_t chol_tc_products(const chol_handle* h) {
+  const DeviceState* D = h->dev;
+  if (!D) return 0;
+  const bool factor = D->sg_ready == 1;
+  return (factor ? 1 : 0) | (factor && D->vs_ready == 1 ? 2 : 0) | (chol_adjoint_split(h) ? 4 : 0);
+}
 
 // Gives the workspaces back; later factorizations run on the binary64 pipe.
 void chol_sg_release(chol_handle* h) {
