@@ -111,6 +111,15 @@ def bf16_sustained_tflops():
         return BF16_SUSTAINED_TFLOPS
 
 
+def syrk_route(tc_products, achieved):
+    """(on the tensor cores, kernels, peak, rate against it) of the SYRK class that ran
+    at `achieved` binary64 GFLOP/s (or None), by the route that the handle reports."""
+    if tc_products & 1:
+        return (True, "k_sg_split_rows + k_sg_syrk", bf16_sustained_tflops() * 1e3,
+                achieved * SLICE_PRODUCTS if achieved else None)
+    return False, "k_syrk", FP64_PEAK_GFLOPS, achieved
+
+
 def max_over_ranks(dist, values, device):
     """Element-wise maximum of per-rank timings (every rank gets the result)."""
     import torch
@@ -622,11 +631,8 @@ def run_ours(args, rank, world, local_rank):
         stored_ratio = S.info.flops_stored / flops
         rc_p, dfma, dfma_ghz = P.chol_probe_fp64(0, 3)
         rc_q, dmma, dmma_ghz = P.chol_probe_fp64(1, 3)
-        tensor = achieved is not None and achieved > FP64_PEAK_GFLOPS   # else the binary64 pipe's kernel ran
-        peak = bf16_sustained_tflops() * 1e3 if tensor else FP64_PEAK_GFLOPS
-        done = achieved * SLICE_PRODUCTS if tensor else achieved
-        roof = {"bound": "tensor" if tensor else "alu",
-                "kernel": "k_sg_split_rows + k_sg_syrk" if tensor else "k_syrk",
+        tensor, kernel, peak, done = syrk_route(P.chol_get_info(S.h).tc_products, achieved)
+        roof = {"bound": "tensor" if tensor else "alu", "kernel": kernel,
                 # tensor: bf16 flops of the slice products, splitting included in the time
                 "achieved": done, "peak": peak, "unit": "GFLOP/s",
                 "frac": (done / peak) if done else None,
