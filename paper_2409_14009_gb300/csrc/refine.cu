@@ -253,7 +253,11 @@ extern "C" int chol_solve_refine(chol_handle* h, const double* b, double* x, int
   const unsigned gsp = grid1d((int64_t)n * 32, kT);
   // a warp per row wastes most lanes on rows of a few entries
   const bool few_per_row = h->csr_ptr[n] <= 16 * (int64_t)n;
-  const bool many_per_row = h->csr_ptr[n] > 256 * (int64_t)n;
+  // 8 lanes a row, or 32 for long rows (8 / 32 lanes, us, one right-hand side: 257
+  // entries in each of 30,000 rows 27 / 35, of 93,385 72 / 108; 600 in 10,000 24 / 24; 1,200
+  // in 10,000 55 / 41; 2,400 in 10,000 102 / 70. With 8 right-hand sides 8 lanes are 4 to 40%
+  // faster at all of these)
+  const bool many_per_row = h->csr_ptr[n] > 600 * (int64_t)n;
   const auto k_res = many_per_row ? k_residual<32> : k_residual<8>;
   const unsigned gres = grid1d((int64_t)n * (many_per_row ? 32 : 8), kT);
 
