@@ -841,10 +841,10 @@ void build(chol_handle* h, const int64_t* colptr, const int32_t* rowind) {
           const int32_t rows = dir ? d.s : d.len - d.s, K = dir ? d.len - d.s : d.s;
           for (int32_t r0 = 0; r0 < rows; r0 += 1 << SPLIT_ROWS_LOG2(K))
             h->vs_tasks.push_back({2 * (P.vs_b + q) + dir, r0});
-          // parts of at least 8 K blocks, two tiles an SM
+          // parts of at least 8 K blocks, at most as many as give every SM two tiles
           const int32_t nblk = (K + 31) / 32;
           const int32_t parts = (int32_t)std::max<int64_t>(
-              1, std::min<int64_t>(nblk / 8, (304 + tiles[dir] - 1) / std::max<int64_t>(tiles[dir], 1)));
+              1, std::min<int64_t>(nblk / 8, (kSolveTiles + tiles[dir] - 1) / std::max<int64_t>(tiles[dir], 1)));
           for (int32_t r0 = 0; r0 < rows; r0 += 128) {
             for (int32_t p = 0; p < parts; ++p)
               h->vs_tiles.push_back({J, r0, (int32_t)((int64_t)nblk * p / parts), (int32_t)((int64_t)nblk * (p + 1) / parts),

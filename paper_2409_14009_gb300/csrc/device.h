@@ -245,6 +245,6 @@ int chol_vs_ensure(chol_handle* h, cudaStream_t st);   // 1: available
 void chol_vs_release(chol_handle* h);
 void chol_vs_products(chol_handle* h, const LevelPlan& P, bool trans, double* Y, double* W, int nr, cudaStream_t st);
 void chol_sg_release(chol_handle* h);
-void chol_sg_trailing(chol_handle* h, const TileTask* tasks, int n, int grid, int buf, cudaStream_t st);
+void chol_sg_trailing(chol_handle* h, const TileTask* tasks, int n, int buf, cudaStream_t st);
 void chol_gather_zrr(chol_handle* h, const LevelPlan& P, const double* Z, double* ZRR, cudaStream_t st);
 void chol_sg_syrk(chol_handle* h, const LevelPlan& P, cudaStream_t st);

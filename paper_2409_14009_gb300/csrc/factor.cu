@@ -1404,13 +1404,13 @@ int enqueue_steps_sg(chol_handle* h, const LevelPlan& P, cudaStream_t st) {
     }
     if (s.sgt_near > 0) {
       KScope ks(h, CHOL_K_GEMM, ms, flops(s.sgt_near), 32.0 * kTile * kTile * s.sgt_near);
-      chol_sg_trailing(h, tiles + s.sgt_c, s.sgt_near, INT_MAX, buf, ms);
+      chol_sg_trailing(h, tiles + s.sgt_c, s.sgt_near, buf, ms);
     }
     CHOL_CUDA_TRY(cudaEventRecord(D->mev[kNear], ms));
     near_pending = true;
     if (nrest > 0) {
       KScope ks(h, CHOL_K_GEMM, ls, flops(nrest), 32.0 * kTile * kTile * nrest);
-      chol_sg_trailing(h, tiles + s.sgt_c + s.sgt_near, nrest, INT_MAX, buf, ls);
+      chol_sg_trailing(h, tiles + s.sgt_c + s.sgt_near, nrest, buf, ls);
       CHOL_CUDA_TRY(cudaEventRecord(D->lev[1], ls));
       rest_pending = true;
     }

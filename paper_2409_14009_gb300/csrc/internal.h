@@ -266,6 +266,7 @@ constexpr int kTrsmRowsHost = 32; // TRSM task height (rows; binary64 tasks take
 constexpr int kSolveSmallCols = 32;   // supernodes solved by one warp: s <= 32 and
 constexpr int kSolveSmallRows = 256;  // len <= 256
 constexpr int kSplitTasks = 608;      // binary64 solve panel products: split levels with fewer tasks (4 x 152 SMs)
+constexpr int kSolveTiles = 304;      // ... on the tensor cores: levels with fewer tiles (2 x 152 SMs)
 constexpr int kMaxSplit = 16;         // ... into at most this many parts
 constexpr int kSplitMin = 128;        // ... of at least this many columns (gemv) or rows (bpanel)
 constexpr int kRlbSmallRows = 1024;   // RLB: rows of a supernode on the one-CTA kernel (small_max_rows cap)

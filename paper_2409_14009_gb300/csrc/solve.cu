@@ -850,7 +850,7 @@ __device__ __forceinline__ unsigned group_mask() {
 }
 
 template <class T>
-__device__ __forceinline__ T pivot_recip(const T* __restrict__ P, const SnodeDev& d, int i, bool rm,
+__device__ __forceinline__ T pivot_recip(const T* __restrict__ P, const SnodeDev& d, int i,
                                          const double* __restrict__ rdiag) {
   if constexpr (sizeof(T) == 8) return rdiag[d.f + i];
   else return T(1) / P[(int64_t)i * d.ld + i];
@@ -869,7 +869,7 @@ k_sv_small_fwd(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list
   const int b = d.len - d.s;
   T* Wj = W + d.wpre * nrhs;
   constexpr bool kScaled = sizeof(T) == 8;
-  const T rd = g < d.s ? pivot_recip<T>(P, d, g, RM, rdiag) : T(0);
+  const T rd = g < d.s ? pivot_recip<T>(P, d, g, rdiag) : T(0);
   T lrow[G];   // L(g, k) (binary64: / L(g, g)), k < g < s, else 0
 #pragma unroll
   for (int k = 0; k < G; ++k) lrow[k] = (k < g && g < d.s) ? lval<T, RM>(P, d, g, k) * (kScaled ? rd : T(1)) : T(0);
@@ -912,7 +912,7 @@ k_sv_small_bwd(const SnodeDev* __restrict__ sn, const int32_t* __restrict__ list
   const int b = d.len - d.s;
   const int32_t* rj = rows + d.roff + d.s;
   constexpr bool kScaled = sizeof(T) == 8;
-  const T rd = g < d.s ? pivot_recip<T>(P, d, g, RM, rdiag) : T(0);
+  const T rd = g < d.s ? pivot_recip<T>(P, d, g, rdiag) : T(0);
   T lcol[G];   // L(k, g) (binary64: / L(g, g)), g < k < s, else 0
 #pragma unroll
   for (int k = 0; k < G; ++k) lcol[k] = (k > g && k < d.s) ? lval<T, RM>(P, d, k, g) * (kScaled ? rd : T(1)) : T(0);

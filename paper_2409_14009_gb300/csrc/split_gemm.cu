@@ -65,17 +65,16 @@ __device__ __forceinline__ uint32_t smem_base(const unsigned char* p) { return (
 // K = 64, one chunk per tile. The thread's entries of C are loaded before the wait for the products.
 __global__ void __launch_bounds__(sg::kThreads, 1)
 k_sg_trailing(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, const TileTask* __restrict__ tasks,
-              int ntasks, const unsigned char* __restrict__ slab, const int32_t* __restrict__ exps,
+              const unsigned char* __restrict__ slab, const int32_t* __restrict__ exps,
               double* __restrict__ L, sg::Waits waits) {
   extern __shared__ unsigned char sg_smem[];
   __shared__ __align__(8) sg::Shared S;
   const uint32_t base = smem_base(sg_smem);
   const uint32_t tmem = sg::setup(S);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  auto next = [&](int i, sg::Tile& t) {
-    const int64_t q = blockIdx.x + (int64_t)i * gridDim.x;
-    if (q >= ntasks) return false;
-    const TileTask k = tasks[q];
+  auto next = [&](int i, sg::Tile& t) {   // one tile a CTA
+    if (i > 0) return false;
+    const TileTask k = tasks[blockIdx.x];
     const SplitDev z = sd[k.J];
     t.a = {slab + z.toff * 64, exps + z.trow0, z.trows, k.r0};
     t.b = {slab + z.toff * 64, exps + z.trow0, z.trows, k.c0};
@@ -88,21 +87,21 @@ k_sg_trailing(const SnodeDev* __restrict__ sn, const SplitDev* __restrict__ sd, 
     if (lane == 0) sg::mma_loop(S, base, tmem, next, waits);
   } else {
     sg::Tile t;
-    for (int i = 0; next(i, t); ++i) {
-      const TileTask k = tasks[blockIdx.x + (int64_t)i * gridDim.x];
-      const SnodeDev d = sn[k.J];
-      const int r = k.r0 + sg::epi_row(), c0 = k.c0 + sg::epi_col();
-      // the thread's columns c0 .. c0 + n - 1 (on or below the diagonal)
-      const int n = r < min(d.len, k.r0 + k.k0) ? min(sg::kCols, min(d.s, r + 1) - c0) : 0;
-      const int32_t ea = n > 0 ? t.a.exps[r] : 0;
-      double* C = L + d.loff + r + (int64_t)c0 * d.ld;
-      double cv[sg::kCols];
+    next(0, t);
+    const TileTask k = tasks[blockIdx.x];
+    const SnodeDev d = sn[k.J];
+    const int r = k.r0 + sg::epi_row(), c0 = k.c0 + sg::epi_col();
+    // the thread's columns c0 .. c0 + n - 1 (on or below the diagonal)
+    const int n = r < min(d.len, k.r0 + k.k0) ? min(sg::kCols, min(d.s, r + 1) - c0) : 0;
+    const int32_t ea = n > 0 ? t.a.exps[r] : 0;
+    double* C = L + d.loff + r + (int64_t)c0 * d.ld;
+    double cv[sg::kCols];
 #pragma unroll
-      for (int c = 0; c < sg::kCols; ++c) cv[c] = c < n ? C[(int64_t)c * d.ld] : 0.0;
-      long long hi[sg::kCols], lo[sg::kCols];
+    for (int c = 0; c < sg::kCols; ++c) cv[c] = c < n ? C[(int64_t)c * d.ld] : 0.0;
+    long long hi[sg::kCols], lo[sg::kCols];
 #pragma unroll
-      for (int c = 0; c < sg::kCols; ++c) hi[c] = lo[c] = 0;
-      if (!sg::drain(S, tmem, i, hi, lo, waits)) break;
+    for (int c = 0; c < sg::kCols; ++c) hi[c] = lo[c] = 0;
+    if (sg::drain(S, tmem, 0, hi, lo, waits)) {
 #pragma unroll
       for (int c = 0; c < sg::kCols; ++c)
         if (c < n) C[(int64_t)c * d.ld] = cv[c] - sg::combine(hi[c], lo[c], ea, t.b.exps[c0 + c]);
@@ -270,12 +269,12 @@ int chol_sg_ensure(chol_handle* h) {
   return CHOL_OK;
 }
 
-// Trailing tiles from the slices in buffer `buf` (written by k_trsm).
-void chol_sg_trailing(chol_handle* h, const TileTask* tasks, int n, int grid, int buf, cudaStream_t st) {
+// n > 0 trailing tiles from the slices in buffer `buf` (written by k_trsm).
+void chol_sg_trailing(chol_handle* h, const TileTask* tasks, int n, int buf, cudaStream_t st) {
   DeviceState* D = h->dev;
-  k_sg_trailing<<<std::min(n, grid), sg::kThreads, sg::kSmemBytes, st>>>(D->sn, D->sg_dev, tasks, n, D->sgt_slab[buf],
-                                                                        D->sgt_exps[buf], D->L,
-                                                                        sg::Waits{D->sg_err, chol_test_wait(h, kTestWaitFactor)});
+  const sg::Waits waits{D->sg_err, chol_test_wait(h, kTestWaitFactor)};
+  k_sg_trailing<<<n, sg::kThreads, sg::kSmemBytes, st>>>(D->sn, D->sg_dev, tasks, D->sgt_slab[buf], D->sgt_exps[buf], D->L,
+                                                         waits);
 }
 
 // U_J of every blocked supernode of a level (RLB: subtracted from the ancestors).
