@@ -1747,7 +1747,8 @@ int chol_finish_factor(chol_handle* h, cudaStream_t st) {
   }
 #endif
   const int32_t s = D->status_host[0];
-  if (s != INT_MAX) return s;
+  // after a lost wait of a product a bad pivot says nothing about the matrix
+  if (s != INT_MAX && !D->status_host[2]) return s;
   if (h->opt.precision != CHOL_PREC_FP64) {
     const int rc = chol_tc_status(h);
     if (rc) return rc;
