@@ -6,7 +6,7 @@ grid (n = 262,144), conductances log-uniform in [1e-2, 1e2], diagonal = incident
 sum + 1e-6, geometric nested-dissection ordering; FP64 factor + solve with 8
 right-hand sides U(-1, 1). One step = value scatter + numeric factorization +
 8-RHS forward/backward solve + logdet, inputs resident in HBM (the factor panels,
-1.4 GB, exceed the 129 MB L2, so no flush is needed between steps).
+1.65 GB, exceed the 129 MB L2, so no flush is needed between steps).
 
 value = symbolic factor flops (sum_j c_j^2) / step time, summed over ranks
 (independent replicas: the single factorization does not shard).
@@ -676,7 +676,7 @@ def run_ours(args, rank, world, local_rank):
                            "merge_growth": args.merge, "supernodes": S.info.nsuper_storage,
                            "flops_stored_over_symbolic": S.info.flops_stored / flops,
                            "parallelism": "replicas" if world > 1 else "single",
-                           "l2": "inputs larger than L2 (panels 1.4 GB)"},
+                           "l2": "inputs larger than L2 (panels 1.65 GB)"},
                 "analyze_ms": analyze_ms, "factor_ms": factor_ms, "solve_ms": solve_ms,
                 "factor_gflops": flops / (factor_ms * 1e-3) / 1e9, "flops": flops,
                 "backward_error": float(eta), "logdet": ld[0],
