@@ -329,7 +329,7 @@ int chol_solve_refine(chol_handle* h, const double* b, double* x, int32_t nrhs, 
  * through the relative positions, Z_JJ = T^T T - Uhat^T Z_RJ). The first call
  * builds the level plan and its workspaces (largest level's sum of s^2,
  * b s and s^2 / 2 doubles, and the slices of its largest group of products, which
- * run on the tensor cores where chol_factor's do). CHOL_PREC_FP64 handles only (else CHOL_ENOTSUP).
+ * run on the tensor cores where chol_factor's do, with the same accuracy). CHOL_PREC_FP64 handles only (else CHOL_ENOTSUP).
  * A call captured in a CUDA graph (after a plain one, which builds the plan) computes
  * at each of the graph's replays, from the factor of that moment. Asynchronous.
  */
