@@ -20,7 +20,8 @@
 // So an entry's error is its one rounding plus about sqrt(K) 2^-62, at most about
 // K 2^-60 (equal entries), times the product of the two rows' largest entries.
 // Normwise that is less than the error of K binary64 FMAs (K 2^-53), and it does
-// not change when rows are scaled by powers of two. It is not relative to the sum's
+// not change when rows are scaled by powers of two (nor does the result, but for
+// last bits where the rows' exponents add to more than 900). It is not relative to the sum's
 // own terms, as the FMAs' is: an entry below 2^-10 of its row's largest keeps fewer
 // than 53 bits and one below 2^-63 none, so where every large entry of one row
 // meets a small one of the other (graded rows), the result has fewer correct
